@@ -31,7 +31,7 @@
 #include <mutex>
 #include <vector>
 
-#include "bdc_internal.cuh"
+#include "bdc_dense.cuh"
 
 namespace bdc {
 
@@ -211,19 +211,6 @@ cudaError_t dgemm(int ta, int tb, int M, int N, int K, double alpha, const doubl
 }
 
 // ------------------------------------------------------------ grid barrier
-struct GridBar {
-    unsigned count, gen;
-    int err;
-    int pad;
-};
-constexpr unsigned long long kBarNs = 2000000000ull;
-
-__device__ __forceinline__ unsigned long long gtime() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // all CTAs of a cooperative launch; false (and the error word set) when the
 // wait gave up or another CTA gave up before
 __device__ bool grid_sync(GridBar *gb) {
@@ -713,7 +700,7 @@ int coop_blocks(const void *fn, int threads, size_t smem) {
 
 // workspace layout of the dense routines (bytes from an aligned base)
 struct DenseWs {
-    size_t bar, PW, QW, yraw, tv, xpart, part, Y, Ti, Z, split, split_doubles, total;
+    size_t bar, PW, QW, yraw, tv, xpart, part, Y, Ti, Z, split, split_doubles, res, total;
 };
 constexpr int kChunkW = 128;   // columns per partial sum of A u
 
@@ -734,6 +721,7 @@ DenseWs dense_ws(int m, int n, int b, int zcols) {
     w.Z = o; o += al256(sizeof(double) * (size_t)b * std::max(std::max(m, n), zcols));
     w.split_doubles = (size_t)16 * b * std::max(std::max(m, n), zcols);
     w.split = o; o += al256(sizeof(double) * w.split_doubles);
+    w.res = o; o += al256(sizeof(double) * resident_scratch_doubles(n));
     w.total = o + 256;
     return w;
 }
@@ -767,14 +755,18 @@ cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, 
     const DenseWs w = dense_ws(m, n, b, n);
     SplitScope split_scope(ws, w);
     GridBar *bar = (GridBar *)(ws + w.bar);
-    cudaError_t err = cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), st);   // count, gen (not the error word)
+    cudaError_t err = cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st);   // the counters (not the error word)
     if (err != cudaSuccess) return err;
     // CTAs per panel by the work of its steps (the products with the
     // trailing matrix, ~ml nl FMAs): a small trailing matrix cannot use the
     // whole GPU, and every barrier costs more with more CTAs
     const int gmax = std::min(coop_blocks((const void *)k_labrd, 256, 0), 4 * 256);
+    unsigned bars = 0;
     for (int i0 = 0; i0 < n; i0 += b) {
         const int nb = std::min(b, n - i0), ml = m - i0, nl = n - i0;
+        if (resident_fits(ml, nl))
+            return launch_gebd2_resident(ml, nl, A + i0 + (size_t)i0 * lda, lda, d + i0, e + i0, tauq + i0, taup + i0,
+                                         (double *)(ws + w.res), bar, &bars, st);
         const int grid = (int)std::max<long long>(8, std::min<long long>(gmax, (long long)ml * nl / kLabrdWork));
         LabrdArgs a{A + i0 + (size_t)i0 * lda, lda, ml, nl, nb, b,
                     d + i0, e + i0, tauq + i0, taup + i0,
@@ -802,7 +794,7 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
     const DenseWs w = dense_ws(m, n, b, n);
     SplitScope split_scope(ws, w);
     GridBar *bar = (GridBar *)(ws + w.bar);
-    cudaError_t err = cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), st);   // count, gen (not the error word)
+    cudaError_t err = cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st);   // the counters (not the error word)
     if (err != cudaSuccess) return err;
     // enough CTAs for ~4 panel rows per thread: the per-column reductions over
     // the CTAs' partial sums grow with the grid

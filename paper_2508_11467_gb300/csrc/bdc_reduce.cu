@@ -1,0 +1,580 @@
+// Bidiagonalization of a matrix held on chip (Sec. 4.1, FP64).
+//
+// The blocked reduction (bdc_dense.cu) passes over the trailing matrix twice
+// per column step and separates its phases by grid barriers.  When the matrix
+// fits the SMs' shared memory (about 30 MB on 152 SMs) k_gebd2_resident loads
+// it once, keeps a set of rows per CTA, applies every reflector pair at once
+// (no panels V, X, Y, U, no trailing product) and needs two barriers a step.
+#include <algorithm>
+#include <mutex>
+#include <type_traits>
+
+#include "bdc_dense.cuh"
+
+namespace bdc {
+
+namespace {
+
+// All CTAs of a cooperative launch wait until `target` arrivals have been
+// counted (a counter that only grows: no reset, no generation).  One thread
+// arrives with release order and polls with acquire order.  The wait is
+// bounded (kBarNs); false when it gave up here or elsewhere.
+__device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned v;
+        int ok = 1;
+        __threadfence();
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gb->mono) : "memory");
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&gb->mono) : "memory");
+        if ((int)(v - target) < 0) {
+            const unsigned long long t0 = gtime();
+            unsigned spins = 0;
+            do {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&gb->mono) : "memory");
+                if ((++spins & 255u) == 0) {
+                    if (*(volatile int *)&gb->err) { ok = 0; break; }
+                    if (gtime() - t0 > kBarNs) {
+                        atomicExch(&gb->err, 1);
+                        ok = 0;
+                        break;
+                    }
+                }
+            } while ((int)(v - target) < 0);
+        }
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// Householder reflector from alpha and ||x_2..||^2 = sig2 (LAPACK's sign
+// convention): beta = -sign(alpha) ||x||, tau = (beta - alpha) / beta, the
+// vector's tail scaled by 1 / (alpha - beta); sig2 = 0 gives tau = 0 (H = I).
+// On the critical path of every step, and every FP64 instruction of a warp
+// takes 64 cycles here: 12 of them instead of the about 40 of a library
+// square root and two divisions (a step at n = 64: 2 x 2300 -> 2 x 1450 cycles
+// in this part).  With y
+// the hardware estimate of 1 / sqrt(s) (20 bits) and r = 1 - s y^2, the
+// series sqrt(s) = s y (1 - r)^(-1/2) = s y (1 + r/2 + 3 r^2/8 + O(r^3))
+// leaves 2^-58; 1 / sqrt(s) is the same series on y, and 1 / (alpha - beta)
+// the geometric series of quot().  Outside 2^-900..2^900 the library calls.
+__device__ __forceinline__ double reflector_fast(double alpha, double sig2, double &tau, double &beta) {
+    if (__double_as_longlong(sig2) == 0) {
+        tau = 0.0;
+        beta = alpha;
+        return 0.0;
+    }
+    const double s = fma(alpha, alpha, sig2);
+    const long long sb = __double_as_longlong(s);
+    const bool neg = __double_as_longlong(alpha) < 0;      // (alpha = -0 reflects to +||x||)
+    if (sb < (123ll << 52) || sb > (1923ll << 52)) {       // also NaN, infinity
+        const double nrm = sqrt(s);
+        beta = neg ? nrm : -nrm;
+        tau = (beta - alpha) / beta;
+        return 1.0 / (alpha - beta);
+    }
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
+    const double g = s * y;
+    const double r = fma(-g, y, 1.0);
+    const double q = fma(0.375, r, 0.5) * r;
+    const double nrm = fma(g, q, g);
+    beta = neg ? nrm : -nrm;
+    const double D = alpha - beta;                          // no cancellation: the signs differ
+    tau = fabs(D) * fma(y, q, y);
+    double z;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(D));
+    const double e = fma(-D, z, 1.0);
+    return fma(z, fma(e, e, e), z);
+}
+
+// ---- exchange between CTAs without barriers
+// A slot is 16 bytes: the two halves of a double, each beside the step
+// number that wrote it, so that a reader that polls a slot knows from the
+// slot itself when the value is there: no fence and no counter (333 x 333:
+// 3.64 ms with two grid barriers a step and plain loads behind them, 3.00 ms
+// with slots; 1000 x 1000: 15.5 and 11.5 ms, the row passes included).  Each
+// 8-byte half is written and read as one access.
+typedef ulonglong2 Slot;
+
+__device__ __forceinline__ void slot_put(Slot *p, double v, unsigned tag) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"((b & 0xffffffffull) | t),
+                 "l"((b >> 32) | t)
+                 : "memory");
+}
+
+__device__ __forceinline__ Slot slot_load(const Slot *p) {
+    Slot s;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(s.x), "=l"(s.y) : "l"(p) : "memory");
+    return s;
+}
+
+// K slots at once (all loads in flight together; p[k] may repeat), polled
+// until each carries `tag`.  Bounded: after kBarNs, or when another wait of
+// the grid gave up, sets the error word and *s_err and returns.
+template <int K>
+__device__ __forceinline__ void slot_get(const Slot *(&p)[K], unsigned tag, double (&v)[K], GridBar *gb,
+                                         int *s_err) {
+    unsigned spins = 0;
+    unsigned long long t0 = 0;
+    for (;;) {
+        Slot s[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) s[k] = slot_load(p[k]);
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            ok = ok && (unsigned)(s[k].x >> 32) == tag && (unsigned)(s[k].y >> 32) == tag;
+            v[k] = __longlong_as_double((long long)((s[k].x & 0xffffffffull) | (s[k].y << 32)));
+        }
+        if (ok) return;
+        if ((++spins & 127u) == 0) {
+            if (t0 == 0) t0 = gtime();
+            if (*(volatile int *)&gb->err || gtime() - t0 > kBarNs) {
+                atomicExch(&gb->err, 1);
+                *(volatile int *)s_err = 1;
+                return;
+            }
+        }
+    }
+}
+
+constexpr int NT = 128;            // threads per CTA: one warp per SM sub-partition
+constexpr int kRedLd = NT + 8;     // row stride of the reduction buffer
+constexpr int LR = 8;              // rows of a CTA handled together
+
+// f(integral_constant<K>) for K = k in 1..LR: straight-line code per row
+// count, so that the loads, FMAs and stores of all rows are scheduled
+// together (one warp per scheduler: nothing else hides a latency; with a
+// test per row the passes ran at a third of this rate)
+template <int LR, typename F>
+__device__ __forceinline__ void rows_dispatch(int k, F f) {
+    if constexpr (LR >= 1) {
+        if (k == LR) f(std::integral_constant<int, LR>{});
+        else rows_dispatch<LR - 1>(k, f);
+    }
+}
+
+// A -= v y^T on K rows and this thread's columns i + 1.., red[q][t] = this
+// thread's part of A r over the columns i + 2..
+template <int K>
+__device__ __forceinline__ void pass_left(double *W, int ldw, const double *vv, const double *sy, const double *sr,
+                                          int i, int n, int t, double *red) {
+    double acc[K], v[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        acc[q] = 0.0;
+        v[q] = -vv[q];
+    }
+    int c = i + 1 + t;
+    if constexpr (K <= 4) {     // two columns at once
+        for (; c + NT < n; c += 2 * NT) {
+            const double y0 = sy[c], y1 = sy[c + NT], r0 = (c > i + 1) ? sr[c] : 0.0, r1 = sr[c + NT];
+            double x[K], z[K];
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                x[q] = W[(size_t)q * ldw + c];
+                z[q] = W[(size_t)q * ldw + c + NT];
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                x[q] = fma(v[q], y0, x[q]);
+                z[q] = fma(v[q], y1, z[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) acc[q] = fma(x[q], r0, acc[q]);
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                W[(size_t)q * ldw + c] = x[q];
+                W[(size_t)q * ldw + c + NT] = z[q];
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) acc[q] = fma(z[q], r1, acc[q]);
+        }
+    }
+    for (; c < n; c += NT) {
+        const double y0 = sy[c], r0 = (c > i + 1) ? sr[c] : 0.0;
+        double x[K];
+#pragma unroll
+        for (int q = 0; q < K; ++q) x[q] = W[(size_t)q * ldw + c];
+#pragma unroll
+        for (int q = 0; q < K; ++q) x[q] = fma(v[q], y0, x[q]);
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            W[(size_t)q * ldw + c] = x[q];
+            acc[q] = fma(x[q], r0, acc[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < K; ++q) red[q * kRedLd + t] = acc[q];
+}
+
+// A -= x u^T on K rows and this thread's columns, su[c] = u_c; sums of A^T a
+// over the rows: from 0 (first) or sum[c], into sum[c] or (gp) the slots
+template <int K>
+__device__ __forceinline__ void pass_right(double *W, int ldw, const double *xv, const double *av, const double *su,
+                                           double *sum, bool first, Slot *gp, int i, int n, int t,
+                                           unsigned tag) {
+    double xr[K], ar[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        xr[q] = -xv[q];
+        ar[q] = av[q];
+    }
+    int c = i + 1 + t;
+    if constexpr (K <= 4) {
+        for (; c + NT < n; c += 2 * NT) {
+            const double u0 = su[c], u1 = su[c + NT];
+            double x[K], z[K];
+            double s0 = first ? 0.0 : sum[c], s1 = first ? 0.0 : sum[c + NT];
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                x[q] = W[(size_t)q * ldw + c];
+                z[q] = W[(size_t)q * ldw + c + NT];
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                x[q] = fma(xr[q], u0, x[q]);
+                z[q] = fma(xr[q], u1, z[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                s0 = fma(ar[q], x[q], s0);
+                s1 = fma(ar[q], z[q], s1);
+            }
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                W[(size_t)q * ldw + c] = x[q];
+                W[(size_t)q * ldw + c + NT] = z[q];
+            }
+            if (gp) {
+                slot_put(gp + c, s0, tag);
+                slot_put(gp + c + NT, s1, tag);
+            } else {
+                sum[c] = s0;
+                sum[c + NT] = s1;
+            }
+        }
+    }
+    for (; c < n; c += NT) {
+        const double u0 = su[c];
+        double x[K];
+        double s0 = first ? 0.0 : sum[c];
+#pragma unroll
+        for (int q = 0; q < K; ++q) x[q] = W[(size_t)q * ldw + c];
+#pragma unroll
+        for (int q = 0; q < K; ++q) x[q] = fma(xr[q], u0, x[q]);
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            W[(size_t)q * ldw + c] = x[q];
+            s0 = fma(ar[q], x[q], s0);
+        }
+        if (gp) slot_put(gp + c, s0, tag);
+        else sum[c] = s0;
+    }
+}
+
+struct Gebd2Args {
+    double *A;
+    int lda, m, n;
+    double *d, *e, *tauq, *taup;
+    Slot *gp;                      // [grid][n]: per-CTA partial sums of A^T a (column i: of a^T a)
+    Slot *row, *yr, *scal;         // [n] top row; [2 n] y and row i after H_i; [1] column scale
+    GridBar *bar;
+    unsigned base;                 // arrivals before this launch
+};
+
+// CTA g holds rows g, g + G, g + 2G, ... (cyclic: the rows that drop out
+// step by step leave every CTA with the same share) in shared memory, row
+// major.  With a = column i of the current matrix, step i is
+//   Y phase (a block of columns per CTA): g_c = sum over CTAs of A[:, c]^T a
+//     (tail rows), sig2 = the same for a itself -> H_i's scalars (every CTA
+//     forms them), y_c = tau (A[i, c] + sc g_c), row i: r_c = A[i, c] - y_c
+//   X phase (own rows): v = sc a; one pass A -= v y^T with h = A r; block
+//     reduction of h and ||r||^2 -> G_i's scalars; x = pi A u with u = [1;
+//     scr r]; next column a' = A[:, i+1] - x; one pass A -= x u^T with the
+//     partial sums of A^T a' and a'^T a' for step i + 1, and the next top row
+// The products are taken with the unscaled a and r, so that no phase waits
+// for a norm.  Four FMAs per entry and step; FP64 runs at two lanes per
+// clock and SM, so four warps fill the pipe and the block reduction (one add
+// per thread and row) is kept small by them.  The phases exchange their
+// vectors through slots (above).  One buffer of each is enough: a CTA writes
+// its sums of step i + 1 after it has the y of every column of step i, which
+// their owners sent after reading all sums of step i; and an owner sends
+// step i + 1's y after the sums of every CTA, which each sent after reading
+// all of step i's y.
+// What bounds it: the two exchanges (about 4500 cycles each) and the
+// dependent FP64 chains of a step (64 cycles an operation), above n ~ 1000
+// the FP64 pipe.  333 x 333: 18.9 ms (k_labrd's seven barriers a step) ->
+// 3.0 ms; 1000 x 1000: 71 -> 11.5 ms; 1500 x 1100: 82 -> 16.5 ms.
+__global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
+    extern __shared__ double smem[];
+    __shared__ int s_err;
+    const int G = gridDim.x, g = blockIdx.x, t = threadIdx.x;
+    const int m = a.m, n = a.n, ldw = a.n;
+    const int lr = (m - g + G - 1) / G;             // own rows (g < G <= m)
+    const int lrmax = (m + G - 1) / G;
+    double *W = smem;                               // [lr][ldw]
+    double *sy = W + (size_t)lrmax * ldw;           // this thread's columns of y, r (written and read by one thread)
+    double *sr = sy + ldw;
+    double *red = sr + ldw;                         // [LR + 1][kRedLd]
+    double *av = red + (LR + 1) * kRedLd;           // [lrmax] a, x, v of the own rows; h sums
+    double *xv = av + lrmax, *vv = xv + lrmax, *hs = vv + lrmax;
+    double *A = a.A;
+    const size_t lda = a.lda;
+
+    if (t == 0) s_err = 0;
+    for (int c = t; c < n; c += NT)
+        for (int l = 0; l < lr; ++l) W[(size_t)l * ldw + c] = A[(size_t)c * lda + g + (size_t)G * l];
+    // clear the slots' step numbers
+    const Slot zero = {0ull, 0ull};
+    for (int c = t; c < n; c += NT) a.gp[(size_t)g * ldw + c] = zero;
+    for (int c = g * NT + t; c < n; c += G * NT) a.row[c] = a.yr[2 * c] = a.yr[2 * c + 1] = zero;
+    if (g == 0 && t == 0) a.scal[0] = zero;
+    if (!grid_wait(a.bar, a.base + G)) return;
+    for (int l = t; l < lr; l += NT) av[l] = W[(size_t)l * ldw];
+    __syncthreads();
+    for (int c = t; c < n; c += NT) {               // sums of step 0
+        double s = 0.0;
+        for (int l = (g == 0); l < lr; ++l) s = fma(av[l], W[(size_t)l * ldw + c], s);
+        if (g == 0) slot_put(a.row + c, W[c], 1u);
+        slot_put(a.gp + (size_t)g * ldw + c, s, 1u);
+    }
+
+    for (int i = 0; i < n; ++i) {
+        const unsigned tag = (unsigned)i + 1u;
+        // ---- Y phase
+        const int ncol = n - 1 - i, cb = (ncol + G - 1) / G;
+        const int c0 = i + 1 + g * cb, nc = max(0, min(cb, n - c0));
+        if (nc > 0 || g == 0) {
+            // sums over the CTAs of nc columns and of column i (slot nc)
+            const int slots = nc + 1;
+            int sp = 1;
+            while (sp < slots) sp <<= 1;            // slots per pass (power of two, at most 32)
+            if (sp > 32) sp = 32;
+            const int sub = t / sp, subs = NT / sp;
+            double alpha = 0.0, top = 0.0, tau, beta;
+            for (int s0 = 0; s0 < slots; s0 += sp) {
+                const int s = s0 + (t & (sp - 1));
+                double v0 = 0.0;
+                // eight CTAs' slots per round (one round for most sizes); the
+                // first round also takes alpha and this thread's top-row entry
+                const Slot *p = a.gp + (s < nc ? c0 + s : i);
+                for (int k = sub; k < G; k += 8 * subs) {
+                    const Slot *q[10];
+                    double v[10];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) q[j] = p + (size_t)(k + j * subs < G ? k + j * subs : k) * ldw;
+                    q[8] = a.row + i;
+                    q[9] = a.row + (t < nc ? c0 + t : i);
+                    slot_get<10>(q, tag, v, a.bar, &s_err);
+                    alpha = v[8];
+                    top = v[9];
+                    v0 += v[0];
+#pragma unroll
+                    for (int j = 1; j < 8; ++j)
+                        if (k + j * subs < G) v0 += v[j];
+                }
+                for (int o = sp; o < 32; o <<= 1) v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+                if (s0 > 0) __syncthreads();
+                if ((t & 31) < sp) red[(t >> 5) * 32 + (t & 31)] = v0;
+                __syncthreads();
+                if (slots > sp && t < sp && s0 + t < slots)
+                    sy[s0 + t] = (red[t] + red[32 + t]) + (red[64 + t] + red[96 + t]);
+            }
+            const bool one = slots <= sp;
+            if (!one) __syncthreads();
+            const double sig2 = one ? (red[nc] + red[32 + nc]) + (red[64 + nc] + red[96 + nc]) : sy[nc];
+            const double sc = reflector_fast(alpha, sig2, tau, beta);
+            for (int q = t; q < nc; q += NT) {
+                const int c = c0 + q;
+                double rw = top;
+                if (q != t) {
+                    const Slot *z[1] = {a.row + c};
+                    double v[1];
+                    slot_get<1>(z, tag, v, a.bar, &s_err);
+                    rw = v[0];
+                }
+                const double gs = one ? (red[q] + red[32 + q]) + (red[64 + q] + red[96 + q]) : sy[q];
+                const double y = tau * fma(sc, gs, rw);
+                slot_put(a.yr + 2 * c, y, tag);
+                slot_put(a.yr + 2 * c + 1, rw - y, tag);
+            }
+            if (g == 0 && t == 0) {
+                slot_put(a.scal, sc, tag);
+                a.d[i] = beta;
+                a.tauq[i] = tau;
+                A[(size_t)i * lda + i] = beta;
+            }
+            __syncthreads();                        // red, sy are reused below
+        }
+        // ---- X phase
+        const int l0 = (i < g) ? 0 : (i - g) / G + 1;   // first own row below i
+        const bool more = i + 1 < n;
+        double sc = 0.0, alr = 0.0;
+        {   // wait on one slot per thread, so that the waiting CTAs do not load L2 with all of theirs
+            const Slot *q[1] = {i + 1 + t < n ? a.yr + 2 * (i + 1 + t) + 1 : a.scal};
+            double v[1];
+            slot_get<1>(q, tag, v, a.bar, &s_err);
+        }
+        for (int c = i + 1 + t, first = 1; first || c < n; c += 4 * NT, first = 0) {
+            // four columns of y and r per round; every round also has the scale and r's first entry
+            const Slot *q[10];
+            double v[10];
+            q[8] = a.scal;
+            q[9] = more ? a.yr + 2 * (i + 1) + 1 : a.scal;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                q[2 * j] = c + j * NT < n ? a.yr + 2 * (c + j * NT) : q[9];
+                q[2 * j + 1] = c + j * NT < n ? a.yr + 2 * (c + j * NT) + 1 : q[9];
+            }
+            slot_get<10>(q, tag, v, a.bar, &s_err);
+            sc = v[8];
+            alr = v[9];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c + j * NT < n) {
+                    sy[c + j * NT] = v[2 * j];
+                    sr[c + j * NT] = v[2 * j + 1];
+                }
+        }
+        for (int l = l0 + t; l < lr; l += NT) {
+            const double v = sc * av[l];
+            vv[l] = v;
+            A[(size_t)i * lda + g + (size_t)G * l] = v;
+        }
+        __syncthreads();
+        if (s_err || !more) return;                 // a wait gave up (uniform: read after the barrier), or done
+        // A -= v y^T with the products h = A r (the tail of row i: columns
+        // i + 2...) in chunks of LR rows; slot LR of the last chunk: ||r||^2
+        double pi, betr;
+        for (int b0 = l0;; b0 += LR) {
+            const int nq = max(0, min(LR, lr - b0));    // rows of this chunk
+            const bool lastc = b0 + LR >= lr;
+            double nrm = 0.0;                           // slot nq of the reduction: ||r||^2 (last chunk)
+            if (lastc)
+                for (int c = i + 1 + t; c < n; c += NT) {
+                    const double rt = (c > i + 1) ? sr[c] : 0.0;
+                    nrm = fma(rt, rt, nrm);
+                }
+            red[nq * kRedLd + t] = nrm;
+            rows_dispatch<LR>(nq, [&](auto K) {
+                pass_left<decltype(K)::value>(W + (size_t)b0 * ldw, ldw, vv + b0, sy, sr, i, n, t, red);
+            });
+            __syncthreads();
+            // block reduction: P lanes per row (all the rows at once)
+            const int rows = nq + 1;
+            const int P = rows <= 4 ? 32 : rows <= 8 ? 16 : 8;
+            {
+                const int q = t / P, p = t & (P - 1);
+                double s0 = 0.0;
+                if (q < rows) {
+                    s0 = red[q * kRedLd + p];
+                    for (int k = p + P; k < NT; k += P) s0 += red[q * kRedLd + k];
+                }
+                for (int o = P >> 1; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+                if (q < rows && p == 0) hs[q == nq ? lrmax : b0 + q] = s0;
+            }
+            __syncthreads();
+            if (lastc) break;
+        }
+        const double scr = reflector_fast(alr, hs[lrmax], pi, betr);
+        for (int l = l0 + t; l < lr; l += NT) {
+            const double w = W[(size_t)l * ldw + i + 1];
+            const double x = pi * fma(scr, hs[l], w);
+            xv[l] = x;
+            av[l] = w - x;
+        }
+        if (g == 0 && t == 0) {
+            a.e[i] = betr;
+            a.taup[i] = pi;
+            A[(size_t)(i + 1) * lda + i] = betr;
+        }
+        __syncthreads();
+        // A -= x u^T, the partial sums of the next step, its top row
+        const bool topmine = l0 < lr && g + G * l0 == i + 1;
+        const int l1 = l0 + (topmine ? 1 : 0);
+        double *ug = g == i % G ? A + i : nullptr;       // this CTA stores row i's reflector
+        const double xt = topmine ? xv[l0] : 0.0;
+        for (int c = i + 1 + t; c < n; c += NT) {
+            const double u = (c == i + 1) ? 1.0 : scr * sr[c];
+            if (ug && c > i + 1) ug[(size_t)c * lda] = u;
+            if (topmine) slot_put(a.row + c, fma(-xt, u, W[(size_t)l0 * ldw + c]), tag + 1u);
+            sr[c] = u;
+            if (l1 >= lr) slot_put(a.gp + (size_t)g * ldw + c, 0.0, tag + 1u);
+        }
+        for (int b0 = l1; b0 < lr; b0 += LR) {
+            const int nq = min(LR, lr - b0);
+            Slot *gp = b0 + LR >= lr ? a.gp + (size_t)g * ldw : nullptr;
+            rows_dispatch<LR>(nq, [&](auto K) {
+                pass_right<decltype(K)::value>(W + (size_t)b0 * ldw, ldw, xv + b0, av + b0, sr, sy, b0 == l1, gp, i, n,
+                                               t, tag + 1u);
+            });
+        }
+    }
+}
+
+// shared memory of a grid of G CTAs (bytes)
+size_t res_smem(int m, int n, int G) {
+    const size_t lr = (m + G - 1) / G, ldw = n;
+    return sizeof(double) * (lr * ldw + 2 * ldw + (size_t)(LR + 1) * kRedLd + 4 * lr + 2);
+}
+
+struct DevInfo {
+    int sms = 0, smem = 0;
+};
+DevInfo dev_info() {
+    static std::mutex mu;
+    static DevInfo cache[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return {};
+    std::lock_guard<std::mutex> lk(mu);
+    DevInfo &d = cache[dev];
+    if (d.sms == 0) {
+        cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&d.smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    }
+    return d;
+}
+
+}  // namespace
+
+size_t resident_scratch_doubles(int n) {
+    // a matrix with m >= n that fits has n^2 doubles in kResGrid SMs of 227 KB
+    const size_t nn = std::min(n, 2200);
+    return 2 * ((size_t)kResGrid * nn + 3 * nn + 8);
+}
+
+int res_grid(int m) {
+    const DevInfo d = dev_info();
+    return std::max(1, std::min(std::min(d.sms, kResGrid), m));
+}
+
+bool resident_fits(int m, int n) {
+    const DevInfo d = dev_info();
+    if (d.sms <= 0 || n < 1 || n > 2200) return false;
+    const int G = res_grid(m);
+    return res_smem(m, n, G) <= (size_t)d.smem;
+}
+
+cudaError_t launch_gebd2_resident(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup,
+                                  double *scratch, GridBar *bar, unsigned *bars, cudaStream_t st) {
+    const int G = res_grid(m);
+    const size_t smem = res_smem(m, n, G);
+    Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * n, *yr = row + n, *scal = yr + 2 * n;
+    Gebd2Args a{A, lda, m, n, d, e, tauq, taup, gp, row, yr, scal, bar, *bars};
+    *bars += (unsigned)G;
+    // the device's maximum, not this launch's size: another thread may be
+    // between its own call and its launch
+    cudaError_t err =
+        cudaFuncSetAttribute(k_gebd2_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, dev_info().smem);
+    if (err != cudaSuccess) return err;
+    void *params[] = {&a};
+    return cudaLaunchCooperativeKernel((const void *)k_gebd2_resident, dim3(G), dim3(NT), params, smem, st);
+}
+
+}  // namespace bdc
