@@ -537,6 +537,7 @@ DevInfo dev_info() {
     if (d.sms == 0) {
         cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&d.smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        d.smem -= 128;   // the kernels' static shared memory
     }
     return d;
 }
