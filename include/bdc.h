@@ -415,7 +415,7 @@ int bdc_mlp_train(const bdc_opts *o, const bdc_mlp_train_opts *t, float *params,
 /* Bidiagonalization A = Q1 B P1^T (Sec. 4.1, Algorithm 1), m >= n: per
  * panel the b column and row reflectors (H_i, G_i, Eq. gebrd-house) with the
  * vectors y_i, x_i of Eqs. (bidiag-y-k3, bidiag-x-k3), then the merged
- * rank-(2b) update A -= P Q^T of Eq. (bidiag-A-trail3) as one FP64
+ * rank-(2b) update A -= P Q^T of Eq. (bidiag-A-trail3) as one
  * tensor-core product.  On exit d[n] / e[n-1] hold B's diagonal and
  * superdiagonal, A holds y_i below the diagonal of column i and u_i right of
  * the superdiagonal of row i (u_i[i+1] = 1 implicit), tauq[n], taup[n] the
@@ -426,9 +426,11 @@ int bdc_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *ta
 
 /* Back-transformation with the reflectors of bdc_gebrd (Sec. 4.3, ormqr /
  * ormlq): vect = 0: C (m x cdim, ldc >= m) := Q1 C; vect = 1: C (cdim x n,
- * ldc >= cdim) := C P1^T.  Each block of b reflectors is applied in the
- * modified compact-WY form: T^{-1} = Y^T Y with diagonal 1/tau (Eqs. inv_t,
- * larft_update), Z = Y^T C, a triangular solve with T^{-1}, C -= Y W. */
+ * ldc >= cdim) := C P1^T.  Each block of reflectors I - Y T Y^T is applied
+ * with T formed from T^{-1} = Y^T Y with diagonal 1/tau (Eqs. inv_t,
+ * larft_update): Z = Y^T C, C -= (Y T) Z, the products by error-free BF16
+ * slices on the tensor cores (56 bits), in FP64 below 64 reflectors.  A
+ * bounded wait of the products that gives up fills C with NaN. */
 size_t bdc_ormbr_workspace(int m, int n, int cdim);
 int bdc_ormbr(int vect, int m, int n, const double *A, int lda, const double *tau, double *C, int ldc, int cdim,
               void *work, size_t lwork, bdc_stream_t stream);

@@ -11,18 +11,30 @@
 //   Sec. 4.3  QR of a tall-and-skinny A (cooperative panel k_geqr2 plus a
 //             block-reflector update of the trailing columns), the explicit Q
 //             (Eq. orgqr-q), and the back-transformations U = Q1 U2 and
-//             V^T = V2^T P1^T.  Every block reflector I - Y T Y^T is applied
-//             in the modified compact-WY form of Eqs. (inv_t, larft_update):
-//             T^{-1} = Y^T Y (one product) with the diagonal 1 / tau, then
-//             Z = Y^T C (product), W = T Z by a triangular solve with T^{-1},
-//             C -= Y W (product): products and a small triangular solve only.
+//             V^T = V2^T P1^T.  A block reflector I - Y T Y^T is applied with
+//             T formed explicitly from the modified compact-WY relation of
+//             Eqs. (inv_t, larft_update), T^{-1} = the upper part of Y^T Y with
+//             the diagonal 1 / tau: products only, no solve per column.
 //
-// The products are FP64 on the tensor cores (mma.sync.m8n8k4.f64, k_dgemm):
-// C = alpha op(A) op(B) + beta C with either operand transposed.  The panel
+// Products: from 64 reflectors on (and for the trailing updates) error-free
+// BF16 slices on the tcgen05 tensor cores (split_products, bdc_gemm_mixed.cu:
+// 56 bits below each row's maximum), smaller ones FP64 mma.sync.m8n8k4
+// (k_dgemm: C = alpha op(A) op(B) + beta C with either operand transposed).
+// mma.sync FP64 runs at 1.67 multiply-adds a clock and SM on GB300 (measured,
+// any shape and occupancy; the plain FMA 1.9), so the FP64 products were
+// most of a large SVD: back-transformation of 4096 x 4096, one side, 181 ms
+// (165 ms without the triangular solves) -> 10.5 ms; trailing updates of its
+// reduction about 85 -> 8 ms; 333 x 333, one side, 2.4 -> 0.64 ms.  Error:
+// U^T U - I and the residual of gesvd as with FP64 products (333 to 2048:
+// 5.5e-14 to 4.2e-13 and 2.8e-15 to 7.6e-15 either way).
+//
+// The panel
 // kernels run as cooperative launches (all CTAs resident) and separate their
 // phases with a grid barrier whose wait is bounded (2 s of %globaltimer): a
 // barrier that gives up sets an error word, every CTA leaves at its next
-// barrier, and the entry point reports BDC_ERR_TIMEOUT.
+// barrier, and the entry point reports BDC_ERR_TIMEOUT (the products' bounded
+// waits set the same word; the entry points without a status fill their
+// result with NaN then).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -56,33 +68,42 @@ __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
                  : "d"(a), "d"(b));
 }
 
-// 64 x 64 CTA tile, four warps of 32 x 32 (4 x 4 fragments 8 x 8), K step 16,
-// operands staged k-major in padded shared tiles, next step prefetched
-constexpr int DBM = 64, DBN = 64, DBK = 16, DSA = DBM + 8, DSB = DBK + 4;
+// Four warps of 32 x 32 (4 x 4 fragments 8 x 8), K step 16, operands staged
+// k-major in padded shared tiles, next step prefetched.  CTA tile 64 x 64, or
+// 32 x 128 for products of at most 32 rows (the QR panels' Y^T C), where the
+// lower half of a 64 x 64 tile would leave two SM sub-partitions idle.
+constexpr int DBK = 16, DSB = DBK + 4;
+template <int DBM, int DBN>
 __global__ void __launch_bounds__(128) k_dgemm(DGemm g) {
+    constexpr int DSA = DBM + 8, WN = DBN / 32;
+    static_assert(DBM / 32 * WN == 4, "four warps");
     __shared__ double As[DBK * DSA];   // As[k][m]
     __shared__ double Bs[DBN * DSB];   // Bs[n][k]
     const int tilesN = (g.N + DBN - 1) / DBN;
     const int m0 = (blockIdx.x / tilesN) * DBM, n0 = (blockIdx.x % tilesN) * DBN;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+    const int wm = (warp / WN) * 32, wn = (warp % WN) * 32;
     const int gr = lane >> 2, tg = lane & 3;
     double acc[4][4][2];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
-    constexpr int L = DBM * DBK / 128;   // 8 elements per thread per operand
-    double ra[L], rb[L];
+    constexpr int LA = DBM * DBK / 128, LB = DBN * DBK / 128;   // elements per thread per operand
+    double ra[LA], rb[LB];
     auto load = [&](int k0) {
 #pragma unroll
-        for (int r = 0; r < L; ++r) {
+        for (int r = 0; r < LA; ++r) {
             const int idx = tid + r * 128;
             int am, ak;
             if (!g.ta) { am = idx % DBM; ak = idx / DBM; } else { ak = idx % DBK; am = idx / DBK; }
             const int gm = m0 + am, gk = k0 + ak;
             ra[r] = (gm < g.M && gk < g.K) ? (g.ta ? g.A[(size_t)gm * g.lda + gk] : g.A[(size_t)gk * g.lda + gm])
                                            : 0.0;
+        }
+#pragma unroll
+        for (int r = 0; r < LB; ++r) {
+            const int idx = tid + r * 128;
             int bk, bn;
             if (!g.tb) { bk = idx % DBK; bn = idx / DBK; } else { bn = idx % DBN; bk = idx / DBN; }
             const int gn = n0 + bn, gk2 = k0 + bk;
@@ -92,12 +113,17 @@ __global__ void __launch_bounds__(128) k_dgemm(DGemm g) {
     };
     auto store = [&]() {
 #pragma unroll
-        for (int r = 0; r < L; ++r) {
+        for (int r = 0; r < LA; ++r) {
             const int idx = tid + r * 128;
-            int am, ak, bk, bn;
+            int am, ak;
             if (!g.ta) { am = idx % DBM; ak = idx / DBM; } else { ak = idx % DBK; am = idx / DBK; }
-            if (!g.tb) { bk = idx % DBK; bn = idx / DBK; } else { bn = idx % DBN; bk = idx / DBN; }
             As[ak * DSA + am] = ra[r];
+        }
+#pragma unroll
+        for (int r = 0; r < LB; ++r) {
+            const int idx = tid + r * 128;
+            int bk, bn;
+            if (!g.tb) { bk = idx % DBK; bn = idx / DBK; } else { bn = idx % DBN; bk = idx / DBN; }
             Bs[bn * DSB + bk] = rb[r];
         }
     };
@@ -151,19 +177,6 @@ __global__ void __launch_bounds__(128) k_dgemm(DGemm g) {
     }
 }
 
-// C = beta C + alpha sum_y part[y] (the split-K partial products, summed in
-// a fixed order)
-__global__ void k_dgemm_reduce(const double *__restrict__ part, int splits, int M, int N, double alpha, double beta,
-                               double *C, int ldc) {
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (long long)M * N) return;
-    const int n = (int)(k / M), m = (int)(k % M);
-    double s = 0.0;
-    for (int y = 0; y < splits; ++y) s += part[(size_t)y * M * N + k];
-    double *c = C + (size_t)n * ldc + m;
-    *c = (beta == 0.0) ? alpha * s : fma(beta, *c, alpha * s);
-}
-
 // scratch for split-K partial products (set per call sequence by the driver)
 thread_local double *g_split_buf = nullptr;
 thread_local size_t g_split_cap = 0;   // doubles
@@ -178,36 +191,52 @@ int sm_count_dense() {
     return n;
 }
 
-// C = alpha op(A) op(B) + beta C.  Products with few output tiles and a long
-// K (the Y^T C and C Y of the block reflectors: 32 x n outputs, K = the
-// panel's rows) split K over several CTAs into partial products, summed in a
-// fixed order by k_dgemm_reduce, so that the whole GPU works on them
+cudaError_t dgemm_launch(const DGemm &g, int splits, cudaStream_t st) {
+    if (g.M <= 32) {
+        const long long tiles = (long long)((g.M + 31) / 32) * ((g.N + 127) / 128);
+        if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
+        k_dgemm<32, 128><<<dim3((unsigned)tiles, (unsigned)splits), 128, 0, st>>>(g);
+    } else {
+        const long long tiles = (long long)((g.M + 63) / 64) * ((g.N + 63) / 64);
+        if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
+        k_dgemm<64, 64><<<dim3((unsigned)tiles, (unsigned)splits), 128, 0, st>>>(g);
+    }
+    return cudaGetLastError();
+}
+
+// C = alpha op(A) op(B) + beta C
 cudaError_t dgemm(int ta, int tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B,
                   int ldb, double beta, double *C, int ldc, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    const long long tiles = (long long)((M + DBM - 1) / DBM) * ((N + DBN - 1) / DBN);
-    if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
-    DGemm g{A, B, C, lda, ldb, ldc, M, N, std::max(K, 0), ta, tb, alpha, beta, 0, nullptr};
-    int splits = 1;
-    const int sms = sm_count_dense();
-    if (K >= 128 && tiles < 2 * sms && g_split_buf) {
-        splits = (int)std::min<long long>((2 * sms + tiles - 1) / tiles, K / 64);
-        splits = std::min(splits, 64);
-        while (splits > 1 && (size_t)splits * M * N > g_split_cap) --splits;
+    return dgemm_launch(DGemm{A, B, C, lda, ldb, ldc, M, N, std::max(K, 0), ta, tb, alpha, beta, 0, nullptr}, 1, st);
+}
+
+// op(A) op(B) as `splits` partial products over ranges of K, part y at
+// g_split_buf + y M N (column-major M x N): the products with few output
+// tiles and a long K (Y^T C and C Y of the block reflectors) then use the
+// whole GPU.  The split count fills whole rounds of two CTAs per SM (the
+// FP64 tensor pipe is full with one warp per sub-partition, so a round's time
+// does not depend on how full it is) and keeps at least 64 of K per part.
+cudaError_t dgemm_parts(int ta, int tb, int M, int N, int K, const double *A, int lda, const double *B, int ldb,
+                        int &splits, cudaStream_t st) {
+    const long long tiles = M <= 32 ? (long long)((N + 127) / 128) : (long long)((M + 63) / 64) * ((N + 63) / 64);
+    const long long sms = sm_count_dense();
+    const long long cap = std::max<long long>(1, (long long)(g_split_cap / ((size_t)M * N)));
+    const long long most = std::max<long long>(1, std::min<long long>({cap, 64, K / 64}));
+    // the split with the least work on the fullest SM, the smallest within 3 %
+    splits = 1;
+    double best = 0.0;
+    for (long long s = 1; s <= most; ++s) {
+        const double c = (double)((tiles * s + sms - 1) / sms) / (double)s;
+        if (s == 1 || c < 0.97 * best) {
+            best = c;
+            splits = (int)s;
+        }
     }
-    if (splits > 1) {
-        g.kchunk = ((K + splits - 1) / splits + DBK - 1) / DBK * DBK;
-        splits = (K + g.kchunk - 1) / g.kchunk;
-        g.part = g_split_buf;
-        k_dgemm<<<dim3((unsigned)tiles, (unsigned)splits), 128, 0, st>>>(g);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        const long long cnt = (long long)M * N;
-        k_dgemm_reduce<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(g_split_buf, splits, M, N, alpha, beta, C, ldc);
-        return cudaGetLastError();
-    }
-    k_dgemm<<<(unsigned)tiles, 128, 0, st>>>(g);
-    return cudaGetLastError();
+    DGemm g{A, B, nullptr, lda, ldb, 0, M, N, K, ta, tb, 1.0, 0.0, 0, g_split_buf};
+    g.kchunk = ((K + splits - 1) / splits + DBK - 1) / DBK * DBK;
+    splits = (K + g.kchunk - 1) / g.kchunk;
+    return dgemm_launch(g, splits, st);
 }
 
 // ------------------------------------------------------------ grid barrier
@@ -583,84 +612,495 @@ __global__ void k_form_y(double *Y, int rows, int nb, const double *src, long lo
     Y[k] = (r < j) ? 0.0 : (r == j) ? 1.0 : src[(size_t)j * sc + (size_t)r * sr];
 }
 
-// T^{-1} = Y^T Y with the diagonal 1 / tau (Eqs. inv_t, larft_update; only the
-// upper triangle is read): the product is done by k_dgemm, this fixes the
-// diagonal; a zero tau (H = I) is marked by a zero diagonal entry
-__global__ void k_tinv_diag(double *Ti, int nb, const double *tau) {
-    const int j = threadIdx.x;
-    if (j < nb) Ti[(size_t)j * nb + j] = (tau[j] != 0.0) ? 1.0 / tau[j] : 0.0;
-}
+// ---- T of the compact WY form I - Y T Y^T = H_1 ... H_nb, for every block
+// of kTB reflectors of a call at once.  T^{-1} is the strictly upper part of
+// Y^T Y plus the diagonal 1 / tau (Eqs. inv_t, larft_update); it is inverted
+// here once (zero row and column where tau = 0), so that applying a block is
+// two products and a small one with T instead of a triangular solve per right
+// hand side (one thread each, 64 x 64 / 2 dependent FMAs: 4096 x 4096, one
+// side, 181 ms of which the solves were about 130).
+constexpr int kTB = 64;
 
-// Triangular solve with T^{-1} (nb x nb, upper, in Ti) on many right-hand
-// sides: mode 0: W = T Z  (T^{-1} W = Z, column vectors of Z, nb x ncol, ld ldz)
-//        mode 1: W = T^T Z (T^{-T} W = Z)
-//        mode 2: W = Z T   (W T^{-1} = Z, row vectors of Z, nrow x nb, ld ldz)
-//        mode 3: W = Z T^T (W T^{-T} = Z)
-// in place; a zero diagonal entry (tau = 0) makes that component of W zero.
-__global__ void __launch_bounds__(128) k_tsolve(const double *__restrict__ Ti, int nb, double *Z, int ldz,
-                                                int count, int mode) {
-    extern __shared__ double st[];   // T^{-1}, nb x nb
-    for (int k = threadIdx.x; k < nb * nb; k += blockDim.x) st[k] = Ti[k];
-    __syncthreads();
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= count) return;
-    // element p of this right-hand side
-    const bool colwise = mode < 2;
-    auto at = [&](int p) -> double & { return colwise ? Z[(size_t)v * ldz + p] : Z[(size_t)p * ldz + v]; };
-    auto tij = [&](int i, int j) { return st[(size_t)j * nb + i]; };   // T^{-1}(i, j), i <= j
-    const bool upper_solve = (mode == 0) || (mode == 3);   // T^{-1} W = Z or W T^{-T} = Z: back substitution
-    if (upper_solve) {
-        for (int p = nb - 1; p >= 0; --p) {
-            const double dp = tij(p, p);
-            if (dp == 0.0) { at(p) = 0.0; continue; }
-            double s = at(p);
-            for (int q = p + 1; q < nb; ++q) s -= tij(p, q) * at(q);
-            at(p) = s / dp;
+// the reflectors of a call: block j holds kTB of them from reflector i0 = j
+// kTB, entry r of reflector i0 + c at src + i0 (sr + sc) + r sr + c sc for r
+// > c (1 at r = c, 0 above), rows - i0 entries long
+struct Reflectors {
+    const double *src;
+    long long sr, sc;
+    int rows, count;
+};
+
+// partial Y^T Y of block blockIdx.x over the rows of chunk blockIdx.y
+__global__ void __launch_bounds__(128) k_gram(Reflectors f, int kchunk, double *part) {
+    constexpr int LD = kTB + 4;
+    __shared__ double Ys[16 * LD];   // [row][reflector]
+    const int i0 = blockIdx.x * kTB, nb = min(kTB, f.count - i0), rows = f.rows - i0;
+    const double *src = f.src + (size_t)i0 * (f.sr + f.sc);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32, gr = lane >> 2, tg = lane & 3;
+    const int kb = blockIdx.y * kchunk, ke = min(rows, kb + kchunk);
+    double acc[4][4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+    for (int k0 = kb; k0 < ke; k0 += 16) {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 16 * kTB / 128; ++q) {
+            const int idx = tid + q * 128;
+            int r, c;   // the contiguous index fastest
+            if (f.sr == 1) { r = idx % 16; c = idx / 16; } else { c = idx % kTB; r = idx / kTB; }
+            const int gk = k0 + r;
+            double v = 0.0;
+            if (gk < ke && c < nb && gk >= c) v = (gk == c) ? 1.0 : src[(size_t)gk * f.sr + (size_t)c * f.sc];
+            Ys[r * LD + c] = v;
         }
-    } else {
-        for (int p = 0; p < nb; ++p) {
-            const double dp = tij(p, p);
-            if (dp == 0.0) { at(p) = 0.0; continue; }
-            double s = at(p);
-            for (int q = 0; q < p; ++q) s -= tij(q, p) * at(q);
-            at(p) = s / dp;
+        __syncthreads();
+        if (wm > wn) continue;       // below the diagonal: not needed
+#pragma unroll
+        for (int kk = 0; kk < 16; kk += 4) {
+            double af[4], bf[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                af[i] = Ys[(kk + tg) * LD + wm + i * 8 + gr];
+                bf[i] = Ys[(kk + tg) * LD + wn + i * 8 + gr];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) dmma(acc[i][j], af[i], bf[j]);
         }
     }
+    double *out = part + ((size_t)blockIdx.x * gridDim.y + blockIdx.y) * kTB * kTB;
+    if (wm <= wn)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    out[(size_t)(wm + i * 8 + gr) * kTB + wn + j * 8 + 2 * tg + h] = acc[i][j][h];
+}
+
+// C (rm x cn, row stride ldc) = sgn A (rm x kn) B (kn x cn) in shared memory, 8 x 8 fragments over the CTA's warps
+__device__ __forceinline__ void smem_mm(double *C, int ldc, const double *A, int lda, const double *B, int ldb, int rm,
+                                        int cn, int kn, double sgn) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int gr = lane >> 2, tg = lane & 3;
+    const int tn = cn / 8, tiles = rm / 8 * tn;
+    for (int q = warp; q < tiles; q += nw) {
+        const int r0 = q / tn * 8, c0 = q % tn * 8;
+        double acc[2] = {0.0, 0.0};
+        for (int k = 0; k < kn; k += 4) dmma(acc, A[(r0 + gr) * lda + k + tg], B[(k + tg) * ldb + c0 + gr]);
+        C[(r0 + gr) * ldc + c0 + 2 * tg] = sgn * acc[0];
+        C[(r0 + gr) * ldc + c0 + 2 * tg + 1] = sgn * acc[1];
+    }
+}
+
+// T (kTB x kTB, row-major, zero below the diagonal and beyond the block's
+// reflectors) of block blockIdx.x: the 16 x 16 diagonal blocks by the column
+// recursion T(:, j) = -tau_j T G(:, j), a warp each; then pairs of blocks by
+// T_12 = -T_11 G_12 T_22.  Block x is sub-block x % per of group x / per:
+// its G and T lie at group (x / per) gstride + (x % per) kTB (ld + 1), row
+// stride ld; G is the sum of `chunks` copies cstride apart.
+constexpr int kTLd = kTB + 4;
+struct TForm {
+    const double *G;
+    double *T;
+    const double *tau;
+    int ld, per, chunks, count;
+    long long gstride_g, gstride_t, cstride;
+};
+__global__ void __launch_bounds__(256) k_tform(TForm f) {
+    extern __shared__ double tsm[];
+    double *Gs = tsm, *Ts = tsm + kTB * kTLd, *Xs = Ts + kTB * kTLd;   // G, T, 32 x 32 product
+    const int i0 = blockIdx.x * kTB, nb = min(kTB, f.count - i0);
+    const int sub = blockIdx.x % f.per, grp = blockIdx.x / f.per;
+    const double *p = f.G + grp * f.gstride_g + (long long)sub * kTB * (f.ld + 1);
+    const double *tau = f.tau;
+    double *Tall = f.T + grp * f.gstride_t + (long long)sub * kTB * (f.ld + 1);
+    for (int k = threadIdx.x; k < kTB * kTB; k += blockDim.x) {
+        const int r = k / kTB, c = k % kTB;
+        double s = 0.0;
+        if (r < c && c < nb)
+            for (int y = 0; y < f.chunks; ++y) s += p[y * f.cstride + (long long)r * f.ld + c];
+        Gs[r * kTLd + c] = s;
+        Ts[r * kTLd + c] = 0.0;
+    }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < kTB / 16) {
+        const int o = warp * 16;
+        for (int j = 0; j < 16; ++j) {
+            const double tj = (o + j < nb) ? tau[i0 + o + j] : 0.0;
+            double s = 0.0;
+            if (lane < j)
+                for (int k = lane; k < j; ++k) s = fma(Ts[(o + lane) * kTLd + o + k], Gs[(o + k) * kTLd + o + j], s);
+            if (lane <= j) Ts[(o + lane) * kTLd + o + j] = (lane == j) ? tj : -tj * s;
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int h = 16; h < kTB; h *= 2)
+        for (int o = 0; o < kTB; o += 2 * h) {
+            smem_mm(Xs, kTLd, Gs + o * kTLd + o + h, kTLd, Ts + (o + h) * kTLd + o + h, kTLd, h, h, h, 1.0);
+            __syncthreads();
+            smem_mm(Ts + o * kTLd + o + h, kTLd, Ts + o * kTLd + o, kTLd, Xs, kTLd, h, h, h, -1.0);
+            __syncthreads();
+        }
+    for (int k = threadIdx.x; k < kTB * kTB; k += blockDim.x)
+        Tall[(long long)(k / kTB) * f.ld + k % kTB] = Ts[(k / kTB) * kTLd + k % kTB];
+}
+constexpr size_t kTformSmem = sizeof(double) * (2 * kTB + 32) * kTLd;
+
+// T of every block of the reflectors into Tall (blocks x kTB x kTB)
+cudaError_t form_t(const Reflectors &f, const double *tau, double *Tall, cudaStream_t st) {
+    if (f.count <= 0) return cudaSuccess;
+    const int blocks = (f.count + kTB - 1) / kTB;
+    // chunks of at least 256 rows, about four CTAs per SM over all blocks
+    const long long cap = (long long)(g_split_cap / ((size_t)blocks * kTB * kTB));
+    long long chunks = std::min<long long>((f.rows + 255) / 256, std::max(1, 4 * sm_count_dense() / blocks));
+    chunks = std::max<long long>(1, std::min(chunks, cap));
+    if (cap < 1) return cudaErrorInvalidValue;
+    int kchunk = (int)((f.rows + chunks - 1) / chunks + 15) / 16 * 16;
+    chunks = (f.rows + kchunk - 1) / kchunk;
+    k_gram<<<dim3(blocks, (unsigned)chunks), 128, 0, st>>>(f, kchunk, g_split_buf);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_tform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTformSmem)) !=
+        cudaSuccess)
+        return e;
+    k_tform<<<blocks, 256, kTformSmem, st>>>(TForm{g_split_buf, Tall, tau, kTB, 1, (int)chunks, f.count,
+                                                   (long long)chunks * kTB * kTB, (long long)kTB * kTB,
+                                                   (long long)kTB * kTB});
+    return cudaGetLastError();
+}
+
+// W = M Z for the summed partial products Z of dgemm_parts, M = T or T^T
+// (tr), nb x nb.  left: Z is nb x count (column-major), a vector per column;
+// right: Z is count x nb, a vector per row (W^T = M Z^T).  16 vectors per
+// CTA; each warp takes 8 rows of M, its fragments straight from L2.  add: Z +=
+// the first nb rows of add (left; the unit entries' share).
+__global__ void __launch_bounds__(256) k_tz(const double *__restrict__ T, int nb, int tr, const double *__restrict__ part,
+                                            int splits, int right, int count, double *__restrict__ W,
+                                            const double *__restrict__ add, int ldadd) {
+    constexpr int V = 16, LD = V + 4;
+    __shared__ double Zs[kTB * LD];   // [k][vector]
+    const int v0 = blockIdx.x * V;
+    const size_t mn = (size_t)nb * count;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gr = lane >> 2, tg = lane & 3;
+    const int i0 = warp * 8;
+    double mf[kTB / 4];
+#pragma unroll
+    for (int k = 0; k < kTB / 4; ++k) {
+        const int i = i0 + gr, j = 4 * k + tg;
+        mf[k] = T[tr ? j * kTB + i : i * kTB + j];
+    }
+    for (int k = threadIdx.x; k < kTB * V; k += blockDim.x) {
+        int p, v;
+        if (right) { v = k % V; p = k / V; } else { p = k % kTB; v = k / kTB; }
+        double s = 0.0;
+        if (p < nb && v0 + v < count) {
+            const double *q = part + (right ? (size_t)p * count + v0 + v : (size_t)(v0 + v) * nb + p);
+            for (int y = 0; y < splits; ++y) s += q[(size_t)y * mn];
+            if (add) s += add[(size_t)(v0 + v) * ldadd + p];
+        }
+        Zs[p * LD + v] = s;
+    }
+    __syncthreads();
+    if (i0 >= nb) return;
+    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+    for (int k = 0; k < kTB / 4; ++k) {
+        // M is triangular: T has only k >= i, T^T only k <= i
+        if (tr ? 4 * k > i0 + 7 : 4 * k + 3 < i0) continue;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) dmma(acc[j], mf[k], Zs[(4 * k + tg) * LD + j * 8 + gr]);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int v = v0 + j * 8 + 2 * tg + h, i = i0 + gr;
+            if (i < nb && v < count) W[right ? (size_t)i * count + v : (size_t)v * nb + i] = acc[j][h];
+        }
 }
 
 // C (rows x cols, ldc) := H C or H^T C (left) or C H or C H^T (right), H =
 // I - Y T Y^T = H_1 ... H_nb for the explicit Y (left: rows x nb; right:
-// cols x nb), modified compact WY: T^{-1} = Y^T Y (diag 1/tau), Z = Y^T C
-// (or C Y), W = T Z / T^T Z (or Z T / Z T^T) by the triangular solve, C -= Y W
-// (or W Y^T).  Scratch: Ti (nb x nb), Z (nb x cols or rows x nb).
-cudaError_t apply_block(int left, int trans, int rows, int cols, const double *Y, int nb, const double *tau,
-                        double *C, int ldc, double *Ti, double *Z, cudaStream_t st) {
+// cols x nb) and its T: Z = Y^T C (or C Y) in partial products, W = T Z or
+// T^T Z (or Z T, Z T^T), C -= Y W (or W Y^T).
+cudaError_t apply_block(int left, int trans, int rows, int cols, const double *Y, int nb, const double *T, double *C,
+                        int ldc, double *W, cudaStream_t st) {
     if (rows <= 0 || cols <= 0 || nb <= 0) return cudaSuccess;
-    const int ry = left ? rows : cols;   // rows of Y
-    cudaError_t e = dgemm(1, 0, nb, nb, ry, 1.0, Y, ry, Y, ry, 0.0, Ti, nb, st);
-    if (e != cudaSuccess) return e;
-    k_tinv_diag<<<1, ((nb + 31) / 32) * 32, 0, st>>>(Ti, nb, tau);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t smem = sizeof(double) * nb * nb;
-    if (smem > 48 * 1024) {   // T^{-1} above the static limit: opt in to more dynamic shared memory
-        static std::once_flag once;
-        static cudaError_t attr = cudaSuccess;
-        std::call_once(once, [] {
-            attr = cudaFuncSetAttribute(k_tsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        });
-        if (attr != cudaSuccess) return attr;
-        if (smem > 200 * 1024) return cudaErrorInvalidValue;
-    }
+    cudaError_t e;
+    int splits;
     if (left) {
-        if ((e = dgemm(1, 0, nb, cols, rows, 1.0, Y, rows, C, ldc, 0.0, Z, nb, st)) != cudaSuccess) return e;
-        k_tsolve<<<(cols + 127) / 128, 128, smem, st>>>(Ti, nb, Z, nb, cols, trans ? 1 : 0);
+        if ((e = dgemm_parts(1, 0, nb, cols, rows, Y, rows, C, ldc, splits, st)) != cudaSuccess) return e;
+        k_tz<<<(cols + 15) / 16, 256, 0, st>>>(T, nb, trans ? 1 : 0, g_split_buf, splits, 0, cols, W, nullptr, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return dgemm(0, 0, rows, cols, nb, -1.0, Y, rows, Z, nb, 1.0, C, ldc, st);
+        return dgemm(0, 0, rows, cols, nb, -1.0, Y, rows, W, nb, 1.0, C, ldc, st);
     }
-    if ((e = dgemm(0, 0, rows, nb, cols, 1.0, C, ldc, Y, cols, 0.0, Z, rows, st)) != cudaSuccess) return e;
-    k_tsolve<<<(rows + 127) / 128, 128, smem, st>>>(Ti, nb, Z, rows, rows, trans ? 3 : 2);
+    if ((e = dgemm_parts(0, 0, rows, nb, cols, C, ldc, Y, cols, splits, st)) != cudaSuccess) return e;
+    k_tz<<<(rows + 15) / 16, 256, 0, st>>>(T, nb, trans ? 0 : 1, g_split_buf, splits, 1, rows, W, nullptr, 0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return dgemm(0, 1, rows, cols, nb, -1.0, Z, rows, Y, cols, 1.0, C, ldc, st);
+    return dgemm(0, 1, rows, cols, nb, -1.0, W, rows, Y, cols, 1.0, C, ldc, st);
+}
+
+// ---- blocks of kWide reflectors on the split-BF16 products (split_products):
+// V = Y T is formed for every block of a call at once (Y read in place from
+// the panel through the slicing's mask), then per block Z = Y^T C (partial
+// products over K) and C -= V Z.
+constexpr int kWide = 256;
+constexpr int kGramMost = 9;     // partial products of one block's Y^T Y at most
+
+// G = Y^T Y above the diagonal from the partial products of Y without its unit
+// entries (symmetric): entry (r, c), r < c, adds reflector r's row c times
+// reflector c's unit entry.  T zeroed.
+__global__ void k_gram_sum(const double *__restrict__ part, Reflectors f, int chunks, double *__restrict__ G,
+                           double *__restrict__ T) {
+    const size_t w2 = (size_t)kWide * kWide;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, r = k / kWide, c = k % kWide;
+    const int i0 = blockIdx.y * kWide, nb = min(kWide, f.count - i0);
+    const double *p = part + (size_t)blockIdx.y * chunks * w2 + k;
+    double s = 0.0;
+    if (r < c && c < nb) {
+        for (int y = 0; y < chunks; ++y) s += p[(size_t)y * w2];
+        s += f.src[(size_t)i0 * (f.sr + f.sc) + (size_t)c * f.sr + (size_t)r * f.sc];
+    }
+    G[blockIdx.y * w2 + k] = s;
+    T[blockIdx.y * w2 + k] = 0.0;
+}
+
+// the off-diagonal blocks of T from its h x h diagonal blocks, one 8 x 8
+// fragment per warp, operands from L2: phase 0: X = G_12 T_22, phase 1: T_12 =
+// -T_11 X (row-major, kWide x kWide per block; a fragment's K range skips the
+// zero half of the triangular factor)
+__global__ void __launch_bounds__(128) k_tmerge(const double *G, double *T, double *X, int h, int phase) {
+    const size_t w2 = (size_t)kWide * kWide;
+    const double *g = G + blockIdx.y * w2;
+    double *t = T + blockIdx.y * w2, *x = X + blockIdx.y * w2;
+    const int lane = threadIdx.x & 31, gr = lane >> 2, tg = lane & 3;
+    const int per = (h / 8) * (h / 8);
+    const int q = blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int o = q / per * 2 * h, r0 = q % per / (h / 8) * 8, c0 = q % per % (h / 8) * 8;
+    if (o + 2 * h > kWide) return;
+    const double *A = phase == 0 ? g + (size_t)o * kWide + o + h : t + (size_t)o * kWide + o;
+    const double *B = phase == 0 ? t + (size_t)(o + h) * kWide + o + h : x + (size_t)o * kWide + o + h;
+    double acc[2] = {0.0, 0.0};
+    const int kb = phase == 0 ? 0 : r0, ke = phase == 0 ? c0 + 8 : h;
+#pragma unroll 8
+    for (int k = kb; k < ke; k += 4)
+        dmma(acc, A[(size_t)(r0 + gr) * kWide + k + tg], B[(size_t)(k + tg) * kWide + c0 + gr]);
+    double *out = (phase == 0 ? x : t) + (size_t)(o + r0 + gr) * kWide + o + h + c0 + 2 * tg;
+    out[0] = phase == 0 ? acc[0] : -acc[0];
+    out[1] = phase == 0 ? acc[1] : -acc[1];
+}
+
+// workspace of the split path: G, T, X (blocks x kWide^2), V (rows x count,
+// also the partial Y^T Y before it), Z parts, slices
+struct SplitWs {
+    double *G, *T, *X, *V, *Z;
+    size_t zcap;       // doubles at Z
+    char *slices;
+    size_t slice_bytes;
+    int *err;
+};
+
+// op(Y) sides of a block (reflectors i0 .. i0 + nb - 1 of f, rows k0 ..).  The
+// vectors leave out the unit entry: it would be the maximum that scales the
+// slices of a reflector whose other entries are about 1 / sqrt(rows), and its
+// product is the row of C itself, added in FP64 (I - Q^T Q of 1000 x 1000:
+// 4.0e-14 by FP64 products, 5.3e-14 with the unit entry sliced).
+SplitSide y_vectors(const Reflectors &f, int i0, int nb, int k0) {   // a vector per reflector, K = rows
+    const double *p = f.src + (size_t)i0 * (f.sr + f.sc) + (size_t)k0 * f.sr;
+    return f.sr == 1 ? SplitSide{p, 0, (int)f.sc, 0, nb, 1, 1, k0, 0} : SplitSide{p, 0, (int)f.sr, 1, nb, 1, 1, k0, 0};
+}
+SplitSide y_rows(const Reflectors &f, int i0, int rows) {            // a vector per row, K = reflectors
+    const double *p = f.src + (size_t)i0 * (f.sr + f.sc);
+    return f.sr == 1 ? SplitSide{p, 0, (int)f.sc, 1, rows, 1, 2, 0, 0} : SplitSide{p, 0, (int)f.sr, 0, rows, 1, 2, 0, 0};
+}
+
+// runs products in sets that fit kSplitMax and the slice scratch
+struct SplitSet {
+    const SplitWs &w;
+    cudaStream_t st;
+    std::vector<SplitProd> v;
+    long long rows = 0, cols = 0, tiles = 0;
+    int kmax = 0;
+    cudaError_t add(const SplitProd &p) {
+        auto need = [&](long long r, long long c, int k, long long t) { return split_scratch(r, c, k, t); };
+        const long long t = (long long)((p.a.n + 127) / 128) * ((p.b.n + 127) / 128);
+        const int k = std::max(kmax, p.K);
+        if (!v.empty() && ((int)v.size() == kSplitMax || need(rows + p.a.n, cols + p.b.n, k, tiles + t) > w.slice_bytes)) {
+            if (cudaError_t e = run()) return e;
+        }
+        v.push_back(p);
+        rows += p.a.n; cols += p.b.n; tiles += t;
+        kmax = std::max(kmax, p.K);
+        return cudaSuccess;
+    }
+    cudaError_t run() {
+        cudaError_t e = split_products(v.data(), (int)v.size(), w.slices, w.slice_bytes, w.err, st);
+        v.clear();
+        rows = cols = tiles = 0;
+        kmax = 0;
+        return e;
+    }
+};
+
+// V = Y T of every kWide block of the reflectors (row-major T): V of block j
+// at w.V + i0 f.rows, column-major, f.rows - i0 rows, leading dimension f.rows
+cudaError_t form_v(const Reflectors &f, const double *tau, const SplitWs &w, cudaStream_t st) {
+    const int blocks = (f.count + kWide - 1) / kWide;
+    const size_t w2 = (size_t)kWide * kWide;
+    cudaError_t e;
+    // the same number of chunks for every block (empty ones are zeroed)
+    const int chunk = std::max(512, ((f.rows + 7) / 8 + 31) / 32 * 32);
+    const int chunks = (f.rows + chunk - 1) / chunk;
+    if ((e = cudaMemsetAsync(w.V, 0, sizeof(double) * w2 * blocks * chunks, st)) != cudaSuccess) return e;
+    SplitSet set{w, st};
+    for (int j = 0; j < blocks; ++j) {
+        const int i0 = j * kWide, nb = std::min(kWide, f.count - i0), rows = f.rows - i0;
+        for (int y = 0, k0 = 0; k0 < rows; ++y, k0 += chunk) {
+            SplitProd p{};
+            p.a = p.b = y_vectors(f, i0, nb, k0);
+            p.C = w.V + ((size_t)j * chunks + y) * w2;
+            p.ldc = kWide;
+            p.K = std::min(chunk, rows - k0);
+            if ((e = set.add(p)) != cudaSuccess) return e;
+        }
+    }
+    if ((e = set.run()) != cudaSuccess) return e;
+    k_gram_sum<<<dim3((unsigned)(w2 / 256), blocks), 256, 0, st>>>(w.V, f, chunks, w.G, w.T);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_tform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTformSmem)) !=
+        cudaSuccess)
+        return e;
+    k_tform<<<(f.count + kTB - 1) / kTB, 256, kTformSmem, st>>>(
+        TForm{w.G, w.T, tau, kWide, kWide / kTB, 1, f.count, (long long)w2, (long long)w2, 0});
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    for (int h = kTB; h < kWide && h < f.count; h *= 2)
+        for (int phase = 0; phase < 2; ++phase) {
+            const int tiles = kWide / (2 * h) * (h / 8) * (h / 8);
+            k_tmerge<<<dim3((tiles + 3) / 4, blocks), 128, 0, st>>>(w.G, w.T, w.X, h, phase);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+    for (int j = 0; j < blocks; ++j) {
+        const int i0 = j * kWide, nb = std::min(kWide, f.count - i0), rows = f.rows - i0;
+        SplitProd p{};
+        p.a = y_rows(f, i0, rows);
+        p.b = SplitSide{w.T + j * w2, 0, kWide, 1, nb, 1, 0, 0, 0};
+        p.C = w.V + (size_t)i0 * f.rows;
+        p.ldc = f.rows;
+        p.K = nb;
+        if ((e = set.add(p)) != cudaSuccess) return e;
+    }
+    return set.run();
+}
+
+// C := (I - V Y^T) C (left, C rows x cols) or C (I - Y V^T) (right), with Y
+// the `nb` reflectors given as K-along vectors yk(k0) and V nb columns (ld ldv)
+template <typename YK>
+cudaError_t apply_wide(int left, int rows, int cols, YK yk, int nb, const double *V, int ldv, double *C, int ldc,
+                       const SplitWs &w, cudaStream_t st) {
+    cudaError_t e;
+    const int K = left ? rows : cols, other = left ? cols : rows;
+    // slabs of the untouched dimension that fit the slice scratch and the Z parts
+    const int tb = (nb + 127) / 128;
+    int slab = (other + 127) / 128 * 128;
+    auto parts_of = [&](int s) {
+        const int t = tb * ((s + 127) / 128);
+        return std::max({1, (K + kSplitMostK - 1) / kSplitMostK, std::min({kSplitMax, 152 / std::max(t, 1), K / 256})});
+    };
+    for (; slab > 128; slab = (slab / 2 + 127) / 128 * 128) {
+        const int np = parts_of(slab), kc = ((K + np - 1) / np + 31) / 32 * 32;
+        if ((size_t)np * nb * slab <= w.zcap &&
+            split_scratch((long long)np * nb, (long long)np * slab, kc, (long long)np * tb * (slab / 128)) <= w.slice_bytes &&
+            split_scratch(slab, K, nb, (long long)(slab / 128) * ((K + 127) / 128)) <= w.slice_bytes &&
+            split_scratch(K, slab, nb, (long long)(slab / 128) * ((K + 127) / 128)) <= w.slice_bytes)
+            break;
+    }
+    for (int s0 = 0; s0 < other; s0 += slab) {
+        const int ns = std::min(slab, other - s0);
+        const int np0 = parts_of(ns), kc = ((K + np0 - 1) / np0 + 31) / 32 * 32, np = (K + kc - 1) / kc;
+        double *c = C + (left ? (size_t)s0 * ldc : (size_t)s0);
+        const long long zs = (long long)nb * ns;
+        SplitSet set{w, st};
+        for (int y = 0; y < np; ++y) {
+            SplitProd p{};
+            p.K = std::min(kc, K - y * kc);
+            p.C = w.Z + y * zs;
+            if (left) {        // Z (nb x ns) = Y^T C
+                p.a = yk(y * kc);
+                p.b = SplitSide{c + y * kc, 0, ldc, 0, ns, 1, 0, 0, 0};
+                p.ldc = nb;
+            } else {           // Z (ns x nb) = C Y
+                p.a = SplitSide{c + (size_t)y * kc * ldc, 0, ldc, 1, ns, 1, 0, 0, 0};
+                p.b = yk(y * kc);
+                p.ldc = ns;
+            }
+            if ((e = set.add(p)) != cudaSuccess) return e;
+        }
+        if ((e = set.run()) != cudaSuccess) return e;
+        SplitProd p{};
+        p.K = nb;
+        p.C = c;
+        p.ldc = ldc;
+        p.sub = 1;
+        if (left) {            // C -= V Z
+            p.a = SplitSide{V, 0, ldv, 1, rows, 1, 0, 0, 0};
+            p.b = SplitSide{w.Z, zs, nb, 0, ns, np, 0, 0, 0, nullptr, 0, 0, c, ldc, 1};   // + C's first nb rows
+        } else {               // C -= Z V^T
+            p.a = SplitSide{w.Z, zs, ns, 1, ns, np, 0, 0, 0, nullptr, 0, 0, c, 1, ldc};   // + C's first nb columns
+            p.b = SplitSide{V, 0, ldv, 1, cols, 1, 0, 0, 0};
+        }
+        if ((e = set.add(p)) != cudaSuccess) return e;
+        if ((e = set.run()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// H^T C for one panel of at most kTB reflectors with its T (row-major, ld
+// kTB): Z = Y^T C in split-K parts, W = T^T Z in FP64 (small), C -= Y W
+cudaError_t apply_panel(const Reflectors &f, const double *T, int rows, int cols, double *C, int ldc, double *W,
+                        const SplitWs &w, cudaStream_t st) {
+    const int nb = f.count, tiles = (cols + 127) / 128;
+    int np = std::max(1, std::min({kSplitMax, 152 / tiles, rows / 256}));
+    const int kc = std::max((rows + np - 1) / np + 31, 32) / 32 * 32;
+    np = (rows + kc - 1) / kc;
+    const long long zs = (long long)nb * cols;
+    cudaError_t e;
+    SplitSet set{w, st};
+    for (int y = 0; y < np; ++y) {
+        SplitProd p{};
+        p.a = y_vectors(f, 0, nb, y * kc);
+        p.b = SplitSide{C + y * kc, 0, ldc, 0, cols, 1, 0, 0, 0};
+        p.C = w.Z + y * zs;
+        p.ldc = nb;
+        p.K = std::min(kc, rows - y * kc);
+        if ((e = set.add(p)) != cudaSuccess) return e;
+    }
+    if ((e = set.run()) != cudaSuccess) return e;
+    k_tz<<<(cols + 15) / 16, 256, 0, st>>>(T, nb, 1, w.Z, np, 0, cols, W, C, ldc);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    SplitProd p{};
+    p.a = y_rows(f, 0, rows);
+    p.b = SplitSide{W, 0, nb, 0, cols, 1, 0, 0, 0};
+    p.C = C;
+    p.ldc = ldc;
+    p.K = nb;
+    p.sub = 1;
+    if ((e = set.add(p)) != cudaSuccess) return e;
+    return set.run();
+}
+
+// a bounded wait of the products gave up: the result must not pass for one
+__global__ void k_poison(const int *err, double *C, long long rows, long long cols, long long ld) {
+    if (*err == 0) return;
+    for (long long k = threadIdx.x; k < rows * cols; k += blockDim.x)
+        C[k / rows * ld + k % rows] = __longlong_as_double(0x7ff8000000000000ll);
 }
 
 __global__ void k_fill(double *X, long long rows, long long cols, long long ld, double diag_val) {
@@ -668,6 +1108,14 @@ __global__ void k_fill(double *X, long long rows, long long cols, long long ld, 
     if (k >= rows * cols) return;
     const long long c = k / rows, r = k % rows;
     X[c * ld + r] = (r == c) ? diag_val : 0.0;
+}
+
+// columns of the identity: column c has its one in row r0 + c
+__global__ void k_identity(double *X, long long rows, long long cols, long long ld, int r0) {
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= rows * cols) return;
+    const long long c = k / rows, r = k % rows;
+    X[c * ld + r] = (r == c + r0) ? 1.0 : 0.0;
 }
 
 __global__ void k_copy_upper(const double *A, long long lda, double *R, long long ldr, int n) {
@@ -698,9 +1146,18 @@ int coop_blocks(const void *fn, int threads, size_t smem) {
     return std::max(1, sms * std::max(per, 1));
 }
 
+// panel and block sizes
+constexpr int kDenseBlock = 32;   // b: columns / rows per panel (reflectors per block)
+// reflectors per block when they are applied (back-transformation, explicit
+// Q) in FP64: wider blocks pass over C fewer times (Z = Y^T C and C -= Y W
+// with K = kApplyBlock)
+constexpr int kApplyBlock = kTB;
+constexpr int kWsBlock = kApplyBlock > kDenseBlock ? kApplyBlock : kDenseBlock;   // workspace sizing
+
 // workspace layout of the dense routines (bytes from an aligned base)
 struct DenseWs {
     size_t bar, PW, QW, yraw, tv, xpart, part, Y, Ti, Z, split, split_doubles, res, total;
+    size_t wG, wT, wX, wV, wZ, wZcap, wS, wSbytes;   // split path
 };
 constexpr int kChunkW = 128;   // columns per partial sum of A u
 
@@ -716,14 +1173,35 @@ DenseWs dense_ws(int m, int n, int b, int zcols) {
     w.tv = o; o += al256(sizeof(double) * 4 * (size_t)b);
     w.xpart = o; o += al256(sizeof(double) * (size_t)chunks * m);
     w.part = o; o += al256(sizeof(double) * (size_t)grid * (b + 1));
-    w.Y = o; o += al256(sizeof(double) * (size_t)std::max(m, n) * b);
-    w.Ti = o; o += al256(sizeof(double) * (size_t)b * b);
+    w.Y = o; o += al256(sizeof(double) * (size_t)std::max(m, n) * std::max(b, kWide));
+    w.Ti = o; o += al256(sizeof(double) * (size_t)kTB * (std::max(m, n) + kTB));   // T of every block
     w.Z = o; o += al256(sizeof(double) * (size_t)b * std::max(std::max(m, n), zcols));
-    w.split_doubles = (size_t)16 * b * std::max(std::max(m, n), zcols);
+    w.split_doubles = std::max<size_t>((size_t)16 * b * std::max(std::max(m, n), zcols), (size_t)16 * kTB * kTB);
     w.split = o; o += al256(sizeof(double) * w.split_doubles);
     w.res = o; o += al256(sizeof(double) * resident_scratch_doubles(n));
+    // split path: every block's G, T, X; V and the partial Y^T Y; parts of Z; slices
+    {
+        const size_t D = std::max(std::max(m, n), zcols), blocks = (n + kWide - 1) / kWide, w2 = (size_t)kWide * kWide;
+        w.wG = o; o += al256(sizeof(double) * blocks * w2);
+        w.wT = o; o += al256(sizeof(double) * blocks * w2);
+        w.wX = o; o += al256(sizeof(double) * blocks * w2);
+        w.wV = o; o += al256(sizeof(double) * std::max(D * n, blocks * kGramMost * w2));
+        w.wZcap = std::max<size_t>((size_t)kWide * 2 * (D + 256), (size_t)kWide * 4096);
+        w.wZ = o; o += al256(sizeof(double) * w.wZcap);
+        // enough for whole products up to about 340 MB, then slabs of 128
+        const size_t Dp = (D + 31) / 32 * 32 + 32;
+        const size_t all = 2 * (D + 2 * kWide + 256) * std::max<size_t>(Dp, 544);
+        const size_t most = std::max<size_t>((size_t)24 << 20, (size_t)(2 * kWide + 512) * Dp);
+        w.wSbytes = 14 * std::min(all, most) + (size_t)64 * (D + 4096) + ((size_t)1 << 20);
+        w.wS = o; o += al256(w.wSbytes);
+    }
     w.total = o + 256;
     return w;
+}
+
+SplitWs split_ws(char *ws, const DenseWs &w) {
+    return SplitWs{(double *)(ws + w.wG), (double *)(ws + w.wT), (double *)(ws + w.wX), (double *)(ws + w.wV),
+                   (double *)(ws + w.wZ), w.wZcap, ws + w.wS, w.wSbytes, &((GridBar *)(ws + w.bar))->err};
 }
 
 // the split-K scratch of the calling thread's dense routine
@@ -746,6 +1224,22 @@ cudaError_t launch_coop(const void *fn, int grid, void *args, cudaStream_t st) {
 }  // namespace
 
 // ---------------------------------------------------------------- drivers
+// Blocks of kWide reflectors on the split products, or of kTB in FP64: the
+// split path's fixed cost (about 50 launches) is below one FP64 block's three
+// products from 64 reflectors on (100 x 100: 0.4 ms either way; 333 x 333:
+// 0.64 against 1.39 ms; 600 x 600: 0.88 against 2.3 ms)
+bool use_wide(int refl, int rows, int other) {
+    return refl >= 64 && other >= 64 && rows <= 8 * kSplitMostK;   // Y^T Y in at most kGramMost parts
+}
+// a QR panel's trailing update on the split products: from about 300 x 300
+bool panel_split(int rows, int cols, const SplitWs &w) {
+    return (long long)rows * cols >= 100 * 1000 && rows <= kSplitMax * (kSplitMostK - 64) &&
+           (size_t)cols * 32 * kSplitMax <= w.zcap &&
+           split_scratch((long long)kSplitMax * 32, (long long)kSplitMax * cols, (rows + kSplitMax - 1) / kSplitMax + 64,
+                         (long long)kSplitMax * ((cols + 127) / 128)) <= w.slice_bytes &&
+           split_scratch(rows, cols, 32, (long long)((rows + 127) / 128) * ((cols + 127) / 128)) <= w.slice_bytes;
+}
+
 // Bidiagonalization, Algorithm 1 (m >= n): per panel of b, k_labrd, then the
 // merged rank-(2b) update of the trailing matrix (one product).
 constexpr long long kLabrdWork = 8192;   // trailing-matrix entries per CTA of the panel kernel
@@ -779,6 +1273,21 @@ cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, 
             // blocks, zero in the columns a short last panel does not use, so
             // the whole update is ONE product with K = 2b
             const double *P = (const double *)(ws + w.PW), *Q = (const double *)(ws + w.QW);
+            const SplitWs sw = split_ws(ws, w);
+            const long long tr = ml - nb, tc = nl - nb;
+            if (split_scratch(tr, tc, 2 * b, ((tr + 127) / 128) * ((tc + 127) / 128)) <= sw.slice_bytes) {
+                // V and Y are brought to X's and U's scale by the exponent of
+                // the panel's first diagonal entry (a column norm)
+                SplitProd p{};
+                p.a = SplitSide{P + nb, 0, ml, 1, (int)tr, 1, 0, 0, 0, d + i0, b, 1};
+                p.b = SplitSide{Q + nb, 0, nl, 1, (int)tc, 1, 0, 0, 0, d + i0, b, -1};
+                p.C = A + i0 + nb + (size_t)(i0 + nb) * lda;
+                p.ldc = lda;
+                p.K = 2 * b;
+                p.sub = 1;
+                if ((err = split_products(&p, 1, sw.slices, sw.slice_bytes, sw.err, st)) != cudaSuccess) return err;
+                continue;
+            }
             if ((err = dgemm(0, 1, ml - nb, nl - nb, 2 * b, -1.0, P + nb, ml, Q + nb, nl, 1.0,
                              A + i0 + nb + (size_t)(i0 + nb) * lda, lda, st)) != cudaSuccess)
                 return err;
@@ -801,16 +1310,28 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
     const int grid = std::max(1, std::min(coop_blocks((const void *)k_geqr2, 256, 0), (m + 1023) / 1024));
     double *Y = (double *)(ws + w.Y), *Ti = (double *)(ws + w.Ti), *Z = (double *)(ws + w.Z);
     const int kmax = std::min(m, n);
+    const SplitWs sw = split_ws(ws, w);
     for (int i0 = 0; i0 < kmax; i0 += b) {
         const int nb = std::min(b, kmax - i0), ml = m - i0;
         Geqr2Args a{A + i0 + (size_t)i0 * lda, lda, ml, nb, b, tau + i0, (double *)(ws + w.part), bar};
         if ((err = launch_coop((const void *)k_geqr2, grid, &a, st)) != cudaSuccess) return err;
         if (i0 + nb < n) {
+            const int cols = n - i0 - nb;
+            if (panel_split(ml, cols, sw)) {
+                const Reflectors f{A + i0 + (size_t)i0 * lda, 1, lda, ml, nb};
+                if ((err = form_t(f, tau + i0, Ti, st)) != cudaSuccess) return err;
+                if ((err = apply_panel(f, Ti, ml, cols, A + i0 + (size_t)(i0 + nb) * lda, lda, Z, sw, st)) !=
+                    cudaSuccess)
+                    return err;
+                continue;
+            }
             const long long cnt = (long long)ml * nb;
             k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
-            if ((err = apply_block(1, 1, ml, n - i0 - nb, Y, nb, tau + i0, A + i0 + (size_t)(i0 + nb) * lda, lda, Ti,
-                                   Z, st)) != cudaSuccess)
+            if ((err = form_t(Reflectors{A + i0 + (size_t)i0 * lda, 1, lda, ml, nb}, tau + i0, Ti, st)) != cudaSuccess)
+                return err;
+            if ((err = apply_block(1, 1, ml, n - i0 - nb, Y, nb, Ti, A + i0 + (size_t)(i0 + nb) * lda, lda, Z, st)) !=
+                cudaSuccess)
                 return err;
         }
     }
@@ -834,6 +1355,25 @@ cudaError_t dense_orgqr(int m, int n, int k, double *A, int lda, const double *t
         k_fill<<<(unsigned)((c2 + 255) / 256), 256, 0, st>>>(A + k + (size_t)k * lda, m - k, n - k, lda, 1.0);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
     }
+    if (use_wide(k, m, n)) {
+        const SplitWs sw = split_ws(ws, w);
+        const Reflectors f{A, 1, lda, m, k};
+        if ((err = form_v(f, tau, sw, st)) != cudaSuccess) return err;
+        for (int i0 = (k - 1) / kWide * kWide; i0 >= 0; i0 -= kWide) {
+            const int nb = std::min(kWide, k - i0), ml = m - i0;
+            const long long cnt = (long long)ml * nb, c2 = (long long)m * nb;
+            k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
+            if ((err = cudaGetLastError()) != cudaSuccess) return err;
+            k_identity<<<(unsigned)((c2 + 255) / 256), 256, 0, st>>>(A + (size_t)i0 * lda, m, nb, lda, i0);
+            if ((err = cudaGetLastError()) != cudaSuccess) return err;
+            const Reflectors fy{Y, 1, ml, ml, nb};
+            err = apply_wide(1, ml, n - i0, [&](int k0) { return y_vectors(fy, 0, nb, k0); }, nb,
+                             sw.V + (size_t)i0 * m, m, A + i0 + (size_t)i0 * lda, lda, sw, st);
+            if (err != cudaSuccess) return err;
+        }
+        return cudaSuccess;
+    }
+    if ((err = form_t(Reflectors{A, 1, lda, m, k}, tau, Ti, st)) != cudaSuccess) return err;
     const int last = ((k - 1) / b) * b;
     for (int i0 = last; i0 >= 0; i0 -= b) {
         const int nb = std::min(b, k - i0), ml = m - i0;
@@ -846,7 +1386,7 @@ cudaError_t dense_orgqr(int m, int n, int k, double *A, int lda, const double *t
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         k_fill<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(A + i0 + (size_t)i0 * lda, ml, nb, lda, 1.0);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        if ((err = apply_block(1, 0, ml, n - i0, Y, nb, tau + i0, A + i0 + (size_t)i0 * lda, lda, Ti, Z, st)) !=
+        if ((err = apply_block(1, 0, ml, n - i0, Y, nb, Ti + (size_t)i0 * kTB, A + i0 + (size_t)i0 * lda, lda, Z, st)) !=
             cudaSuccess)
             return err;
     }
@@ -862,20 +1402,37 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
     SplitScope split_scope(ws, w);
     double *Y = (double *)(ws + w.Y), *Ti = (double *)(ws + w.Ti), *Z = (double *)(ws + w.Z);
     cudaError_t err = cudaSuccess;
+    const int refl = vect == 0 ? n : n - 1;
+    if (use_wide(refl, vect == 0 ? m : n - 1, cdim)) {
+        const SplitWs sw = split_ws(ws, w);
+        const Reflectors f = vect == 0 ? Reflectors{A, 1, lda, m, n} : Reflectors{A + lda, lda, 1, n - 1, n - 1};
+        if ((err = form_v(f, tau, sw, st)) != cudaSuccess) return err;
+        for (int i0 = (refl - 1) / kWide * kWide; i0 >= 0; i0 -= kWide) {
+            const int nb = std::min(kWide, refl - i0), ry = f.rows - i0;
+            auto yk = [&](int k0) { return y_vectors(f, i0, nb, k0); };
+            const double *V = sw.V + (size_t)i0 * f.rows;
+            err = vect == 0 ? apply_wide(1, ry, cdim, yk, nb, V, f.rows, C + i0, ldc, sw, st)
+                            : apply_wide(0, cdim, ry, yk, nb, V, f.rows, C + (size_t)(i0 + 1) * ldc, ldc, sw, st);
+            if (err != cudaSuccess) return err;
+        }
+        return cudaSuccess;
+    }
     if (vect == 0) {
+        if ((err = form_t(Reflectors{A, 1, lda, m, n}, tau, Ti, st)) != cudaSuccess) return err;
         const int last = ((n - 1) / b) * b;
         for (int i0 = last; i0 >= 0; i0 -= b) {
             const int nb = std::min(b, n - i0), ml = m - i0;
             const long long cnt = (long long)ml * nb;
             k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
-            if ((err = apply_block(1, 0, ml, cdim, Y, nb, tau + i0, C + i0, ldc, Ti, Z, st)) != cudaSuccess)
+            if ((err = apply_block(1, 0, ml, cdim, Y, nb, Ti + (size_t)i0 * kTB, C + i0, ldc, Z, st)) != cudaSuccess)
                 return err;
         }
         return cudaSuccess;
     }
     if (n < 2) return cudaSuccess;
     const int nr = n - 1;   // row reflectors G_0 .. G_{n-2}, acting on columns 1..n-1
+    if ((err = form_t(Reflectors{A + lda, lda, 1, n - 1, nr}, tau, Ti, st)) != cudaSuccess) return err;
     const int last = ((nr - 1) / b) * b;
     for (int i0 = last; i0 >= 0; i0 -= b) {
         const int nb = std::min(b, nr - i0), ny = n - 1 - i0;
@@ -883,7 +1440,7 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
         // Y[r][j] = u_{i0+j} at column i0 + 1 + r: row i0 + j of A from column i0 + 1
         k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ny, nb, A + i0 + (size_t)(i0 + 1) * lda, lda, 1);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        if ((err = apply_block(0, 1, cdim, ny, Y, nb, tau + i0, C + (size_t)(i0 + 1) * ldc, ldc, Ti, Z, st)) !=
+        if ((err = apply_block(0, 1, cdim, ny, Y, nb, Ti + (size_t)i0 * kTB, C + (size_t)(i0 + 1) * ldc, ldc, Z, st)) !=
             cudaSuccess)
             return err;
     }
@@ -898,6 +1455,10 @@ cudaError_t dense_read_err(char *ws, int *info, cudaStream_t st) {
     k_read_err<<<1, 1, 0, st>>>((const GridBar *)(ws + dense_ws(1, 1, 1, 1).bar), info);
     return cudaGetLastError();
 }
+cudaError_t dense_poison(char *ws, double *C, int rows, int cols, int ld, cudaStream_t st) {
+    k_poison<<<1, 1024, 0, st>>>(&((const GridBar *)(ws + dense_ws(1, 1, 1, 1).bar))->err, C, rows, cols, ld);
+    return cudaGetLastError();
+}
 cudaError_t dense_copy_upper(const double *A, int lda, double *R, int ldr, int n, cudaStream_t st) {
     const long long cnt = (long long)n * n;
     k_copy_upper<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(A, lda, R, ldr, n);
@@ -909,11 +1470,29 @@ cudaError_t dense_zero_rows(double *X, int ld, int r0, int r1, int cols, cudaStr
     k_zero_rows<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(X, ld, r0, r1, cols);
     return cudaGetLastError();
 }
-cudaError_t dense_dgemm(int ta, int tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B,
-                        int ldb, double beta, double *C, int ldc, cudaStream_t st) {
-    return dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, st);
+// C (m x n) = A (m x n, lda) B (n x n, ld n), in row slabs that fit the slices
+cudaError_t dense_product(int m, int n, const double *A, int lda, const double *B, double *C, int ldc, char *ws,
+                          cudaStream_t st) {
+    const DenseWs w = dense_ws(m, n, kWsBlock, std::max(m, n));
+    const SplitWs sw = split_ws(ws, w);
+    auto fits = [&](int r) {
+        return split_scratch(r, n, n, (long long)((r + 127) / 128) * ((n + 127) / 128)) <= sw.slice_bytes;
+    };
+    int slab = m;
+    while (slab > 128 && !fits(slab)) slab = (slab / 2 + 127) / 128 * 128;
+    if (n < 64 || n > kSplitMostK || !fits(slab))
+        return dgemm(0, 0, m, n, n, 1.0, A, lda, B, n, 0.0, C, ldc, st);
+    for (int r0 = 0; r0 < m; r0 += slab) {
+        SplitProd p{};
+        p.a = SplitSide{A + r0, 0, lda, 1, std::min(slab, m - r0), 1, 0, 0, 0};
+        p.b = SplitSide{B, 0, n, 0, n, 1, 0, 0, 0};
+        p.C = C + r0;
+        p.ldc = ldc;
+        p.K = n;
+        if (cudaError_t e = split_products(&p, 1, sw.slices, sw.slice_bytes, sw.err, st)) return e;
+    }
+    return cudaSuccess;
 }
-
 
 }  // namespace bdc
 
@@ -922,12 +1501,6 @@ using namespace bdc;
 
 namespace {
 
-constexpr int kDenseBlock = 32;   // b: columns / rows per panel (reflectors per block)
-// reflectors per block when they are applied (back-transformation, explicit
-// Q): wider blocks pass over C fewer times (Z = Y^T C and C -= Y W with
-// K = kApplyBlock); T^{-1} (kApplyBlock^2 doubles) stays in shared memory
-constexpr int kApplyBlock = 64;
-constexpr int kWsBlock = kApplyBlock > kDenseBlock ? kApplyBlock : kDenseBlock;   // workspace sizing
 constexpr double kQrRatio = 1.6;  // m >= 1.6 n: QR first (Sec. 4.3)
 
 char *align_ws(void *work) { return (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255); }
@@ -993,8 +1566,11 @@ int bdc_ormbr(int vect, int m, int n, const double *A, int lda, const double *ta
     if (!work) return -10;
     const size_t need = dense_ws_bytes(std::max(m, cdim), std::max(n, cdim), kWsBlock) + 512;
     if (lwork < need) return -11;
-    return note_cuda(dense_ormbr(vect, m, n, A, lda, tau, C, ldc, cdim, kApplyBlock, align_ws(work),
-                                 (cudaStream_t)stream));
+    cudaStream_t st = (cudaStream_t)stream;
+    char *ws = align_ws(work);
+    if (int r = note_cuda(dense_clear_err(ws, st))) return r;
+    if (int r = note_cuda(dense_ormbr(vect, m, n, A, lda, tau, C, ldc, cdim, kApplyBlock, ws, st))) return r;
+    return note_cuda(dense_poison(ws, C, vect == 0 ? m : cdim, vect == 0 ? cdim : n, ldc, st));
 }
 
 size_t bdc_ormbr_workspace(int m, int n, int cdim) {
@@ -1035,7 +1611,11 @@ int bdc_orgqr(int m, int n, double *A, int lda, const double *tau, void *work, s
     if (n == 0) return 0;
     if (!work) return -6;
     if (lwork < bdc_geqrf_workspace(m, n)) return -7;
-    return note_cuda(dense_orgqr(m, n, n, A, lda, tau, kApplyBlock, align_ws(work), (cudaStream_t)stream));
+    cudaStream_t st = (cudaStream_t)stream;
+    char *ws = align_ws(work);
+    if (int r = note_cuda(dense_clear_err(ws, st))) return r;
+    if (int r = note_cuda(dense_orgqr(m, n, n, A, lda, tau, kApplyBlock, ws, st))) return r;
+    return note_cuda(dense_poison(ws, A, m, n, lda, st));
 }
 
 size_t bdc_gesvd_workspace(int m, int n, const bdc_opts *o) {
@@ -1079,7 +1659,7 @@ int bdc_gesvd(int m, int n, double *A, int lda, double *S, double *U, int ldu, d
         if ((rc = bdc_svd_ex(n, d, e, UR, S, VT, n, ldvt, o, ws + L.bdc, lwb, d_info, stream))) return rc;
         if ((rc = note_cuda(dense_ormbr(0, n, n, R, n, tq, UR, n, n, kApplyBlock, dws, st)))) return rc;
         if ((rc = note_cuda(dense_ormbr(1, n, n, R, n, tp, VT, ldvt, n, kApplyBlock, dws, st)))) return rc;
-        if ((rc = note_cuda(dense_dgemm(0, 0, m, n, n, 1.0, A, lda, UR, n, 0.0, U, ldu, st)))) return rc;
+        if ((rc = note_cuda(dense_product(m, n, A, lda, UR, U, ldu, dws, st)))) return rc;
     } else {
         if ((rc = note_cuda(dense_gebrd(m, n, A, lda, d, e, tq, tp, b, dws, st)))) return rc;
         if ((rc = bdc_svd_ex(n, d, e, U, S, VT, ldu, ldvt, o, ws + L.bdc, lwb, d_info, stream))) return rc;

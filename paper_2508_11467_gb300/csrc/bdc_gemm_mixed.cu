@@ -43,7 +43,7 @@
 #include <mutex>
 #include <vector>
 
-#include "bdc_internal.cuh"
+#include "bdc_dense.cuh"
 
 namespace bdc {
 
@@ -53,7 +53,8 @@ struct MixProb {
     int tile0;    // first tile of the product in the launch grid
     int tilesN;   // tiles along N (for the host-known bound Nmax)
     int Mmax, Nmax;
-    int pad0, pad1;
+    int sub;      // 1: C -= A B (the merge products store C = A B)
+    int pad1;
 };
 
 namespace {
@@ -434,14 +435,22 @@ __global__ void __launch_bounds__(256) k_slice_b(const GemmProb *__restrict__ pr
 //            accumulator buffers alternate per stage.  Adds 2^(E+F-16) SL to C.
 //   MODE_X3  BF16x3: (hi, lo) pairs (0,0), (0,1), (1,0) in one accumulator
 //            over the whole K.  Writes C.
-enum { MODE_E = 0, MODE_L = 1, MODE_X3 = 2 };
+//   MODE_LW  MODE_L for operands whose rows hold one entry far above the rest
+//            (a reflector's unit entry over entries of 1 / sqrt(rows)): group S
+//            as well (the pairs i + j = S + 2 whose slices exist), and group 4
+//            summed over the stages in 32-bit integers (below 2^22 a stage: K
+//            up to 16384 of them).  MODE_L's dropped pairs and FP32 sums are
+//            each a few 1e-16 sqrt(K / 333) of max|A_r| max|B_c| for S = 7, far
+//            above an FP64 product's error on such operands.
+//   MODE_EW  MODE_E that also takes C -= A B (MODE_LW does too).
+enum { MODE_E = 0, MODE_L = 1, MODE_X3 = 2, MODE_LW = 3, MODE_EW = 4 };
 
 // Slices loaded per stage (MODE_E multiplies slices 1..4 only), bytes per
 // stage, and ring depth: as many stages as fit in ~200 KB of shared memory,
 // 2 to 4 (a deeper ring hides more TMA latency; the operand traffic per
 // MMA is what bounds these small-K products)
 template <int S, int MODE>
-__host__ __device__ constexpr int stage_slices() { return (MODE == MODE_E && S > 4) ? 4 : S; }
+__host__ __device__ constexpr int stage_slices() { return ((MODE == MODE_E || MODE == MODE_EW) && S > 4) ? 4 : S; }
 template <int S, int MODE>
 __host__ __device__ constexpr int stage_bytes() { return 2 * stage_slices<S, MODE>() * TM * TK * 2; }
 template <int S, int MODE>
@@ -589,7 +598,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                         }
                         umma_commit(&empty[buf]);
                         if (s == nk - 1) { umma_commit(&accfull[0]); ++nA; }
-                    } else if constexpr (MODE == MODE_L) {
+                    } else if constexpr (MODE == MODE_L || MODE == MODE_LW) {
                         const int b = G & 1;                   // accumulator buffer of this stage
                         if (G >= 2) {
                             if (!mbar_wait(&accempty[b], ((G >> 1) - 1) & 1, err, abort_flag, wait_ns)) { ok = false; break; }
@@ -604,7 +613,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                                     mma(c4, i, 4 - i, kk, (kk == 0 && i == 0) ? 0u : 1u);
                             bool first = true;
 #pragma unroll
-                            for (int g = 5; g <= S - 1; ++g)
+                            for (int g = 5; g <= (MODE == MODE_LW ? S : S - 1); ++g)
 #pragma unroll
                                 for (int i = 0; i <= g; ++i) {
                                     const int j = g - i;
@@ -693,7 +702,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                     cml[h2] = cok ? (pr.cmap ? pr.cmap[col] : col) : 0;
                 }
             };
-            if constexpr (MODE == MODE_E) {
+            if constexpr (MODE == MODE_E || MODE == MODE_EW) {
                 // unsigned: the magic offsets wrap modulo 2^64 and cancel exactly at the end
                 unsigned long long L[CPT];
 #pragma unroll
@@ -760,20 +769,34 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                             F[i] = __shfl_sync(0xffffffffu, fbl[k >> 5], k & 31);
                             cj[i] = __shfl_sync(0xffffffffu, cml[k >> 5], k & 31);
                         }
+                        double cold[8];                    // C -= A B: the old entries, loaded together
+                        if constexpr (MODE == MODE_EW) {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                cold[i] = (mx.sub && rowok && c0 + 8 * cb + i < pr.N) ? pr.C[cj[i] * ldc + row] : 0.0;
+                        }
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const int k = 8 * cb + i;
-                            if (rowok && c0 + k < pr.N)
-                                pr.C[cj[i] * ldc + row] = i64_ldexp((long long)(L[k] - corr), Er + F[i] - 40);
+                            if (rowok && c0 + k < pr.N) {
+                                const double v = i64_ldexp((long long)(L[k] - corr), Er + F[i] - 40);
+                                if constexpr (MODE == MODE_EW) pr.C[cj[i] * ldc + row] = mx.sub ? cold[i] - v : v;
+                                else pr.C[cj[i] * ldc + row] = v;
+                            }
                         }
                     }
                 }
-            } else if constexpr (MODE == MODE_L) {
+            } else if constexpr (MODE == MODE_L || MODE == MODE_LW) {
                 // group 4 is exact per stage (and weighs <= 2^-32), groups >= 5 weigh
                 // <= 2^-40: both are summed over the stages in FP32 registers
                 float SL[CPT];
+                int I4[MODE == MODE_LW ? CPT : 1];     // MODE_LW: group 4 in units of 2^-32, exact over the stages
 #pragma unroll
                 for (int i = 0; i < CPT; ++i) SL[i] = 0.f;
+                if constexpr (MODE == MODE_LW) {
+#pragma unroll
+                    for (int i = 0; i < CPT; ++i) I4[i] = 0;
+                }
                 // the final read-modify-write of C waits on its loads while the
                 // next tile's stages wait on this warp: pull this warp's 32 rows of
                 // its CPT columns into L2 now (lane = column, 256 B each), while
@@ -804,7 +827,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                         tmem_wait_ld();
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            SL[8 * cb + i] += v4[i];
+                            if constexpr (MODE == MODE_LW)
+                                I4[8 * cb + i] += __float_as_int(fmaf(v4[i], 4294967296.0f, 12582912.0f)) - 0x4B400000;
+                            else
+                                SL[8 * cb + i] += v4[i];
                             if (S > 5) SL[8 * cb + i] += vl[i];
                         }
                     }
@@ -830,7 +856,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const int k = 8 * cb + i;
-                            if (rowok && c0 + k < pr.N) pr.C[off[i] + row] = cv[i] + f32_ldexp(SL[k], Er + F[i] - 16);
+                            double v;
+                            if constexpr (MODE == MODE_LW)
+                                v = i64_ldexp(((long long)I4[k] << 16) + __float2ll_rn(SL[k] * 0x1p48f), Er + F[i] - 64);
+                            else
+                                v = f32_ldexp(SL[k], Er + F[i] - 16);
+                            if (MODE == MODE_LW && mx.sub) v = -v;
+                            if (rowok && c0 + k < pr.N) pr.C[off[i] + row] = cv[i] + v;
                         }
                     }
                 }
@@ -954,6 +986,37 @@ int sm_count() {
     return n;
 }
 
+template <int S, int MODE>
+constexpr size_t mma_smem() { return (size_t)stage_bytes<S, MODE>() * stage_count<S, MODE>() + 1024 + 256; }
+
+// the kernels' shared memory opted into once per process
+template <int S, bool EXACT>
+cudaError_t mma_attributes() {
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(once, [&] {
+        if constexpr (EXACT) {
+            attr_err = cudaFuncSetAttribute(k_mma<S, MODE_E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)mma_smem<S, MODE_E>());
+            if (attr_err == cudaSuccess)
+                attr_err = cudaFuncSetAttribute(k_mma<S, MODE_L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)mma_smem<S, MODE_L>());
+            if constexpr (S == 7) {
+                if (attr_err == cudaSuccess)
+                    attr_err = cudaFuncSetAttribute(k_mma<S, MODE_LW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)mma_smem<S, MODE_LW>());
+                if (attr_err == cudaSuccess)
+                    attr_err = cudaFuncSetAttribute(k_mma<S, MODE_EW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)mma_smem<S, MODE_EW>());
+            }
+        } else {
+            attr_err = cudaFuncSetAttribute(k_mma<S, MODE_X3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)mma_smem<S, MODE_X3>());
+        }
+    });
+    return attr_err;
+}
+
 template <int S, bool EXACT>
 cudaError_t run_mixed(const GemmProb *probs, int nprobs, const std::vector<MixProb> &hm, int rowsA, int colsB,
                       int Kld, char *scratch, const Layout &L, int *err, int phase, cudaStream_t st) {
@@ -1032,23 +1095,8 @@ cudaError_t run_mixed(const GemmProb *probs, int nprobs, const std::vector<MixPr
         return cudaErrorInvalidValue;
     if (EXACT && (!make_map(&mae, As, rowsA, Kld, S, SE, TM) || !make_map(&mbe, Bs, colsB, Kld, S, SE, TNX)))
         return cudaErrorInvalidValue;
-    auto smem_of = [](int stage, int count) { return (size_t)stage * count + 1024 + 256; };
-    const size_t smemE = smem_of(stage_bytes<S, MODE_E>(), stage_count<S, MODE_E>());
-    const size_t smemL = smem_of(stage_bytes<S, MODE_L>(), stage_count<S, MODE_L>());
-    const size_t smemX = smem_of(stage_bytes<S, MODE_X3>(), stage_count<S, MODE_X3>());
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [&] {
-        if constexpr (EXACT) {
-            attr_err = cudaFuncSetAttribute(k_mma<S, MODE_E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemE);
-            if (attr_err == cudaSuccess)
-                attr_err =
-                    cudaFuncSetAttribute(k_mma<S, MODE_L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemL);
-        } else {
-            attr_err = cudaFuncSetAttribute(k_mma<S, MODE_X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemX);
-        }
-    });
-    if (attr_err != cudaSuccess) return attr_err;
+    const size_t smemE = mma_smem<S, MODE_E>(), smemL = mma_smem<S, MODE_L>(), smemX = mma_smem<S, MODE_X3>();
+    if ((e = mma_attributes<S, EXACT>()) != cudaSuccess) return e;
     if (tiles <= 0) return cudaSuccess;
     StageScope mma_scope(st, BDC_STAGE_GEMM, (EXACT && S > 4) ? 3 : 2, 0.0);
     const unsigned long long wait_ns = test_wait_ns();
@@ -1123,5 +1171,262 @@ cudaError_t launch_gemm_mixed(const GemmProb *probs, int nprobs, const int *Mmax
                                  st);
 }
 
+
+// ------------------------------------------------ products of the dense path
+// The same slicing and kernels for products whose sizes the host knows (the
+// block reflectors and trailing updates of bdc_dense.cu): either operand
+// stored along K or across it, optionally as the unit lower trapezoid of a
+// reflector panel, summed from split-K parts; C = A B or C -= A B.  On GB300
+// mma.sync FP64 runs at 1.67 multiply-adds a clock and SM (the plain FMA's
+// rate, 1.05 TFLOP/s in all), the 34 slice products at 128 x 128 x 32 in
+// about 3.2 us a tile: 50 times the FP64 rate.
+namespace {
+
+constexpr int DS = 7;                      // slices: 56 bits below the row's maximum
+
+struct SplitTab {
+    SplitProd p[kSplitMax];
+    int count;
+};
+
+// tables of the launch: products, exponent maxima cleared, tile list
+__global__ void __launch_bounds__(256) k_split_tab(const __grid_constant__ SplitTab t, GemmProb *probs, MixProb *mix,
+                                                   unsigned long long *maxA, unsigned long long *maxB, int2 *tiles,
+                                                   int *ntiles) {
+    int base = 0;
+    for (int q = 0; q < t.count; ++q) {
+        const SplitProd &p = t.p[q];
+        const int tm = (p.a.n + TM - 1) / TM, tn = (p.b.n + TNX - 1) / TNX, cnt = tm * tn;
+        if (blockIdx.x == 0) {
+            if (threadIdx.x == 0) {
+                probs[q] = GemmProb{p.a.p, p.b.p, p.C, 0, 0, p.ldc, p.a.n, p.b.n, p.K, nullptr};
+                MixProb m{};
+                m.a_row0 = p.a.row0; m.b_col0 = p.b.row0; m.tile0 = base; m.tilesN = tn;
+                m.Mmax = p.a.n; m.Nmax = p.b.n; m.sub = p.sub;
+                mix[q] = m;
+            }
+        }
+        constexpr int G = 8;               // bands of 8 row blocks, as in k_tile_list
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
+            const int band = k / (G * tn), in_band = k % (G * tn);
+            const int bm0 = band * G, bsz = min(G, tm - bm0);
+            tiles[base + k] = make_int2(q, ((bm0 + in_band % bsz) << 16) | (in_band / bsz));
+        }
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.a.n; k += gridDim.x * blockDim.x)
+            maxA[p.a.row0 + k] = 0ull;
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.b.n; k += gridDim.x * blockDim.x)
+            maxB[p.b.row0 + k] = 0ull;
+        base += cnt;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ntiles = base;
+}
+
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// entry k of vector v
+__device__ __forceinline__ double split_at(const SplitSide &s, int v, int k) {
+    if (s.mask) {                          // reflector panel
+        const int r = (s.mask == 1 ? k : v) + s.moff, c = s.mask == 1 ? v : k;
+        if (r <= c) return (r == c && s.mask == 2) ? 1.0 : 0.0;
+    }
+    const double *p = s.p + (s.tr ? (size_t)k * s.ld + v : (size_t)v * s.ld + k);
+    double x = *p;
+    for (int q = 1; q < s.parts; ++q) x += p[(size_t)q * s.pstride];
+    if (s.add) x += s.add[v * s.add_v + k * s.add_k];
+    if (s.ref && k < s.kref) {             // times 2^(+-e), 2^e <= |*ref| < 2^(e+1)
+        const int e = (int)((mag_bits(*s.ref) >> 52)) - 1023;
+        if (e > -1023 && e < 1024) x = ldexp_safe(x, s.rsign * e);
+    }
+    return x;
+}
+// vectors stored along K: a warp each, two neighbouring entries per lane (the
+// second pass finds them in cache); grid (vectors / 8, products, sides)
+__global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ SplitTab t, __nv_bfloat16 *As,
+                                                     __nv_bfloat16 *Bs, int *Ea, int *Fb, int rowsA, int colsB,
+                                                     int Kld) {
+    const SplitProd &p = t.p[blockIdx.y];
+    const SplitSide s = blockIdx.z ? p.b : p.a;
+    const int v = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (s.tr || v >= s.n) return;
+    const int K = p.K, Kend = (K + TK - 1) / TK * TK;
+    unsigned long long m = 0;
+#pragma unroll 4
+    for (int k = 2 * lane; k < K; k += 64) {
+        m = max(m, mag_bits(split_at(s, v, k)));
+        if (k + 1 < K) m = max(m, mag_bits(split_at(s, v, k + 1)));
+    }
+    for (int o = 16; o > 0; o >>= 1) m = max(m, (unsigned long long)__shfl_xor_sync(0xffffffffu, m, o));
+    const int E = scale_exp(m);
+    const int rows = blockIdx.z ? colsB : rowsA;
+    if (lane == 0) (blockIdx.z ? Fb : Ea)[s.row0 + v] = E;
+    __nv_bfloat16 *dst = (blockIdx.z ? Bs : As) + (size_t)(s.row0 + v) * Kld;
+#pragma unroll 2
+    for (int k = 2 * lane; k < Kend; k += 64) {
+        const double x0 = k < K ? split_at(s, v, k) : 0.0, x1 = k + 1 < K ? split_at(s, v, k + 1) : 0.0;
+        int n0[DS], n1[DS];
+        digits<DS>(x0, E, n0);
+        digits<DS>(x1, E, n1);
+#pragma unroll
+        for (int q = 0; q < DS; ++q)
+            *reinterpret_cast<__nv_bfloat162 *>(dst + (size_t)q * rows * Kld + k) =
+                __nv_bfloat162(slice_bf16(n0[q], q), slice_bf16(n1[q], q));
+    }
+}
+
+// vectors stored across K: maxima of 32 vectors over 128 of K per CTA
+// (an ordered-integer maximum: the result does not depend on the order);
+// grid (vectors / 32, K / 128, products x sides)
+__global__ void __launch_bounds__(256) k_split_max(const __grid_constant__ SplitTab t, unsigned long long *maxA,
+                                                   unsigned long long *maxB) {
+    __shared__ unsigned long long sm[8][33];
+    const SplitProd &p = t.p[blockIdx.z >> 1];
+    const SplitSide s = (blockIdx.z & 1) ? p.b : p.a;
+    const int tr = threadIdx.x & 31, tc = threadIdx.x >> 5, v = blockIdx.x * 32 + tr;
+    if (!s.tr || blockIdx.x * 32 >= s.n || blockIdx.y * 128 >= p.K) return;
+    unsigned long long m = 0;
+    if (v < s.n) {
+#pragma unroll 8
+        for (int q = 0; q < 16; ++q) {
+            const int k = blockIdx.y * 128 + tc + 8 * q;
+            if (k < p.K) m = max(m, mag_bits(split_at(s, v, k)));
+        }
+    }
+    sm[tc][tr] = m;
+    __syncthreads();
+    if (tc == 0 && v < s.n) {
+        for (int q = 1; q < 8; ++q) m = max(m, sm[q][tr]);
+        atomicMax(((blockIdx.z & 1) ? maxB : maxA) + s.row0 + v, m);
+    }
+}
+
+// ... and their digits, 32 vectors x 64 of K per CTA transposed through
+// shared memory; grid (vectors / 32, K / 64, products x sides)
+__global__ void __launch_bounds__(256) k_split_across(const __grid_constant__ SplitTab t, __nv_bfloat16 *As,
+                                                      __nv_bfloat16 *Bs, const unsigned long long *maxA,
+                                                      const unsigned long long *maxB, int *Ea, int *Fb, int rowsA,
+                                                      int colsB, int Kld) {
+    __shared__ __nv_bfloat16 tile[DS][32][72];
+    const SplitProd &p = t.p[blockIdx.z >> 1];
+    const int side = blockIdx.z & 1;
+    const SplitSide s = side ? p.b : p.a;
+    const int tr = threadIdx.x & 31, tc = threadIdx.x >> 5, v = blockIdx.x * 32 + tr;
+    const int K = p.K, Kend = (K + TK - 1) / TK * TK, k0 = blockIdx.y * 64;
+    if (!s.tr || blockIdx.x * 32 >= s.n || k0 >= Kend) return;
+    const int E = v < s.n ? scale_exp((side ? maxB : maxA)[s.row0 + v]) : 0;
+    if (blockIdx.y == 0 && tc == 0 && v < s.n) (side ? Fb : Ea)[s.row0 + v] = E;
+    double x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int k = k0 + tc + 8 * q;
+        x[q] = (v < s.n && k < K) ? split_at(s, v, k) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        int n[DS];
+        digits<DS>(x[q], E, n);
+#pragma unroll
+        for (int z = 0; z < DS; ++z) tile[z][tr][tc + 8 * q] = slice_bf16(n[z], z);
+    }
+    __syncthreads();
+    const int rows = side ? colsB : rowsA;
+    __nv_bfloat16 *dst = side ? Bs : As;
+    for (int idx = threadIdx.x; idx < DS * 256; idx += 256) {
+        const int z = idx >> 8, rr = (idx >> 3) & 31, seg = idx & 7;
+        if (blockIdx.x * 32 + rr < s.n && k0 + seg * 8 < Kend)
+            *reinterpret_cast<uint4 *>(dst + ((size_t)z * rows + s.row0 + blockIdx.x * 32 + rr) * Kld + k0 + seg * 8) =
+                *reinterpret_cast<const uint4 *>(&tile[z][rr][seg * 8]);
+    }
+}
+
+struct SplitLayout {
+    size_t A, B, E, F, mA, mB, probs, mix, tiles, total;
+};
+SplitLayout split_layout(long long rowsA, long long colsB, int Kld, long long tiles) {
+    SplitLayout L{};
+    size_t o = 0;
+    L.A = o; o += align256((size_t)DS * rowsA * Kld * 2);
+    L.B = o; o += align256((size_t)DS * colsB * Kld * 2);
+    L.E = o; o += align256(sizeof(int) * rowsA);
+    L.F = o; o += align256(sizeof(int) * colsB);
+    L.mA = o; o += align256(8 * rowsA);
+    L.mB = o; o += align256(8 * colsB);
+    L.probs = o; o += align256(sizeof(GemmProb) * kSplitMax) + 256;
+    L.mix = o; o += align256(sizeof(MixProb) * kSplitMax);
+    L.tiles = o; o += align256(sizeof(int2) * tiles);
+    L.total = o;
+    return L;
+}
+
+}  // namespace
+
+size_t split_scratch(long long rowsA, long long colsB, int K, long long tiles) {
+    return split_layout(rowsA + TM, colsB + TNX, (K + TK - 1) / TK * TK, tiles).total + 256;
+}
+
+cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t bytes, int *err, cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+    if (count > kSplitMax) return cudaErrorInvalidValue;
+    SplitTab t{};
+    long long rows = 0, cols = 0, tiles = 0;
+    int kmax = 1, mv = 0, mt = 0, kt = 0;
+    for (int q = 0; q < count; ++q) {
+        SplitProd &p = prods[q];
+        if (p.a.n <= 0 || p.b.n <= 0 || p.K <= 0 || p.K > kSplitMostK) return cudaErrorInvalidValue;
+        p.a.row0 = (int)rows;
+        p.b.row0 = (int)cols;
+        rows += p.a.n;
+        cols += p.b.n;
+        kmax = std::max(kmax, p.K);
+        tiles += (long long)((p.a.n + TM - 1) / TM) * ((p.b.n + TNX - 1) / TNX);
+        for (const SplitSide *s : {&p.a, &p.b}) {
+            if (s->tr) { mt = std::max(mt, s->n); kt = std::max(kt, p.K); }
+            else mv = std::max(mv, s->n);
+        }
+        t.p[q] = p;
+    }
+    t.count = count;
+    const int Kld = (kmax + TK - 1) / TK * TK, ra = (int)rows + TM, cb = (int)cols + TNX;
+    const SplitLayout L = split_layout(ra, cb, Kld, tiles);
+    char *sc = (char *)(((uintptr_t)scratch + 255) & ~(uintptr_t)255);
+    if (L.total + 256 > bytes) return cudaErrorInvalidValue;
+    __nv_bfloat16 *As = (__nv_bfloat16 *)(sc + L.A), *Bs = (__nv_bfloat16 *)(sc + L.B);
+    int *E = (int *)(sc + L.E), *F = (int *)(sc + L.F);
+    unsigned long long *mA = (unsigned long long *)(sc + L.mA), *mB = (unsigned long long *)(sc + L.mB);
+    GemmProb *probs = (GemmProb *)(sc + L.probs);
+    MixProb *mix = (MixProb *)(sc + L.mix);
+    int2 *tl = (int2 *)(sc + L.tiles);
+    int *nt = (int *)(sc + L.mix - 256);
+    CUtensorMap ma, mb, mae, mbe;
+    constexpr int SE = stage_slices<DS, MODE_EW>();
+    if (!make_map(&ma, As, ra, Kld, DS, DS, TM) || !make_map(&mb, Bs, cb, Kld, DS, DS, TNX) ||
+        !make_map(&mae, As, ra, Kld, DS, SE, TM) || !make_map(&mbe, Bs, cb, Kld, DS, SE, TNX))
+        return cudaErrorInvalidValue;
+    cudaError_t e;
+    if ((e = mma_attributes<DS, true>()) != cudaSuccess) return e;
+    const int most = (int)std::max<long long>(std::max(rows, cols), tiles);
+    k_split_tab<<<std::min((most + 255) / 256, 64), 256, 0, st>>>(t, probs, mix, mA, mB, tl, nt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (mv > 0) {
+        k_split_along<<<dim3((mv + 7) / 8, count, 2), 256, 0, st>>>(t, As, Bs, E, F, ra, cb, Kld);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (mt > 0) {
+        k_split_max<<<dim3((mt + 31) / 32, (kt + 127) / 128, 2 * count), 256, 0, st>>>(t, mA, mB);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_split_across<<<dim3((mt + 31) / 32, (kt + 63) / 64, 2 * count), 256, 0, st>>>(t, As, Bs, mA, mB, E, F, ra, cb,
+                                                                                       Kld);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    const int grid = (int)std::min<long long>(tiles, sm_count());
+    const unsigned long long wait_ns = test_wait_ns();
+    k_mma<DS, MODE_EW><<<grid, THREADS, mma_smem<DS, MODE_EW>(), st>>>(mae, mbe, probs, mix, count, E, F, err, tl, nt,
+                                                                        wait_ns, 0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_mma<DS, MODE_LW><<<grid, THREADS, mma_smem<DS, MODE_LW>(), st>>>(ma, mb, probs, mix, count, E, F, err, tl, nt,
+                                                                        wait_ns, 0);
+    return cudaGetLastError();
+}
 
 }  // namespace bdc

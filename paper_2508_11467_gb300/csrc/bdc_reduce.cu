@@ -54,13 +54,12 @@ __device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
 // convention): beta = -sign(alpha) ||x||, tau = (beta - alpha) / beta, the
 // vector's tail scaled by 1 / (alpha - beta); sig2 = 0 gives tau = 0 (H = I).
 // On the critical path of every step, and every FP64 instruction of a warp
-// takes 64 cycles here: 12 of them instead of the about 40 of a library
+// takes 64 cycles here: 17 of them instead of the about 40 of a library
 // square root and two divisions (a step at n = 64: 2 x 2300 -> 2 x 1450 cycles
-// in this part).  With y
-// the hardware estimate of 1 / sqrt(s) (20 bits) and r = 1 - s y^2, the
-// series sqrt(s) = s y (1 - r)^(-1/2) = s y (1 + r/2 + 3 r^2/8 + O(r^3))
-// leaves 2^-58; 1 / sqrt(s) is the same series on y, and 1 / (alpha - beta)
-// the geometric series of quot().  Outside 2^-900..2^900 the library calls.
+// in this part).  With y the hardware estimate of 1 / sqrt(s) and r = 1 - s
+// y^2 (at most 2^-19.0 measured over [1, 4)), the series sqrt(s) = s y (1 -
+// r)^(-1/2) = s y (1 + r/2 + 3 r^2/8 + 5 r^3/16 ...) leaves 2^-58 and a residual
+// step the rounding of the last bit; the quotients are quot()'s.  Outside 2^-900..2^900 the library calls.
 __device__ __forceinline__ double reflector_fast(double alpha, double sig2, double &tau, double &beta) {
     if (__double_as_longlong(sig2) == 0) {
         tau = 0.0;
@@ -81,10 +80,11 @@ __device__ __forceinline__ double reflector_fast(double alpha, double sig2, doub
     const double g = s * y;
     const double r = fma(-g, y, 1.0);
     const double q = fma(0.375, r, 0.5) * r;
-    const double nrm = fma(g, q, g);
+    double nrm = fma(g, q, g);
+    nrm = fma(fma(-nrm, nrm, s), 0.5 * y, nrm);             // one residual step: the last bit
     beta = neg ? nrm : -nrm;
     const double D = alpha - beta;                          // no cancellation: the signs differ
-    tau = fabs(D) * fma(y, q, y);
+    tau = quot(fabs(D), nrm);
     double z;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(D));
     const double e = fma(-D, z, 1.0);
