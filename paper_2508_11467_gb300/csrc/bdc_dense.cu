@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(128) k_gram(Reflectors f, int kchunk, double *
             Ys[r * LD + c] = v;
         }
         __syncthreads();
-        if (wm > wn) continue;       // below the diagonal: not needed
+        if (wm > wn || wn >= nb) continue;   // below the diagonal, past the reflectors
 #pragma unroll
         for (int kk = 0; kk < 16; kk += 4) {
             double af[4], bf[4];
@@ -724,6 +724,7 @@ __global__ void __launch_bounds__(256) k_tform(TForm f) {
         const int r = k / kTB, c = k % kTB;
         double s = 0.0;
         if (r < c && c < nb)
+#pragma unroll 8
             for (int y = 0; y < f.chunks; ++y) s += p[y * f.cstride + (long long)r * f.ld + c];
         Gs[r * kTLd + c] = s;
         Ts[r * kTLd + c] = 0.0;
@@ -742,7 +743,7 @@ __global__ void __launch_bounds__(256) k_tform(TForm f) {
         }
     }
     __syncthreads();
-    for (int h = 16; h < kTB; h *= 2)
+    for (int h = 16; h < kTB && h < nb; h *= 2)
         for (int o = 0; o < kTB; o += 2 * h) {
             smem_mm(Xs, kTLd, Gs + o * kTLd + o + h, kTLd, Ts + (o + h) * kTLd + o + h, kTLd, h, h, h, 1.0);
             __syncthreads();
@@ -753,6 +754,13 @@ __global__ void __launch_bounds__(256) k_tform(TForm f) {
         Tall[(long long)(k / kTB) * f.ld + k % kTB] = Ts[(k / kTB) * kTLd + k % kTB];
 }
 constexpr size_t kTformSmem = sizeof(double) * (2 * kTB + 32) * kTLd;
+cudaError_t launch_tform(const TForm &f, int blocks, cudaStream_t st) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_tform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTformSmem);
+    if (e != cudaSuccess) return e;
+    k_tform<<<blocks, 256, kTformSmem, st>>>(f);
+    return cudaGetLastError();
+}
 
 // T of every block of the reflectors into Tall (blocks x kTB x kTB)
 cudaError_t form_t(const Reflectors &f, const double *tau, double *Tall, cudaStream_t st) {
@@ -768,13 +776,8 @@ cudaError_t form_t(const Reflectors &f, const double *tau, double *Tall, cudaStr
     k_gram<<<dim3(blocks, (unsigned)chunks), 128, 0, st>>>(f, kchunk, g_split_buf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_tform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTformSmem)) !=
-        cudaSuccess)
-        return e;
-    k_tform<<<blocks, 256, kTformSmem, st>>>(TForm{g_split_buf, Tall, tau, kTB, 1, (int)chunks, f.count,
-                                                   (long long)chunks * kTB * kTB, (long long)kTB * kTB,
-                                                   (long long)kTB * kTB});
-    return cudaGetLastError();
+    return launch_tform(TForm{g_split_buf, Tall, tau, kTB, 1, (int)chunks, f.count, (long long)chunks * kTB * kTB,
+                              (long long)kTB * kTB, (long long)kTB * kTB}, blocks, st);
 }
 
 // W = M Z for the summed partial products Z of dgemm_parts, M = T or T^T
@@ -803,6 +806,7 @@ __global__ void __launch_bounds__(256) k_tz(const double *__restrict__ T, int nb
         double s = 0.0;
         if (p < nb && v0 + v < count) {
             const double *q = part + (right ? (size_t)p * count + v0 + v : (size_t)(v0 + v) * nb + p);
+#pragma unroll 8
             for (int y = 0; y < splits; ++y) s += q[(size_t)y * mn];
             if (add) s += add[(size_t)(v0 + v) * ldadd + p];
         }
@@ -866,6 +870,7 @@ __global__ void k_gram_sum(const double *__restrict__ part, Reflectors f, int ch
     const double *p = part + (size_t)blockIdx.y * chunks * w2 + k;
     double s = 0.0;
     if (r < c && c < nb) {
+#pragma unroll 4
         for (int y = 0; y < chunks; ++y) s += p[(size_t)y * w2];
         s += f.src[(size_t)i0 * (f.sr + f.sc) + (size_t)c * f.sr + (size_t)r * f.sc];
     }
@@ -975,12 +980,9 @@ cudaError_t form_v(const Reflectors &f, const double *tau, const SplitWs &w, cud
     if ((e = set.run()) != cudaSuccess) return e;
     k_gram_sum<<<dim3((unsigned)(w2 / 256), blocks), 256, 0, st>>>(w.V, f, chunks, w.G, w.T);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_tform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTformSmem)) !=
-        cudaSuccess)
+    if ((e = launch_tform(TForm{w.G, w.T, tau, kWide, kWide / kTB, 1, f.count, (long long)w2, (long long)w2, 0},
+                          (f.count + kTB - 1) / kTB, st)) != cudaSuccess)
         return e;
-    k_tform<<<(f.count + kTB - 1) / kTB, 256, kTformSmem, st>>>(
-        TForm{w.G, w.T, tau, kWide, kWide / kTB, 1, f.count, (long long)w2, (long long)w2, 0});
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int h = kTB; h < kWide && h < f.count; h *= 2)
         for (int phase = 0; phase < 2; ++phase) {
             const int tiles = kWide / (2 * h) * (h / 8) * (h / 8);
@@ -1311,15 +1313,23 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
     double *Y = (double *)(ws + w.Y), *Ti = (double *)(ws + w.Ti), *Z = (double *)(ws + w.Z);
     const int kmax = std::min(m, n);
     const SplitWs sw = split_ws(ws, w);
+    unsigned bars = 0;
     for (int i0 = 0; i0 < kmax; i0 += b) {
         const int nb = std::min(b, kmax - i0), ml = m - i0;
         Geqr2Args a{A + i0 + (size_t)i0 * lda, lda, ml, nb, b, tau + i0, (double *)(ws + w.part), bar};
-        if ((err = launch_coop((const void *)k_geqr2, grid, &a, st)) != cudaSuccess) return err;
+        const bool resident = geqr2_resident_fits(ml, nb);   // also leaves Y^T Y in gram
+        double *gram = Ti + (size_t)kTB * kTB;
+        err = resident ? launch_geqr2_resident(ml, nb, a.A, lda, a.tau, gram, kTB, (double *)(ws + w.res), bar,
+                                                                  &bars, st)
+                                          : launch_coop((const void *)k_geqr2, grid, &a, st);
+        if (err != cudaSuccess) return err;
         if (i0 + nb < n) {
             const int cols = n - i0 - nb;
+            const Reflectors f{A + i0 + (size_t)i0 * lda, 1, lda, ml, nb};
+            err = resident ? launch_tform(TForm{gram, Ti, tau + i0, kTB, 1, 1, nb, 0, 0, 0}, 1, st)
+                           : form_t(f, tau + i0, Ti, st);
+            if (err != cudaSuccess) return err;
             if (panel_split(ml, cols, sw)) {
-                const Reflectors f{A + i0 + (size_t)i0 * lda, 1, lda, ml, nb};
-                if ((err = form_t(f, tau + i0, Ti, st)) != cudaSuccess) return err;
                 if ((err = apply_panel(f, Ti, ml, cols, A + i0 + (size_t)(i0 + nb) * lda, lda, Z, sw, st)) !=
                     cudaSuccess)
                     return err;
@@ -1328,8 +1338,6 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
             const long long cnt = (long long)ml * nb;
             k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
-            if ((err = form_t(Reflectors{A + i0 + (size_t)i0 * lda, 1, lda, ml, nb}, tau + i0, Ti, st)) != cudaSuccess)
-                return err;
             if ((err = apply_block(1, 1, ml, n - i0 - nb, Y, nb, Ti, A + i0 + (size_t)(i0 + nb) * lda, lda, Z, st)) !=
                 cudaSuccess)
                 return err;

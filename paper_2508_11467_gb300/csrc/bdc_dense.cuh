@@ -34,6 +34,12 @@ bool resident_fits(int m, int n);
 cudaError_t launch_gebd2_resident(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup,
                                   double *scratch, GridBar *bar, unsigned *bars, cudaStream_t st);
 
+// QR of an m x nb panel (nb <= 32) held on chip, likewise; gram[c ldg + i] =
+// v_c^T v_i for c < i
+bool geqr2_resident_fits(int m, int nb);
+cudaError_t launch_geqr2_resident(int m, int nb, double *A, int lda, double *tau, double *gram, int ldg,
+                                  double *scratch, GridBar *bar, unsigned *bars, cudaStream_t st);
+
 // One operand of a product of split_products(): n vectors of K entries (the
 // rows of A, the columns of B).  tr = 0: vector v at p + v ld, along K; tr =
 // 1: entry k of vector v at p + k ld + v.  parts > 1: the sum of `parts`

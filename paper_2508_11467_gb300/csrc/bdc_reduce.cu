@@ -1,4 +1,5 @@
-// Bidiagonalization of a matrix held on chip (Sec. 4.1, FP64).
+// Bidiagonalization of a matrix held on chip (Sec. 4.1, FP64), and the QR
+// panels (Sec. 4.3).
 //
 // The blocked reduction (bdc_dense.cu) passes over the trailing matrix twice
 // per column step and separates its phases by grid barriers.  When the matrix
@@ -542,12 +543,192 @@ DevInfo dev_info() {
     return d;
 }
 
+// -------------------------------------------------------------- QR panel
+constexpr int kQp = 32;            // panel columns: a lane each
+constexpr int kQld = kQp + 1;      // row stride in shared memory
+
+struct Geqr2ResArgs {
+    double *A;
+    int lda, m, nb;
+    double *tau, *gram;            // gram[c ldg + i]: v_c^T v_i, c < i (what T is formed from)
+    int ldg;
+    Slot *gp;                      // [grid][32]: per-CTA partial sums a^T A[:, c] (column i: a^T a)
+    Slot *row, *sv, *scal;         // [32] top row; [32] update factors; [1] column scale
+    GridBar *bar;
+    unsigned base;
+};
+
+// Householder QR of an m x nb panel (Sec. 4.3, step 1) held on chip: a block
+// of rows per CTA in shared memory (row major), a column per lane, the rows
+// over four warps.  With a = column i (unscaled; v = sc a, v_i = 1):
+//   owners  column c > i is owned by one warp of the grid: g_c = sum over CTAs
+//           of a^T A[:, c] and sig2 = a^T a (tail rows) -> H_i's scalars, s_c =
+//           tau (A[i, c] + sc g_c); R[i, c] = A[i, c] - s_c is final; sc s_c
+//           goes to every CTA.  Column i's owner stores tau, beta and sends sc.
+//           A finished column's owner (c < i) gets v_c^T v_i the same way: its
+//           lane would idle, and T needs those products (a separate pass over
+//           a 10000 x 32 panel for them measured 335 us, this kernel 200).
+//   rows    one pass A[r, c] -= a_r (sc s_c) with the partial sums of the next
+//           column a' = A[:, i + 1] (a lane broadcast) against all columns
+// Two slot exchanges per column (buffers reused as in k_gebd2_resident)
+// instead of three grid barriers with the panel read from L2.  What bounds
+// it: the exchanges; two FP64 operations per row and column are about 2000
+// cycles of a column at 66 rows a CTA.
+__global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
+    extern __shared__ double smem[];
+    __shared__ int s_err;
+    __shared__ double s_red[4][kQp], s_fac[kQp], s_sc[kQp];
+    const int G = gridDim.x, g = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int m = a.m, nb = a.nb;
+    const int rb = (m + G - 1) / G, r0 = min(m, g * rb), nr = min(m, r0 + rb) - r0;
+    double *W = smem;              // [nr][kQld]
+    double *A = a.A;
+    const size_t lda = a.lda;
+    if (t == 0) s_err = 0;
+    for (int c = warp; c < kQp; c += 4)
+        for (int r = lane; r < nr; r += 32) W[r * kQld + c] = c < nb ? A[(size_t)c * lda + r0 + r] : 0.0;
+    const Slot zero = {0ull, 0ull};
+    if (t < kQp) a.gp[g * kQp + t] = zero;
+    if (g == 0 && t < kQp) a.row[t] = a.sv[t] = zero;
+    if (g == 0 && t == 0) a.scal[0] = zero;
+    if (!grid_wait(a.bar, a.base + G)) return;
+
+    auto publish = [&](double acc, unsigned tag) {
+        s_red[warp][lane] = acc;
+        __syncthreads();
+        if (warp == 0 && lane < nb)
+            slot_put(a.gp + g * kQp + lane, (s_red[0][lane] + s_red[1][lane]) + (s_red[2][lane] + s_red[3][lane]), tag);
+    };
+    {
+        double acc = 0.0;
+        for (int r = warp; r < nr; r += 4) {
+            const double x = W[r * kQld + lane], y = W[r * kQld];
+            if (r0 + r == 0) {
+                if (lane < nb) slot_put(a.row + lane, x, 1u);
+            } else {
+                acc = fma(y, x, acc);
+            }
+        }
+        publish(acc, 1u);
+    }
+    for (int i = 0; i < nb; ++i) {
+        const unsigned tag = (unsigned)i + 1u;
+        // ---- owners: the k-th column other than i for k = g + G warp; column i itself: the last CTA's last warp
+        {
+            const int k = g + G * warp, c = k < i ? k : k + 1;
+            const bool own = c < nb, self = g == G - 1 && warp == 3;
+            if (own || self) {
+                // lanes 0-15 sum column c, lanes 16-31 column i
+                const int col = (lane < 16 && own) ? c : i;
+                double s = 0.0, alpha = 0.0, rw = 0.0;
+                for (int q0 = lane & 15; q0 < G; q0 += 128) {
+                    const Slot *q[10];
+                    double v[10];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) q[j] = a.gp + (q0 + 16 * j < G ? q0 + 16 * j : q0) * kQp + col;
+                    q[8] = a.row + i;
+                    q[9] = a.row + col;
+                    slot_get<10>(q, tag, v, a.bar, &s_err);
+                    alpha = v[8];
+                    rw = v[9];
+                    s += v[0];
+#pragma unroll
+                    for (int j = 1; j < 8; ++j)
+                        if (q0 + 16 * j < G) s += v[j];
+                }
+                for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                const double sig2 = __shfl_sync(0xffffffffu, s, 16);
+                double tau, beta;
+                const double sc = reflector_fast(alpha, sig2, tau, beta);
+                if (own && c < i && lane == 0) a.gram[(size_t)c * a.ldg + i] = s_sc[c] * fma(sc, s, rw);
+                if (own && c > i && lane == 0) {
+                    const double sfac = tau * fma(sc, s, rw);
+                    slot_put(a.sv + c, sc * sfac, tag);
+                    A[(size_t)c * lda + i] = rw - sfac;
+                }
+                if (self && lane == 0) {
+                    slot_put(a.scal, sc, tag);
+                    a.tau[i] = tau;
+                    A[(size_t)i * lda + i] = beta;
+                }
+            }
+        }
+        // ---- rows
+        if (warp == 0) {
+            const Slot *q[2] = {a.scal, lane > i && lane < nb ? a.sv + lane : a.scal};
+            double v[2];
+            slot_get<2>(q, tag, v, a.bar, &s_err);
+            s_fac[lane] = lane > i && lane < nb ? -v[1] : 0.0;
+            if (lane == 0) s_sc[i] = v[0];
+        }
+        __syncthreads();
+        if (s_err) return;         // uniform: read after the barrier
+        if (i + 1 == nb) break;
+        const double f = s_fac[lane];
+        const int rl = max(0, i + 1 - r0);              // own rows below i
+        double acc = 0.0;
+        int r = rl + warp;
+        if (r0 + rl == i + 1 && rl < nr && warp == 0) { // the next top row
+            const double x = fma(W[r * kQld + i], f, W[r * kQld + lane]);
+            if (lane < nb) slot_put(a.row + lane, x, tag + 1u);
+            r += 4;
+        }
+        for (; r + 12 < nr; r += 16) {
+            double x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] = W[(r + 4 * j) * kQld + lane];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] = fma(W[(r + 4 * j) * kQld + i], f, x[j]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc = fma(__shfl_sync(0xffffffffu, x[j], i + 1), x[j], acc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) W[(r + 4 * j) * kQld + lane] = x[j];   // (lanes <= i: unchanged, f = 0)
+        }
+        for (; r < nr; r += 4) {
+            const double x = fma(W[r * kQld + i], f, W[r * kQld + lane]);
+            acc = fma(__shfl_sync(0xffffffffu, x, i + 1), x, acc);
+            W[r * kQld + lane] = x;
+        }
+        publish(acc, tag + 1u);
+    }
+    // the reflectors' entries, scaled
+    for (int c = warp; c < nb; c += 4)
+        for (int r = lane; r < nr; r += 32)
+            if (r0 + r > c) A[(size_t)c * lda + r0 + r] = s_sc[c] * W[r * kQld + c];
+}
+
 }  // namespace
 
 size_t resident_scratch_doubles(int n) {
     // a matrix with m >= n that fits has n^2 doubles in kResGrid SMs of 227 KB
-    const size_t nn = std::min(n, 2200);
+    const size_t nn = std::max(std::min(n, 2200), kQp);   // (at least a QR panel's slots)
     return 2 * ((size_t)kResGrid * nn + 3 * nn + 8);
+}
+
+// rows of a QR panel's CTA: about 64, at least 8 CTAs (the owners of 31
+// columns are a warp each), as many as there are SMs
+static int qr_grid(int m) {
+    const DevInfo d = dev_info();
+    return std::max(8, std::min({(m + 63) / 64, d.sms, kResGrid}));
+}
+static size_t qr_smem(int m, int G) { return sizeof(double) * (size_t)((m + G - 1) / G) * kQld + 64; }
+
+bool geqr2_resident_fits(int m, int nb) {
+    const DevInfo d = dev_info();
+    return d.sms >= 8 && nb >= 1 && nb <= kQp && m >= nb && qr_smem(m, qr_grid(m)) <= (size_t)d.smem - 4096;
+}
+
+cudaError_t launch_geqr2_resident(int m, int nb, double *A, int lda, double *tau, double *gram, int ldg,
+                                  double *scratch, GridBar *bar, unsigned *bars, cudaStream_t st) {
+    const int G = qr_grid(m);
+    Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * kQp, *sv = row + kQp, *scal = sv + kQp;
+    Geqr2ResArgs a{A, lda, m, nb, tau, gram, ldg, gp, row, sv, scal, bar, *bars};
+    *bars += (unsigned)G;
+    cudaError_t err =
+        cudaFuncSetAttribute(k_geqr2_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, dev_info().smem - 4096);
+    if (err != cudaSuccess) return err;
+    void *params[] = {&a};
+    return cudaLaunchCooperativeKernel((const void *)k_geqr2_resident, dim3(G), dim3(NT), params, qr_smem(m, G), st);
 }
 
 int res_grid(int m) {
