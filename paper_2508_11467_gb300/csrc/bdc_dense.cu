@@ -1,7 +1,7 @@
 // Dense front and back end of the SVD (FP64), all on the GPU:
 //
 //   Sec. 4.1, Algorithm 1  bidiagonalization A = Q1 B P1^T (m >= n) by blocks
-//             of b columns and rows: one cooperative panel kernel (k_labrd)
+//             of b columns and rows: one cooperative panel kernel (k_labrd_panel, bdc_reduce.cu)
 //             forms the b column reflectors H_i, row reflectors G_i and the
 //             vectors y_i, x_i of Eqs. (bidiag-y-k3) and (bidiag-x-k3), the
 //             corrections of the not yet updated trailing matrix merged into
@@ -303,48 +303,6 @@ __device__ double grid_partials(const double *part, int count, int stride, doubl
     return block_sum((s0 + s1) + (s2 + s3), sh);
 }
 
-// dot product of x[r] y[r] over r = r0 + lane, r0 + lane + 32, ... < r1 by
-// sum over j < cnt of a[j sa] b[j sb] + c[j sa] d[j sb] (the panel's
-// earlier columns, cnt < b): two independent FMA chains and the loads of
-// eight j in flight, instead of one dependent chain waiting on each j's loads
-__device__ __forceinline__ double dot2(const double *__restrict__ a, const double *__restrict__ b,
-                                       const double *__restrict__ c, const double *__restrict__ d, long long sa,
-                                       long long sb, int cnt) {
-    double s0 = 0.0, s1 = 0.0;
-    int j = 0;
-#pragma unroll 4
-    for (; j + 1 < cnt; j += 2) {
-        s0 = fma(a[j * sa], b[j * sb], s0);
-        s1 = fma(a[(j + 1) * sa], b[(j + 1) * sb], s1);
-        s0 = fma(c[j * sa], d[j * sb], s0);
-        s1 = fma(c[(j + 1) * sa], d[(j + 1) * sb], s1);
-    }
-    if (j < cnt) {
-        s0 = fma(a[j * sa], b[j * sb], s0);
-        s0 = fma(c[j * sa], d[j * sb], s0);
-    }
-    return s0 + s1;
-}
-
-// one warp (result in every lane): four independent accumulators so that
-// four pairs of loads are in flight per lane
-__device__ __forceinline__ double warp_dot(const double *__restrict__ x, const double *__restrict__ y, int r0,
-                                           int r1) {
-    const int lane = threadIdx.x & 31;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    int r = r0 + lane;
-    for (; r + 96 < r1; r += 128) {
-        s0 = fma(x[r], y[r], s0);
-        s1 = fma(x[r + 32], y[r + 32], s1);
-        s2 = fma(x[r + 64], y[r + 64], s2);
-        s3 = fma(x[r + 96], y[r + 96], s3);
-    }
-    for (; r < r1; r += 32) s0 = fma(x[r], y[r], s0);
-    double s = (s0 + s1) + (s2 + s3);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-}
-
 // Householder reflector from alpha and ||x_2..||^2 = sig2 (LAPACK's sign
 // convention, Sec. 4.1's first display): beta = -sign(alpha) ||x||, tau =
 // (beta - alpha) / beta, the vector's tail scaled by 1 / (alpha - beta);
@@ -359,156 +317,6 @@ __device__ __forceinline__ double reflector(double alpha, double sig2, double &t
     beta = alpha >= 0.0 ? -nrm : nrm;
     tau = (beta - alpha) / beta;
     return 1.0 / (alpha - beta);
-}
-
-// -------------------------------------------------------- gebrd panel
-// Panel of Algorithm 1 (labrd) on the local m x n trailing matrix A (ld lda):
-// nb column and row reflectors.  Workspace (all column-major):
-//   PW  m x 2b: [V | X], QW  n x 2b: [Y | U] (explicit, zero outside their
-//   supports), yraw[n], tv[4b] (the small products of Eqs. bidiag-y-k3 /
-//   x-k3), xpart[chunks][m] (column-chunk partial sums of A u), part[grid][2]
-//   (partial sums of squares).
-struct LabrdArgs {
-    double *A;
-    int lda, m, n, nb, b;
-    double *d, *e, *tauq, *taup;   // offset to the panel's first index
-    double *PW, *QW, *yraw, *tv, *xpart, *part;
-    int chunks, chunkw;            // column chunks of the row-wise product A u
-    GridBar *bar;
-};
-
-__global__ void __launch_bounds__(256) k_labrd(LabrdArgs a) {
-    __shared__ double sh[32];
-    const int T = blockDim.x, G = gridDim.x;
-    const int gtid = blockIdx.x * T + threadIdx.x, gthreads = G * T;
-    const int lane = threadIdx.x & 31;
-    const int gwarp = gtid >> 5, gwarps = gthreads >> 5;
-    const int m = a.m, n = a.n, b = a.b;
-    double *A = a.A;
-    const long long lda = a.lda;
-    double *V = a.PW, *X = a.PW + (size_t)b * m, *Y = a.QW, *U = a.QW + (size_t)b * n;
-    double *t1 = a.tv, *t2 = a.tv + b, *t3 = a.tv + 2 * b, *t4 = a.tv + 3 * b;
-
-    // zero the workspace matrices (supports are filled step by step)
-    for (size_t k = gtid; k < (size_t)2 * b * m; k += gthreads) a.PW[k] = 0.0;
-    for (size_t k = gtid; k < (size_t)2 * b * n; k += gthreads) a.QW[k] = 0.0;
-    if (!grid_sync(a.bar)) return;
-
-    for (int i = 0; i < a.nb; ++i) {
-        // (a) column i of the panel, rows i..m-1: A - V Y^T - X U^T (Eq. bidiag-y-k2 form)
-        double ss = 0.0;
-        for (int r = i + gtid; r < m; r += gthreads) {
-            double v = A[(size_t)i * lda + r];
-            v -= dot2(V + r, Y + i, X + r, U + i, m, n, i);
-            A[(size_t)i * lda + r] = v;
-            if (r > i) ss = fma(v, v, ss);
-        }
-        ss = block_sum(ss, sh);
-        if (threadIdx.x == 0) a.part[2 * blockIdx.x] = ss;
-        if (!grid_sync(a.bar)) return;
-        // (b) the column reflector H_i (every CTA forms the same scalars)
-        double sig2 = grid_partials(a.part, G, 2, sh);
-        const double alpha = A[(size_t)i * lda + i];
-        double tau, beta;
-        const double sc = reflector(alpha, sig2, tau, beta);
-        for (int r = i + 1 + gtid; r < m; r += gthreads) {
-            const double v = A[(size_t)i * lda + r] * sc;
-            A[(size_t)i * lda + r] = v;
-            V[(size_t)i * m + r] = v;
-        }
-        if (gtid == 0) {
-            V[(size_t)i * m + i] = 1.0;
-            a.d[i] = beta;
-            a.tauq[i] = tau;
-        }
-        if (!grid_sync(a.bar)) return;
-        if (gtid == 0) A[(size_t)i * lda + i] = beta;   // v_i[i] = 1 is implicit from here on
-        // (c) yraw = A^T v over the trailing columns, t1 = V^T v, t2 = X^T v
-        // (Eq. bidiag-y-k3); one warp per dot product, rows i..m-1
-        const int ncol = n - i - 1;
-        for (int w = gwarp; w < ncol + 2 * i; w += gwarps) {
-            const double *col;
-            if (w < ncol) col = A + (size_t)(i + 1 + w) * lda;
-            else if (w < ncol + i) col = V + (size_t)(w - ncol) * m;
-            else col = X + (size_t)(w - ncol - i) * m;
-            const double s = warp_dot(col, V + (size_t)i * m, i, m);
-            if (lane == 0) {
-                if (w < ncol) a.yraw[i + 1 + w] = s;
-                else if (w < ncol + i) t1[w - ncol] = s;
-                else t2[w - ncol - i] = s;
-            }
-        }
-        if (!grid_sync(a.bar)) return;
-        if (ncol == 0) continue;   // the last column of the matrix: no row reflector
-        // (d) y_i = tau (yraw - Y t1 - U t2), then row i, columns i+1..n-1:
-        // A - V Y^T - X U^T with the new v_i, y_i (Eq. bidiag-x-k3 form)
-        ss = 0.0;
-        for (int c = i + 1 + gtid; c < n; c += gthreads) {
-            double y = a.yraw[c];
-            y -= dot2(Y + c, t1, U + c, t2, n, 1, i);
-            y *= tau;
-            Y[(size_t)i * n + c] = y;
-            double v = A[(size_t)c * lda + i] - y;   // V[i][i] = 1
-            v -= dot2(Y + c, V + i, U + c, X + i, n, m, i);
-            A[(size_t)c * lda + i] = v;
-            if (c > i + 1) ss = fma(v, v, ss);
-        }
-        ss = block_sum(ss, sh);
-        if (threadIdx.x == 0) a.part[2 * blockIdx.x + 1] = ss;
-        if (!grid_sync(a.bar)) return;
-        // (e) the row reflector G_i
-        sig2 = grid_partials(a.part + 1, G, 2, sh);
-        const double alr = A[(size_t)(i + 1) * lda + i];
-        double pi, betr;
-        const double scr = reflector(alr, sig2, pi, betr);
-        for (int c = i + 2 + gtid; c < n; c += gthreads) {
-            const double u = A[(size_t)c * lda + i] * scr;
-            A[(size_t)c * lda + i] = u;
-            U[(size_t)i * n + c] = u;
-        }
-        if (gtid == 0) {
-            U[(size_t)i * n + i + 1] = 1.0;
-            a.e[i] = betr;
-            a.taup[i] = pi;
-        }
-        if (!grid_sync(a.bar)) return;
-        if (gtid == 0) A[(size_t)(i + 1) * lda + i] = betr;
-        // (f) xpart = A u by column chunks (rows i+1..m-1), t3 = Y^T u, t4 = U^T u
-        const int rows = m - i - 1;
-        const long long items = (long long)a.chunks * rows;
-        for (long long t = gtid; t < items; t += gthreads) {
-            const int ch = (int)(t / rows), r = i + 1 + (int)(t % rows);
-            const int c0 = i + 1 + ch * a.chunkw, c1 = min(n, c0 + a.chunkw);
-            const double *ui = U + (size_t)i * n;
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            int c = c0;
-            for (; c + 3 < c1; c += 4) {
-                s0 = fma(A[(size_t)c * lda + r], ui[c], s0);
-                s1 = fma(A[(size_t)(c + 1) * lda + r], ui[c + 1], s1);
-                s2 = fma(A[(size_t)(c + 2) * lda + r], ui[c + 2], s2);
-                s3 = fma(A[(size_t)(c + 3) * lda + r], ui[c + 3], s3);
-            }
-            for (; c < c1; ++c) s0 = fma(A[(size_t)c * lda + r], ui[c], s0);
-            a.xpart[(size_t)ch * m + r] = (s0 + s1) + (s2 + s3);
-        }
-        for (int w = gwarp; w < 2 * i + 1; w += gwarps) {
-            const double *col = (w <= i) ? Y + (size_t)w * n : U + (size_t)(w - i - 1) * n;
-            const double s = warp_dot(col, U + (size_t)i * n, i + 1, n);
-            if (lane == 0) {
-                if (w <= i) t3[w] = s;
-                else t4[w - i - 1] = s;
-            }
-        }
-        if (!grid_sync(a.bar)) return;
-        // (g) x_i = pi (A u - V t3 - X t4), rows i+1..m-1
-        for (int r = i + 1 + gtid; r < m; r += gthreads) {
-            double x = 0.0;
-            for (int ch = 0; ch < a.chunks; ++ch) x += a.xpart[(size_t)ch * m + r];
-            x -= dot2(V + r, t3, X + r, t4, m, 1, i) + V[(size_t)i * m + r] * t3[i];
-            X[(size_t)i * m + r] = pi * x;
-        }
-        if (!grid_sync(a.bar)) return;
-    }
 }
 
 // ---------------------------------------------------------- QR panel
@@ -1158,28 +966,24 @@ constexpr int kWsBlock = kApplyBlock > kDenseBlock ? kApplyBlock : kDenseBlock; 
 
 // workspace layout of the dense routines (bytes from an aligned base)
 struct DenseWs {
-    size_t bar, PW, QW, yraw, tv, xpart, part, Y, Ti, Z, split, split_doubles, res, total;
+    size_t bar, PW, QW, part, Y, Ti, Z, split, split_doubles, res, lab, total;
     size_t wG, wT, wX, wV, wZ, wZcap, wS, wSbytes;   // split path
 };
-constexpr int kChunkW = 128;   // columns per partial sum of A u
 
 DenseWs dense_ws(int m, int n, int b, int zcols) {
     DenseWs w{};
     size_t o = 0;
-    const int chunks = (n + kChunkW - 1) / kChunkW;
     const int grid = 4 * 256;   // upper bound of the cooperative grid (partial arrays)
     w.bar = o; o += 256;
     w.PW = o; o += al256(sizeof(double) * 2 * (size_t)b * m);
     w.QW = o; o += al256(sizeof(double) * 2 * (size_t)b * n);
-    w.yraw = o; o += al256(sizeof(double) * (size_t)n);
-    w.tv = o; o += al256(sizeof(double) * 4 * (size_t)b);
-    w.xpart = o; o += al256(sizeof(double) * (size_t)chunks * m);
     w.part = o; o += al256(sizeof(double) * (size_t)grid * (b + 1));
     w.Y = o; o += al256(sizeof(double) * (size_t)std::max(m, n) * std::max(b, kWide));
     w.Ti = o; o += al256(sizeof(double) * (size_t)kTB * (std::max(m, n) + kTB));   // T of every block
     w.Z = o; o += al256(sizeof(double) * (size_t)b * std::max(std::max(m, n), zcols));
     w.split_doubles = std::max<size_t>((size_t)16 * b * std::max(std::max(m, n), zcols), (size_t)16 * kTB * kTB);
     w.split = o; o += al256(sizeof(double) * w.split_doubles);
+    w.lab = o; o += al256(sizeof(double) * labrd_scratch_doubles(m, n));
     w.res = o; o += al256(sizeof(double) * resident_scratch_doubles(n));
     // split path: every block's G, T, X; V and the partial Y^T Y; parts of Z; slices
     {
@@ -1242,10 +1046,8 @@ bool panel_split(int rows, int cols, const SplitWs &w) {
            split_scratch(rows, cols, 32, (long long)((rows + 127) / 128) * ((cols + 127) / 128)) <= w.slice_bytes;
 }
 
-// Bidiagonalization, Algorithm 1 (m >= n): per panel of b, k_labrd, then the
-// merged rank-(2b) update of the trailing matrix (one product).
-constexpr long long kLabrdWork = 8192;   // trailing-matrix entries per CTA of the panel kernel
-
+// Bidiagonalization, Algorithm 1 (m >= n): on chip once it fits; before that,
+// per panel of b, k_labrd_panel, then the merged rank-(2b) update of the trailing matrix (one product).
 cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup, int b,
                         char *ws, cudaStream_t st) {
     const DenseWs w = dense_ws(m, n, b, n);
@@ -1253,22 +1055,16 @@ cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, 
     GridBar *bar = (GridBar *)(ws + w.bar);
     cudaError_t err = cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st);   // the counters (not the error word)
     if (err != cudaSuccess) return err;
-    // CTAs per panel by the work of its steps (the products with the
-    // trailing matrix, ~ml nl FMAs): a small trailing matrix cannot use the
-    // whole GPU, and every barrier costs more with more CTAs
-    const int gmax = std::min(coop_blocks((const void *)k_labrd, 256, 0), 4 * 256);
     unsigned bars = 0;
     for (int i0 = 0; i0 < n; i0 += b) {
         const int nb = std::min(b, n - i0), ml = m - i0, nl = n - i0;
         if (resident_fits(ml, nl))
             return launch_gebd2_resident(ml, nl, A + i0 + (size_t)i0 * lda, lda, d + i0, e + i0, tauq + i0, taup + i0,
                                          (double *)(ws + w.res), bar, &bars, st);
-        const int grid = (int)std::max<long long>(8, std::min<long long>(gmax, (long long)ml * nl / kLabrdWork));
-        LabrdArgs a{A + i0 + (size_t)i0 * lda, lda, ml, nl, nb, b,
-                    d + i0, e + i0, tauq + i0, taup + i0,
-                    (double *)(ws + w.PW), (double *)(ws + w.QW), (double *)(ws + w.yraw), (double *)(ws + w.tv),
-                    (double *)(ws + w.xpart), (double *)(ws + w.part), (nl + kChunkW - 1) / kChunkW, kChunkW, bar};
-        if ((err = launch_coop((const void *)k_labrd, grid, &a, st)) != cudaSuccess) return err;
+        if ((err = launch_labrd_panel(ml, nl, nb, A + i0 + (size_t)i0 * lda, lda, d + i0, e + i0, tauq + i0, taup + i0,
+                                      (double *)(ws + w.PW), (double *)(ws + w.QW), (double *)(ws + w.lab), bar, &bars,
+                                      st)) != cudaSuccess)
+            return err;
         if (nb < nl) {
             // the merged rank-(2b) update A[nb:, nb:] -= P Q^T (Eq. bidiag-A-trail3):
             // P = [V X] (ml x 2b) and Q = [Y U] (nl x 2b) are contiguous column

@@ -6,7 +6,7 @@
 
 namespace bdc {
 
-// count, gen: the reusable barrier of k_geqr2 and k_labrd (bdc_dense.cu);
+// count, gen: the reusable barrier of k_geqr2 (bdc_dense.cu);
 // mono: the monotonic arrival counter of the kernels of bdc_reduce.cu; err:
 // set by the barrier wait that gave up (all CTAs leave at their next barrier)
 struct GridBar {
@@ -34,6 +34,12 @@ bool resident_fits(int m, int n);
 cudaError_t launch_gebd2_resident(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup,
                                   double *scratch, GridBar *bar, unsigned *bars, cudaStream_t st);
 
+// one panel of nb <= 32 columns and rows of the blocked reduction of the m x n
+// matrix A: V, X at PW (m x 32 each), Y, U at QW (n x 32 each)
+size_t labrd_scratch_doubles(int m, int n);
+cudaError_t launch_labrd_panel(int m, int n, int nb, double *A, int lda, double *d, double *e, double *tauq,
+                               double *taup, double *PW, double *QW, double *scratch, GridBar *bar, unsigned *bars,
+                               cudaStream_t st);
 // QR of an m x nb panel (nb <= 32) held on chip, likewise; gram[c ldg + i] =
 // v_c^T v_i for c < i
 bool geqr2_resident_fits(int m, int nb);

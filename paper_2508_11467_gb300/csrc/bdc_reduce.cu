@@ -17,23 +17,34 @@ namespace bdc {
 namespace {
 
 // All CTAs of a cooperative launch wait until `target` arrivals have been
-// counted (a counter that only grows: no reset, no generation).  One thread
-// arrives with release order and polls with acquire order.  The wait is
-// bounded (kBarNs); false when it gave up here or elsewhere.
+// counted (a counter that only grows: no reset, no generation); one thread
+// arrives and polls.  ORDERED: what any thread of the grid wrote before is
+// visible after (the arrival releases, the poll acquires, and the CTA's
+// barriers carry both to its other threads).  Not ORDERED: only a hint that
+// the other CTAs have got here, for readers of slots (below).  152 CTAs of
+// 128 threads: 2480 cycles ordered, 1620 as a hint, 3260 with full fences
+// around it; one thread polling per CTA matters: a flag per CTA polled by as
+// many threads took 5000 to 14000.  The wait is bounded (kBarNs); false when
+// it gave up here or elsewhere.
+template <bool ORDERED = true>
 __device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned v;
         int ok = 1;
-        __threadfence();
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gb->mono) : "memory");
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&gb->mono) : "memory");
+        auto poll = [&] {
+            if (ORDERED) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&gb->mono) : "memory");
+            else asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&gb->mono) : "memory");
+        };
+        if (ORDERED) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gb->mono) : "memory");
+        else asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(&gb->mono) : "memory");
+        poll();
         if ((int)(v - target) < 0) {
             const unsigned long long t0 = gtime();
             unsigned spins = 0;
             do {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&gb->mono) : "memory");
+                poll();
                 if ((++spins & 255u) == 0) {
                     if (*(volatile int *)&gb->err) { ok = 0; break; }
                     if (gtime() - t0 > kBarNs) {
@@ -44,7 +55,6 @@ __device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
                 }
             } while ((int)(v - target) < 0);
         }
-        __threadfence();
         s_ok = ok;
     }
     __syncthreads();
@@ -92,13 +102,14 @@ __device__ __forceinline__ double reflector_fast(double alpha, double sig2, doub
     return fma(z, fma(e, e, e), z);
 }
 
-// ---- exchange between CTAs without barriers
+// ---- exchange between CTAs without fences
 // A slot is 16 bytes: the two halves of a double, each beside the step
-// number that wrote it, so that a reader that polls a slot knows from the
-// slot itself when the value is there: no fence and no counter (333 x 333:
-// 3.64 ms with two grid barriers a step and plain loads behind them, 3.00 ms
-// with slots; 1000 x 1000: 15.5 and 11.5 ms, the row passes included).  Each
-// 8-byte half is written and read as one access.
+// number that wrote it, so that a reader knows from the slot itself whether
+// the value is there.  The CTAs wait for one another by an unordered
+// grid_wait and then read: the rare slot that is still on its way is read
+// again.  (Polling the slots alone, without that wait, kept L2 busy with 128
+// threads a CTA: a 333 x 333 step took 18000 cycles, 16400 with the wait.)
+// Each 8-byte half is written and read as one access.
 typedef ulonglong2 Slot;
 
 __device__ __forceinline__ void slot_put(Slot *p, double v, unsigned tag) {
@@ -114,18 +125,23 @@ __device__ __forceinline__ Slot slot_load(const Slot *p) {
     return s;
 }
 
-// K slots at once (all loads in flight together; p[k] may repeat), polled
+// K slots at once (all loads in flight together), polled
 // until each carries `tag`.  Bounded: after kBarNs, or when another wait of
 // the grid gave up, sets the error word and *s_err and returns.
+// A null p[k] is skipped (v[k] = 0).
 template <int K>
 __device__ __forceinline__ void slot_get(const Slot *(&p)[K], unsigned tag, double (&v)[K], GridBar *gb,
                                          int *s_err) {
+    const unsigned long long want = (unsigned long long)tag << 32;
     unsigned spins = 0;
     unsigned long long t0 = 0;
     for (;;) {
         Slot s[K];
 #pragma unroll
-        for (int k = 0; k < K; ++k) s[k] = slot_load(p[k]);
+        for (int k = 0; k < K; ++k) {
+            s[k] = Slot{want, want};
+            if (p[k]) s[k] = slot_load(p[k]);
+        }
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -308,10 +324,10 @@ struct Gebd2Args {
 // their owners sent after reading all sums of step i; and an owner sends
 // step i + 1's y after the sums of every CTA, which each sent after reading
 // all of step i's y.
-// What bounds it: the two exchanges (about 4500 cycles each) and the
+// What bounds it: the two exchanges (about 3500 cycles each) and the
 // dependent FP64 chains of a step (64 cycles an operation), above n ~ 1000
-// the FP64 pipe.  333 x 333: 18.9 ms (k_labrd's seven barriers a step) ->
-// 3.0 ms; 1000 x 1000: 71 -> 11.5 ms; 1500 x 1100: 82 -> 16.5 ms.
+// the FP64 pipe.  333 x 333: 18.9 ms (blocked panels, seven barriers a step)
+// -> 2.8 ms; 1000 x 1000: 71 -> 12 ms; 1500 x 1100: 82 -> 17 ms.
 __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
     extern __shared__ double smem[];
     __shared__ int s_err;
@@ -336,7 +352,8 @@ __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
     for (int c = t; c < n; c += NT) a.gp[(size_t)g * ldw + c] = zero;
     for (int c = g * NT + t; c < n; c += G * NT) a.row[c] = a.yr[2 * c] = a.yr[2 * c + 1] = zero;
     if (g == 0 && t == 0) a.scal[0] = zero;
-    if (!grid_wait(a.bar, a.base + G)) return;
+    unsigned target = a.base + G;
+    if (!grid_wait(a.bar, target)) return;
     for (int l = t; l < lr; l += NT) av[l] = W[(size_t)l * ldw];
     __syncthreads();
     for (int c = t; c < n; c += NT) {               // sums of step 0
@@ -345,6 +362,7 @@ __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
         if (g == 0) slot_put(a.row + c, W[c], 1u);
         slot_put(a.gp + (size_t)g * ldw + c, s, 1u);
     }
+    if (!grid_wait<false>(a.bar, target += G)) return;
 
     for (int i = 0; i < n; ++i) {
         const unsigned tag = (unsigned)i + 1u;
@@ -369,9 +387,9 @@ __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
                     const Slot *q[10];
                     double v[10];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) q[j] = p + (size_t)(k + j * subs < G ? k + j * subs : k) * ldw;
+                    for (int j = 0; j < 8; ++j) q[j] = k + j * subs < G && s < slots ? p + (size_t)(k + j * subs) * ldw : nullptr;
                     q[8] = a.row + i;
-                    q[9] = a.row + (t < nc ? c0 + t : i);
+                    q[9] = t < nc ? a.row + c0 + t : nullptr;
                     slot_get<10>(q, tag, v, a.bar, &s_err);
                     alpha = v[8];
                     top = v[9];
@@ -411,27 +429,22 @@ __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
                 a.tauq[i] = tau;
                 A[(size_t)i * lda + i] = beta;
             }
-            __syncthreads();                        // red, sy are reused below
         }
+        if (!grid_wait<false>(a.bar, target += G)) return;
         // ---- X phase
         const int l0 = (i < g) ? 0 : (i - g) / G + 1;   // first own row below i
         const bool more = i + 1 < n;
         double sc = 0.0, alr = 0.0;
-        {   // wait on one slot per thread, so that the waiting CTAs do not load L2 with all of theirs
-            const Slot *q[1] = {i + 1 + t < n ? a.yr + 2 * (i + 1 + t) + 1 : a.scal};
-            double v[1];
-            slot_get<1>(q, tag, v, a.bar, &s_err);
-        }
         for (int c = i + 1 + t, first = 1; first || c < n; c += 4 * NT, first = 0) {
             // four columns of y and r per round; every round also has the scale and r's first entry
             const Slot *q[10];
             double v[10];
             q[8] = a.scal;
-            q[9] = more ? a.yr + 2 * (i + 1) + 1 : a.scal;
+            q[9] = more ? a.yr + 2 * (i + 1) + 1 : nullptr;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                q[2 * j] = c + j * NT < n ? a.yr + 2 * (c + j * NT) : q[9];
-                q[2 * j + 1] = c + j * NT < n ? a.yr + 2 * (c + j * NT) + 1 : q[9];
+                q[2 * j] = c + j * NT < n ? a.yr + 2 * (c + j * NT) : nullptr;
+                q[2 * j + 1] = c + j * NT < n ? a.yr + 2 * (c + j * NT) + 1 : nullptr;
             }
             slot_get<10>(q, tag, v, a.bar, &s_err);
             sc = v[8];
@@ -516,6 +529,7 @@ __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
                                                t, tag + 1u);
             });
         }
+        if (!grid_wait<false>(a.bar, target += G)) return;
     }
 }
 
@@ -541,6 +555,365 @@ DevInfo dev_info() {
         d.smem -= 128;   // the kernels' static shared memory
     }
     return d;
+}
+
+// ------------------------------------------------------ blocked panel
+// Panel of Algorithm 1 (labrd) on the m x n trailing matrix A, for matrices
+// that do not fit on chip: nb column and row reflectors, the corrections of
+// the not yet updated trailing matrix kept in V, X (m x b, ld m) and Y, U (n x
+// b, ld n).  Four phases a step, separated by grid_wait:
+//   P1  own rows: x_{i-1} (the products with r_{i-1} are sums of partial
+//       products), column i: a_i
+//   P2  a_i^T A over the trailing columns, V^T a_i, X^T a_i, a_i^T a_i
+//   P3  own columns: y_i, row i: r_i; the scaled reflector v_i
+//   P4  A r_i over the trailing rows, Y^T r_i, U^T r_i, r_i^T r_i
+// The products take the unscaled a and r, so that no phase waits for a norm,
+// and each norm is one more dot product.  P2 and P4 cut the flattened
+// (columns x rows) space evenly over the grid's warps (a warp's range may
+// span several columns; partial sums, at most kParts per result, are added by
+// their reader), 16 warps an SM with 20 loads in flight a lane.
+// What bounds it: P2 and P4 at the FP64 pipe and L2 (16 bytes a clock and SM
+// at the pipe's two lanes): 65000 cycles each at n = 4096, of which
+// 55000 are the FMAs at two a clock.  P1 and P3 are chains of FP64 operations and L2 trips,
+// 10600 and 8500 cycles, and a barrier 3100.  FP64 instructions of a CTA's
+// warps queue at the pipe (64 cycles each), so the scalars are one warp's and
+// the short sums are cut so that few warps hold full ones.  4096 x 4096: 126 us
+// a step behind seven barriers -> 84 at the first panel, 31 at order 1900;
+// whole reduction 533 -> 178 ms.
+constexpr int kLT = 512, kLW = kLT / 32, kParts = 32, kLb = 32;
+
+struct Labrd2Args {
+    double *A;
+    int lda, m, n, nb;
+    double *d, *e, *tauq, *taup;
+    double *V, *X, *Y, *U;
+    double *av, *rv;               // a_i (m), r_i (n)
+    double *cpart, *hpart, *tpart; // partial sums: P2 (n + 2b + 1) x kParts, P4 rows ceil(m/32) x kParts x 32, P4 dots
+    GridBar *bar;
+    unsigned base;
+};
+
+// How `groups` results of `blocks` blocks each are cut over nw warps: every
+// result in `parts` equal ranges of `size` blocks, so that readers know the
+// count of partial sums; the count (a lane tries each) that leaves the warps
+// with the fewest blocks, a range's start counted as two.
+struct Cut {
+    int parts, size;
+};
+__device__ __forceinline__ Cut cut_of(int groups, int blocks, int nw) {
+    const int s = (threadIdx.x & 31) + 1, size = (blocks + s - 1) / s;
+    const unsigned rounds = (unsigned)(groups * s + nw - 1) / (unsigned)nw;
+    const unsigned cost = s <= blocks ? min(rounds * (unsigned)(size + 2), 0x3ffffffu) : 0x3ffffffu;
+    const int parts = (int)(__reduce_min_sync(0xffffffffu, cost << 6 | (unsigned)s) & 63u);
+    return Cut{parts, (blocks + parts - 1) / parts};
+}
+static_assert(kParts == 32, "a lane per count");
+
+// x over four columns p[0..3] against y, entries [r0, r1) in lane steps of 32:
+// four accumulators reduced together; lane 8 c ends with column c's sum
+__device__ __forceinline__ double dot4(const double *const (&p)[4], const double *y, int r0, int r1, int lane) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    int r = r0 + lane;
+    for (; r + 96 < r1; r += 128) {
+        double yv[4], x[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) yv[k] = __ldcg(y + r + 32 * k);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[c][k] = __ldcg(p[c] + r + 32 * k);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) s[c] = fma(x[c][k], yv[k], s[c]);
+    }
+    for (; r < r1; r += 32) {
+        const double yv = __ldcg(y + r);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[c] = fma(__ldcg(p[c] + r), yv, s[c]);
+    }
+    // halves exchange two columns, quarters one: six adds instead of twenty
+    const bool hi = lane & 16;
+    double a0 = hi ? s[2] : s[0], a1 = hi ? s[3] : s[1];
+    a0 += __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[2], 16);
+    a1 += __shfl_xor_sync(0xffffffffu, hi ? s[1] : s[3], 16);
+    const bool q = lane & 8;
+    double b = q ? a1 : a0;
+    b += __shfl_xor_sync(0xffffffffu, q ? a0 : a1, 8);
+    for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    return b;                      // lanes 8 c .. 8 c + 7: column (c >> 1) * 2 + (c & 1)
+}
+
+// the dot products of `count` vectors (ptr(k)) with y over [r0, r1), cut over
+// the grid's warps; partial sums at part[k kParts + p]
+template <typename F>
+__device__ __forceinline__ void dots(int count, F ptr, const double *y, int r0, int r1, double *part, int gwarp, int nw,
+                                     int lane) {
+    const int groups = (count + 3) / 4, blocks = (r1 - r0 + 31) / 32;
+    if (blocks <= 0) return;
+    const Cut cut = cut_of(groups, blocks, nw);
+    for (int u = gwarp; u < groups * cut.parts; u += nw) {
+        const int g = u / cut.parts, q = u - g * cut.parts;
+        const int b0 = q * cut.size, b1 = min(blocks, b0 + cut.size);
+        const double *p[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) p[c] = ptr(min(4 * g + c, count - 1));
+        const double s = dot4(p, y, r0 + 32 * b0, min(r1, r0 + 32 * b1), lane);   // (0 for an empty range)
+        const int c = 4 * g + (lane >> 3);
+        if ((lane & 7) == 0 && c < count) __stcg(part + (size_t)c * kParts + q, s);
+    }
+}
+// the sums of results first .. first + count - 1 of dots(total, ..) into out,
+// eight lanes each
+__device__ __forceinline__ void dot_sums(const double *part, int total, int r0, int r1, int nw, int first, int count,
+                                         double *out) {
+    const int groups = (total + 3) / 4, blocks = (r1 - r0 + 31) / 32;
+    const Cut cut = blocks > 0 ? cut_of(groups, blocks, nw) : Cut{0, 0};
+    const int l = threadIdx.x & 7;
+    for (int k0 = 0; k0 < count; k0 += kLT / 8) {
+        const int k = k0 + threadIdx.x / 8;
+        if (k0 + (int)(threadIdx.x >> 5) * 4 >= count) break;   // whole warps
+        double v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            v[q] = k < count && l + 8 * q < cut.parts ? __ldcg(part + (size_t)(first + k) * kParts + l + 8 * q) : 0.0;
+        double s = v[0];
+#pragma unroll
+        for (int q = 1; q < 4; ++q)
+            if (8 * q < cut.parts) s += v[q];
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (l == 0 && k < count) out[k] = s;
+    }
+}
+
+// A panel phase's own 32 rows (or columns) r, a lane each: sums over the
+// panel's earlier columns j of P[r, j] f1[j] + Q[r, j] f2[j] and of P[r, j]
+// f3[j] + Q[r, j] f4[j], P's cp and Q's cq columns split over eight warps
+// (loaded before the factors are known); the partial sums of a product over
+// four more warps.
+struct Rows {
+    double p[4], q[4], h[8];
+    __device__ __forceinline__ void load(const double *P, int cp, const double *Q, int cq, int ld, int r, bool ok,
+                                         const double *hp, size_t hstride, int parts, int warp) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int j = warp + 8 * k;
+            p[k] = ok && warp < 8 && j < cp ? __ldcg(P + (size_t)j * ld + r) : 0.0;
+            q[k] = ok && warp < 8 && j < cq ? __ldcg(Q + (size_t)j * ld + r) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int z = warp - 8 + 4 * k;
+            h[k] = ok && warp >= 8 && warp < 12 && z < parts ? __ldcg(hp + z * hstride) : 0.0;
+        }
+    }
+    __device__ __forceinline__ void sum(int cp, int cq, const double *f1, const double *f2, const double *f3,
+                                        const double *f4, int parts, double (*red)[2][32], int warp, int lane) {
+        if (warp < 8) {
+            double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = warp + 8 * k;
+                if (j < cp) { s0 = fma(p[k], f1[j], s0); s1 = fma(p[k], f3[j], s1); }
+                if (j < cq) { s0 = fma(q[k], f2[j], s0); s1 = fma(q[k], f4[j], s1); }
+            }
+            red[warp][0][lane] = s0;
+            red[warp][1][lane] = s1;
+        } else if (warp < 12) {
+            double s = h[0];
+#pragma unroll
+            for (int k = 1; k < 8; ++k)
+                if (warp - 8 + 4 * k < parts) s += h[k];
+            red[warp][0][lane] = s;
+        }
+    }
+};
+__device__ __forceinline__ double red8(const double (*red)[2][32], int k, int lane) {
+    return ((red[0][k][lane] + red[1][k][lane]) + (red[2][k][lane] + red[3][k][lane])) +
+           ((red[4][k][lane] + red[5][k][lane]) + (red[6][k][lane] + red[7][k][lane]));
+}
+__device__ __forceinline__ double red4(const double (*red)[2][32], int lane) {
+    return (red[8][0][lane] + red[9][0][lane]) + (red[10][0][lane] + red[11][0][lane]);
+}
+
+__global__ void __launch_bounds__(kLT, 1) k_labrd_panel(Labrd2Args a) {
+    __shared__ double s_t[2 * kLb + 2], s_1[kLb], s_2[kLb], s_3[kLb], s_4[kLb];
+    __shared__ double s_red[12][2][32], s_x[32], s_c[2];
+    const int G = gridDim.x, g = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int m = a.m, n = a.n, nw = G * kLW, gwarp = warp * G + g;   // consecutive ranges on different SMs
+    double *A = a.A, *V = a.V, *X = a.X, *Y = a.Y, *U = a.U;
+    const size_t lda = a.lda;
+    unsigned target = a.base;
+
+    for (int i = 0;; ++i) {
+        const bool last = i == a.nb;
+        // ---- P1
+        {
+            const int rb = (m - i + G - 1) / G, ra = i + g * rb, rz = min(m, ra + rb);
+            const int cblocks = i > 0 ? (n - i - 1 + 15) / 16 : 0;           // P4's cut of step i - 1
+            const Cut hc = cblocks > 0 ? cut_of((m - i + 31) / 32, cblocks, nw) : Cut{0, 0};
+            const int cp = i, cq = max(0, i - 1);
+            Rows rows;
+            double a0 = 0.0;
+            auto load = [&](int r0) {
+                const int r = r0 + lane, rg = (r - i) >> 5, rl = (r - i) & 31;
+                rows.load(V, cp, X, cq, m, r, r < rz, a.hpart + (size_t)rg * kParts * 32 + rl, 32, hc.parts, warp);
+                if (warp < 2 && r < rz) a0 = __ldcg(A + (size_t)min(i, n - 1) * lda + r);
+            };
+            load(ra);
+            double pi = 0.0, scr = 0.0, betr = 0.0;
+            if (i > 0) {
+                const int nd = 2 * i;
+                const double alr = __ldcg(a.rv + i);
+                if (t >= 384 && t < 384 + i) s_3[t - 384] = __ldcg(Y + (size_t)(t - 384) * n + i);
+                if (t >= 448 && t < 448 + i - 1) s_4[t - 448] = __ldcg(U + (size_t)(t - 448) * n + i);
+                dot_sums(a.tpart, nd, i + 1, n, nw, 0, nd, s_t);
+                __syncthreads();
+                if (warp == 0) {   // one warp: each further one would take its turn at the FP64 pipe
+                    scr = reflector_fast(alr, s_t[nd - 1], pi, betr);
+                    if (lane < i) s_1[lane] = fma(scr, s_t[lane], s_3[lane]);
+                    if (lane < i - 1) s_2[lane] = fma(scr, s_t[i + lane], s_4[lane]);
+                    if (lane == 0) { s_c[0] = scr; s_c[1] = betr; }
+                }
+            }
+            for (int r0 = ra; r0 < rz; r0 += 32) {
+                const int r = r0 + lane;
+                if (r0 > ra) load(r0);
+                __syncthreads();   // s_1 .. s_4, s_c; s_red, s_x of the previous rows
+                if (i > 0) rows.sum(cp, cq, s_1, s_2, s_3, s_4, hc.parts, s_red, warp, lane);
+                __syncthreads();
+                double sa = 0.0;
+                if (i > 0 && warp == 0) {
+                    const double x = pi * (fma(scr, red4(s_red, lane), a0) - red8(s_red, 0, lane));
+                    s_x[lane] = x;
+                    if (r < rz) __stcg(X + (size_t)(i - 1) * m + r, x);
+                } else if (i > 0 && warp == 1) {
+                    sa = red8(s_red, 1, lane);
+                }
+                __syncthreads();
+                if (warp == 1 && r < rz && !last) __stcg(a.av + r, i > 0 ? (a0 - sa) - s_x[lane] : a0);
+            }
+            // the row reflector i - 1
+            if (i > 0) {
+                if (ra >= rz) __syncthreads();   // s_c
+                scr = s_c[0];
+                betr = s_c[1];
+                const int cb = (n - i + G - 1) / G, c0 = i + g * cb;
+                for (int c = c0 + t - 64; c < min(n, c0 + cb); c += kLT - 64) {
+                    if (c < c0) continue;
+                    const double u = c == i ? 1.0 : scr * __ldcg(a.rv + c);
+                    __stcg(U + (size_t)(i - 1) * n + c, u);
+                    A[(size_t)c * lda + i - 1] = c == i ? betr : u;
+                }
+                if (g == 0 && t == 0) {
+                    a.e[i - 1] = betr;
+                    a.taup[i - 1] = pi;
+                }
+            }
+        }
+        if (last) return;
+        if (!grid_wait(a.bar, target += G)) return;
+        // ---- P2
+        const int nc = n - 1 - i, n2 = nc + 2 * i + 1;
+        dots(n2, [&](int k) {
+                return (const double *)(k < nc ? A + (size_t)(i + 1 + k) * lda
+                                        : k < nc + i ? V + (size_t)(k - nc) * m
+                                        : k < nc + 2 * i ? X + (size_t)(k - nc - i) * m : a.av);
+            }, a.av, i + 1, m, a.cpart, gwarp, nw, lane);
+        if (!grid_wait(a.bar, target += G)) return;
+        // ---- P3
+        {
+            const int nd = 2 * i + 1, blocks = (m - i - 1 + 31) / 32;
+            const int cb = (nc + G - 1) / G, ca = i + 1 + g * cb, cz = min(n, ca + cb);
+            const Cut gc = blocks > 0 ? cut_of((n2 + 3) / 4, blocks, nw) : Cut{0, 0};
+            Rows rows;
+            double a0 = 0.0;
+            auto load = [&](int c0) {
+                const int c = c0 + lane;
+                rows.load(Y, i, U, i, n, c, c < cz, a.cpart + (size_t)(c - i - 1) * kParts, 1, gc.parts, warp);
+                if (warp < 2 && c < cz) a0 = __ldcg(A + (size_t)c * lda + i);
+            };
+            load(ca);
+            const double alpha = __ldcg(a.av + i);
+            if (t >= 384 && t < 384 + i) s_3[t - 384] = __ldcg(V + (size_t)(t - 384) * m + i);
+            if (t >= 448 && t < 448 + i) s_4[t - 448] = __ldcg(X + (size_t)(t - 448) * m + i);
+            dot_sums(a.cpart, n2, i + 1, m, nw, nc, nd, s_t);
+            __syncthreads();
+            double tau = 0.0, beta = 0.0, sc = 0.0;
+            if (warp == 0) {
+                sc = reflector_fast(alpha, s_t[2 * i], tau, beta);
+                if (lane < i) {
+                    s_1[lane] = fma(sc, s_t[lane], s_3[lane]);
+                    s_2[lane] = fma(sc, s_t[i + lane], s_4[lane]);
+                }
+                if (lane == 0) s_c[0] = sc;
+            }
+            for (int c0 = ca; c0 < cz; c0 += 32) {
+                const int c = c0 + lane;
+                if (c0 > ca) load(c0);
+                __syncthreads();
+                rows.sum(i, i, s_1, s_2, s_3, s_4, gc.parts, s_red, warp, lane);
+                __syncthreads();
+                double sr = 0.0;
+                if (warp == 0) {
+                    const double y = tau * (fma(sc, red4(s_red, lane), a0) - red8(s_red, 0, lane));
+                    s_x[lane] = y;
+                    if (c < cz) __stcg(Y + (size_t)i * n + c, y);
+                } else if (warp == 1) {
+                    sr = red8(s_red, 1, lane);
+                }
+                __syncthreads();
+                if (warp == 1 && c < cz) __stcg(a.rv + c, (a0 - sr) - s_x[lane]);
+            }
+            // the column reflector i
+            if (ca >= cz) __syncthreads();   // s_c
+            sc = s_c[0];
+            const int rb = (m - i - 1 + G - 1) / G, ra = i + 1 + g * rb;
+            for (int r = ra + t - 64; r < min(m, ra + rb); r += kLT - 64) {
+                if (r < ra) continue;
+                const double v = sc * __ldcg(a.av + r);
+                __stcg(V + (size_t)i * m + r, v);
+                A[(size_t)i * lda + r] = v;
+            }
+            if (g == 0 && t == 0) {
+                a.d[i] = beta;
+                a.tauq[i] = tau;
+                A[(size_t)i * lda + i] = beta;
+            }
+            if (nc == 0) return;   // the last column of the matrix: no row reflector
+        }
+        if (!grid_wait(a.bar, target += G)) return;
+        // ---- P4: rows i + 1 .. by groups of 32 (a row per lane), columns i + 2 .. by 16
+        {
+            const int groups = (m - i - 1 + 31) / 32, cblocks = (n - i - 2 + 15) / 16;
+            if (groups > 0 && cblocks > 0) {
+                const Cut cut = cut_of(groups, cblocks, nw);
+                for (int u = gwarp; u < groups * cut.parts; u += nw) {
+                    const int rg = u / cut.parts, q = u - rg * cut.parts;
+                    const int b0 = q * cut.size, b1 = min(cblocks, b0 + cut.size);
+                    const int r = i + 1 + 32 * rg + lane, ce = min(n, i + 2 + 16 * b1);
+                    const double *p = A + min(r, m - 1);
+                    double s0 = 0.0, s1 = 0.0;
+                    for (int c = i + 2 + 16 * b0; c < ce; c += 16) {
+                        const double rr = c + (lane & 15) < ce ? __ldcg(a.rv + c + (lane & 15)) : 0.0;
+                        double x[16];
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) x[k] = __ldcg(p + (size_t)min(c + k, ce - 1) * lda);
+#pragma unroll
+                        for (int k = 0; k < 16; k += 2) {
+                            s0 = fma(x[k], __shfl_sync(0xffffffffu, rr, k), s0);
+                            s1 = fma(x[k + 1], __shfl_sync(0xffffffffu, rr, k + 1), s1);
+                        }
+                    }
+                    __stcg(a.hpart + ((size_t)rg * kParts + q) * 32 + lane, s0 + s1);
+                }
+            }
+            dots(2 * i + 2, [&](int k) {
+                    return (const double *)(k <= i ? Y + (size_t)k * n : k <= 2 * i ? U + (size_t)(k - i - 1) * n : a.rv);
+                }, a.rv, i + 2, n, a.tpart, nw - 1 - gwarp, nw, lane);
+        }
+        if (!grid_wait(a.bar, target += G)) return;
+    }
 }
 
 // -------------------------------------------------------------- QR panel
@@ -591,7 +964,8 @@ __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
     if (t < kQp) a.gp[g * kQp + t] = zero;
     if (g == 0 && t < kQp) a.row[t] = a.sv[t] = zero;
     if (g == 0 && t == 0) a.scal[0] = zero;
-    if (!grid_wait(a.bar, a.base + G)) return;
+    unsigned target = a.base + G;
+    if (!grid_wait(a.bar, target)) return;
 
     auto publish = [&](double acc, unsigned tag) {
         s_red[warp][lane] = acc;
@@ -613,6 +987,7 @@ __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
     }
     for (int i = 0; i < nb; ++i) {
         const unsigned tag = (unsigned)i + 1u;
+        if (!grid_wait<false>(a.bar, target += G)) return;
         // ---- owners: the k-th column other than i for k = g + G warp; column i itself: the last CTA's last warp
         {
             const int k = g + G * warp, c = k < i ? k : k + 1;
@@ -625,7 +1000,7 @@ __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
                     const Slot *q[10];
                     double v[10];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) q[j] = a.gp + (q0 + 16 * j < G ? q0 + 16 * j : q0) * kQp + col;
+                    for (int j = 0; j < 8; ++j) q[j] = q0 + 16 * j < G ? a.gp + (q0 + 16 * j) * kQp + col : nullptr;
                     q[8] = a.row + i;
                     q[9] = a.row + col;
                     slot_get<10>(q, tag, v, a.bar, &s_err);
@@ -653,9 +1028,10 @@ __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
                 }
             }
         }
+        if (!grid_wait<false>(a.bar, target += G)) return;
         // ---- rows
         if (warp == 0) {
-            const Slot *q[2] = {a.scal, lane > i && lane < nb ? a.sv + lane : a.scal};
+            const Slot *q[2] = {a.scal, lane > i && lane < nb ? a.sv + lane : nullptr};
             double v[2];
             slot_get<2>(q, tag, v, a.bar, &s_err);
             s_fac[lane] = lane > i && lane < nb ? -v[1] : 0.0;
@@ -705,6 +1081,26 @@ size_t resident_scratch_doubles(int n) {
     return 2 * ((size_t)kResGrid * nn + 3 * nn + 8);
 }
 
+size_t labrd_scratch_doubles(int m, int n) {
+    return (size_t)m + n + 64 + (size_t)kParts * ((size_t)n + 2 * kLb + 8) + (size_t)kParts * 32 * ((m + 31) / 32 + 1) +
+           (size_t)kParts * (2 * kLb + 8);
+}
+
+cudaError_t launch_labrd_panel(int m, int n, int nb, double *A, int lda, double *d, double *e, double *tauq,
+                               double *taup, double *PW, double *QW, double *scratch, GridBar *bar, unsigned *bars,
+                               cudaStream_t st) {
+    if (nb > kLb) return cudaErrorInvalidValue;
+    const int G = std::max(1, dev_info().sms);
+    double *av = scratch, *rv = av + m, *cp = rv + n + 32, *hp = cp + (size_t)kParts * (n + 2 * kLb + 8);
+    double *tp = hp + (size_t)kParts * 32 * ((m + 31) / 32 + 1);
+    Labrd2Args a{A, lda, m, n, nb, d, e, tauq, taup, PW, PW + (size_t)kLb * m, QW, QW + (size_t)kLb * n, av, rv, cp, hp,
+                 tp, bar, *bars};
+    // four waits a step; the matrix's last column (no row reflector) ends after two
+    *bars += (unsigned)G * (nb == n ? 4u * (unsigned)(nb - 1) + 2u : 4u * (unsigned)nb);
+    void *params[] = {&a};
+    return cudaLaunchCooperativeKernel((const void *)k_labrd_panel, dim3(G), dim3(kLT), params, 0, st);
+}
+
 // rows of a QR panel's CTA: about 64, at least 8 CTAs (the owners of 31
 // columns are a warp each), as many as there are SMs
 static int qr_grid(int m) {
@@ -723,7 +1119,7 @@ cudaError_t launch_geqr2_resident(int m, int nb, double *A, int lda, double *tau
     const int G = qr_grid(m);
     Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * kQp, *sv = row + kQp, *scal = sv + kQp;
     Geqr2ResArgs a{A, lda, m, nb, tau, gram, ldg, gp, row, sv, scal, bar, *bars};
-    *bars += (unsigned)G;
+    *bars += (unsigned)G * (1u + 2u * (unsigned)nb);
     cudaError_t err =
         cudaFuncSetAttribute(k_geqr2_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, dev_info().smem - 4096);
     if (err != cudaSuccess) return err;
@@ -749,7 +1145,7 @@ cudaError_t launch_gebd2_resident(int m, int n, double *A, int lda, double *d, d
     const size_t smem = res_smem(m, n, G);
     Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * n, *yr = row + n, *scal = yr + 2 * n;
     Gebd2Args a{A, lda, m, n, d, e, tauq, taup, gp, row, yr, scal, bar, *bars};
-    *bars += (unsigned)G;
+    *bars += (unsigned)G * (1u + 2u * (unsigned)n);   // load, first sums, n Y phases, n - 1 X phases
     // the device's maximum, not this launch's size: another thread may be
     // between its own call and its launch
     cudaError_t err =
