@@ -133,17 +133,25 @@ __device__ __forceinline__ Sums pole_sums(const real_t *__restrict__ d, const re
     if constexpr (G < 32) {
         // several roots per warp split their poles at different k: one loop
         // over all poles (the same trip count for every group of the warp)
+        // with one pair of accumulators: a lane's poles ascend, so its sums
+        // are psi's up to its first pole past k and phi's from there (two
+        // FP64 operations a pole for every lane; a branch per pole made a
+        // warp whose groups split at different k issue both sides, four)
+        real_t s0 = R(0.0), s1 = R(0.0);
+        bool right = false;
         for (int j = lane; j < N; j += G, ++t) {
             const real_t zj = z[j];
             const real_t tq = quot(zj, shifted(j) - x);
-            if (j <= k) {
-                s.psi = fma(zj, tq, s.psi);
-                s.dpsi = fma(tq, tq, s.dpsi);
-            } else {
-                s.phi = fma(zj, tq, s.phi);
-                s.dphi = fma(tq, tq, s.dphi);
+            if (!right && j > k) {
+                right = true;
+                s.psi = s0; s.dpsi = s1;
+                s0 = R(0.0); s1 = R(0.0);
             }
+            s0 = fma(zj, tq, s0);
+            s1 = fma(tq, tq, s1);
         }
+        if (right) { s.phi = s0; s.dphi = s1; }
+        else { s.psi = s0; s.dpsi = s1; }
     } else {
         for (int j = lane; j <= k; j += G, ++t) {
             const real_t zj = z[j];
