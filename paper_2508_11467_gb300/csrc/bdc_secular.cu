@@ -267,22 +267,50 @@ __device__ __forceinline__ int root_iterate(const real_t *__restrict__ d, const 
 // then finishes from there.  Other poles within ~2^-23 relative of the
 // origin are only approximate in FP32: that costs FP64 steps, never
 // accuracy.  Updates r.x (r.lo, r.hi untouched); all lanes agree.
-template <int G>
-__device__ __forceinline__ void fp32_phase(const float *__restrict__ d32, const float *__restrict__ z32, int N,
-                                           int i, bool last, RootState &r) {
+// (fp32_iterate: T = the poles per lane it holds in registers, which do not
+// change between the steps (0: any number, read again each step); loads,
+// divisions and the straight-line sums of a step then overlap.  Few roots a
+// sub-partition are bound by this phase's instruction count: of the 12500
+// instructions a warp issued for n = 100's last merge, 550 were FP64.)
+template <int G, int T>
+__device__ __forceinline__ void fp32_iterate(const float *__restrict__ d32, const float *__restrict__ z32, int N,
+                                             int k, bool last, RootState &r) {
     const int lane = threadIdx.x & (G - 1);
-    const int k = last ? i - 1 : i;
     const float lamL = (float)r.lamL, lamR = (float)r.lamR;
     const float dor = d32[r.o];
     float x = (float)r.x, lo = (float)r.lo, hi = (float)r.hi;
+    float cj[T > 0 ? T : 1], zj[T > 0 ? T : 1];
+    if constexpr (T > 0) {
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const int j = lane + G * t;
+            const bool ok = j < N;
+            const float dj = ok ? d32[j] : 0.f;
+            zj[t] = ok ? z32[j] : 0.f;
+            cj[t] = (j == k) ? lamL : (j == k + 1) ? lamR : (dj - dor) * (dj + dor);
+        }
+    }
     for (int it = 0; it < 16; ++it) {
         float psi = 0.f, dpsi = 0.f, phi = 0.f, dphi = 0.f;
-        for (int j = lane; j < N; j += G) {
-            const float dj = d32[j], zj = z32[j];
-            const float c = (j == k) ? lamL : (j == k + 1) ? lamR : (dj - dor) * (dj + dor);
-            const float t = __fdividef(zj, c - x);   // approximate: this phase only starts the FP64 one
-            if (j <= k) { psi = fmaf(zj, t, psi); dpsi = fmaf(t, t, dpsi); }
-            else { phi = fmaf(zj, t, phi); dphi = fmaf(t, t, dphi); }
+        if constexpr (T > 0) {
+            float q[T];
+#pragma unroll
+            for (int t = 0; t < T; ++t)      // approximate: this phase only starts the FP64 one
+                q[t] = lane + G * t < N ? __fdividef(zj[t], cj[t] - x) : 0.f;
+#pragma unroll
+            for (int t = 0; t < T; ++t) {
+                const float l = lane + G * t <= k ? q[t] : 0.f, u = lane + G * t <= k ? 0.f : q[t];
+                psi = fmaf(zj[t], l, psi); dpsi = fmaf(l, l, dpsi);
+                phi = fmaf(zj[t], u, phi); dphi = fmaf(u, u, dphi);
+            }
+        } else {
+            for (int j = lane; j < N; j += G) {
+                const float dj = d32[j], zv = z32[j];
+                const float c = (j == k) ? lamL : (j == k + 1) ? lamR : (dj - dor) * (dj + dor);
+                const float t = __fdividef(zv, c - x);
+                if (j <= k) { psi = fmaf(zv, t, psi); dpsi = fmaf(t, t, dpsi); }
+                else { phi = fmaf(zv, t, phi); dphi = fmaf(t, t, dphi); }
+            }
         }
         psi = group_sum<G>(psi); dpsi = group_sum<G>(dpsi); phi = group_sum<G>(phi); dphi = group_sum<G>(dphi);
         const float f = 1.f + psi + phi;
@@ -296,6 +324,16 @@ __device__ __forceinline__ void fp32_phase(const float *__restrict__ d32, const 
     }
     const real_t xd = (real_t)x;
     if (xd > r.lo && xd < r.hi) r.x = xd;
+}
+
+template <int G>
+__device__ __forceinline__ void fp32_phase(const float *__restrict__ d32, const float *__restrict__ z32, int N,
+                                           int i, bool last, RootState &r) {
+    const int k = last ? i - 1 : i;
+    if (N <= 4 * G) fp32_iterate<G, 4>(d32, z32, N, k, last, r);
+    else if (N <= 8 * G) fp32_iterate<G, 8>(d32, z32, N, k, last, r);
+    else if (N <= 16 * G) fp32_iterate<G, 16>(d32, z32, N, k, last, r);
+    else fp32_iterate<G, 0>(d32, z32, N, k, last, r);
 }
 
 // Solve root i of (d, z) (N entries, d[0] = 0 < d[1] < ...).  Returns the
