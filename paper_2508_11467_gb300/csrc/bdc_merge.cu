@@ -37,7 +37,11 @@ namespace {
 
 constexpr int PREP_THREADS = 512;
 // chunks of 32 positions whose loads the deflation and numbering loops of
-// the prep issue together (one round trip per batch instead of per chunk)
+// the prep issue together (one round trip per batch instead of per chunk).
+// Merges with at most one chunk per warp take batches of one: their prep is a
+// single pass through this code, and the unrolled batches, predicated off,
+// were most of the 2800 instructions (and of the instruction fetches) of a
+// merge of order 12.
 constexpr int kDeflBatch = 8;
 constexpr int kNumBatch = 4;      // the same for the survivor numbering (more loads per chunk)
 constexpr int FL_START = 16, FL_MEMBER = 32;
@@ -128,6 +132,7 @@ __device__ __forceinline__ int col_side(int c, int nl) { return c == 0 ? 0 : (c 
 // each rotated pair, and the final z of every survivor in place in zs.
 // src (may be null) gives the pre-deflation column of each position, used to
 // type survivors.  Returns the number ns of small-z survivors.
+template <int kDB>
 __device__ int deflate_core(int m, real_t tol, const real_t *ds, real_t *zs, const int *src, int nl,
                             int *slist, int *sidx, int *role, real_t *rc, real_t *rs, int *wsum,
                             int *a_out) {
@@ -143,36 +148,36 @@ __device__ int deflate_core(int m, real_t tol, const real_t *ds, real_t *zs, con
     const rbits_t tolb = abits(tol);
     // survivors (position 0 and |z| > tol), numbered in ascending position
     // order.  Warp w takes the positions [wb, we) in chunks of 32 consecutive
-    // ones (lane = position: coalesced), the loads of kDeflBatch chunks in
+    // ones (lane = position: coalesced), the loads of kDB chunks in
     // flight together; a chunk's survivors are counted by a ballot and
     // numbered by the population count of the lower lanes.
     const int wspan = ((m + nw - 1) / nw + 31) & ~31;
     const int wb = min(m, (t >> 5) * wspan), we = min(m, wb + wspan);
     int cnt = 0;
-    for (int c0 = wb; c0 < we; c0 += 32 * kDeflBatch) {
-        rbits_t zb[kDeflBatch];
+    for (int c0 = wb; c0 < we; c0 += 32 * kDB) {
+        rbits_t zb[kDB];
 #pragma unroll
-        for (int u = 0; u < kDeflBatch; ++u) {
+        for (int u = 0; u < kDB; ++u) {
             const int p = c0 + 32 * u + lane;
             zb[u] = (p < we) ? abits(zs[p]) : (rbits_t)0;
         }
 #pragma unroll
-        for (int u = 0; u < kDeflBatch; ++u) {
+        for (int u = 0; u < kDB; ++u) {
             const int p = c0 + 32 * u + lane;
             cnt += __popc(__ballot_sync(0xffffffffu, p < we && (p == 0 || zb[u] > tolb)));
         }
     }
     int ns;
     int k = __shfl_sync(0xffffffffu, block_excl_scan(lane == 0 ? cnt : 0, wsum, ns), 0);
-    for (int c0 = wb; c0 < we; c0 += 32 * kDeflBatch) {
-        rbits_t zb[kDeflBatch];
+    for (int c0 = wb; c0 < we; c0 += 32 * kDB) {
+        rbits_t zb[kDB];
 #pragma unroll
-        for (int u = 0; u < kDeflBatch; ++u) {
+        for (int u = 0; u < kDB; ++u) {
             const int p = c0 + 32 * u + lane;
             zb[u] = (p < we) ? abits(zs[p]) : (rbits_t)0;
         }
 #pragma unroll
-        for (int u = 0; u < kDeflBatch; ++u) {
+        for (int u = 0; u < kDB; ++u) {
             const int p = c0 + 32 * u + lane;
             const bool keep = p < we && (p == 0 || zb[u] > tolb);
             const unsigned b = __ballot_sync(0xffffffffu, keep);
@@ -327,6 +332,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_merge_order(const NodeDesc *_
 }
 
 // ordered = 1: k_merge_order has written ds, src and zs at positions 1..m-1
+template <int kDB, int kNB>
 __global__ void __launch_bounds__(PREP_THREADS) k_merge_prep(const NodeDesc *__restrict__ nodes,
                                                              const MatDesc *__restrict__ mats,
                                                              NodeState *__restrict__ state,
@@ -389,30 +395,30 @@ __global__ void __launch_bounds__(PREP_THREADS) k_merge_prep(const NodeDesc *__r
     __syncthreads();
     // z of every position: alpha times the last row of a left child's right
     // vector, beta times the first row of a right child's.  Four positions
-    // per thread in flight: each level of the chain (source column, its
+    // per thread in flight (kNB): each level of the chain (source column, its
     // slot, the slot's range and entry) is loaded for all four before the
     // next, and the slot entry unconditionally (it lies inside the slot
     // column whatever its range), so the loads do not wait on one another.
-    for (int pos0 = 1 + t; !ordered && pos0 < m; pos0 += 4 * T) {
-        int jx[4];
-        bool left[4];
+    for (int pos0 = 1 + t; !ordered && pos0 < m; pos0 += kNB * T) {
+        int jx[kNB];
+        bool left[kNB];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kNB; ++u) {
             const int pos = pos0 + u * T;
             const int c = (pos < m) ? src[pos] : 1;
             left[u] = c <= nl;
             jx[u] = left[u] ? r0L + c - 1 : r0R + (c - nl - 1);
         }
-        real_t zv[4];
+        real_t zv[kNB];
         if (md.vals) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) zv[u] = left[u] ? md.vl[1 - nd.buf][jx[u]] : md.vf[1 - nd.buf][jx[u]];
+            for (int u = 0; u < kNB; ++u) zv[u] = left[u] ? md.vl[1 - nd.buf][jx[u]] : md.vf[1 - nd.buf][jx[u]];
         } else {
-            int g[4];
+            int g[kNB];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) g[u] = cvs[jx[u]];
+            for (int u = 0; u < kNB; ++u) g[u] = cvs[jx[u]];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < kNB; ++u) {
                 const long long row = left[u] ? r0L + nl : r0R;
                 const int lo = md.vlo[g[u]], hi = md.vhi[g[u]];
                 const real_t v = md.V[(size_t)g[u] * ld + row];
@@ -420,7 +426,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_merge_prep(const NodeDesc *__r
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kNB; ++u) {
             const int pos = pos0 + u * T;
             if (pos < m) zs[pos] = (left[u] ? alpha : beta) * zv[u];
         }
@@ -449,7 +455,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_merge_prep(const NodeDesc *__r
 
     // ---- deflation
     int a;
-    const int ns = deflate_core(m, tol, ds, zs, src, nl, md.slist + r0, md.sidx + r0, md.role + r0,
+    const int ns = deflate_core<kDB>(m, tol, ds, zs, src, nl, md.slist + r0, md.sidx + r0, md.role + r0,
                                 md.rc + r0, md.rs + r0, wsum, &a);
     (void)ns;
     const int *role = md.role + r0;
@@ -475,15 +481,15 @@ __global__ void __launch_bounds__(PREP_THREADS) k_merge_prep(const NodeDesc *__r
         return (code == ROLE_ZERO) ? 4 : 5;
     };
     int cnt[6] = {0, 0, 0, 0, 0, 0};             // this warp's counts (lane 0 keeps them)
-    for (int c0 = wb; c0 < we; c0 += 32 * kDeflBatch) {
-        int rr[kDeflBatch];                      // the roles of kDeflBatch chunks, loaded together
+    for (int c0 = wb; c0 < we; c0 += 32 * kDB) {
+        int rr[kDB];                      // the roles of kDB chunks, loaded together
 #pragma unroll
-        for (int u = 0; u < kDeflBatch; ++u) {
+        for (int u = 0; u < kDB; ++u) {
             const int p = c0 + 32 * u + lane;
             rr[u] = (p < we) ? role[p] : 0;
         }
 #pragma unroll
-        for (int u = 0; u < kDeflBatch; ++u) {
+        for (int u = 0; u < kDB; ++u) {
             const int p = c0 + 32 * u + lane;
             int grp = -1, cat = -1;
             if (p < we) cat = category(p, rr[u], grp);
@@ -516,28 +522,28 @@ __global__ void __launch_bounds__(PREP_THREADS) k_merge_prep(const NodeDesc *__r
     int *nus = slots ? md.us[nd.buf] + r0 : nullptr, *nvs = slots ? md.vs[nd.buf] + r0 : nullptr;
     auto slot_u = [&](int c) { return c == 0 ? r0 + nl : (c <= nl ? cus[r0L + c - 1] : cus[r0R + (c - nl - 1)]); };
     auto slot_v = [&](int c) { return c == 0 ? cvs[r0L + nl] : (c <= nl ? cvs[r0L + c - 1] : cvs[r0R + (c - nl - 1)]); };
-    // batches of kNumBatch chunks (nothing read here is written in this
+    // batches of kNB chunks (nothing read here is written in this
     // loop): the roles, values and sources of a batch are loaded together,
     // then the slots of its sources, before any of its stores
     auto ld_pos = [&](int q, int &rq, real_t &dq, real_t &zq, int &cq) {
         if (q < we) { rq = role[q]; dq = ds[q]; zq = zs[q]; cq = slots ? src[q] : 0; }
     };
-    for (int c0 = wb; c0 < we; c0 += 32 * kNumBatch) {
-        int rq[kNumBatch], cq[kNumBatch], suq[kNumBatch], svq[kNumBatch];
-        real_t dq[kNumBatch], zq[kNumBatch];
+    for (int c0 = wb; c0 < we; c0 += 32 * kNB) {
+        int rq[kNB], cq[kNB], suq[kNB], svq[kNB];
+        real_t dq[kNB], zq[kNB];
 #pragma unroll
-        for (int u = 0; u < kNumBatch; ++u) {
+        for (int u = 0; u < kNB; ++u) {
             rq[u] = cq[u] = suq[u] = svq[u] = 0;
             dq[u] = zq[u] = R(0);
             ld_pos(c0 + 32 * u + lane, rq[u], dq[u], zq[u], cq[u]);
         }
         if (slots) {
 #pragma unroll
-            for (int u = 0; u < kNumBatch; ++u)
+            for (int u = 0; u < kNB; ++u)
                 if (c0 + 32 * u + lane < we) { suq[u] = slot_u(cq[u]); svq[u] = slot_v(cq[u]); }
         }
 #pragma unroll
-        for (int u = 0; u < kNumBatch; ++u) {
+        for (int u = 0; u < kNB; ++u) {
             const int p = c0 + 32 * u + lane;
             const bool in = p < we;
             const int rp = rq[u], su = suq[u], sv = svq[u];
@@ -976,7 +982,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_deflate_single(int m, const re
     for (int p = threadIdx.x; p < m; p += blockDim.x) zs[p] = z[p];
     __syncthreads();
     int a;
-    deflate_core(m, tol, d, zs, nullptr, 0, slist, sidx, role, rc, rs, wsum, &a);
+    deflate_core<kDeflBatch>(m, tol, d, zs, nullptr, 0, slist, sidx, role, rc, rs, wsum, &a);
     for (int p = threadIdx.x; p < m; p += blockDim.x) {
         const int code = role[p] & 15;
         keep[p] = (code == ROLE_KEEP);
@@ -1005,7 +1011,8 @@ cudaError_t launch_merge_prep(const NodeDesc *nodes, int nnodes, const MatDesc *
     }
     // a warp per 32 entries of the largest node, up to PREP_THREADS
     const int T = std::min(PREP_THREADS, std::max(32, (mmax + 1 + 31) / 32 * 32));
-    k_merge_prep<<<nnodes, T, 0, st>>>(nodes, mats, state, probs, scans, ordered);
+    if (mmax <= T) k_merge_prep<1, 1><<<nnodes, T, 0, st>>>(nodes, mats, state, probs, scans, ordered);
+    else k_merge_prep<kDeflBatch, kNumBatch><<<nnodes, T, 0, st>>>(nodes, mats, state, probs, scans, ordered);
     return cudaGetLastError();
 }
 

@@ -136,7 +136,21 @@ __device__ __forceinline__ Sums pole_sums(const real_t *__restrict__ d, const re
         // with one pair of accumulators: a lane's poles ascend, so its sums
         // are psi's up to its first pole past k and phi's from there (two
         // FP64 operations a pole for every lane; a branch per pole made a
-        // warp whose groups split at different k issue both sides, four)
+        // warp whose groups split at different k issue both sides, four.
+        // In FP32 the branch's extra two cost less than the bookkeeping.)
+#ifdef BDC_FP32
+        for (int j = lane; j < N; j += G, ++t) {
+            const real_t zj = z[j];
+            const real_t tq = quot(zj, shifted(j) - x);
+            if (j <= k) {
+                s.psi = fma(zj, tq, s.psi);
+                s.dpsi = fma(tq, tq, s.dpsi);
+            } else {
+                s.phi = fma(zj, tq, s.phi);
+                s.dphi = fma(tq, tq, s.dphi);
+            }
+        }
+#else
         real_t s0 = R(0.0), s1 = R(0.0);
         bool right = false;
         for (int j = lane; j < N; j += G, ++t) {
@@ -152,6 +166,7 @@ __device__ __forceinline__ Sums pole_sums(const real_t *__restrict__ d, const re
         }
         if (right) { s.phi = s0; s.dphi = s1; }
         else { s.psi = s0; s.dpsi = s1; }
+#endif
     } else {
         for (int j = lane; j <= k; j += G, ++t) {
             const real_t zj = z[j];
@@ -360,7 +375,11 @@ __device__ __forceinline__ int solve_root(const real_t *__restrict__ d, const re
     const real_t dl = d[i];
     const real_t du = last ? sqrt(dl * dl + zz) : d[i + 1];
     const real_t h = R(0.5) * (du - dl);
+#ifdef BDC_FP32
+    constexpr bool pre32 = false;    // (the code of the phase costs the FP32 kernel registers: 538 -> 728 us a batch)
+#else
     const bool pre32 = d32 != nullptr;
+#endif
     const bool use_mlp = !last && ((vstart == vstart) || pre32);
     RootState r;
     r.dl = dl;
@@ -915,7 +934,11 @@ __global__ void __launch_bounds__(kLgThreads) k_vectors_warp(const NodeDesc *__r
     // keeps N <= 16 G there)
     const bool wu = md.want_u != 0;
     switch (G) {
-    case 4: vectors_group<4, 16>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu); break;
+    case 4:   // (merges of a few survivors: code for a few entries a lane)
+        if (N <= 16) vectors_group<4, 4>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu);
+        else if (N <= 32) vectors_group<4, 8>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu);
+        else vectors_group<4, 16>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu);
+        break;
     case 8: vectors_group<8, 16>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu); break;
     case 16: vectors_group<16, 16>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu); break;
     default:
