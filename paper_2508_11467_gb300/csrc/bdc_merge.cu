@@ -699,17 +699,18 @@ struct ColSrc {
 // to dst, by nthr threads from tid: four loads in flight per thread before
 // their stores (source and destination may not alias as far as the compiler
 // knows, so it would not hoist them itself)
+constexpr int kCopy = 4;   // loads in flight per thread
 __device__ __forceinline__ void copy_slot(real_t *__restrict__ dst, const real_t *__restrict__ src, int n,
                                           long long lo, long long hi, int tid, int nthr) {
-    for (int r = tid; r < n; r += 4 * nthr) {
-        real_t v[4];
+    for (int r = tid; r < n; r += kCopy * nthr) {
+        real_t v[kCopy];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kCopy; ++u) {
             const int row = r + u * nthr;
             v[u] = (row < n && row >= lo && row < hi) ? src[row] : R(0);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kCopy; ++u) {
             const int row = r + u * nthr;
             if (row < n) dst[row] = v[u];
         }
@@ -1016,11 +1017,17 @@ cudaError_t launch_merge_prep(const NodeDesc *nodes, int nnodes, const MatDesc *
     return cudaGetLastError();
 }
 
+// A warp per column task up to this order, a CTA per task above: a task is a
+// chain of six dependent descriptor loads and a copy, so tasks in flight count
+// (64 a SM by warps, 8 by CTAs), as long as a column is a few rounds of a
+// warp's loads.  512 matrices to order 1024: 4.49 -> 3.84 ms (FP32), 22.6 ->
+// 21.5 ms (FP64) against CTAs above 256; one matrix of 16384: 7.02 -> 6.96 ms.
+constexpr int kGatherWarpMax = 2048;
 cudaError_t launch_merge_gather(const NodeDesc *nodes, int nnodes, const MatDesc *mats,
                                 const NodeState *state, int mmax, cudaStream_t st) {
     if (nnodes <= 0) return cudaSuccess;
     const int ntasks = nnodes * mmax;
-    if (mmax <= 256) {
+    if (mmax <= kGatherWarpMax) {
         // a warp per column task, four per CTA
         k_merge_gather<4><<<(unsigned)(ntasks + 3) / 4, 128, 0, st>>>(nodes, mats, state, mmax, ntasks);
     } else {
