@@ -75,6 +75,7 @@ __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
 constexpr int DBK = 16, DSB = DBK + 4;
 template <int DBM, int DBN>
 __global__ void __launch_bounds__(128) k_dgemm(DGemm g) {
+    pdl_begin();
     constexpr int DSA = DBM + 8, WN = DBN / 32;
     static_assert(DBM / 32 * WN == 4, "four warps");
     __shared__ double As[DBK * DSA];   // As[k][m]
@@ -195,11 +196,11 @@ cudaError_t dgemm_launch(const DGemm &g, int splits, cudaStream_t st) {
     if (g.M <= 32) {
         const long long tiles = (long long)((g.M + 31) / 32) * ((g.N + 127) / 128);
         if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
-        k_dgemm<32, 128><<<dim3((unsigned)tiles, (unsigned)splits), 128, 0, st>>>(g);
+        launch_pdl(k_dgemm<32, 128>, dim3((unsigned)tiles, (unsigned)splits), 128, 0, st, g);
     } else {
         const long long tiles = (long long)((g.M + 63) / 64) * ((g.N + 63) / 64);
         if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
-        k_dgemm<64, 64><<<dim3((unsigned)tiles, (unsigned)splits), 128, 0, st>>>(g);
+        launch_pdl(k_dgemm<64, 64>, dim3((unsigned)tiles, (unsigned)splits), 128, 0, st, g);
     }
     return cudaGetLastError();
 }
@@ -414,6 +415,7 @@ __global__ void __launch_bounds__(256) k_geqr2(Geqr2Args a) {
 // of row j of A's panel, read with ldsrc = 1 and stride lda, off = 0 on the
 // shifted rows).
 __global__ void k_form_y(double *Y, int rows, int nb, const double *src, long long sr, long long sc) {
+    pdl_begin();
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= (long long)rows * nb) return;
     const int j = (int)(k / rows), r = (int)(k % rows);
@@ -440,6 +442,7 @@ struct Reflectors {
 
 // partial Y^T Y of block blockIdx.x over the rows of chunk blockIdx.y
 __global__ void __launch_bounds__(128) k_gram(Reflectors f, int kchunk, double *part) {
+    pdl_begin();
     constexpr int LD = kTB + 4;
     __shared__ double Ys[16 * LD];   // [row][reflector]
     const int i0 = blockIdx.x * kTB, nb = min(kTB, f.count - i0), rows = f.rows - i0;
@@ -521,6 +524,7 @@ struct TForm {
     long long gstride_g, gstride_t, cstride;
 };
 __global__ void __launch_bounds__(256) k_tform(TForm f) {
+    pdl_begin();
     extern __shared__ double tsm[];
     double *Gs = tsm, *Ts = tsm + kTB * kTLd, *Xs = Ts + kTB * kTLd;   // G, T, 32 x 32 product
     const int i0 = blockIdx.x * kTB, nb = min(kTB, f.count - i0);
@@ -566,7 +570,7 @@ cudaError_t launch_tform(const TForm &f, int blocks, cudaStream_t st) {
     cudaError_t e =
         cudaFuncSetAttribute(k_tform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTformSmem);
     if (e != cudaSuccess) return e;
-    k_tform<<<blocks, 256, kTformSmem, st>>>(f);
+    launch_pdl(k_tform, blocks, 256, kTformSmem, st, f);
     return cudaGetLastError();
 }
 
@@ -581,7 +585,7 @@ cudaError_t form_t(const Reflectors &f, const double *tau, double *Tall, cudaStr
     if (cap < 1) return cudaErrorInvalidValue;
     int kchunk = (int)((f.rows + chunks - 1) / chunks + 15) / 16 * 16;
     chunks = (f.rows + kchunk - 1) / kchunk;
-    k_gram<<<dim3(blocks, (unsigned)chunks), 128, 0, st>>>(f, kchunk, g_split_buf);
+    launch_pdl(k_gram, dim3(blocks, (unsigned)chunks), 128, 0, st, f, kchunk, g_split_buf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_tform(TForm{g_split_buf, Tall, tau, kTB, 1, (int)chunks, f.count, (long long)chunks * kTB * kTB,
@@ -596,6 +600,7 @@ cudaError_t form_t(const Reflectors &f, const double *tau, double *Tall, cudaStr
 __global__ void __launch_bounds__(256) k_tz(const double *__restrict__ T, int nb, int tr, const double *__restrict__ part,
                                             int splits, int right, int count, double *__restrict__ W,
                                             const double *__restrict__ add, int ldadd) {
+    pdl_begin();
     constexpr int V = 16, LD = V + 4;
     __shared__ double Zs[kTB * LD];   // [k][vector]
     const int v0 = blockIdx.x * V;
@@ -650,12 +655,12 @@ cudaError_t apply_block(int left, int trans, int rows, int cols, const double *Y
     int splits;
     if (left) {
         if ((e = dgemm_parts(1, 0, nb, cols, rows, Y, rows, C, ldc, splits, st)) != cudaSuccess) return e;
-        k_tz<<<(cols + 15) / 16, 256, 0, st>>>(T, nb, trans ? 1 : 0, g_split_buf, splits, 0, cols, W, nullptr, 0);
+        launch_pdl(k_tz, (cols + 15) / 16, 256, 0, st, T, nb, trans ? 1 : 0, g_split_buf, splits, 0, cols, W, nullptr, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         return dgemm(0, 0, rows, cols, nb, -1.0, Y, rows, W, nb, 1.0, C, ldc, st);
     }
     if ((e = dgemm_parts(0, 0, rows, nb, cols, C, ldc, Y, cols, splits, st)) != cudaSuccess) return e;
-    k_tz<<<(rows + 15) / 16, 256, 0, st>>>(T, nb, trans ? 0 : 1, g_split_buf, splits, 1, rows, W, nullptr, 0);
+    launch_pdl(k_tz, (rows + 15) / 16, 256, 0, st, T, nb, trans ? 0 : 1, g_split_buf, splits, 1, rows, W, nullptr, 0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return dgemm(0, 1, rows, cols, nb, -1.0, W, rows, Y, cols, 1.0, C, ldc, st);
 }
@@ -670,16 +675,18 @@ constexpr int kGramMost = 9;     // partial products of one block's Y^T Y at mos
 // G = Y^T Y above the diagonal from the partial products of Y without its unit
 // entries (symmetric): entry (r, c), r < c, adds reflector r's row c times
 // reflector c's unit entry.  T zeroed.
-__global__ void k_gram_sum(const double *__restrict__ part, Reflectors f, int chunks, double *__restrict__ G,
+__global__ void k_gram_sum(const double *__restrict__ part, Reflectors f, int chunk, int chunks, double *__restrict__ G,
                            double *__restrict__ T) {
+    pdl_begin();
     const size_t w2 = (size_t)kWide * kWide;
     const int k = blockIdx.x * blockDim.x + threadIdx.x, r = k / kWide, c = k % kWide;
     const int i0 = blockIdx.y * kWide, nb = min(kWide, f.count - i0);
     const double *p = part + (size_t)blockIdx.y * chunks * w2 + k;
     double s = 0.0;
     if (r < c && c < nb) {
+        const int own = (f.rows - i0 + chunk - 1) / chunk;   // this block's partial products
 #pragma unroll 4
-        for (int y = 0; y < chunks; ++y) s += p[(size_t)y * w2];
+        for (int y = 0; y < own; ++y) s += p[(size_t)y * w2];
         s += f.src[(size_t)i0 * (f.sr + f.sc) + (size_t)c * f.sr + (size_t)r * f.sc];
     }
     G[blockIdx.y * w2 + k] = s;
@@ -691,6 +698,7 @@ __global__ void k_gram_sum(const double *__restrict__ part, Reflectors f, int ch
 // -T_11 X (row-major, kWide x kWide per block; a fragment's K range skips the
 // zero half of the triangular factor)
 __global__ void __launch_bounds__(128) k_tmerge(const double *G, double *T, double *X, int h, int phase) {
+    pdl_begin();
     const size_t w2 = (size_t)kWide * kWide;
     const double *g = G + blockIdx.y * w2;
     double *t = T + blockIdx.y * w2, *x = X + blockIdx.y * w2;
@@ -769,10 +777,9 @@ cudaError_t form_v(const Reflectors &f, const double *tau, const SplitWs &w, cud
     const int blocks = (f.count + kWide - 1) / kWide;
     const size_t w2 = (size_t)kWide * kWide;
     cudaError_t e;
-    // the same number of chunks for every block (empty ones are zeroed)
+    // (a block below the first has as many chunks or fewer)
     const int chunk = std::max(512, ((f.rows + 7) / 8 + 31) / 32 * 32);
     const int chunks = (f.rows + chunk - 1) / chunk;
-    if ((e = cudaMemsetAsync(w.V, 0, sizeof(double) * w2 * blocks * chunks, st)) != cudaSuccess) return e;
     SplitSet set{w, st};
     for (int j = 0; j < blocks; ++j) {
         const int i0 = j * kWide, nb = std::min(kWide, f.count - i0), rows = f.rows - i0;
@@ -786,7 +793,7 @@ cudaError_t form_v(const Reflectors &f, const double *tau, const SplitWs &w, cud
         }
     }
     if ((e = set.run()) != cudaSuccess) return e;
-    k_gram_sum<<<dim3((unsigned)(w2 / 256), blocks), 256, 0, st>>>(w.V, f, chunks, w.G, w.T);
+    launch_pdl(k_gram_sum, dim3((unsigned)(w2 / 256), blocks), 256, 0, st, w.V, f, chunk, chunks, w.G, w.T);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = launch_tform(TForm{w.G, w.T, tau, kWide, kWide / kTB, 1, f.count, (long long)w2, (long long)w2, 0},
                           (f.count + kTB - 1) / kTB, st)) != cudaSuccess)
@@ -794,7 +801,7 @@ cudaError_t form_v(const Reflectors &f, const double *tau, const SplitWs &w, cud
     for (int h = kTB; h < kWide && h < f.count; h *= 2)
         for (int phase = 0; phase < 2; ++phase) {
             const int tiles = kWide / (2 * h) * (h / 8) * (h / 8);
-            k_tmerge<<<dim3((tiles + 3) / 4, blocks), 128, 0, st>>>(w.G, w.T, w.X, h, phase);
+            launch_pdl(k_tmerge, dim3((tiles + 3) / 4, blocks), 128, 0, st, w.G, w.T, w.X, h, phase);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     for (int j = 0; j < blocks; ++j) {
@@ -893,7 +900,7 @@ cudaError_t apply_panel(const Reflectors &f, const double *T, int rows, int cols
         if ((e = set.add(p)) != cudaSuccess) return e;
     }
     if ((e = set.run()) != cudaSuccess) return e;
-    k_tz<<<(cols + 15) / 16, 256, 0, st>>>(T, nb, 1, w.Z, np, 0, cols, W, C, ldc);
+    launch_pdl(k_tz, (cols + 15) / 16, 256, 0, st, T, nb, 1, w.Z, np, 0, cols, W, C, ldc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     SplitProd p{};
     p.a = y_rows(f, 0, rows);
@@ -922,6 +929,7 @@ __global__ void k_fill(double *X, long long rows, long long cols, long long ld, 
 
 // columns of the identity: column c has its one in row r0 + c
 __global__ void k_identity(double *X, long long rows, long long cols, long long ld, int r0) {
+    pdl_begin();
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= rows * cols) return;
     const long long c = k / rows, r = k % rows;
@@ -943,6 +951,7 @@ __global__ void k_zero_rows(double *X, long long ld, int r0, int r1, int cols) {
     X[(size_t)c * ld + r] = 0.0;
 }
 
+__global__ void k_clear_bar(GridBar *bar) { *bar = GridBar{0, 0, 0, 0}; }
 __global__ void k_read_err(const GridBar *bar, int *info) {
     if (bar->err) *info = BDC_ERR_TIMEOUT;
 }
@@ -1132,7 +1141,7 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
                 continue;
             }
             const long long cnt = (long long)ml * nb;
-            k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
+            launch_pdl(k_form_y, (unsigned)((cnt + 255) / 256), 256, 0, st, Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
             if ((err = apply_block(1, 1, ml, n - i0 - nb, Y, nb, Ti, A + i0 + (size_t)(i0 + nb) * lda, lda, Z, st)) !=
                 cudaSuccess)
@@ -1166,9 +1175,9 @@ cudaError_t dense_orgqr(int m, int n, int k, double *A, int lda, const double *t
         for (int i0 = (k - 1) / kWide * kWide; i0 >= 0; i0 -= kWide) {
             const int nb = std::min(kWide, k - i0), ml = m - i0;
             const long long cnt = (long long)ml * nb, c2 = (long long)m * nb;
-            k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
+            launch_pdl(k_form_y, (unsigned)((cnt + 255) / 256), 256, 0, st, Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
-            k_identity<<<(unsigned)((c2 + 255) / 256), 256, 0, st>>>(A + (size_t)i0 * lda, m, nb, lda, i0);
+            launch_pdl(k_identity, (unsigned)((c2 + 255) / 256), 256, 0, st, A + (size_t)i0 * lda, m, nb, lda, i0);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
             const Reflectors fy{Y, 1, ml, ml, nb};
             err = apply_wide(1, ml, n - i0, [&](int k0) { return y_vectors(fy, 0, nb, k0); }, nb,
@@ -1182,7 +1191,7 @@ cudaError_t dense_orgqr(int m, int n, int k, double *A, int lda, const double *t
     for (int i0 = last; i0 >= 0; i0 -= b) {
         const int nb = std::min(b, k - i0), ml = m - i0;
         const long long cnt = (long long)ml * nb;
-        k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
+        launch_pdl(k_form_y, (unsigned)((cnt + 255) / 256), 256, 0, st, Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         // the panel's columns become identity columns (rows i0.., zero above)
         const long long c2 = (long long)m * nb;
@@ -1227,7 +1236,7 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
         for (int i0 = last; i0 >= 0; i0 -= b) {
             const int nb = std::min(b, n - i0), ml = m - i0;
             const long long cnt = (long long)ml * nb;
-            k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
+            launch_pdl(k_form_y, (unsigned)((cnt + 255) / 256), 256, 0, st, Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
             if ((err = apply_block(1, 0, ml, cdim, Y, nb, Ti + (size_t)i0 * kTB, C + i0, ldc, Z, st)) != cudaSuccess)
                 return err;
@@ -1242,7 +1251,7 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
         const int nb = std::min(b, nr - i0), ny = n - 1 - i0;
         const long long cnt = (long long)ny * nb;
         // Y[r][j] = u_{i0+j} at column i0 + 1 + r: row i0 + j of A from column i0 + 1
-        k_form_y<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(Y, ny, nb, A + i0 + (size_t)(i0 + 1) * lda, lda, 1);
+        launch_pdl(k_form_y, (unsigned)((cnt + 255) / 256), 256, 0, st, Y, ny, nb, A + i0 + (size_t)(i0 + 1) * lda, lda, 1);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         if ((err = apply_block(0, 1, cdim, ny, Y, nb, Ti + (size_t)i0 * kTB, C + (size_t)(i0 + 1) * ldc, ldc, Z, st)) !=
             cudaSuccess)
@@ -1252,8 +1261,10 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
 }
 
 size_t dense_ws_bytes(int m, int n, int b) { return dense_ws(m, n, b, std::max(m, n)).total; }
+// (a kernel, not a memset: overlapped launches may follow it directly)
 cudaError_t dense_clear_err(char *ws, cudaStream_t st) {
-    return cudaMemsetAsync(ws + dense_ws(1, 1, 1, 1).bar, 0, sizeof(GridBar), st);
+    k_clear_bar<<<1, 1, 0, st>>>((GridBar *)(ws + dense_ws(1, 1, 1, 1).bar));
+    return cudaGetLastError();
 }
 cudaError_t dense_read_err(char *ws, int *info, cudaStream_t st) {
     k_read_err<<<1, 1, 0, st>>>((const GridBar *)(ws + dense_ws(1, 1, 1, 1).bar), info);
@@ -1345,6 +1356,7 @@ int bdc_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *ta
     if (n > 0 && (!d || !tauq || !taup || (n > 1 && !e))) return -5;
     if (!d_info) return -12;
     cudaStream_t st = (cudaStream_t)stream;
+    const OverlapScope overlapped(st);
     if (int r = note_cuda(cudaMemsetAsync(d_info, 0, sizeof(int), st))) return r;
     if (n == 0) return 0;
     if (!work) return -10;
@@ -1371,6 +1383,7 @@ int bdc_ormbr(int vect, int m, int n, const double *A, int lda, const double *ta
     const size_t need = dense_ws_bytes(std::max(m, cdim), std::max(n, cdim), kWsBlock) + 512;
     if (lwork < need) return -11;
     cudaStream_t st = (cudaStream_t)stream;
+    const OverlapScope overlapped(st);
     char *ws = align_ws(work);
     if (int r = note_cuda(dense_clear_err(ws, st))) return r;
     if (int r = note_cuda(dense_ormbr(vect, m, n, A, lda, tau, C, ldc, cdim, kApplyBlock, ws, st))) return r;
@@ -1396,6 +1409,7 @@ int bdc_geqrf(int m, int n, double *A, int lda, double *tau, void *work, size_t 
     if (std::min(m, n) > 0 && !tau) return -5;
     if (!d_info) return -9;
     cudaStream_t st = (cudaStream_t)stream;
+    const OverlapScope overlapped(st);
     if (int r = note_cuda(cudaMemsetAsync(d_info, 0, sizeof(int), st))) return r;
     if (std::min(m, n) == 0) return 0;
     if (!work) return -6;
@@ -1416,6 +1430,7 @@ int bdc_orgqr(int m, int n, double *A, int lda, const double *tau, void *work, s
     if (!work) return -6;
     if (lwork < bdc_geqrf_workspace(m, n)) return -7;
     cudaStream_t st = (cudaStream_t)stream;
+    const OverlapScope overlapped(st);
     char *ws = align_ws(work);
     if (int r = note_cuda(dense_clear_err(ws, st))) return r;
     if (int r = note_cuda(dense_orgqr(m, n, n, A, lda, tau, kApplyBlock, ws, st))) return r;
@@ -1438,6 +1453,7 @@ int bdc_gesvd(int m, int n, double *A, int lda, double *S, double *U, int ldu, d
     if (ldvt < std::max(1, n)) return -9;
     if (!d_info) return -13;
     cudaStream_t st = (cudaStream_t)stream;
+    const OverlapScope overlapped(st);
     if (int r = note_cuda(cudaMemsetAsync(d_info, 0, sizeof(int), st))) return r;
     if (n == 0) return 0;
     if (o && o->vectors != BDC_VEC_BOTH) return -10;

@@ -356,12 +356,14 @@ __global__ void __launch_bounds__(1024) k_scale(const MatDesc *__restrict__ mats
 // launch of the call (error word *err) makes every matrix report the timeout
 __global__ void k_info(const MatDesc *__restrict__ mats, int nmat, const int *__restrict__ err,
                        int *__restrict__ out) {
+    pdl_begin();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m < nmat) out[m] = (*err != 0) ? BDC_ERR_TIMEOUT : *mats[m].info;
 }
 
 // values only: S descending and unscaled
 __global__ void k_final_values(const MatDesc *__restrict__ mats) {
+    pdl_begin();
     const MatDesc &md = mats[blockIdx.y];
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < md.n) md.So[c] = md.D[md.Q[md.n - 1 - c]] * md.scale[0];
@@ -375,6 +377,7 @@ __global__ void k_final_values(const MatDesc *__restrict__ mats) {
 // store, so the loads of a tile are in flight together.
 constexpr int FINAL_ROWS = 512;
 __global__ void __launch_bounds__(256) k_final(const MatDesc *__restrict__ mats, int tiles_per_side) {
+    pdl_begin();
     __shared__ real_t tile[32][33];
     const MatDesc &md = mats[blockIdx.z];
     const int n = md.n;
@@ -591,6 +594,11 @@ double g_fp64[BDC_NSTAGES] = {0};
 
 }  // namespace
 
+bool &overlap() {
+    thread_local bool on = false;
+    return on;
+}
+
 StageScope::StageScope(cudaStream_t s, int k, long long l, double w) : st(s), stage(k), launches(l), work(w) {
     if (g_prof.on) {
         cudaEventCreate(&a);
@@ -719,6 +727,7 @@ int run_plan(const Plan &p, const bdc_opts &o, char *work, std::vector<MatDesc> 
     }
     cudaError_t e = upload(p, work, mats, st);
     if (e != cudaSuccess) return note(e);
+    const OverlapScope overlapped(st, !g_prof.on);
     SideStream *side = nullptr;
     if (!p.vals && !p.heights.empty() && (e = side_stream(side)) != cudaSuccess) return note(e);
     int *derr = (int *)(work + p.off_err);
@@ -837,7 +846,7 @@ int run_plan(const Plan &p, const bdc_opts &o, char *work, std::vector<MatDesc> 
                 return note(e);
             {
                 StageScope sc(side->s, BDC_STAGE_FINISH, 1, 24.0 * msum);
-                if ((e = launch_merge_finish(dn, nn, dmats, dstate, mm, side->s)) != cudaSuccess) return note(e);
+                if ((e = launch_merge_finish(dn, nn, dmats, dstate, mm, false, side->s)) != cudaSuccess) return note(e);
             }
             if ((e = cudaEventRecord(side->join, side->s)) != cudaSuccess) return note(e);
         }
@@ -873,7 +882,7 @@ int run_plan(const Plan &p, const bdc_opts &o, char *work, std::vector<MatDesc> 
         }
         if (!overlap) {   // node values and their order (O(m) per merge)
             StageScope sc(st, BDC_STAGE_FINISH, 1, 24.0 * msum);
-            if ((e = launch_merge_finish(dn, nn, dmats, dstate, mm, st)) != cudaSuccess) return note(e);
+            if ((e = launch_merge_finish(dn, nn, dmats, dstate, mm, true, st)) != cudaSuccess) return note(e);
         }
     }
     g_prof_level = -1;
@@ -881,7 +890,7 @@ int run_plan(const Plan &p, const bdc_opts &o, char *work, std::vector<MatDesc> 
         StageScope sc(st, BDC_STAGE_FINAL, (p.nmat + 65534) / 65535, 0.0);
         for (int m0 = 0; m0 < p.nmat; m0 += 65535) {
             const int nm = std::min(65535, p.nmat - m0);
-            k_final_values<<<dim3((unsigned)(p.nmax + 255) / 256, nm), 256, 0, st>>>(dmats + m0);
+            launch_pdl(k_final_values, dim3((unsigned)(p.nmax + 255) / 256, nm), 256, 0, st, dmats + m0);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return note(e);
     } else if (p.nmat > 0) {
@@ -893,7 +902,7 @@ int run_plan(const Plan &p, const bdc_opts &o, char *work, std::vector<MatDesc> 
         for (int m0 = 0; m0 < p.nmat; m0 += 65535) {
             const int nm = std::min(65535, p.nmat - m0);
             dim3 grid((unsigned)tps, (unsigned)(p.nmax + FINAL_ROWS - 1) / FINAL_ROWS, nm);
-            k_final<<<grid, 256, 0, st>>>(dmats + m0, tps);
+            launch_pdl(k_final, grid, 256, 0, st, dmats + m0, tps);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return note(e);
     }
@@ -912,7 +921,7 @@ int run_plan(const Plan &p, const bdc_opts &o, char *work, std::vector<MatDesc> 
     if (o.checked && p.nmat > 0 && (e = launch_check_final(dmats, p.nmat, st)) != cudaSuccess) return note(e);
     // gather the per-matrix status words into the caller's d_info
     if (p.nmat > 0) {
-        k_info<<<(p.nmat + 255) / 256, 256, 0, st>>>(dmats, p.nmat, derr, d_info_out);
+        launch_pdl(k_info, (p.nmat + 255) / 256, 256, 0, st, dmats, p.nmat, derr, d_info_out);
         if ((e = cudaGetLastError()) != cudaSuccess) return note(e);
     }
     return 0;

@@ -469,6 +469,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                                                      int *__restrict__ err, const int2 *__restrict__ tiles,
                                                      const int *__restrict__ ntiles, unsigned long long wait_ns,
                                                      int stall) {
+    pdl_begin();
     constexpr int TILE = TM * TK * 2;                 // one 128 x 32 BF16 slice tile (A or B)
     constexpr int SL = stage_slices<S, MODE>();       // slices per operand in a stage
     constexpr int STAGE_BYTES = stage_bytes<S, MODE>();
@@ -1105,15 +1106,12 @@ cudaError_t run_mixed(const GemmProb *probs, int nprobs, const std::vector<MixPr
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int grid = tiles < sm_count() ? tiles : sm_count();   // persistent: one CTA per SM
     if constexpr (EXACT) {
-        k_mma<S, MODE_E><<<grid, THREADS, smemE, st>>>(mae, mbe, probs, dmix, nprobs, E, F, err, tlist, ntiles,
-                                                       wait_ns, stall);
+        launch_pdl(k_mma<S, MODE_E>, grid, THREADS, smemE, st, mae, mbe, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, stall);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if constexpr (S > 4)
-            k_mma<S, MODE_L><<<grid, THREADS, smemL, st>>>(ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles,
-                                                           wait_ns, 0);
+            launch_pdl(k_mma<S, MODE_L>, grid, THREADS, smemL, st, ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, 0);
     } else {
-        k_mma<S, MODE_X3><<<grid, THREADS, smemX, st>>>(ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles,
-                                                        wait_ns, stall);
+        launch_pdl(k_mma<S, MODE_X3>, grid, THREADS, smemX, st, ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, stall);
     }
     return cudaGetLastError();
 }
@@ -1193,6 +1191,7 @@ struct SplitTab {
 __global__ void __launch_bounds__(256) k_split_tab(const __grid_constant__ SplitTab t, GemmProb *probs, MixProb *mix,
                                                    unsigned long long *maxA, unsigned long long *maxB, int2 *tiles,
                                                    int *ntiles) {
+    pdl_begin();
     int base = 0;
     for (int q = 0; q < t.count; ++q) {
         const SplitProd &p = t.p[q];
@@ -1246,6 +1245,7 @@ __device__ __forceinline__ double split_at(const SplitSide &s, int v, int k) {
 __global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ SplitTab t, __nv_bfloat16 *As,
                                                      __nv_bfloat16 *Bs, int *Ea, int *Fb, int rowsA, int colsB,
                                                      int Kld) {
+    pdl_begin();
     const SplitProd &p = t.p[blockIdx.y];
     const SplitSide s = blockIdx.z ? p.b : p.a;
     const int v = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -1280,6 +1280,7 @@ __global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ Spl
 // grid (vectors / 32, K / 128, products x sides)
 __global__ void __launch_bounds__(256) k_split_max(const __grid_constant__ SplitTab t, unsigned long long *maxA,
                                                    unsigned long long *maxB) {
+    pdl_begin();
     __shared__ unsigned long long sm[8][33];
     const SplitProd &p = t.p[blockIdx.z >> 1];
     const SplitSide s = (blockIdx.z & 1) ? p.b : p.a;
@@ -1307,6 +1308,7 @@ __global__ void __launch_bounds__(256) k_split_across(const __grid_constant__ Sp
                                                       __nv_bfloat16 *Bs, const unsigned long long *maxA,
                                                       const unsigned long long *maxB, int *Ea, int *Fb, int rowsA,
                                                       int colsB, int Kld) {
+    pdl_begin();
     __shared__ __nv_bfloat16 tile[DS][32][72];
     const SplitProd &p = t.p[blockIdx.z >> 1];
     const int side = blockIdx.z & 1;
@@ -1406,26 +1408,23 @@ cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t by
     cudaError_t e;
     if ((e = mma_attributes<DS, true>()) != cudaSuccess) return e;
     const int most = (int)std::max<long long>(std::max(rows, cols), tiles);
-    k_split_tab<<<std::min((most + 255) / 256, 64), 256, 0, st>>>(t, probs, mix, mA, mB, tl, nt);
+    launch_pdl(k_split_tab, std::min((most + 255) / 256, 64), 256, 0, st, t, probs, mix, mA, mB, tl, nt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (mv > 0) {
-        k_split_along<<<dim3((mv + 7) / 8, count, 2), 256, 0, st>>>(t, As, Bs, E, F, ra, cb, Kld);
+        launch_pdl(k_split_along, dim3((mv + 7) / 8, count, 2), 256, 0, st, t, As, Bs, E, F, ra, cb, Kld);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (mt > 0) {
-        k_split_max<<<dim3((mt + 31) / 32, (kt + 127) / 128, 2 * count), 256, 0, st>>>(t, mA, mB);
+        launch_pdl(k_split_max, dim3((mt + 31) / 32, (kt + 127) / 128, 2 * count), 256, 0, st, t, mA, mB);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_split_across<<<dim3((mt + 31) / 32, (kt + 63) / 64, 2 * count), 256, 0, st>>>(t, As, Bs, mA, mB, E, F, ra, cb,
-                                                                                       Kld);
+        launch_pdl(k_split_across, dim3((mt + 31) / 32, (kt + 63) / 64, 2 * count), 256, 0, st, t, As, Bs, mA, mB, E, F, ra, cb, Kld);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const int grid = (int)std::min<long long>(tiles, sm_count());
     const unsigned long long wait_ns = test_wait_ns();
-    k_mma<DS, MODE_EW><<<grid, THREADS, mma_smem<DS, MODE_EW>(), st>>>(mae, mbe, probs, mix, count, E, F, err, tl, nt,
-                                                                        wait_ns, 0);
+    launch_pdl(k_mma<DS, MODE_EW>, grid, THREADS, mma_smem<DS, MODE_EW>(), st, mae, mbe, probs, mix, count, E, F, err, tl, nt, wait_ns, 0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_mma<DS, MODE_LW><<<grid, THREADS, mma_smem<DS, MODE_LW>(), st>>>(ma, mb, probs, mix, count, E, F, err, tl, nt,
-                                                                        wait_ns, 0);
+    launch_pdl(k_mma<DS, MODE_LW>, grid, THREADS, mma_smem<DS, MODE_LW>(), st, ma, mb, probs, mix, count, E, F, err, tl, nt, wait_ns, 0);
     return cudaGetLastError();
 }
 

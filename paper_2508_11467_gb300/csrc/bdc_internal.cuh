@@ -29,6 +29,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <tuple>
+#include <utility>
 #include <vector>
 
 #include "../../include/bdc.h"
@@ -244,6 +246,51 @@ __device__ __forceinline__ void set_error(int *info, int code) {
     atomicCAS(info, 0, code);
 }
 
+// ------------------------------------------- launches that overlap their start
+// A solve is a chain of some 30 to 120 short kernels.  Those that directly
+// follow another kernel in their stream are launched with programmatic stream
+// serialization, which lets a kernel be set up while the one before still
+// runs; pdl_begin(), the first statement of each of them, waits until that
+// kernel has completed and its writes are visible (so a kernel completes only
+// after all before it have, and may rely on that).  No kernel triggers its
+// successor early (griddepcontrol.launch_dependents): CTAs that became
+// resident while the kernel before still ran were dealt unevenly to the SMs
+// (n = 16384: 6.99 ms with plain launches, 6.82 ms so, 7.35 ms with the early
+// trigger; n = 1001 1291, 1192, 1315 us; n = 100 585, 534, 541 us; values of
+// n = 10007 2.53, 2.34, 2.71 ms).  launch_pdl falls back to plain launches
+// where overlap() is off (graph capture, stage profiling).  A launch after an
+// event wait, a copy or a memset is a plain one.
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+bool &overlap();   // of the calling thread (bdc_driver.cu)
+// overlap() on for a scope unless `st` is being captured
+struct OverlapScope {
+    bool was;
+    explicit OverlapScope(cudaStream_t st, bool allowed = true) : was(overlap()) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        overlap() = allowed && cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+    }
+    ~OverlapScope() { overlap() = was; }
+};
+
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...a) {
+    std::tuple<P...> args(static_cast<P>(std::forward<A>(a))...);
+    void *ptrs[sizeof...(P)];
+    std::apply([&](auto &...x) { int i = 0; ((ptrs[i++] = (void *)&x), ...); }, args);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = overlap() ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, (const void *)k, ptrs);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // ------------------------------------------------------ host-side launchers
 // (each returns cudaGetLastError() of its launches)
 cudaError_t launch_scale(const MatDesc *mats, int nmat, int nmax, cudaStream_t st);
@@ -268,7 +315,7 @@ cudaError_t launch_gather_rows(const NodeDesc *nodes, int nnodes, const MatDesc 
 cudaError_t launch_rows_update(const NodeDesc *nodes, int nnodes, const MatDesc *mats,
                                const NodeState *state, int mmax, cudaStream_t st);
 cudaError_t launch_merge_finish(const NodeDesc *nodes, int nnodes, const MatDesc *mats,
-                                const NodeState *state, int mmax, cudaStream_t st);
+                                const NodeState *state, int mmax, bool after_kernel, cudaStream_t st);
 cudaError_t launch_final(const MatDesc *mats, int nmat, int nmax, cudaStream_t st);
 
 // checked mode (bdc_check.cu): invariants after the deflation, after the

@@ -112,6 +112,7 @@ __global__ void __launch_bounds__(32) k_leaf_rotations(const NodeDesc *__restric
                                                        const MatDesc *__restrict__ mats, int nleaves, int L,
                                                        int per_warp, int max_sweeps, int ccap,
                                                        char *__restrict__ log, NodeState *__restrict__ state) {
+    pdl_begin();
     extern __shared__ real_t sm[];
     const int lane = threadIdx.x;
     const int li = blockIdx.x * per_warp + lane;
@@ -487,6 +488,7 @@ __device__ __forceinline__ void chain_pivot(real_t *x, int ld, int first, int st
 __global__ void __launch_bounds__(32) k_leaf_vectors(const NodeDesc *__restrict__ leaves,
                                                      const MatDesc *__restrict__ mats, int L, int max_sweeps,
                                                      const char *__restrict__ log) {
+    pdl_begin();
     extern __shared__ real_t sm[];
     const int lane = threadIdx.x;
     const NodeDesc nd = leaves[blockIdx.x];
@@ -645,8 +647,7 @@ cudaError_t launch_leaves(const NodeDesc *leaves, int nleaves, const MatDesc *ma
                                              (int)smem1);
         if (e != cudaSuccess) return e;
     }
-    k_leaf_rotations<<<(nleaves + per_warp - 1) / per_warp, 32, smem1, st>>>(leaves, mats, nleaves, L, per_warp,
-                                                                             max_sweeps, ccap, (char *)log, state);
+    launch_pdl(k_leaf_rotations, (nleaves + per_warp - 1) / per_warp, 32, smem1, st, leaves, mats, nleaves, L, per_warp, max_sweeps, ccap, (char *)log, state);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || vals) return e;
     const size_t smem2 = sizeof(real_t) * ((size_t)L * L + (size_t)(L + 1) * (L + 1) + 6 * (size_t)(L + 1)) +
@@ -655,7 +656,7 @@ cudaError_t launch_leaves(const NodeDesc *leaves, int nleaves, const MatDesc *ma
         e = cudaFuncSetAttribute(k_leaf_vectors, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
         if (e != cudaSuccess) return e;
     }
-    k_leaf_vectors<<<nleaves, 32, smem2, st>>>(leaves, mats, L, max_sweeps, (const char *)log);
+    launch_pdl(k_leaf_vectors, nleaves, 32, smem2, st, leaves, mats, L, max_sweeps, (const char *)log);
     return cudaGetLastError();
 }
 

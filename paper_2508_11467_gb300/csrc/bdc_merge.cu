@@ -264,6 +264,7 @@ constexpr int ORDER_THREADS = 256, ORDER_SPAN = 4, ORDER_MIN = 4096;
 
 __global__ void __launch_bounds__(ORDER_THREADS) k_merge_order(const NodeDesc *__restrict__ nodes,
                                                                const MatDesc *__restrict__ mats) {
+    pdl_begin();
     const NodeDesc nd = nodes[blockIdx.y];
     const MatDesc &md = mats[nd.mat];
     const int m = nd.m, nl = nd.nl, nr = m - nl - 1;
@@ -338,6 +339,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_merge_prep(const NodeDesc *__r
                                                              NodeState *__restrict__ state,
                                                              GemmProb *__restrict__ probs, int scans,
                                                              int ordered) {
+    pdl_begin();
     __shared__ int wsum[PREP_THREADS / 32 + 1];
     __shared__ real_t dsum[PREP_THREADS / 32 + 1];
     const NodeDesc nd = nodes[blockIdx.x];
@@ -873,6 +875,7 @@ struct RowSrc {
 __global__ void __launch_bounds__(128) k_gather_rows(const NodeDesc *__restrict__ nodes,
                                                      const MatDesc *__restrict__ mats,
                                                      const NodeState *__restrict__ state, int mmax, int nnodes) {
+    pdl_begin();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int node = (int)(idx / mmax), p = (int)(idx % mmax);
     if (node >= nnodes) return;
@@ -938,6 +941,7 @@ __global__ void __launch_bounds__(128) k_gather_rows(const NodeDesc *__restrict_
 __global__ void __launch_bounds__(256) k_merge_finish(const NodeDesc *__restrict__ nodes,
                                                       const MatDesc *__restrict__ mats,
                                                       const NodeState *__restrict__ state) {
+    pdl_begin();
     const NodeDesc nd = nodes[blockIdx.y];
     const MatDesc &md = mats[nd.mat];
     const NodeState ns = state[nd.id];
@@ -1005,15 +1009,15 @@ cudaError_t launch_merge_prep(const NodeDesc *nodes, int nnodes, const MatDesc *
         const int chunks = (mmax + ORDER_THREADS * ORDER_SPAN - 1) / (ORDER_THREADS * ORDER_SPAN);
         for (int n0 = 0; n0 < nnodes; n0 += 65535) {     // grid y: at most 65535 nodes per launch
             const int nn = std::min(65535, nnodes - n0);
-            k_merge_order<<<dim3((unsigned)chunks, (unsigned)nn), ORDER_THREADS, 0, st>>>(nodes + n0, mats);
+            launch_pdl(k_merge_order, dim3((unsigned)chunks, (unsigned)nn), ORDER_THREADS, 0, st, nodes + n0, mats);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }
     }
     // a warp per 32 entries of the largest node, up to PREP_THREADS
     const int T = std::min(PREP_THREADS, std::max(32, (mmax + 1 + 31) / 32 * 32));
-    if (mmax <= T) k_merge_prep<1, 1><<<nnodes, T, 0, st>>>(nodes, mats, state, probs, scans, ordered);
-    else k_merge_prep<kDeflBatch, kNumBatch><<<nnodes, T, 0, st>>>(nodes, mats, state, probs, scans, ordered);
+    if (mmax <= T) launch_pdl(k_merge_prep<1, 1>, nnodes, T, 0, st, nodes, mats, state, probs, scans, ordered);
+    else launch_pdl(k_merge_prep<kDeflBatch, kNumBatch>, nnodes, T, 0, st, nodes, mats, state, probs, scans, ordered);
     return cudaGetLastError();
 }
 
@@ -1040,18 +1044,19 @@ cudaError_t launch_gather_rows(const NodeDesc *nodes, int nnodes, const MatDesc 
                                const NodeState *state, int mmax, cudaStream_t st) {
     if (nnodes <= 0) return cudaSuccess;
     const long long t = (long long)nnodes * mmax;
-    k_gather_rows<<<(unsigned)((t + 127) / 128), 128, 0, st>>>(nodes, mats, state, mmax, nnodes);
+    launch_pdl(k_gather_rows, (unsigned)((t + 127) / 128), 128, 0, st, nodes, mats, state, mmax, nnodes);
     return cudaGetLastError();
 }
 
 cudaError_t launch_merge_finish(const NodeDesc *nodes, int nnodes, const MatDesc *mats,
-                                const NodeState *state, int mmax, cudaStream_t st) {
+                                const NodeState *state, int mmax, bool after_kernel, cudaStream_t st) {
     if (nnodes <= 0) return cudaSuccess;
     const int T = std::min(256, std::max(32, (mmax + 31) / 32 * 32));
     const int chunks = std::max(1, mmax / (16 * 256));   // about 16 positions per thread for large merges
     for (int n0 = 0; n0 < nnodes; n0 += 65535) {         // grid y: at most 65535 nodes per launch
         const int nn = std::min(65535, nnodes - n0);
-        k_merge_finish<<<dim3((unsigned)chunks, (unsigned)nn), T, 0, st>>>(nodes + n0, mats, state);
+        if (after_kernel) launch_pdl(k_merge_finish, dim3((unsigned)chunks, (unsigned)nn), T, 0, st, nodes + n0, mats, state);
+        else k_merge_finish<<<dim3((unsigned)chunks, (unsigned)nn), T, 0, st>>>(nodes + n0, mats, state);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

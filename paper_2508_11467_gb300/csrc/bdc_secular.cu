@@ -630,6 +630,7 @@ __global__ void __launch_bounds__(kLgThreads, 16 / kLgWarps) k_secular(const Nod
                                                  const MatDesc *__restrict__ mats,
                                                  NodeState *__restrict__ state, int wpn,
                                                  int max_iter, int nnodes, int seed_mode, int fp32_start) {
+    pdl_begin();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int node = warp / wpn, w = warp % wpn;
     if (node >= nnodes) return;
@@ -758,6 +759,7 @@ __device__ __forceinline__ real_t lowner_one(const real_t *__restrict__ d, const
 __global__ void __launch_bounds__(kLgThreads) k_lowner(const NodeDesc *__restrict__ nodes,
                                                 const MatDesc *__restrict__ mats,
                                                 const NodeState *__restrict__ state, int wpn, int nnodes) {
+    pdl_begin();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int node = warp / wpn, w = warp % wpn;
     if (node >= nnodes) return;
@@ -915,6 +917,7 @@ __global__ void __launch_bounds__(kLgThreads) k_vectors_warp(const NodeDesc *__r
                                                       const MatDesc *__restrict__ mats,
                                                       const NodeState *__restrict__ state, int wpn,
                                                       int nnodes) {
+    pdl_begin();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int node = warp / wpn, w = warp % wpn;
     if (node >= nnodes) return;
@@ -979,6 +982,7 @@ __device__ __forceinline__ void rows_group(const real_t *__restrict__ d, const r
 __global__ void __launch_bounds__(kLgThreads) k_rows_update(const NodeDesc *__restrict__ nodes,
                                                      const MatDesc *__restrict__ mats,
                                                      const NodeState *__restrict__ state, int wpn, int nnodes) {
+    pdl_begin();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int node = warp / wpn, w = warp % wpn;
     if (node >= nnodes) return;
@@ -1040,14 +1044,12 @@ cudaError_t launch_secular(const NodeDesc *nodes, int nnodes, const MatDesc *mat
     }
 #endif
     const long long swarps = (long long)nnodes * secular_group_warps(mmax);
-    k_secular<<<(unsigned)((swarps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st>>>(
-        nodes, mats, state, secular_group_warps(mmax), max_iter, nnodes, seed_mode, fp32_start);
+    launch_pdl(k_secular, (unsigned)((swarps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st,  nodes, mats, state, secular_group_warps(mmax), max_iter, nnodes, seed_mode, fp32_start);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     }
     StageScope sc(st, BDC_STAGE_LOWNER, 1, 0.0);
-    k_lowner<<<(unsigned)((gwarps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st>>>(nodes, mats, state,
-                                                                                   group_warps(mmax), nnodes);
+    launch_pdl(k_lowner, (unsigned)((gwarps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st, nodes, mats, state, group_warps(mmax), nnodes);
     return cudaGetLastError();
 }
 
@@ -1055,8 +1057,7 @@ cudaError_t launch_vectors(const NodeDesc *nodes, int nnodes, const MatDesc *mat
                            int mmax, cudaStream_t st) {
     if (nnodes <= 0) return cudaSuccess;
     const long long warps = (long long)nnodes * group_warps(mmax);
-    k_vectors_warp<<<(unsigned)((warps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st>>>(nodes, mats, state,
-                                                                                        group_warps(mmax), nnodes);
+    launch_pdl(k_vectors_warp, (unsigned)((warps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st, nodes, mats, state, group_warps(mmax), nnodes);
     return cudaGetLastError();
 }
 
@@ -1064,8 +1065,7 @@ cudaError_t launch_rows_update(const NodeDesc *nodes, int nnodes, const MatDesc 
                                int mmax, cudaStream_t st) {
     if (nnodes <= 0) return cudaSuccess;
     const long long warps = (long long)nnodes * group_warps(mmax);
-    k_rows_update<<<(unsigned)((warps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st>>>(nodes, mats, state,
-                                                                                       group_warps(mmax), nnodes);
+    launch_pdl(k_rows_update, (unsigned)((warps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st, nodes, mats, state, group_warps(mmax), nnodes);
     return cudaGetLastError();
 }
 
