@@ -523,8 +523,14 @@ struct TForm {
     int ld, per, chunks, count;
     long long gstride_g, gstride_t, cstride;
 };
-__global__ void __launch_bounds__(256) k_tform(TForm f) {
+constexpr int kPair = 2;   // sets of reflectors (Q1 and P1) served by one launch
+struct TForms {
+    TForm f[kPair];
+};
+__global__ void __launch_bounds__(256) k_tform(const __grid_constant__ TForms fs) {
     pdl_begin();
+    const TForm &f = fs.f[blockIdx.y];
+    if ((int)blockIdx.x * kTB >= f.count) return;
     extern __shared__ double tsm[];
     double *Gs = tsm, *Ts = tsm + kTB * kTLd, *Xs = Ts + kTB * kTLd;   // G, T, 32 x 32 product
     const int i0 = blockIdx.x * kTB, nb = min(kTB, f.count - i0);
@@ -566,11 +572,13 @@ __global__ void __launch_bounds__(256) k_tform(TForm f) {
         Tall[(long long)(k / kTB) * f.ld + k % kTB] = Ts[(k / kTB) * kTLd + k % kTB];
 }
 constexpr size_t kTformSmem = sizeof(double) * (2 * kTB + 32) * kTLd;
-cudaError_t launch_tform(const TForm &f, int blocks, cudaStream_t st) {
+cudaError_t launch_tform(const TForm *f, int jobs, int blocks, cudaStream_t st) {
+    TForms fs{};
+    for (int q = 0; q < jobs; ++q) fs.f[q] = f[q];
     cudaError_t e =
         cudaFuncSetAttribute(k_tform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTformSmem);
     if (e != cudaSuccess) return e;
-    launch_pdl(k_tform, blocks, 256, kTformSmem, st, f);
+    launch_pdl(k_tform, dim3(blocks, jobs), 256, kTformSmem, st, fs);
     return cudaGetLastError();
 }
 
@@ -588,8 +596,9 @@ cudaError_t form_t(const Reflectors &f, const double *tau, double *Tall, cudaStr
     launch_pdl(k_gram, dim3(blocks, (unsigned)chunks), 128, 0, st, f, kchunk, g_split_buf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_tform(TForm{g_split_buf, Tall, tau, kTB, 1, (int)chunks, f.count, (long long)chunks * kTB * kTB,
-                              (long long)kTB * kTB, (long long)kTB * kTB}, blocks, st);
+    const TForm tf{g_split_buf, Tall, tau, kTB, 1, (int)chunks, f.count, (long long)chunks * kTB * kTB,
+                   (long long)kTB * kTB, (long long)kTB * kTB};
+    return launch_tform(&tf, 1, blocks, st);
 }
 
 // W = M Z for the summed partial products Z of dgemm_parts, M = T or T^T
@@ -675,33 +684,50 @@ constexpr int kGramMost = 9;     // partial products of one block's Y^T Y at mos
 // G = Y^T Y above the diagonal from the partial products of Y without its unit
 // entries (symmetric): entry (r, c), r < c, adds reflector r's row c times
 // reflector c's unit entry.  T zeroed.
-__global__ void k_gram_sum(const double *__restrict__ part, Reflectors f, int chunk, int chunks, double *__restrict__ G,
-                           double *__restrict__ T) {
+struct GramSum {
+    const double *part;
+    Reflectors f;
+    int chunk, chunks;
+    double *G, *T;
+};
+struct GramSums {
+    GramSum g[kPair];
+};
+__global__ void k_gram_sum(const __grid_constant__ GramSums gs) {
     pdl_begin();
+    const GramSum &a = gs.g[blockIdx.z];
+    const Reflectors &f = a.f;
     const size_t w2 = (size_t)kWide * kWide;
     const int k = blockIdx.x * blockDim.x + threadIdx.x, r = k / kWide, c = k % kWide;
     const int i0 = blockIdx.y * kWide, nb = min(kWide, f.count - i0);
-    const double *p = part + (size_t)blockIdx.y * chunks * w2 + k;
+    if (nb <= 0) return;
+    const double *p = a.part + (size_t)blockIdx.y * a.chunks * w2 + k;
     double s = 0.0;
     if (r < c && c < nb) {
-        const int own = (f.rows - i0 + chunk - 1) / chunk;   // this block's partial products
+        const int own = (f.rows - i0 + a.chunk - 1) / a.chunk;   // this block's partial products
 #pragma unroll 4
         for (int y = 0; y < own; ++y) s += p[(size_t)y * w2];
         s += f.src[(size_t)i0 * (f.sr + f.sc) + (size_t)c * f.sr + (size_t)r * f.sc];
     }
-    G[blockIdx.y * w2 + k] = s;
-    T[blockIdx.y * w2 + k] = 0.0;
+    a.G[blockIdx.y * w2 + k] = s;
+    a.T[blockIdx.y * w2 + k] = 0.0;
 }
 
 // the off-diagonal blocks of T from its h x h diagonal blocks, one 8 x 8
 // fragment per warp, operands from L2: phase 0: X = G_12 T_22, phase 1: T_12 =
 // -T_11 X (row-major, kWide x kWide per block; a fragment's K range skips the
 // zero half of the triangular factor)
-__global__ void __launch_bounds__(128) k_tmerge(const double *G, double *T, double *X, int h, int phase) {
+struct TMerge {
+    const double *G[kPair];
+    double *T[kPair], *X[kPair];
+    int blocks[kPair];
+};
+__global__ void __launch_bounds__(128) k_tmerge(const __grid_constant__ TMerge a, int h, int phase) {
     pdl_begin();
+    if ((int)blockIdx.y >= a.blocks[blockIdx.z]) return;
     const size_t w2 = (size_t)kWide * kWide;
-    const double *g = G + blockIdx.y * w2;
-    double *t = T + blockIdx.y * w2, *x = X + blockIdx.y * w2;
+    const double *g = a.G[blockIdx.z] + blockIdx.y * w2;
+    double *t = a.T[blockIdx.z] + blockIdx.y * w2, *x = a.X[blockIdx.z] + blockIdx.y * w2;
     const int lane = threadIdx.x & 31, gr = lane >> 2, tg = lane & 3;
     const int per = (h / 8) * (h / 8);
     const int q = blockIdx.x * 4 + (threadIdx.x >> 5);
@@ -771,84 +797,101 @@ struct SplitSet {
     }
 };
 
-// V = Y T of every kWide block of the reflectors (row-major T): V of block j
-// at w.V + i0 f.rows, column-major, f.rows - i0 rows, leading dimension f.rows
-cudaError_t form_v(const Reflectors &f, const double *tau, const SplitWs &w, cudaStream_t st) {
-    const int blocks = (f.count + kWide - 1) / kWide;
+// A set of reflectors to apply: left: C := Q C (C f.rows x other), right: C
+// := C P^T (other x f.rows; C's first column is the reflectors' first row),
+// with workspace of its own (slices and the error word may be shared).
+struct WideJob {
+    Reflectors f;
+    const double *tau;
+    int left, other;
+    double *C;
+    int ldc;
+    SplitWs w;
+    int blocks() const { return (f.count + kWide - 1) / kWide; }
+};
+
+// V = Y T of every kWide block of the jobs' reflectors (row-major T): V of
+// block j at w.V + i0 f.rows, column-major, f.rows - i0 rows, leading
+// dimension f.rows
+cudaError_t form_v(const WideJob *jobs, int njobs, cudaStream_t st) {
     const size_t w2 = (size_t)kWide * kWide;
     cudaError_t e;
-    // (a block below the first has as many chunks or fewer)
-    const int chunk = std::max(512, ((f.rows + 7) / 8 + 31) / 32 * 32);
-    const int chunks = (f.rows + chunk - 1) / chunk;
-    SplitSet set{w, st};
-    for (int j = 0; j < blocks; ++j) {
-        const int i0 = j * kWide, nb = std::min(kWide, f.count - i0), rows = f.rows - i0;
-        for (int y = 0, k0 = 0; k0 < rows; ++y, k0 += chunk) {
-            SplitProd p{};
-            p.a = p.b = y_vectors(f, i0, nb, k0);
-            p.C = w.V + ((size_t)j * chunks + y) * w2;
-            p.ldc = kWide;
-            p.K = std::min(chunk, rows - k0);
-            if ((e = set.add(p)) != cudaSuccess) return e;
+    SplitSet set{jobs[0].w, st};
+    GramSums gs{};
+    TForm tf[kPair];
+    TMerge tm{};
+    int most = 0, count = 0;
+    for (int q = 0; q < njobs; ++q) {
+        const Reflectors &f = jobs[q].f;
+        const SplitWs &w = jobs[q].w;
+        const int blocks = jobs[q].blocks();
+        // (a block below the first has as many chunks or fewer)
+        const int chunk = std::max(512, ((f.rows + 7) / 8 + 31) / 32 * 32);
+        const int chunks = (f.rows + chunk - 1) / chunk;
+        for (int j = 0; j < blocks; ++j) {
+            const int i0 = j * kWide, nb = std::min(kWide, f.count - i0), rows = f.rows - i0;
+            for (int y = 0, k0 = 0; k0 < rows; ++y, k0 += chunk) {
+                SplitProd p{};
+                p.a = p.b = y_vectors(f, i0, nb, k0);
+                p.C = w.V + ((size_t)j * chunks + y) * w2;
+                p.ldc = kWide;
+                p.K = std::min(chunk, rows - k0);
+                if ((e = set.add(p)) != cudaSuccess) return e;
+            }
         }
+        gs.g[q] = GramSum{w.V, f, chunk, chunks, w.G, w.T};
+        tf[q] = TForm{w.G, w.T, jobs[q].tau, kWide, kWide / kTB, 1, f.count, (long long)w2, (long long)w2, 0};
+        tm.G[q] = w.G; tm.T[q] = w.T; tm.X[q] = w.X; tm.blocks[q] = blocks;
+        most = std::max(most, blocks);
+        count = std::max(count, f.count);
     }
     if ((e = set.run()) != cudaSuccess) return e;
-    launch_pdl(k_gram_sum, dim3((unsigned)(w2 / 256), blocks), 256, 0, st, w.V, f, chunk, chunks, w.G, w.T);
+    launch_pdl(k_gram_sum, dim3((unsigned)(w2 / 256), most, njobs), 256, 0, st, gs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = launch_tform(TForm{w.G, w.T, tau, kWide, kWide / kTB, 1, f.count, (long long)w2, (long long)w2, 0},
-                          (f.count + kTB - 1) / kTB, st)) != cudaSuccess)
-        return e;
-    for (int h = kTB; h < kWide && h < f.count; h *= 2)
+    if ((e = launch_tform(tf, njobs, (count + kTB - 1) / kTB, st)) != cudaSuccess) return e;
+    for (int h = kTB; h < kWide && h < count; h *= 2)
         for (int phase = 0; phase < 2; ++phase) {
             const int tiles = kWide / (2 * h) * (h / 8) * (h / 8);
-            launch_pdl(k_tmerge, dim3((tiles + 3) / 4, blocks), 128, 0, st, w.G, w.T, w.X, h, phase);
+            launch_pdl(k_tmerge, dim3((tiles + 3) / 4, most, njobs), 128, 0, st, tm, h, phase);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-    for (int j = 0; j < blocks; ++j) {
-        const int i0 = j * kWide, nb = std::min(kWide, f.count - i0), rows = f.rows - i0;
-        SplitProd p{};
-        p.a = y_rows(f, i0, rows);
-        p.b = SplitSide{w.T + j * w2, 0, kWide, 1, nb, 1, 0, 0, 0};
-        p.C = w.V + (size_t)i0 * f.rows;
-        p.ldc = f.rows;
-        p.K = nb;
-        if ((e = set.add(p)) != cudaSuccess) return e;
-    }
+    for (int q = 0; q < njobs; ++q)
+        for (int j = 0; j < jobs[q].blocks(); ++j) {
+            const Reflectors &f = jobs[q].f;
+            const int i0 = j * kWide, nb = std::min(kWide, f.count - i0);
+            SplitProd p{};
+            p.a = y_rows(f, i0, f.rows - i0);
+            p.b = SplitSide{jobs[q].w.T + j * w2, 0, kWide, 1, nb, 1, 0, 0, 0};
+            p.C = jobs[q].w.V + (size_t)i0 * f.rows;
+            p.ldc = f.rows;
+            p.K = nb;
+            if ((e = set.add(p)) != cudaSuccess) return e;
+        }
     return set.run();
 }
 
-// C := (I - V Y^T) C (left, C rows x cols) or C (I - Y V^T) (right), with Y
-// the `nb` reflectors given as K-along vectors yk(k0) and V nb columns (ld ldv)
-template <typename YK>
-cudaError_t apply_wide(int left, int rows, int cols, YK yk, int nb, const double *V, int ldv, double *C, int ldc,
-                       const SplitWs &w, cudaStream_t st) {
-    cudaError_t e;
-    const int K = left ? rows : cols, other = left ? cols : rows;
-    // slabs of the untouched dimension that fit the slice scratch and the Z parts
-    const int tb = (nb + 127) / 128;
-    int slab = (other + 127) / 128 * 128;
-    auto parts_of = [&](int s) {
-        const int t = tb * ((s + 127) / 128);
-        return std::max({1, (K + kSplitMostK - 1) / kSplitMostK, std::min({kSplitMax, 152 / std::max(t, 1), K / 256})});
-    };
-    for (; slab > 128; slab = (slab / 2 + 127) / 128 * 128) {
-        const int np = parts_of(slab), kc = ((K + np - 1) / np + 31) / 32 * 32;
-        if ((size_t)np * nb * slab <= w.zcap &&
-            split_scratch((long long)np * nb, (long long)np * slab, kc, (long long)np * tb * (slab / 128)) <= w.slice_bytes &&
-            split_scratch(slab, K, nb, (long long)(slab / 128) * ((K + 127) / 128)) <= w.slice_bytes &&
-            split_scratch(K, slab, nb, (long long)(slab / 128) * ((K + 127) / 128)) <= w.slice_bytes)
-            break;
+// One block of a job on ns rows or columns of C from s0: C := (I - V Y^T) C
+// (left) or C (I - Y V^T) (right).  yk(k0): the block's reflectors as K-along
+// vectors from row k0.
+struct WideStep {
+    int left, rows, nb, np, kc, ns;   // rows of the block's reflectors; np products of kc rows each
+    double *c;
+    int ldc;
+    const double *V;
+    int ldv;
+    double *Z;
+    void cut(int parts) {             // K = rows in `parts` products at most
+        np = std::max({1, (rows + kSplitMostK - 1) / kSplitMostK, std::min(parts, rows / 256)});
+        kc = ((rows + np - 1) / np + 31) / 32 * 32;
+        np = (rows + kc - 1) / kc;
     }
-    for (int s0 = 0; s0 < other; s0 += slab) {
-        const int ns = std::min(slab, other - s0);
-        const int np0 = parts_of(ns), kc = ((K + np0 - 1) / np0 + 31) / 32 * 32, np = (K + kc - 1) / kc;
-        double *c = C + (left ? (size_t)s0 * ldc : (size_t)s0);
-        const long long zs = (long long)nb * ns;
-        SplitSet set{w, st};
+    int tiles() const { return (nb + 127) / 128 * ((ns + 127) / 128); }
+    template <typename YK>
+    cudaError_t products(YK yk, SplitSet &set) const {
         for (int y = 0; y < np; ++y) {
             SplitProd p{};
-            p.K = std::min(kc, K - y * kc);
-            p.C = w.Z + y * zs;
+            p.K = std::min(kc, rows - y * kc);
+            p.C = Z + (long long)y * nb * ns;
             if (left) {        // Z (nb x ns) = Y^T C
                 p.a = yk(y * kc);
                 p.b = SplitSide{c + y * kc, 0, ldc, 0, ns, 1, 0, 0, 0};
@@ -858,9 +901,12 @@ cudaError_t apply_wide(int left, int rows, int cols, YK yk, int nb, const double
                 p.b = yk(y * kc);
                 p.ldc = ns;
             }
-            if ((e = set.add(p)) != cudaSuccess) return e;
+            if (cudaError_t e = set.add(p)) return e;
         }
-        if ((e = set.run()) != cudaSuccess) return e;
+        return cudaSuccess;
+    }
+    cudaError_t update(SplitSet &set) const {
+        const long long zs = (long long)nb * ns;
         SplitProd p{};
         p.K = nb;
         p.C = c;
@@ -868,12 +914,98 @@ cudaError_t apply_wide(int left, int rows, int cols, YK yk, int nb, const double
         p.sub = 1;
         if (left) {            // C -= V Z
             p.a = SplitSide{V, 0, ldv, 1, rows, 1, 0, 0, 0};
-            p.b = SplitSide{w.Z, zs, nb, 0, ns, np, 0, 0, 0, nullptr, 0, 0, c, ldc, 1};   // + C's first nb rows
+            p.b = SplitSide{Z, zs, nb, 0, ns, np, 0, 0, 0, nullptr, 0, 0, c, ldc, 1};   // + C's first nb rows
         } else {               // C -= Z V^T
-            p.a = SplitSide{w.Z, zs, ns, 1, ns, np, 0, 0, 0, nullptr, 0, 0, c, 1, ldc};   // + C's first nb columns
-            p.b = SplitSide{V, 0, ldv, 1, cols, 1, 0, 0, 0};
+            p.a = SplitSide{Z, zs, ns, 1, ns, np, 0, 0, 0, nullptr, 0, 0, c, 1, ldc};   // + C's first nb columns
+            p.b = SplitSide{V, 0, ldv, 1, rows, 1, 0, 0, 0};
         }
-        if ((e = set.add(p)) != cudaSuccess) return e;
+        return set.add(p);
+    }
+};
+
+// the step of the whole untouched dimension; its block's C starts at c
+WideStep wide_step(int left, int rows, int other, int nb, const double *V, int ldv, double *c, int ldc,
+                   const SplitWs &w) {
+    return WideStep{left, rows, nb, 1, 0, other, c, ldc, V, ldv, w.Z};
+}
+
+// one block, in slabs of the untouched dimension that fit the slice scratch and the Z parts
+template <typename YK>
+cudaError_t apply_wide(int left, int rows, int other, YK yk, int nb, const double *V, int ldv, double *C, int ldc,
+                       const SplitWs &w, cudaStream_t st) {
+    cudaError_t e;
+    int slab = (other + 127) / 128 * 128;
+    auto step_of = [&](int s) {
+        WideStep x = wide_step(left, rows, s, nb, V, ldv, C, ldc, w);
+        x.cut(std::min(kSplitMax, 152 / std::max(x.tiles(), 1)));
+        return x;
+    };
+    for (; slab > 128; slab = (slab / 2 + 127) / 128 * 128) {
+        const WideStep x = step_of(slab);
+        const long long t = x.tiles();
+        if ((size_t)x.np * nb * slab <= w.zcap &&
+            split_scratch((long long)x.np * nb, (long long)x.np * slab, x.kc, x.np * t) <= w.slice_bytes &&
+            split_scratch(slab, rows, nb, (long long)(slab / 128) * ((rows + 127) / 128)) <= w.slice_bytes &&
+            split_scratch(rows, slab, nb, (long long)(slab / 128) * ((rows + 127) / 128)) <= w.slice_bytes)
+            break;
+    }
+    SplitSet set{w, st};
+    for (int s0 = 0; s0 < other; s0 += slab) {
+        WideStep x = step_of(std::min(slab, other - s0));
+        x.c = C + (left ? (size_t)s0 * ldc : (size_t)s0);
+        if ((e = x.products(yk, set)) != cudaSuccess || (e = set.run()) != cudaSuccess ||
+            (e = x.update(set)) != cudaSuccess || (e = set.run()) != cudaSuccess)
+            return e;
+    }
+    return cudaSuccess;
+}
+
+// where block i0 of a job starts in its C
+double *job_c(const WideJob &j, int i0) { return j.C + (j.left ? (size_t)i0 : (size_t)i0 * j.ldc); }
+
+// the blocks of one job from the last to the first
+cudaError_t apply_job(const WideJob &j, cudaStream_t st) {
+    if (cudaError_t e = form_v(&j, 1, st)) return e;
+    for (int i0 = (j.blocks() - 1) * kWide; i0 >= 0; i0 -= kWide) {
+        const int nb = std::min(kWide, j.f.count - i0), rows = j.f.rows - i0;
+        auto yk = [&](int k0) { return y_vectors(j.f, i0, nb, k0); };
+        if (cudaError_t e = apply_wide(j.left, rows, j.other, yk, nb, j.w.V + (size_t)i0 * j.f.rows, j.f.rows,
+                                       job_c(j, i0), j.ldc, j.w, st))
+            return e;
+    }
+    return cudaSuccess;
+}
+
+// Two jobs side by side (the back-transformations of U and V^T), their
+// products in the same launches: below about order 2000 a block's products
+// leave most SMs without a tile and its time is the launches' and the K loop
+// of a tile's (gesvd of 333 x 333: 4.57 ms one after the other, 4.11 ms so).
+cudaError_t apply_pair(const WideJob (&j)[kPair], cudaStream_t st) {
+    cudaError_t e;
+    if ((e = form_v(j, kPair, st)) != cudaSuccess) return e;
+    SplitSet set{j[0].w, st};
+    for (int b = std::max(j[0].blocks(), j[1].blocks()) - 1; b >= 0; --b) {
+        WideStep x[kPair];
+        int tiles = 0;
+        bool live[kPair];
+        for (int q = 0; q < kPair; ++q) {
+            const int i0 = b * kWide;
+            if (!(live[q] = b < j[q].blocks())) continue;
+            x[q] = wide_step(j[q].left, j[q].f.rows - i0, j[q].other, std::min(kWide, j[q].f.count - i0),
+                             j[q].w.V + (size_t)i0 * j[q].f.rows, j[q].f.rows, job_c(j[q], i0), j[q].ldc, j[q].w);
+            tiles += x[q].tiles();
+        }
+        for (int q = 0; q < kPair; ++q)
+            if (live[q]) {
+                const int fit = (int)(j[q].w.zcap / ((size_t)x[q].nb * x[q].ns));
+                x[q].cut(std::min({kSplitMax / kPair, 152 / std::max(tiles, 1), fit}));
+                if ((e = x[q].products([&](int k0) { return y_vectors(j[q].f, b * kWide, x[q].nb, k0); }, set)) !=
+                    cudaSuccess)
+                    return e;
+            }
+        if ((e = set.run()) != cudaSuccess) return e;
+        for (int q = 0; q < kPair; ++q)
+            if (live[q] && (e = x[q].update(set)) != cudaSuccess) return e;
         if ((e = set.run()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -973,10 +1105,13 @@ constexpr int kDenseBlock = 32;   // b: columns / rows per panel (reflectors per
 constexpr int kApplyBlock = kTB;
 constexpr int kWsBlock = kApplyBlock > kDenseBlock ? kApplyBlock : kDenseBlock;   // workspace sizing
 
+constexpr size_t kPairMost = 2048;   // largest dimension of back-transformations done side by side
+
 // workspace layout of the dense routines (bytes from an aligned base)
 struct DenseWs {
     size_t bar, PW, QW, part, Y, Ti, Z, split, split_doubles, res, lab, total;
     size_t wG, wT, wX, wV, wZ, wZcap, wS, wSbytes;   // split path
+    size_t pG, pT, pX, pV, pZ;                       // ... of a second job (order up to kPairMost)
 };
 
 DenseWs dense_ws(int m, int n, int b, int zcols) {
@@ -1003,6 +1138,13 @@ DenseWs dense_ws(int m, int n, int b, int zcols) {
         w.wV = o; o += al256(sizeof(double) * std::max(D * n, blocks * kGramMost * w2));
         w.wZcap = std::max<size_t>((size_t)kWide * 2 * (D + 256), (size_t)kWide * 4096);
         w.wZ = o; o += al256(sizeof(double) * w.wZcap);
+        if (D <= kPairMost) {
+            w.pG = o; o += al256(sizeof(double) * blocks * w2);
+            w.pT = o; o += al256(sizeof(double) * blocks * w2);
+            w.pX = o; o += al256(sizeof(double) * blocks * w2);
+            w.pV = o; o += al256(sizeof(double) * std::max(D * n, blocks * kGramMost * w2));
+            w.pZ = o; o += al256(sizeof(double) * w.wZcap);
+        }
         // enough for whole products up to about 340 MB, then slabs of 128
         const size_t Dp = (D + 31) / 32 * 32 + 32;
         const size_t all = 2 * (D + 2 * kWide + 256) * std::max<size_t>(Dp, 544);
@@ -1017,6 +1159,13 @@ DenseWs dense_ws(int m, int n, int b, int zcols) {
 SplitWs split_ws(char *ws, const DenseWs &w) {
     return SplitWs{(double *)(ws + w.wG), (double *)(ws + w.wT), (double *)(ws + w.wX), (double *)(ws + w.wV),
                    (double *)(ws + w.wZ), w.wZcap, ws + w.wS, w.wSbytes, &((GridBar *)(ws + w.bar))->err};
+}
+
+SplitWs split_ws2(char *ws, const DenseWs &w) {
+    SplitWs s = split_ws(ws, w);
+    s.G = (double *)(ws + w.pG); s.T = (double *)(ws + w.pT); s.X = (double *)(ws + w.pX);
+    s.V = (double *)(ws + w.pV); s.Z = (double *)(ws + w.pZ);
+    return s;
 }
 
 // the split-K scratch of the calling thread's dense routine
@@ -1131,7 +1280,8 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
         if (i0 + nb < n) {
             const int cols = n - i0 - nb;
             const Reflectors f{A + i0 + (size_t)i0 * lda, 1, lda, ml, nb};
-            err = resident ? launch_tform(TForm{gram, Ti, tau + i0, kTB, 1, 1, nb, 0, 0, 0}, 1, st)
+            const TForm tf{gram, Ti, tau + i0, kTB, 1, 1, nb, 0, 0, 0};
+            err = resident ? launch_tform(&tf, 1, 1, st)
                            : form_t(f, tau + i0, Ti, st);
             if (err != cudaSuccess) return err;
             if (panel_split(ml, cols, sw)) {
@@ -1171,7 +1321,8 @@ cudaError_t dense_orgqr(int m, int n, int k, double *A, int lda, const double *t
     if (use_wide(k, m, n)) {
         const SplitWs sw = split_ws(ws, w);
         const Reflectors f{A, 1, lda, m, k};
-        if ((err = form_v(f, tau, sw, st)) != cudaSuccess) return err;
+        const WideJob job{f, tau, 1, n, A, lda, sw};
+        if ((err = form_v(&job, 1, st)) != cudaSuccess) return err;
         for (int i0 = (k - 1) / kWide * kWide; i0 >= 0; i0 -= kWide) {
             const int nb = std::min(kWide, k - i0), ml = m - i0;
             const long long cnt = (long long)ml * nb, c2 = (long long)m * nb;
@@ -1218,17 +1369,8 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
     const int refl = vect == 0 ? n : n - 1;
     if (use_wide(refl, vect == 0 ? m : n - 1, cdim)) {
         const SplitWs sw = split_ws(ws, w);
-        const Reflectors f = vect == 0 ? Reflectors{A, 1, lda, m, n} : Reflectors{A + lda, lda, 1, n - 1, n - 1};
-        if ((err = form_v(f, tau, sw, st)) != cudaSuccess) return err;
-        for (int i0 = (refl - 1) / kWide * kWide; i0 >= 0; i0 -= kWide) {
-            const int nb = std::min(kWide, refl - i0), ry = f.rows - i0;
-            auto yk = [&](int k0) { return y_vectors(f, i0, nb, k0); };
-            const double *V = sw.V + (size_t)i0 * f.rows;
-            err = vect == 0 ? apply_wide(1, ry, cdim, yk, nb, V, f.rows, C + i0, ldc, sw, st)
-                            : apply_wide(0, cdim, ry, yk, nb, V, f.rows, C + (size_t)(i0 + 1) * ldc, ldc, sw, st);
-            if (err != cudaSuccess) return err;
-        }
-        return cudaSuccess;
+        return apply_job(vect == 0 ? WideJob{{A, 1, lda, m, n}, tau, 1, cdim, C, ldc, sw}
+                                   : WideJob{{A + lda, lda, 1, n - 1, n - 1}, tau, 0, cdim, C + ldc, ldc, sw}, st);
     }
     if (vect == 0) {
         if ((err = form_t(Reflectors{A, 1, lda, m, n}, tau, Ti, st)) != cudaSuccess) return err;
@@ -1258,6 +1400,19 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
             return err;
     }
     return cudaSuccess;
+}
+
+// U := Q1 U (m x n) and VT := VT P1^T (n x n) with the reflectors of gebrd
+cudaError_t dense_ormbr_both(int m, int n, const double *A, int lda, const double *tauq, const double *taup, double *U,
+                             int ldu, double *VT, int ldvt, int b, char *ws, cudaStream_t st) {
+    const DenseWs w = dense_ws(m, n, b, n);
+    if ((size_t)std::max(m, n) <= kPairMost && use_wide(n - 1, m, n)) {
+        const WideJob j[kPair] = {{{A, 1, lda, m, n}, tauq, 1, n, U, ldu, split_ws(ws, w)},
+                                  {{A + lda, lda, 1, n - 1, n - 1}, taup, 0, n, VT + ldvt, ldvt, split_ws2(ws, w)}};
+        return apply_pair(j, st);
+    }
+    if (cudaError_t e = dense_ormbr(0, m, n, A, lda, tauq, U, ldu, n, b, ws, st)) return e;
+    return dense_ormbr(1, m, n, A, lda, taup, VT, ldvt, n, b, ws, st);
 }
 
 size_t dense_ws_bytes(int m, int n, int b) { return dense_ws(m, n, b, std::max(m, n)).total; }
@@ -1328,9 +1483,9 @@ struct GesvdWs {
 GesvdWs gesvd_layout(int m, int n, const bdc_opts *o) {
     GesvdWs w{};
     size_t off = 0;
-    w.dense = off; off += al256(dense_ws_bytes(m, n, kWsBlock));
-    w.vecs = off; off += al256(sizeof(double) * 4 * (size_t)n + 64);
     const bool qr = m >= kQrRatio * n;
+    w.dense = off; off += al256(std::max(dense_ws_bytes(m, n, kWsBlock), qr ? dense_ws_bytes(n, n, kWsBlock) : 0));
+    w.vecs = off; off += al256(sizeof(double) * 4 * (size_t)n + 64);
     w.R = off; off += qr ? al256(sizeof(double) * (size_t)n * n) : 0;
     w.UR = off; off += qr ? al256(sizeof(double) * (size_t)n * n) : 0;
     w.bdc = off; off += al256(bdc_svd_workspace(n, o));
@@ -1477,15 +1632,13 @@ int bdc_gesvd(int m, int n, double *A, int lda, double *S, double *U, int ldu, d
         if ((rc = note_cuda(cudaMemsetAsync(tq, 0, sizeof(double) * n, st)))) return rc;
         if ((rc = note_cuda(dense_gebrd(n, n, R, n, d, e, tq, tp, b, dws, st)))) return rc;
         if ((rc = bdc_svd_ex(n, d, e, UR, S, VT, n, ldvt, o, ws + L.bdc, lwb, d_info, stream))) return rc;
-        if ((rc = note_cuda(dense_ormbr(0, n, n, R, n, tq, UR, n, n, kApplyBlock, dws, st)))) return rc;
-        if ((rc = note_cuda(dense_ormbr(1, n, n, R, n, tp, VT, ldvt, n, kApplyBlock, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_ormbr_both(n, n, R, n, tq, tp, UR, n, VT, ldvt, kApplyBlock, dws, st)))) return rc;
         if ((rc = note_cuda(dense_product(m, n, A, lda, UR, U, ldu, dws, st)))) return rc;
     } else {
         if ((rc = note_cuda(dense_gebrd(m, n, A, lda, d, e, tq, tp, b, dws, st)))) return rc;
         if ((rc = bdc_svd_ex(n, d, e, U, S, VT, ldu, ldvt, o, ws + L.bdc, lwb, d_info, stream))) return rc;
         if ((rc = note_cuda(dense_zero_rows(U, ldu, n, m, n, st)))) return rc;
-        if ((rc = note_cuda(dense_ormbr(0, m, n, A, lda, tq, U, ldu, n, kApplyBlock, dws, st)))) return rc;
-        if ((rc = note_cuda(dense_ormbr(1, m, n, A, lda, tp, VT, ldvt, n, kApplyBlock, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_ormbr_both(m, n, A, lda, tq, tp, U, ldu, VT, ldvt, kApplyBlock, dws, st)))) return rc;
     }
     return note_cuda(dense_read_err(dws, d_info, st));
 }

@@ -162,7 +162,7 @@ __device__ __forceinline__ void slot_get(const Slot *(&p)[K], unsigned tag, doub
 
 constexpr int NT = 128;            // threads per CTA: one warp per SM sub-partition
 constexpr int kRedLd = NT + 8;     // row stride of the reduction buffer
-constexpr int LR = 8;              // rows of a CTA handled together
+constexpr int LR = 12;             // rows of a CTA handled together at most (1500 x 1100: 17.3 ms at 8, 16.5 at 12)
 
 // f(integral_constant<K>) for K = k in 1..LR: straight-line code per row
 // count, so that the loads, FMAs and stores of all rows are scheduled
@@ -328,7 +328,7 @@ struct Gebd2Args {
 // dependent FP64 chains of a step (64 cycles an operation), above n ~ 1000
 // the FP64 pipe.  333 x 333: 18.9 ms (blocked panels, seven barriers a step)
 // -> 2.8 ms; 1000 x 1000: 71 -> 12 ms; 1500 x 1100: 82 -> 17 ms.
-__global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
+__global__ void __launch_bounds__(NT, 1) k_gebd2_resident(Gebd2Args a) {
     extern __shared__ double smem[];
     __shared__ int s_err;
     const int G = gridDim.x, g = blockIdx.x, t = threadIdx.x;
@@ -466,9 +466,11 @@ __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
         // A -= v y^T with the products h = A r (the tail of row i: columns
         // i + 2...) in chunks of LR rows; slot LR of the last chunk: ||r||^2
         double pi, betr;
-        for (int b0 = l0;; b0 += LR) {
-            const int nq = max(0, min(LR, lr - b0));    // rows of this chunk
-            const bool lastc = b0 + LR >= lr;
+        // equal chunks of at most LR rows
+        const int chunks = max(1, (lr - l0 + LR - 1) / LR), rows0 = (lr - l0 + chunks - 1) / chunks;
+        for (int b0 = l0;; b0 += rows0) {
+            const int nq = max(0, min(rows0, lr - b0));   // rows of this chunk
+            const bool lastc = b0 + rows0 >= lr;
             double nrm = 0.0;                           // slot nq of the reduction: ||r||^2 (last chunk)
             if (lastc)
                 for (int c = i + 1 + t; c < n; c += NT) {
@@ -521,9 +523,10 @@ __global__ void __launch_bounds__(NT) k_gebd2_resident(Gebd2Args a) {
             sr[c] = u;
             if (l1 >= lr) slot_put(a.gp + (size_t)g * ldw + c, 0.0, tag + 1u);
         }
-        for (int b0 = l1; b0 < lr; b0 += LR) {
-            const int nq = min(LR, lr - b0);
-            Slot *gp = b0 + LR >= lr ? a.gp + (size_t)g * ldw : nullptr;
+        const int chunks1 = max(1, (lr - l1 + LR - 1) / LR), rows1 = max(1, (lr - l1 + chunks1 - 1) / chunks1);
+        for (int b0 = l1; b0 < lr; b0 += rows1) {
+            const int nq = min(rows1, lr - b0);
+            Slot *gp = b0 + rows1 >= lr ? a.gp + (size_t)g * ldw : nullptr;
             rows_dispatch<LR>(nq, [&](auto K) {
                 pass_right<decltype(K)::value>(W + (size_t)b0 * ldw, ldw, xv + b0, av + b0, sr, sy, b0 == l1, gp, i, n,
                                                t, tag + 1u);
