@@ -83,9 +83,18 @@ constexpr int kSecPoles = 16;
 __host__ __device__ __forceinline__ int secular_group_size(int N) {
     return N <= 4 * kSecPoles ? 4 : N <= 8 * kSecPoles ? 8 : N <= 16 * kSecPoles ? 16 : 32;
 }
-// warps per node: ceil(N G(N) / 32) grows with N, so mmax bounds it
-__host__ __device__ __forceinline__ int secular_group_warps(int mmax) {
-    return (int)(((long long)mmax * secular_group_size(mmax) + 31) / 32);
+// roots per warp: 32 / G, or fewer (>> spread, at least one) when the merges
+// of a height have few roots for the chip: the groups of a warp take their
+// own paths (iterations, origin switches), which the warp issues one after
+// another, so a warp of one root is done when its root is
+__host__ __device__ __forceinline__ int secular_roots_per_warp(int N, int spread) {
+    const int per = (32 / secular_group_size(N)) >> spread;
+    return per < 1 ? 1 : per;
+}
+// warps per node (N <= mmax needs no more: its G is no larger)
+__host__ __device__ __forceinline__ int secular_group_warps(int mmax, int spread) {
+    const int per = secular_roots_per_warp(mmax, spread);
+    return (mmax + per - 1) / per;
 }
 
 // Warps per CTA of the lane-group kernels (k_secular, k_lowner,
@@ -624,21 +633,23 @@ __device__ __forceinline__ void secular_group(const NodeDesc &nd, const MatDesc 
     }
 }
 
-// Warp w of a node (secular_group_warps(mmax) per node) serves roots w * (32 / G) + (lane / G),
-// G = secular_group_size(N) from the node's survivor count, known only here.
+// Warp w of a node (wpn per node) serves roots w * per + (lane / G), per =
+// secular_roots_per_warp, G = secular_group_size(N) from the node's survivor
+// count, known only here.
 __global__ void __launch_bounds__(kLgThreads, 16 / kLgWarps) k_secular(const NodeDesc *__restrict__ nodes,
                                                  const MatDesc *__restrict__ mats,
                                                  NodeState *__restrict__ state, int wpn,
-                                                 int max_iter, int nnodes, int seed_mode, int fp32_start) {
+                                                 int max_iter, int nnodes, int seed_mode, int fp32_start,
+                                                 int spread) {
     pdl_begin();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int node = warp / wpn, w = warp % wpn;
     if (node >= nnodes) return;
     const NodeDesc nd = nodes[node];
     const NodeState ns = state[nd.id];
-    const int N = ns.N, G = secular_group_size(N), per = 32 / G;
+    const int N = ns.N, G = secular_group_size(N), per = secular_roots_per_warp(N, spread);
     const int i = w * per + lane / G;
-    if (i >= N) return;                              // whole groups leave together
+    if (i >= N || lane >= per * G) return;           // whole groups leave together
     const MatDesc &md = mats[nd.mat];
     const real_t zz = ns.rho;                        // sum z^2 (computed by the merge prep)
     __shared__ real_t s_lam[kLgWarps][kLamCache * 32];   // shifted poles of each lane's root (pole_sums)
@@ -1018,6 +1029,13 @@ __global__ void __launch_bounds__(256) k_mvectors_single(int N, const double *d,
 
 }  // namespace
 
+// About one warp per SM sub-partition (4 x 152): up to there a warp with fewer
+// roots takes no FP64 issue from another.  Limits of 0 / 700 / 1300 warps,
+// timed in turn: n = 100 531 / 510 / 517 us, n = 1001 1193 / 1176 / 1176 us,
+// n = 4096 (FP64) 6946 / 6946 / 6959 us; 2600 and more slow the large orders
+// (n = 4096 7036 us, values only at n = 10007 2417 us against 2343 us).
+constexpr long long kSpreadWarps = 700;
+
 cudaError_t launch_secular(const NodeDesc *nodes, int nnodes, const MatDesc *mats, NodeState *state,
                            int mmax, int max_iter, int seed_mode, const float *mlp, int harvest, int fp32_start,
                            cudaStream_t st) {
@@ -1043,8 +1061,12 @@ cudaError_t launch_secular(const NodeDesc *nodes, int nnodes, const MatDesc *mat
         if (e != cudaSuccess) return e;
     }
 #endif
-    const long long swarps = (long long)nnodes * secular_group_warps(mmax);
-    launch_pdl(k_secular, (unsigned)((swarps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st,  nodes, mats, state, secular_group_warps(mmax), max_iter, nnodes, seed_mode, fp32_start);
+    int spread = 0;
+    while (spread < 3 && nnodes * (long long)secular_group_warps(mmax, spread + 1) <= kSpreadWarps) ++spread;
+    const int wpn = secular_group_warps(mmax, spread);
+    const long long swarps = (long long)nnodes * wpn;
+    launch_pdl(k_secular, (unsigned)((swarps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st, nodes, mats, state, wpn,
+               max_iter, nnodes, seed_mode, fp32_start, spread);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     }
