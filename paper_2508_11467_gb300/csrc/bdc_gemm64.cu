@@ -2,9 +2,10 @@
 // all column-major, a batch of independent problems per launch (four per
 // merge node: the top and bottom blocks of W~ U_M and Q~ V_M).
 //
-// FP32 build: CUDA-core FP32 FMA, CTA tile 64 x 64, K step 16, 256 threads
-// of 4 x 4 outputs, operands staged k-major in padded shared tiles (float4
-// reads), the next K step prefetched into registers.
+// FP32 build: CUDA-core FP32 FMA in packed pairs, CTA tiles 64 x 32 or
+// 32 x 32 (launch_gemm64), 8 x 4 outputs a thread, operands staged k-major in
+// two padded shared buffers (float4 reads, one barrier a K step), the next K
+// step prefetched into registers.
 //
 // FP64 build: tensor-core FP64 (DMMA, mma.sync.m8n8k4.f64).  CTA tile 64 x 64
 // (32 x 32, 32 x 64 or 64 x 32 for small problems), K step 16, warps of
@@ -20,60 +21,86 @@ namespace BDC_NS {
 namespace {
 
 #ifdef BDC_FP32
-constexpr int BM = 64, BN = 64, BK = 16, SP = 68;   // SP: padded row stride of both tiles (floats)
+// acc(lo, hi) += a(lo, hi) * b: two FP32 fused multiply-adds, each rounded as
+// fmaf rounds
+__device__ __forceinline__ void ffma2(unsigned long long &acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long pair2(float lo, float hi) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
 
-__global__ void __launch_bounds__(256) k_gemm32(const GemmProb *__restrict__ probs, int tilesN) {
-    __shared__ __align__(16) float As[BK * SP];    // As[k][m]
-    __shared__ __align__(16) float Bs[BK * SP];    // Bs[k][n]
+// RT x CT threads of 8 rows x 4 columns each.  Bound by latency (global loads
+// of a step, shared reads) and by padding of the many small blocks, not by the
+// FMA rate: the tiles are small, the registers capped (MINB) so that ~28 warps
+// an SM are in flight, and BK = 8 halves the staging registers and shared
+// memory.  Both operands of two FMAs ride in one packed instruction.  512
+// matrices of order 32..1024 (whole solve): 64 x 64 tiles of 256 threads and
+// single FMAs 4236 us; 64 x 64 tiles of 128 threads, packed, 3739; 64 x 32
+// 3633; K step 8 and 70 registers 3489 (130 registers: 4008, 64: 3544).
+// 64 x 64 with 8 x 8 outputs a thread: 3793.
+template <int RT, int CT, int BK, int MINB>
+__global__ void __launch_bounds__(RT * CT, MINB) k_gemm32(const GemmProb *__restrict__ probs, int tilesN) {
+    constexpr int BM = 8 * RT, BN = 4 * CT, T = RT * CT;
+    constexpr int SA = BM + 4, SB = BN + 4;          // padded row strides (floats)
+    constexpr int LA = BM * BK / T, LB = BN * BK / T;
+    __shared__ __align__(16) float As[2][BK * SA];   // As[.][k][m]
+    __shared__ __align__(16) float Bs[2][BK * SB];   // Bs[.][k][n]
     const GemmProb pr = probs[blockIdx.y];
     const int m0 = (blockIdx.x / tilesN) * BM, n0 = (blockIdx.x % tilesN) * BN;
     if (m0 >= pr.M || n0 >= pr.N) return;
     const int tid = threadIdx.x;
-    const int tm = (tid >> 4) * 4, tn = (tid & 15) * 4;
+    const int tm = (tid / CT) * 8, tn = (tid % CT) * 4;
     const float *__restrict__ A = pr.A;
     const float *__restrict__ B = pr.B;
     const int M = pr.M, N = pr.N, K = pr.K, lda = pr.lda, ldb = pr.ldb;
-    float acc[4][4];
+    unsigned long long acc[4][4];                   // rows 2 i, 2 i + 1
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    float ra[4], rb[4];
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    float ra[LA], rb[LB];
     auto load = [&](int k0) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int idx = tid + r * 256;       // 0..1023
-            const int am = idx & 63, ak = idx >> 6;
-            const int gm = m0 + am, gk = k0 + ak;
+        for (int r = 0; r < LA; ++r) {
+            const int idx = tid + r * T, gm = m0 + idx % BM, gk = k0 + idx / BM;
             ra[r] = (gm < M && gk < K) ? A[(size_t)gk * lda + gm] : 0.f;
-            const int bk = idx & 15, bn = idx >> 4;
-            const int gn = n0 + bn, gk2 = k0 + bk;
-            rb[r] = (gn < N && gk2 < K) ? B[(size_t)gn * ldb + gk2] : 0.f;
         }
-    };
-    auto store = [&]() {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int idx = tid + r * 256;
-            As[(idx >> 6) * SP + (idx & 63)] = ra[r];
-            Bs[(idx & 15) * SP + (idx >> 4)] = rb[r];
+        for (int r = 0; r < LB; ++r) {
+            const int idx = tid + r * T, gk = k0 + idx % BK, gn = n0 + idx / BK;
+            rb[r] = (gn < N && gk < K) ? B[(size_t)gn * ldb + gk] : 0.f;
         }
     };
     load(0);
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        __syncthreads();
-        store();
+    for (int k0 = 0, buf = 0; k0 < K; k0 += BK, buf ^= 1) {
+        // one barrier a step: the buffer written here was last read two steps
+        // ago, before the barrier of the step between
+#pragma unroll
+        for (int r = 0; r < LA; ++r) {
+            const int idx = tid + r * T;
+            As[buf][(idx / BM) * SA + idx % BM] = ra[r];
+        }
+#pragma unroll
+        for (int r = 0; r < LB; ++r) {
+            const int idx = tid + r * T;
+            Bs[buf][(idx % BK) * SB + idx / BK] = rb[r];
+        }
         __syncthreads();
         if (k0 + BK < K) load(k0 + BK);
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            const float4 a = *reinterpret_cast<const float4 *>(As + kk * SP + tm);
-            const float4 b = *reinterpret_cast<const float4 *>(Bs + kk * SP + tn);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+            const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(&As[buf][kk * SA + tm]);
+            const ulonglong2 a1 = *reinterpret_cast<const ulonglong2 *>(&As[buf][kk * SA + tm + 4]);
+            const unsigned long long av[4] = {a0.x, a0.y, a1.x, a1.y};
+            const float4 b = *reinterpret_cast<const float4 *>(&Bs[buf][kk * SB + tn]);
+            const unsigned long long bv[4] = {pair2(b.x, b.x), pair2(b.y, b.y), pair2(b.z, b.z), pair2(b.w, b.w)};
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+                for (int i = 0; i < 4; ++i) ffma2(acc[i][j], av[i], bv[j]);
         }
     }
     float *__restrict__ C = pr.C;
@@ -84,10 +111,23 @@ __global__ void __launch_bounds__(256) k_gemm32(const GemmProb *__restrict__ pro
         float *__restrict__ Cc = C + gemm_col(pr, gn);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int gm = m0 + tm + i;
-            if (gm < M) Cc[gm] = acc[i][j];
+            const int gm = m0 + tm + 2 * i;
+            if (gm < M) Cc[gm] = __uint_as_float((unsigned)acc[i][j]);
+            if (gm + 1 < M) Cc[gm + 1] = __uint_as_float((unsigned)(acc[i][j] >> 32));
         }
     }
+}
+
+template <int RT, int CT, int BK, int MINB>
+cudaError_t gemm32(const GemmProb *probs, int nprobs, int rows, int cols, cudaStream_t st) {
+    const int tm = (rows + 8 * RT - 1) / (8 * RT), tn = (cols + 4 * CT - 1) / (4 * CT);
+    for (int p0 = 0; p0 < nprobs; p0 += 65535) {
+        const int np = (nprobs - p0 < 65535) ? nprobs - p0 : 65535;
+        k_gemm32<RT, CT, BK, MINB><<<dim3((unsigned)tm * tn, np), RT * CT, 0, st>>>(probs + p0, tn);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 #else
 constexpr int BK = 16;
@@ -316,10 +356,18 @@ cudaError_t gemm64_warp(const GemmProb *probs, int nprobs, int rows, int cols, c
 cudaError_t launch_gemm64(const GemmProb *probs, int nprobs, int mmax_rows, int nmax_cols, cudaStream_t st) {
     if (nprobs <= 0 || mmax_rows <= 0 || nmax_cols <= 0) return cudaSuccess;
 #ifdef BDC_FP32
-    const int bm = BM, bn = BN;
+    // the fewest, longest-running tiles lose to smaller ones while the chip is
+    // not full (four matrices of order 1000, whole solve: 494 us with 64 x 64
+    // tiles, 482 us with 32 x 32 and K step 16), and up to 36 columns anything
+    // wider is mostly padding (2000 matrices of order 24..80: 1005 us with
+    // 32 x 64, 967 us with 32 x 32); elsewhere 64 x 32 (above)
+    const long long tiles = (long long)nprobs * ((mmax_rows + 63) / 64) * ((nmax_cols + 63) / 64);
+    if (tiles < 4 * 152) return gemm32<4, 8, 16, 12>(probs, nprobs, mmax_rows, nmax_cols, st);
+    if (nmax_cols <= 36) return gemm32<4, 8, 8, 20>(probs, nprobs, mmax_rows, nmax_cols, st);
+    return gemm32<8, 8, 8, 14>(probs, nprobs, mmax_rows, nmax_cols, st);
 #else
     // tiles of one, four or sixteen fragments: the largest that still give
-    // every SM sub-partition (4 x 152) kFillWarps of them (by the host's
+    // every SM sub-partition (4 x 152) four of them (by the host's
     // bounds; deflation leaves fewer)
     constexpr long long kFill = 4 * 152 * 4;
     const long long frags = (long long)nprobs * ((mmax_rows + 7) / 8) * ((nmax_cols + 7) / 8);
@@ -329,23 +377,19 @@ cudaError_t launch_gemm64(const GemmProb *probs, int nprobs, int mmax_rows, int 
     // 32-row / 32-column tiles when the problems are that small
     const int wm = mmax_rows <= 32 ? 1 : 2, wn = nmax_cols <= 32 ? 1 : 2;
     const int bm = 32 * wm, bn = 32 * wn;
-#endif
     const int tilesN = (nmax_cols + bn - 1) / bn, tilesM = (mmax_rows + bm - 1) / bm;
     for (int p0 = 0; p0 < nprobs; p0 += 65535) {
         const int np = (nprobs - p0 < 65535) ? nprobs - p0 : 65535;
         dim3 grid((unsigned)tilesN * tilesM, np);
-#ifdef BDC_FP32
-        k_gemm32<<<grid, 256, 0, st>>>(probs + p0, tilesN);
-#else
         if (wm == 1 && wn == 1) k_gemm64<1, 1><<<grid, 32, 0, st>>>(probs + p0, tilesN);
         else if (wm == 1) k_gemm64<1, 2><<<grid, 64, 0, st>>>(probs + p0, tilesN);
         else if (wn == 1) k_gemm64<2, 1><<<grid, 64, 0, st>>>(probs + p0, tilesN);
         else k_gemm64<2, 2><<<grid, 128, 0, st>>>(probs + p0, tilesN);
-#endif
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+#endif
 }
 
 }  // namespace BDC_NS
