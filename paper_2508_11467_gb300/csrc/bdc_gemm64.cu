@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(32 * WM * WN, 3 * 4 / (WM * WN)) k_gemm64(cons
 // ones are faster (the four products of one order-100 merge: 45.9 us at F = 4,
 // 9.7 us at F = 1).  Every output sums its K steps in the same order at any F.
 constexpr int SW_WARPS = 4;
-constexpr int kSmallRows = 64, kSmallCols = 64;   // largest blocks served by 32 x 32 tiles
+constexpr int kSmallRows = 64, kSmallCols = 128;
 
 template <int F>
 __global__ void __launch_bounds__(32 * SW_WARPS, 4) k_gemm64_warp(const GemmProb *__restrict__ probs, int nprobs,
