@@ -245,9 +245,29 @@ __device__ __forceinline__ void digits(double x, int E, int (&n)[S]) {
 // instructions: n becomes an FP32 value exactly by the 1.5 2^23 offset trick
 // (one FP32 add), scales by 2^-8s (one multiply), and having at most 8
 // significant bits its BF16 pattern is the top half of the FP32 pattern
+__device__ __forceinline__ uint32_t slice_word(int n, int s) {
+    return __float_as_uint((__int_as_float(0x4B400000 + n) - 12582912.0f) * __uint_as_float((uint32_t)(127 - 8 * s) << 23));
+}
+
 __device__ __forceinline__ __nv_bfloat16 slice_bf16(int n, int s) {
-    const float f = (__int_as_float(0x4B400000 + n) - 12582912.0f) * __uint_as_float((uint32_t)(127 - 8 * s) << 23);
-    return __ushort_as_bfloat16((unsigned short)(__float_as_uint(f) >> 16));
+    return __ushort_as_bfloat16((unsigned short)(slice_word(n, s) >> 16));
+}
+
+// the slices of x as BF16 patterns in the upper halves of w: the S digits at
+// scale 2^E, or (!EXACT) x rounded to BF16 and what is left of it in FP32
+template <int S, bool EXACT>
+__device__ __forceinline__ void slices(double x, int E, uint32_t (&w)[S]) {
+    if (EXACT) {
+        int n[S];
+        digits<S>(x, E, n);
+#pragma unroll
+        for (int s = 0; s < S; ++s) w[s] = slice_word(n[s], s);
+    } else {
+        const float xf = (float)x;
+        const __nv_bfloat16 h = __float2bfloat16_rn(xf);
+        w[0] = (uint32_t)__bfloat16_as_ushort(h) << 16;
+        w[1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(xf - __bfloat162float(h))) << 16;
+    }
 }
 
 // A operand: 32 rows per CTA (256 threads), A column-major; grid (row blocks
@@ -258,7 +278,7 @@ __global__ void __launch_bounds__(256) k_slice_a(const GemmProb *__restrict__ pr
                                                 int p0, __nv_bfloat16 *__restrict__ As, int *__restrict__ Ea,
                                                 int rowsA, int Kld) {
     __shared__ unsigned long long smax[8][33];
-    __shared__ __nv_bfloat16 tile[S][32][72];
+    __shared__ __align__(16) __nv_bfloat16 tile[S][32][72];
     const int p = p0 + blockIdx.y;
     const GemmProb pr = probs[p];
     const MixProb mx = mix[p];
@@ -289,21 +309,26 @@ __global__ void __launch_bounds__(256) k_slice_a(const GemmProb *__restrict__ pr
     // K-contiguous; only up to the last 32-wide stage the MMA reads
     const int Kend = min(Kld, (K + TK - 1) / TK * TK);
     for (int k0 = 0; k0 < Kend; k0 += 64) {
-        for (int kk = tc; kk < 64; kk += 8) {
-            const int k = k0 + kk;
-            const double x = (rowok && k < K) ? pr.A[(size_t)k * pr.lda + row] : 0.0;
-            if (EXACT) {
-                int n[S];
-                digits<S>(x, E, n);
+        // eight consecutive columns a thread: their slices go to shared memory
+        // as one 16-byte word each (row stride 144 B: conflict-free)
+        double x[8];
+        uint32_t w[S][4];
 #pragma unroll
-                for (int s = 0; s < S; ++s) tile[s][tr][kk] = slice_bf16(n[s], s);
-            } else {
-                const float xf = (float)x;
-                const __nv_bfloat16 h = __float2bfloat16_rn(xf);
-                tile[0][tr][kk] = h;
-                tile[1][tr][kk] = __float2bfloat16_rn(xf - __bfloat162float(h));
-            }
+        for (int q = 0; q < 8; ++q) {
+            const int k = k0 + 8 * tc + q;
+            x[q] = (rowok && k < K) ? pr.A[(size_t)k * pr.lda + row] : 0.0;
         }
+#pragma unroll
+        for (int q = 0; q < 8; q += 2) {
+            uint32_t lo[S], hi[S];
+            slices<S, EXACT>(x[q], E, lo);
+            slices<S, EXACT>(x[q + 1], E, hi);
+#pragma unroll
+            for (int s = 0; s < S; ++s) w[s][q / 2] = __byte_perm(lo[s], hi[s], 0x7632);
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+            *reinterpret_cast<uint4 *>(&tile[s][tr][8 * tc]) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
         __syncthreads();
         // 32 rows x 64 columns x S slices out, 8 columns (16 B) per thread-store
         for (int idx = threadIdx.x; idx < S * 32 * 8; idx += 256) {
@@ -353,7 +378,7 @@ __global__ void __launch_bounds__(256) k_slice_b(const GemmProb *__restrict__ pr
         unsigned long long m = 0;
 #pragma unroll
         for (int q = 0; q < kSliceRegs; ++q) {
-            const int k = l + q * LANES;
+            const int k = 2 * (l + q / 2 * LANES) + q % 2;
             xv[q] = (colok && k < K) ? col[k] : 0.0;
             const unsigned long long b = (unsigned long long)__double_as_longlong(xv[q]) & 0x7FFFFFFFFFFFFFFFull;
             m = b > m ? b : m;
@@ -369,20 +394,15 @@ __global__ void __launch_bounds__(256) k_slice_b(const GemmProb *__restrict__ pr
         }
         const int Kend = min(Kld, (K + TK - 1) / TK * TK);
 #pragma unroll
-        for (int q = 0; q < kSliceRegs; ++q) {
-            const int k = l + q * LANES;
+        for (int q = 0; q < kSliceRegs; q += 2) {
+            const int k = 2 * (l + q / 2 * LANES);
             if (k >= Kend) break;
-            if (EXACT) {
-                int n[S];
-                digits<S>(xv[q], F, n);
+            uint32_t lo[S], hi[S];
+            slices<S, EXACT>(xv[q], F, lo);
+            slices<S, EXACT>(xv[q + 1], F, hi);
 #pragma unroll
-                for (int s2 = 0; s2 < S; ++s2) dst[(size_t)s2 * colsB * Kld + k] = slice_bf16(n[s2], s2);
-            } else {
-                const float xf = (float)xv[q];
-                const __nv_bfloat16 h = __float2bfloat16_rn(xf);
-                dst[k] = h;
-                dst[(size_t)colsB * Kld + k] = __float2bfloat16_rn(xf - __bfloat162float(h));
-            }
+            for (int s = 0; s < S; ++s)
+                *reinterpret_cast<uint32_t *>(dst + (size_t)s * colsB * Kld + k) = __byte_perm(lo[s], hi[s], 0x7632);
         }
         return;
     }
@@ -403,20 +423,14 @@ __global__ void __launch_bounds__(256) k_slice_b(const GemmProb *__restrict__ pr
         if (l == 0) Fb[mx.b_col0 + c] = colok ? F : 0;
     }
     const int Kend = min(Kld, (K + TK - 1) / TK * TK);
-    #pragma unroll 4
-    for (int k = l; k < Kend; k += LANES) {
-        const double x = (colok && k < K) ? col[k] : 0.0;
-        if (EXACT) {
-            int n[S];
-            digits<S>(x, F, n);
+    #pragma unroll 2
+    for (int k = 2 * l; k < Kend; k += 2 * LANES) {
+        uint32_t lo[S], hi[S];
+        slices<S, EXACT>((colok && k < K) ? col[k] : 0.0, F, lo);
+        slices<S, EXACT>((colok && k + 1 < K) ? col[k + 1] : 0.0, F, hi);
 #pragma unroll
-            for (int s = 0; s < S; ++s) dst[(size_t)s * colsB * Kld + k] = slice_bf16(n[s], s);
-        } else {
-            const float xf = (float)x;
-            const __nv_bfloat16 h = __float2bfloat16_rn(xf);
-            dst[k] = h;
-            dst[(size_t)colsB * Kld + k] = __float2bfloat16_rn(xf - __bfloat162float(h));
-        }
+        for (int s = 0; s < S; ++s)
+            *reinterpret_cast<uint32_t *>(dst + (size_t)s * colsB * Kld + k) = __byte_perm(lo[s], hi[s], 0x7632);
     }
 }
 
