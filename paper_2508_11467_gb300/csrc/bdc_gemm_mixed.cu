@@ -348,9 +348,9 @@ constexpr int kSliceRegs = 16;   // entries per lane held in registers by the on
 // B operand: LANES lanes per column (column-major B is K-contiguous),
 // 32 / LANES columns per warp; grid (columns of the host bound of the
 // largest product / (256 / LANES), products from p0).  K is a merge's
-// survivor count: eight lanes per column for the small merges (a few
-// dozen K, where a whole warp per column would mostly wait on its loads),
-// a warp per column for the large ones.  Only the columns the MMA tiles
+// survivor count: eight lanes per column for the small merges and the wide
+// heights (where a whole warp per column would mostly wait on its loads), a
+// warp per column otherwise.  Only the columns the MMA tiles
 // read are written: those below N, and zeros up to N rounded up to the
 // tile width; lanes past them exit (N, the survivor count, is known only on
 // the device and is often far below the host bound).  Columns of up to
@@ -1094,7 +1094,12 @@ cudaError_t run_mixed(const GemmProb *probs, int nprobs, const std::vector<MixPr
         StageScope slice_scope(st, BDC_STAGE_SLICE, 1, 0.0);
         for (int p0 = 0; p0 < nprobs; p0 += 65535) {
             const int np = std::min(nprobs - p0, 65535);
-            if (ncols <= 128)
+            // eight lanes while a column is short, or when there are columns for
+            // several rounds of such warps (4 a warp, 32 warps an SM): a warp on
+            // one column mostly waits.  512 matrices of order 32..1024: 21305 us
+            // with 32 lanes above 128 columns, 20912 us to 600, 20897 us to 1100;
+            // 16 lanes 21028 us, four 21053 us.  One matrix: no difference.
+            if (ncols <= 128 || (ncols <= 576 && (long long)np * ncols >= 65536))
                 k_slice_b<S, EXACT, 8><<<dim3((ncols + 31) / 32, np), 256, 0, st>>>(probs, dmix, p0, Bs, F, colsB, Kld);
             else
                 k_slice_b<S, EXACT, 32><<<dim3((ncols + 7) / 8, np), 256, 0, st>>>(probs, dmix, p0, Bs, F, colsB, Kld);
