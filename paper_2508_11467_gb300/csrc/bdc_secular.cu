@@ -851,8 +851,9 @@ __device__ void vectors_one(const real_t *__restrict__ d, const real_t *__restri
 
 // The same with a lane group per column (G = 4 to 32 lanes, about 16 rows
 // each), for heights whose merges have N <= 1024 survivors: each lane keeps
-// its entries v_j (j = lane, lane + G, ...) in registers between the norm and
-// the write, so every entry costs one division; rows are written at their K
+// its entries v_j (j = lane, lane + G, ...), and up to 16 of them also as u_j,
+// in registers between the norm and the write, so every entry costs one
+// division; rows are written at their K
 // positions (kposM), the padding rows [n1, P1) of the K order as zeros.
 template <int G, int T>
 __device__ __forceinline__ void vectors_group(const real_t *__restrict__ d, const real_t *__restrict__ zt,
@@ -860,20 +861,22 @@ __device__ __forceinline__ void vectors_group(const real_t *__restrict__ d, cons
                                               real_t tau, real_t *__restrict__ UMcol, real_t *__restrict__ VMcol,
                                               int gl, bool wu) {
     const real_t wsum = dor + tau;   // w_i: d_j + w_i formed once per entry (a sum of positives)
-    real_t vr[T];
+    constexpr bool KEEP = T <= 16;   // u_j as well (registers)
+    real_t vr[T], ur[KEEP ? T : 1];
     real_t sv = R(0.0), su = R(0.0);
 #pragma unroll
     for (int t = 0; t < T; ++t) {
         const int j = gl + t * G;
-        real_t v = R(0.0);
+        real_t v = R(0.0), u = R(0.0);
         if (j < N) {
             const real_t dj = d[j];
             v = quot(zt[j], ((dj - dor) - tau) * (dj + wsum));
-            const real_t u = (j == 0) ? -R(1.0) : dj * v;
+            u = (j == 0) ? -R(1.0) : dj * v;
             sv = fma(v, v, sv);
             su = fma(u, u, su);
         }
         vr[t] = v;
+        if constexpr (KEEP) ur[t] = u;
     }
     sv = group_sum<G>(sv);
     su = group_sum<G>(su);
@@ -888,10 +891,20 @@ __device__ __forceinline__ void vectors_group(const real_t *__restrict__ d, cons
         if (j < N) {
             const int kp = kpos[j];
             VMcol[kp] = vr[t] * iv;
-            if (wu) UMcol[kp] = ((j == 0) ? -R(1.0) : d[j] * vr[t]) * iu;
+            if constexpr (KEEP) {
+                if (wu) UMcol[kp] = ur[t] * iu;
+            } else if (wu) {
+                UMcol[kp] = ((j == 0) ? -R(1.0) : d[j] * vr[t]) * iu;
+            }
         }
     }
 }
+
+#ifdef BDC_FP32
+template <bool SMALL> constexpr int kVecCtas = SMALL ? 16 : 14;
+#else
+template <bool SMALL> constexpr int kVecCtas = 8;
+#endif
 
 // the same for N > 32 * 32 survivors, a warp per column: the entries wait for
 // the norms in V's own column (each lane reads back what it wrote).  Bound by
@@ -942,7 +955,14 @@ __device__ __forceinline__ void vectors_warp_long(const real_t *__restrict__ d, 
     }
 }
 
-__global__ void __launch_bounds__(kLgThreads) k_vectors_warp(const NodeDesc *__restrict__ nodes,
+// SMALL: heights whose merges have at most 512 survivors, without the code
+// for longer ones.  Bound by the FP64 pipe (70 % busy), which more warps feed
+// better than registers do: CTAs an SM as below, the long paths with 80 bytes
+// of spills.  One kernel of 148 registers for all, every u_j formed twice ->
+// now: n = 16384 6758 -> 6645 us, clustered n = 4096 10331 -> 10094 us, 512
+// matrices of order 32..1024 20892 -> 20517 us, FP32 3372 -> 3306 us.
+template <bool SMALL>
+__global__ void __launch_bounds__(kLgThreads, kVecCtas<SMALL>) k_vectors_warp(const NodeDesc *__restrict__ nodes,
                                                       const MatDesc *__restrict__ mats,
                                                       const NodeState *__restrict__ state, int wpn,
                                                       int nnodes) {
@@ -974,7 +994,9 @@ __global__ void __launch_bounds__(kLgThreads) k_vectors_warp(const NodeDesc *__r
     case 8: vectors_group<8, 16>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu); break;
     case 16: vectors_group<16, 16>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu); break;
     default:
-        if (N <= 32 * 32) vectors_group<32, 32>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu);
+        if (N <= 32 * 16) vectors_group<32, 16>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu);
+        else if (SMALL) break;
+        else if (N <= 32 * 32) vectors_group<32, 32>(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu);
         else vectors_warp_long(d, zt, kpos, N, ns.n1, ns.P1, dor, tau, UMcol, VMcol, gl, wu);
         break;
     }
@@ -1097,7 +1119,8 @@ cudaError_t launch_vectors(const NodeDesc *nodes, int nnodes, const MatDesc *mat
                            int mmax, cudaStream_t st) {
     if (nnodes <= 0) return cudaSuccess;
     const long long warps = (long long)nnodes * group_warps(mmax);
-    launch_pdl(k_vectors_warp, (unsigned)((warps + kLgWarps - 1) / kLgWarps), kLgThreads, 0, st, nodes, mats, state, group_warps(mmax), nnodes);
+    launch_pdl(mmax <= 512 ? k_vectors_warp<true> : k_vectors_warp<false>, (unsigned)((warps + kLgWarps - 1) / kLgWarps),
+               kLgThreads, 0, st, nodes, mats, state, group_warps(mmax), nnodes);
     return cudaGetLastError();
 }
 
