@@ -26,11 +26,13 @@ namespace {
 // around it; one thread polling per CTA matters: a flag per CTA polled by as
 // many threads took 5000 to 14000.  The wait is bounded (kBarNs); false when
 // it gave up here or elsewhere.
-template <bool ORDERED = true>
-__device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
+// meanwhile() runs on warp 0, thread LEAD arrives and polls.
+template <bool ORDERED, int LEAD, typename F>
+__device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target, F meanwhile) {
     __shared__ int s_ok;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) meanwhile();
+    if (threadIdx.x == LEAD) {
         unsigned v;
         int ok = 1;
         auto poll = [&] {
@@ -59,6 +61,10 @@ __device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
     }
     __syncthreads();
     return s_ok != 0;
+}
+template <bool ORDERED = true>
+__device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
+    return grid_wait<ORDERED, 0>(gb, target, [] {});
 }
 
 // Householder reflector from alpha and ||x_2..||^2 = sig2 (LAPACK's sign
@@ -300,7 +306,7 @@ struct Gebd2Args {
     int lda, m, n;
     double *d, *e, *tauq, *taup;
     Slot *gp;                      // [grid][n]: per-CTA partial sums of A^T a (column i: of a^T a)
-    Slot *row, *yr, *scal;         // [n] top row; [2 n] y and row i after H_i; [1] column scale
+    Slot *row, *gs;                // [2][n] top row, by the step's parity; [n] sums of g over the CTAs
     GridBar *bar;
     unsigned base;                 // arrivals before this launch
 };
@@ -310,27 +316,35 @@ struct Gebd2Args {
 // major.  With a = column i of the current matrix, step i is
 //   Y phase (a block of columns per CTA): g_c = sum over CTAs of A[:, c]^T a
 //     (tail rows), sig2 = the same for a itself -> H_i's scalars (every CTA
-//     forms them), y_c = tau (A[i, c] + sc g_c), row i: r_c = A[i, c] - y_c
-//   X phase (own rows): v = sc a; one pass A -= v y^T with h = A r; block
-//     reduction of h and ||r||^2 -> G_i's scalars; x = pi A u with u = [1;
-//     scr r]; next column a' = A[:, i+1] - x; one pass A -= x u^T with the
+//     forms them, while the sums g travel)
+//   X phase (own rows): y_c = A[i, c] + sc g_c, row i: r_c = A[i, c] - tau
+//     y_c (every CTA, all columns); v = tau sc a; one pass A -= v y^T with h =
+//     A r; block reduction of h and ||r||^2 -> G_i's scalars; x = pi A u with u
+//     = [1; scr r]; next column a' = A[:, i+1] - x; one pass A -= x u^T with the
 //     partial sums of A^T a' and a'^T a' for step i + 1, and the next top row
 // The products are taken with the unscaled a and r, so that no phase waits
 // for a norm.  Four FMAs per entry and step; FP64 runs at two lanes per
 // clock and SM, so four warps fill the pipe and the block reduction (one add
 // per thread and row) is kept small by them.  The phases exchange their
-// vectors through slots (above).  One buffer of each is enough: a CTA writes
-// its sums of step i + 1 after it has the y of every column of step i, which
-// their owners sent after reading all sums of step i; and an owner sends
-// step i + 1's y after the sums of every CTA, which each sent after reading
-// all of step i's y.
+// vectors through slots (above).  One buffer of the sums is enough: a CTA
+// writes its sums of step i + 1 after it has the g of every column of step i,
+// which their owners sent after reading all sums of step i (of column i, which
+// all read, no later sum is written); and an owner sends step i + 1's g after
+// the sums of every CTA, which each sent after reading all of step i's g.  The
+// top row has two: all read step i's in the X phase, where its next owner
+// writes step i + 1's, over that of step i - 1, which all have read before
+// they arrived in the Y phase of step i.
 // What bounds it: the two exchanges (about 3500 cycles each) and the
 // dependent FP64 chains of a step (64 cycles an operation), above n ~ 1000
 // the FP64 pipe.  333 x 333: 18.9 ms (blocked panels, seven barriers a step)
-// -> 2.8 ms; 1000 x 1000: 71 -> 12 ms; 1500 x 1100: 82 -> 17 ms.
+// -> 2.6 ms; 1100 x 1100: 13.9 ms; 1500 x 1100: 82 -> 15.7 ms.  Sending y and
+// r from the owners of the columns, each after its own H_i scalars, put those
+// (1450 cycles) in front of the exchange instead of beside it: 2.8, 14.6 and
+// 16.3 ms.
 __global__ void __launch_bounds__(NT, 1) k_gebd2_resident(Gebd2Args a) {
     extern __shared__ double smem[];
     __shared__ int s_err;
+    __shared__ double s_alpha, s_sc, s_tau;
     const int G = gridDim.x, g = blockIdx.x, t = threadIdx.x;
     const int m = a.m, n = a.n, ldw = a.n;
     const int lr = (m - g + G - 1) / G;             // own rows (g < G <= m)
@@ -350,8 +364,7 @@ __global__ void __launch_bounds__(NT, 1) k_gebd2_resident(Gebd2Args a) {
     // clear the slots' step numbers
     const Slot zero = {0ull, 0ull};
     for (int c = t; c < n; c += NT) a.gp[(size_t)g * ldw + c] = zero;
-    for (int c = g * NT + t; c < n; c += G * NT) a.row[c] = a.yr[2 * c] = a.yr[2 * c + 1] = zero;
-    if (g == 0 && t == 0) a.scal[0] = zero;
+    for (int c = g * NT + t; c < n; c += G * NT) a.row[c] = a.row[n + c] = a.gs[c] = zero;
     unsigned target = a.base + G;
     if (!grid_wait(a.bar, target)) return;
     for (int l = t; l < lr; l += NT) av[l] = W[(size_t)l * ldw];
@@ -369,30 +382,30 @@ __global__ void __launch_bounds__(NT, 1) k_gebd2_resident(Gebd2Args a) {
         // ---- Y phase
         const int ncol = n - 1 - i, cb = (ncol + G - 1) / G;
         const int c0 = i + 1 + g * cb, nc = max(0, min(cb, n - c0));
-        if (nc > 0 || g == 0) {
-            // sums over the CTAs of nc columns and of column i (slot nc)
+        const Slot *row = a.row + (size_t)(i & 1) * n;
+        // sums over the CTAs of nc columns and of column i (slot nc); every
+        // CTA sums column i, in the same order (the cut follows cb, not nc)
+        int sp = 1;
+        while (sp < cb + 1) sp <<= 1;               // slots per pass (power of two, at most 32)
+        if (sp > 32) sp = 32;
+        const bool one = cb + 1 <= sp;
+        {
             const int slots = nc + 1;
-            int sp = 1;
-            while (sp < slots) sp <<= 1;            // slots per pass (power of two, at most 32)
-            if (sp > 32) sp = 32;
             const int sub = t / sp, subs = NT / sp;
-            double alpha = 0.0, top = 0.0, tau, beta;
             for (int s0 = 0; s0 < slots; s0 += sp) {
                 const int s = s0 + (t & (sp - 1));
                 double v0 = 0.0;
-                // eight CTAs' slots per round (one round for most sizes); the
-                // first round also takes alpha and this thread's top-row entry
+                // eight CTAs' slots per round (one round for most sizes), and
+                // alpha
                 const Slot *p = a.gp + (s < nc ? c0 + s : i);
                 for (int k = sub; k < G; k += 8 * subs) {
-                    const Slot *q[10];
-                    double v[10];
+                    const Slot *q[9];
+                    double v[9];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) q[j] = k + j * subs < G && s < slots ? p + (size_t)(k + j * subs) * ldw : nullptr;
-                    q[8] = a.row + i;
-                    q[9] = t < nc ? a.row + c0 + t : nullptr;
-                    slot_get<10>(q, tag, v, a.bar, &s_err);
-                    alpha = v[8];
-                    top = v[9];
+                    q[8] = t == 0 ? row + i : nullptr;
+                    slot_get<9>(q, tag, v, a.bar, &s_err);
+                    if (t == 0) s_alpha = v[8];
                     v0 += v[0];
 #pragma unroll
                     for (int j = 1; j < 8; ++j)
@@ -402,63 +415,54 @@ __global__ void __launch_bounds__(NT, 1) k_gebd2_resident(Gebd2Args a) {
                 if (s0 > 0) __syncthreads();
                 if ((t & 31) < sp) red[(t >> 5) * 32 + (t & 31)] = v0;
                 __syncthreads();
-                if (slots > sp && t < sp && s0 + t < slots)
-                    sy[s0 + t] = (red[t] + red[32 + t]) + (red[64 + t] + red[96 + t]);
-            }
-            const bool one = slots <= sp;
-            if (!one) __syncthreads();
-            const double sig2 = one ? (red[nc] + red[32 + nc]) + (red[64 + nc] + red[96 + nc]) : sy[nc];
-            const double sc = reflector_fast(alpha, sig2, tau, beta);
-            for (int q = t; q < nc; q += NT) {
-                const int c = c0 + q;
-                double rw = top;
-                if (q != t) {
-                    const Slot *z[1] = {a.row + c};
-                    double v[1];
-                    slot_get<1>(z, tag, v, a.bar, &s_err);
-                    rw = v[0];
+                if (t < sp && s0 + t < slots) {
+                    const double gs = (red[t] + red[32 + t]) + (red[64 + t] + red[96 + t]);
+                    if (s0 + t < nc) slot_put(a.gs + c0 + s0 + t, gs, tag);
+                    else if (!one) sy[0] = gs;
                 }
-                const double gs = one ? (red[q] + red[32 + q]) + (red[64 + q] + red[96 + q]) : sy[q];
-                const double y = tau * fma(sc, gs, rw);
-                slot_put(a.yr + 2 * c, y, tag);
-                slot_put(a.yr + 2 * c + 1, rw - y, tag);
-            }
-            if (g == 0 && t == 0) {
-                slot_put(a.scal, sc, tag);
-                a.d[i] = beta;
-                a.tauq[i] = tau;
-                A[(size_t)i * lda + i] = beta;
             }
         }
-        if (!grid_wait<false>(a.bar, target += G)) return;
+        // H_i's scalars while the other CTAs' sums are on their way
+        if (!grid_wait<false, 32>(a.bar, target += G, [&] {
+                const double sig2 = one ? (red[nc] + red[32 + nc]) + (red[64 + nc] + red[96 + nc]) : sy[0];
+                double tau, beta;
+                const double sc = reflector_fast(s_alpha, sig2, tau, beta);
+                if (t == 0) {
+                    s_sc = sc;
+                    s_tau = tau;
+                    if (g == 0) {
+                        a.d[i] = beta;
+                        a.tauq[i] = tau;
+                        A[(size_t)i * lda + i] = beta;
+                    }
+                }
+            }))
+            return;
+        const double sc = s_sc, tau = s_tau;
         // ---- X phase
         const int l0 = (i < g) ? 0 : (i - g) / G + 1;   // first own row below i
         const bool more = i + 1 < n;
-        double sc = 0.0, alr = 0.0;
-        for (int c = i + 1 + t, first = 1; first || c < n; c += 4 * NT, first = 0) {
-            // four columns of y and r per round; every round also has the scale and r's first entry
-            const Slot *q[10];
-            double v[10];
-            q[8] = a.scal;
-            q[9] = more ? a.yr + 2 * (i + 1) + 1 : nullptr;
+        for (int c = i + 1 + t; c < n; c += 4 * NT) {
+            // four columns of g and row i per round
+            const Slot *q[8];
+            double v[8];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                q[2 * j] = c + j * NT < n ? a.yr + 2 * (c + j * NT) : nullptr;
-                q[2 * j + 1] = c + j * NT < n ? a.yr + 2 * (c + j * NT) + 1 : nullptr;
+                q[2 * j] = c + j * NT < n ? a.gs + c + j * NT : nullptr;
+                q[2 * j + 1] = c + j * NT < n ? row + c + j * NT : nullptr;
             }
-            slot_get<10>(q, tag, v, a.bar, &s_err);
-            sc = v[8];
-            alr = v[9];
+            slot_get<8>(q, tag, v, a.bar, &s_err);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if (c + j * NT < n) {
-                    sy[c + j * NT] = v[2 * j];
-                    sr[c + j * NT] = v[2 * j + 1];
+                    const double y = fma(sc, v[2 * j], v[2 * j + 1]);
+                    sy[c + j * NT] = y;
+                    sr[c + j * NT] = fma(-tau, y, v[2 * j + 1]);
                 }
         }
         for (int l = l0 + t; l < lr; l += NT) {
             const double v = sc * av[l];
-            vv[l] = v;
+            vv[l] = tau * v;
             A[(size_t)i * lda + g + (size_t)G * l] = v;
         }
         __syncthreads();
@@ -498,7 +502,7 @@ __global__ void __launch_bounds__(NT, 1) k_gebd2_resident(Gebd2Args a) {
             __syncthreads();
             if (lastc) break;
         }
-        const double scr = reflector_fast(alr, hs[lrmax], pi, betr);
+        const double scr = reflector_fast(sr[i + 1], hs[lrmax], pi, betr);
         for (int l = l0 + t; l < lr; l += NT) {
             const double w = W[(size_t)l * ldw + i + 1];
             const double x = pi * fma(scr, hs[l], w);
@@ -519,7 +523,7 @@ __global__ void __launch_bounds__(NT, 1) k_gebd2_resident(Gebd2Args a) {
         for (int c = i + 1 + t; c < n; c += NT) {
             const double u = (c == i + 1) ? 1.0 : scr * sr[c];
             if (ug && c > i + 1) ug[(size_t)c * lda] = u;
-            if (topmine) slot_put(a.row + c, fma(-xt, u, W[(size_t)l0 * ldw + c]), tag + 1u);
+            if (topmine) slot_put(a.row + (size_t)((i + 1) & 1) * n + c, fma(-xt, u, W[(size_t)l0 * ldw + c]), tag + 1u);
             sr[c] = u;
             if (l1 >= lr) slot_put(a.gp + (size_t)g * ldw + c, 0.0, tag + 1u);
         }
@@ -1146,8 +1150,8 @@ cudaError_t launch_gebd2_resident(int m, int n, double *A, int lda, double *d, d
                                   double *scratch, GridBar *bar, unsigned *bars, cudaStream_t st) {
     const int G = res_grid(m);
     const size_t smem = res_smem(m, n, G);
-    Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * n, *yr = row + n, *scal = yr + 2 * n;
-    Gebd2Args a{A, lda, m, n, d, e, tauq, taup, gp, row, yr, scal, bar, *bars};
+    Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * n, *gs = row + 2 * n;
+    Gebd2Args a{A, lda, m, n, d, e, tauq, taup, gp, row, gs, bar, *bars};
     *bars += (unsigned)G * (1u + 2u * (unsigned)n);   // load, first sums, n Y phases, n - 1 X phases
     // the device's maximum, not this launch's size: another thread may be
     // between its own call and its launch
