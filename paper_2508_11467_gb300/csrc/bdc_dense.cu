@@ -603,14 +603,17 @@ cudaError_t form_t(const Reflectors &f, const double *tau, double *Tall, cudaStr
 
 // W = M Z for the summed partial products Z of dgemm_parts, M = T or T^T
 // (tr), nb x nb.  left: Z is nb x count (column-major), a vector per column;
-// right: Z is count x nb, a vector per row (W^T = M Z^T).  16 vectors per
-// CTA; each warp takes 8 rows of M, its fragments straight from L2.  add: Z +=
-// the first nb rows of add (left; the unit entries' share).
+// right: Z is count x nb, a vector per row (W^T = M Z^T).  V = 16 vectors per
+// CTA, 8 while that leaves SMs without one (the sums of the partial products
+// take most of it: 480 vectors of 31 parts 46 us with 16, 28 with 8); each warp
+// takes 8 rows of M, its fragments straight from L2.  add: Z += the first nb
+// rows of add (left; the unit entries' share).
+template <int V>
 __global__ void __launch_bounds__(256) k_tz(const double *__restrict__ T, int nb, int tr, const double *__restrict__ part,
                                             int splits, int right, int count, double *__restrict__ W,
                                             const double *__restrict__ add, int ldadd) {
     pdl_begin();
-    constexpr int V = 16, LD = V + 4;
+    constexpr int LD = V + 4;
     __shared__ double Zs[kTB * LD];   // [k][vector]
     const int v0 = blockIdx.x * V;
     const size_t mn = (size_t)nb * count;
@@ -628,7 +631,7 @@ __global__ void __launch_bounds__(256) k_tz(const double *__restrict__ T, int nb
         double s = 0.0;
         if (p < nb && v0 + v < count) {
             const double *q = part + (right ? (size_t)p * count + v0 + v : (size_t)(v0 + v) * nb + p);
-#pragma unroll 8
+#pragma unroll 16
             for (int y = 0; y < splits; ++y) s += q[(size_t)y * mn];
             if (add) s += add[(size_t)(v0 + v) * ldadd + p];
         }
@@ -636,21 +639,29 @@ __global__ void __launch_bounds__(256) k_tz(const double *__restrict__ T, int nb
     }
     __syncthreads();
     if (i0 >= nb) return;
-    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+    double acc[V / 8][2];
+#pragma unroll
+    for (int j = 0; j < V / 8; ++j) acc[j][0] = acc[j][1] = 0.0;
 #pragma unroll
     for (int k = 0; k < kTB / 4; ++k) {
         // M is triangular: T has only k >= i, T^T only k <= i
         if (tr ? 4 * k > i0 + 7 : 4 * k + 3 < i0) continue;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) dmma(acc[j], mf[k], Zs[(4 * k + tg) * LD + j * 8 + gr]);
+        for (int j = 0; j < V / 8; ++j) dmma(acc[j], mf[k], Zs[(4 * k + tg) * LD + j * 8 + gr]);
     }
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
+    for (int j = 0; j < V / 8; ++j)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int v = v0 + j * 8 + 2 * tg + h, i = i0 + gr;
             if (i < nb && v < count) W[right ? (size_t)i * count + v : (size_t)v * nb + i] = acc[j][h];
         }
+}
+
+template <typename... Args>
+void launch_tz(int count, cudaStream_t st, Args... args) {
+    if (count <= 8 * sm_count_dense()) launch_pdl(k_tz<8>, (count + 7) / 8, 256, 0, st, args...);
+    else launch_pdl(k_tz<16>, (count + 15) / 16, 256, 0, st, args...);
 }
 
 // C (rows x cols, ldc) := H C or H^T C (left) or C H or C H^T (right), H =
@@ -664,12 +675,12 @@ cudaError_t apply_block(int left, int trans, int rows, int cols, const double *Y
     int splits;
     if (left) {
         if ((e = dgemm_parts(1, 0, nb, cols, rows, Y, rows, C, ldc, splits, st)) != cudaSuccess) return e;
-        launch_pdl(k_tz, (cols + 15) / 16, 256, 0, st, T, nb, trans ? 1 : 0, g_split_buf, splits, 0, cols, W, nullptr, 0);
+        launch_tz(cols, st, T, nb, trans ? 1 : 0, g_split_buf, splits, 0, cols, W, nullptr, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         return dgemm(0, 0, rows, cols, nb, -1.0, Y, rows, W, nb, 1.0, C, ldc, st);
     }
     if ((e = dgemm_parts(0, 0, rows, nb, cols, C, ldc, Y, cols, splits, st)) != cudaSuccess) return e;
-    launch_pdl(k_tz, (rows + 15) / 16, 256, 0, st, T, nb, trans ? 0 : 1, g_split_buf, splits, 1, rows, W, nullptr, 0);
+    launch_tz(rows, st, T, nb, trans ? 0 : 1, g_split_buf, splits, 1, rows, W, nullptr, 0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return dgemm(0, 1, rows, cols, nb, -1.0, W, rows, Y, cols, 1.0, C, ldc, st);
 }
@@ -1032,7 +1043,7 @@ cudaError_t apply_panel(const Reflectors &f, const double *T, int rows, int cols
         if ((e = set.add(p)) != cudaSuccess) return e;
     }
     if ((e = set.run()) != cudaSuccess) return e;
-    launch_pdl(k_tz, (cols + 15) / 16, 256, 0, st, T, nb, 1, w.Z, np, 0, cols, W, C, ldc);
+    launch_tz(cols, st, T, nb, 1, w.Z, np, 0, cols, W, C, ldc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     SplitProd p{};
     p.a = y_rows(f, 0, rows);

@@ -1206,37 +1206,36 @@ struct SplitTab {
     int count;
 };
 
-// tables of the launch: products, exponent maxima cleared, tile list
+// tables of the launch: products, exponent maxima cleared, tile list; grid
+// (blocks, products): the products one after another took 18 us for 31, 2.9
+// for one
 __global__ void __launch_bounds__(256) k_split_tab(const __grid_constant__ SplitTab t, GemmProb *probs, MixProb *mix,
                                                    unsigned long long *maxA, unsigned long long *maxB, int2 *tiles,
                                                    int *ntiles) {
     pdl_begin();
+    const int q = blockIdx.y;
+    const SplitProd &p = t.p[q];
+    const int tm = (p.a.n + TM - 1) / TM, tn = (p.b.n + TNX - 1) / TNX, cnt = tm * tn;
     int base = 0;
-    for (int q = 0; q < t.count; ++q) {
-        const SplitProd &p = t.p[q];
-        const int tm = (p.a.n + TM - 1) / TM, tn = (p.b.n + TNX - 1) / TNX, cnt = tm * tn;
-        if (blockIdx.x == 0) {
-            if (threadIdx.x == 0) {
-                probs[q] = GemmProb{p.a.p, p.b.p, p.C, 0, 0, p.ldc, p.a.n, p.b.n, p.K, nullptr};
-                MixProb m{};
-                m.a_row0 = p.a.row0; m.b_col0 = p.b.row0; m.tile0 = base; m.tilesN = tn;
-                m.Mmax = p.a.n; m.Nmax = p.b.n; m.sub = p.sub;
-                mix[q] = m;
-            }
-        }
-        constexpr int G = 8;               // bands of 8 row blocks, as in k_tile_list
-        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
-            const int band = k / (G * tn), in_band = k % (G * tn);
-            const int bm0 = band * G, bsz = min(G, tm - bm0);
-            tiles[base + k] = make_int2(q, ((bm0 + in_band % bsz) << 16) | (in_band / bsz));
-        }
-        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.a.n; k += gridDim.x * blockDim.x)
-            maxA[p.a.row0 + k] = 0ull;
-        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.b.n; k += gridDim.x * blockDim.x)
-            maxB[p.b.row0 + k] = 0ull;
-        base += cnt;
+    for (int j = 0; j < q; ++j) base += ((t.p[j].a.n + TM - 1) / TM) * ((t.p[j].b.n + TNX - 1) / TNX);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        probs[q] = GemmProb{p.a.p, p.b.p, p.C, 0, 0, p.ldc, p.a.n, p.b.n, p.K, nullptr};
+        MixProb m{};
+        m.a_row0 = p.a.row0; m.b_col0 = p.b.row0; m.tile0 = base; m.tilesN = tn;
+        m.Mmax = p.a.n; m.Nmax = p.b.n; m.sub = p.sub;
+        mix[q] = m;
+        if (q + 1 == t.count) *ntiles = base + cnt;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ntiles = base;
+    constexpr int G = 8;                   // bands of 8 row blocks, as in k_tile_list
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
+        const int band = k / (G * tn), in_band = k % (G * tn);
+        const int bm0 = band * G, bsz = min(G, tm - bm0);
+        tiles[base + k] = make_int2(q, ((bm0 + in_band % bsz) << 16) | (in_band / bsz));
+    }
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.a.n; k += gridDim.x * blockDim.x)
+        maxA[p.a.row0 + k] = 0ull;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < p.b.n; k += gridDim.x * blockDim.x)
+        maxB[p.b.row0 + k] = 0ull;
 }
 
 __device__ __forceinline__ unsigned long long mag_bits(double x) {
@@ -1259,6 +1258,8 @@ __device__ __forceinline__ double split_at(const SplitSide &s, int v, int k) {
     }
     return x;
 }
+constexpr int kAlongRegs = 6;              // entry pairs a lane keeps in registers: K <= 384
+
 // vectors stored along K: a warp each, two neighbouring entries per lane (the
 // second pass finds them in cache); grid (vectors / 8, products, sides)
 __global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ SplitTab t, __nv_bfloat16 *As,
@@ -1270,28 +1271,53 @@ __global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ Spl
     const int v = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (s.tr || v >= s.n) return;
     const int K = p.K, Kend = (K + TK - 1) / TK * TK;
+    const int rows = blockIdx.z ? colsB : rowsA;
+    __nv_bfloat16 *dst = (blockIdx.z ? Bs : As) + (size_t)(s.row0 + v) * Kld;
     unsigned long long m = 0;
+    auto max_exp = [&] {
+        for (int o = 16; o > 0; o >>= 1) m = max(m, (unsigned long long)__shfl_xor_sync(0xffffffffu, m, o));
+        const int E = scale_exp(m);
+        if (lane == 0) (blockIdx.z ? Fb : Ea)[s.row0 + v] = E;
+        return E;
+    };
+    auto put = [&](int k, int E, double x0, double x1) {
+        uint32_t lo[DS], hi[DS];
+        slices<DS, true>(x0, E, lo);
+        slices<DS, true>(x1, E, hi);
+#pragma unroll
+        for (int q = 0; q < DS; ++q)
+            *reinterpret_cast<uint32_t *>(dst + (size_t)q * rows * Kld + k) = __byte_perm(lo[q], hi[q], 0x7632);
+    };
+    // a plain matrix of short vectors: every load issued at once, kept for
+    // the digits (31 products of 480 columns x 323: 49 -> 27 us)
+    if (!s.mask && s.parts <= 1 && !s.add && !s.ref && K <= 64 * kAlongRegs) {
+        const double *x = s.p + (size_t)v * s.ld;
+        double xv[kAlongRegs][2];
+#pragma unroll
+        for (int j = 0; j < kAlongRegs; ++j) {
+            const int k = 2 * lane + 64 * j;
+            xv[j][0] = k < K ? x[k] : 0.0;
+            xv[j][1] = k + 1 < K ? x[k + 1] : 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j < kAlongRegs; ++j) m = max(m, max(mag_bits(xv[j][0]), mag_bits(xv[j][1])));
+        const int E = max_exp();
+#pragma unroll
+        for (int j = 0; j < kAlongRegs; ++j) {
+            const int k = 2 * lane + 64 * j;
+            if (k < Kend) put(k, E, xv[j][0], xv[j][1]);
+        }
+        return;
+    }
 #pragma unroll 4
     for (int k = 2 * lane; k < K; k += 64) {
         m = max(m, mag_bits(split_at(s, v, k)));
         if (k + 1 < K) m = max(m, mag_bits(split_at(s, v, k + 1)));
     }
-    for (int o = 16; o > 0; o >>= 1) m = max(m, (unsigned long long)__shfl_xor_sync(0xffffffffu, m, o));
-    const int E = scale_exp(m);
-    const int rows = blockIdx.z ? colsB : rowsA;
-    if (lane == 0) (blockIdx.z ? Fb : Ea)[s.row0 + v] = E;
-    __nv_bfloat16 *dst = (blockIdx.z ? Bs : As) + (size_t)(s.row0 + v) * Kld;
+    const int E = max_exp();
 #pragma unroll 2
-    for (int k = 2 * lane; k < Kend; k += 64) {
-        const double x0 = k < K ? split_at(s, v, k) : 0.0, x1 = k + 1 < K ? split_at(s, v, k + 1) : 0.0;
-        int n0[DS], n1[DS];
-        digits<DS>(x0, E, n0);
-        digits<DS>(x1, E, n1);
-#pragma unroll
-        for (int q = 0; q < DS; ++q)
-            *reinterpret_cast<__nv_bfloat162 *>(dst + (size_t)q * rows * Kld + k) =
-                __nv_bfloat162(slice_bf16(n0[q], q), slice_bf16(n1[q], q));
-    }
+    for (int k = 2 * lane; k < Kend; k += 64)
+        put(k, E, k < K ? split_at(s, v, k) : 0.0, k + 1 < K ? split_at(s, v, k + 1) : 0.0);
 }
 
 // vectors stored across K: maxima of 32 vectors over 128 of K per CTA
@@ -1426,8 +1452,8 @@ cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t by
         return cudaErrorInvalidValue;
     cudaError_t e;
     if ((e = mma_attributes<DS, true>()) != cudaSuccess) return e;
-    const int most = (int)std::max<long long>(std::max(rows, cols), tiles);
-    launch_pdl(k_split_tab, std::min((most + 255) / 256, 64), 256, 0, st, t, probs, mix, mA, mB, tl, nt);
+    const int most = (int)std::max<long long>(std::max(rows, cols), tiles);   // (all products)
+    launch_pdl(k_split_tab, dim3(std::max(1, std::min((most / t.count + 255) / 256, 64)), t.count), 256, 0, st, t, probs, mix, mA, mB, tl, nt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (mv > 0) {
         launch_pdl(k_split_along, dim3((mv + 7) / 8, count, 2), 256, 0, st, t, As, Bs, E, F, ra, cb, Kld);
