@@ -933,7 +933,7 @@ struct Geqr2ResArgs {
     double *tau, *gram;            // gram[c ldg + i]: v_c^T v_i, c < i (what T is formed from)
     int ldg;
     Slot *gp;                      // [grid][32]: per-CTA partial sums a^T A[:, c] (column i: a^T a)
-    Slot *row, *sv, *scal;         // [32] top row; [32] update factors; [1] column scale
+    Slot *row, *sv;                // [2][32] top row, by the step's parity; [32] sums over the CTAs
     GridBar *bar;
     unsigned base;
 };
@@ -941,23 +941,25 @@ struct Geqr2ResArgs {
 // Householder QR of an m x nb panel (Sec. 4.3, step 1) held on chip: a block
 // of rows per CTA in shared memory (row major), a column per lane, the rows
 // over four warps.  With a = column i (unscaled; v = sc a, v_i = 1):
-//   owners  column c > i is owned by one warp of the grid: g_c = sum over CTAs
-//           of a^T A[:, c] and sig2 = a^T a (tail rows) -> H_i's scalars, s_c =
-//           tau (A[i, c] + sc g_c); R[i, c] = A[i, c] - s_c is final; sc s_c
-//           goes to every CTA.  Column i's owner stores tau, beta and sends sc.
-//           A finished column's owner (c < i) gets v_c^T v_i the same way: its
-//           lane would idle, and T needs those products (a separate pass over
-//           a 10000 x 32 panel for them measured 335 us, this kernel 200).
-//   rows    one pass A[r, c] -= a_r (sc s_c) with the partial sums of the next
+//   owners  column c != i is owned by one warp of the grid: g_c = sum over CTAs
+//           of a^T A[:, c] (tail rows), sent to every CTA; a warp of every CTA
+//           sums sig2 = a^T a and forms H_i's scalars while these travel.  The
+//           finished columns (c < i) give v_c^T v_i: their lanes would idle,
+//           and T needs those products (a separate pass over a 10000 x 32
+//           panel for them measured 335 us, this kernel 200).
+//   rows    s_c = tau (A[i, c] + sc g_c), R[i, c] = A[i, c] - s_c is final;
+//           one pass A[r, c] -= a_r (sc s_c) with the partial sums of the next
 //           column a' = A[:, i + 1] (a lane broadcast) against all columns
 // Two slot exchanges per column (buffers reused as in k_gebd2_resident)
 // instead of three grid barriers with the panel read from L2.  What bounds
 // it: the exchanges; two FP64 operations per row and column are about 2000
-// cycles of a column at 66 rows a CTA.
+// cycles of a column at 66 rows a CTA.  geqrf of 10000 x 32, 10000 x 600 and
+// 2048 x 2048: 355, 8449 and 29191 us with the scalars formed by the owners
+// before they sent their results, 301, 7442 and 27524 us now.
 __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
     extern __shared__ double smem[];
     __shared__ int s_err;
-    __shared__ double s_red[4][kQp], s_fac[kQp], s_sc[kQp];
+    __shared__ double s_red[4][kQp], s_fac[kQp], s_sc[kQp], s_alpha, s_sig2, s_tau;
     const int G = gridDim.x, g = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int m = a.m, nb = a.nb;
     const int rb = (m + G - 1) / G, r0 = min(m, g * rb), nr = min(m, r0 + rb) - r0;
@@ -969,8 +971,7 @@ __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
         for (int r = lane; r < nr; r += 32) W[r * kQld + c] = c < nb ? A[(size_t)c * lda + r0 + r] : 0.0;
     const Slot zero = {0ull, 0ull};
     if (t < kQp) a.gp[g * kQp + t] = zero;
-    if (g == 0 && t < kQp) a.row[t] = a.sv[t] = zero;
-    if (g == 0 && t == 0) a.scal[0] = zero;
+    if (g == 0 && t < kQp) a.row[t] = a.row[kQp + t] = a.sv[t] = zero;
     unsigned target = a.base + G;
     if (!grid_wait(a.bar, target)) return;
 
@@ -995,54 +996,58 @@ __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
     for (int i = 0; i < nb; ++i) {
         const unsigned tag = (unsigned)i + 1u;
         if (!grid_wait<false>(a.bar, target += G)) return;
-        // ---- owners: the k-th column other than i for k = g + G warp; column i itself: the last CTA's last warp
+        const Slot *row = a.row + (i & 1) * kQp;
+        // ---- warps 1-3: the k-th column other than i; warp 0: column i itself
         {
-            const int k = g + G * warp, c = k < i ? k : k + 1;
-            const bool own = c < nb, self = g == G - 1 && warp == 3;
-            if (own || self) {
-                // lanes 0-15 sum column c, lanes 16-31 column i
-                const int col = (lane < 16 && own) ? c : i;
-                double s = 0.0, alpha = 0.0, rw = 0.0;
-                for (int q0 = lane & 15; q0 < G; q0 += 128) {
-                    const Slot *q[10];
-                    double v[10];
+            const int k = g + G * (warp - 1), c = warp == 0 ? i : k < i ? k : k + 1;
+            if (c < nb) {
+                double s = 0.0;
+                for (int q0 = lane; q0 < G; q0 += 160) {
+                    const Slot *q[6];
+                    double v[6];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) q[j] = q0 + 16 * j < G ? a.gp + (q0 + 16 * j) * kQp + col : nullptr;
-                    q[8] = a.row + i;
-                    q[9] = a.row + col;
-                    slot_get<10>(q, tag, v, a.bar, &s_err);
-                    alpha = v[8];
-                    rw = v[9];
+                    for (int j = 0; j < 5; ++j) q[j] = q0 + 32 * j < G ? a.gp + (q0 + 32 * j) * kQp + c : nullptr;
+                    q[5] = warp == 0 ? row + i : nullptr;
+                    slot_get<6>(q, tag, v, a.bar, &s_err);
+                    if (t == 0) s_alpha = v[5];
                     s += v[0];
 #pragma unroll
-                    for (int j = 1; j < 8; ++j)
-                        if (q0 + 16 * j < G) s += v[j];
+                    for (int j = 1; j < 5; ++j)
+                        if (q0 + 32 * j < G) s += v[j];
                 }
-                for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                const double sig2 = __shfl_sync(0xffffffffu, s, 16);
-                double tau, beta;
-                const double sc = reflector_fast(alpha, sig2, tau, beta);
-                if (own && c < i && lane == 0) a.gram[(size_t)c * a.ldg + i] = s_sc[c] * fma(sc, s, rw);
-                if (own && c > i && lane == 0) {
-                    const double sfac = tau * fma(sc, s, rw);
-                    slot_put(a.sv + c, sc * sfac, tag);
-                    A[(size_t)c * lda + i] = rw - sfac;
-                }
-                if (self && lane == 0) {
-                    slot_put(a.scal, sc, tag);
-                    a.tau[i] = tau;
-                    A[(size_t)i * lda + i] = beta;
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) {
+                    if (warp == 0) s_sig2 = s;
+                    else slot_put(a.sv + c, s, tag);
                 }
             }
         }
-        if (!grid_wait<false>(a.bar, target += G)) return;
+        // the scalars of H_i while the other columns' sums are on their way
+        if (!grid_wait<false, 32>(a.bar, target += G, [&] {
+                double tau, beta;
+                const double sc = reflector_fast(s_alpha, s_sig2, tau, beta);
+                if (t == 0) {
+                    s_sc[i] = sc;
+                    s_tau = tau;
+                    if (g == 0) {
+                        a.tau[i] = tau;
+                        A[(size_t)i * lda + i] = beta;
+                    }
+                }
+            }))
+            return;
         // ---- rows
         if (warp == 0) {
-            const Slot *q[2] = {a.scal, lane > i && lane < nb ? a.sv + lane : nullptr};
+            const bool on = lane != i && lane < nb;
+            const Slot *q[2] = {on ? a.sv + lane : nullptr, on ? row + lane : nullptr};
             double v[2];
             slot_get<2>(q, tag, v, a.bar, &s_err);
-            s_fac[lane] = lane > i && lane < nb ? -v[1] : 0.0;
-            if (lane == 0) s_sc[i] = v[0];
+            const double sc = s_sc[i], w = fma(sc, v[0], v[1]), sfac = s_tau * w;
+            s_fac[lane] = lane > i && lane < nb ? -(sc * sfac) : 0.0;
+            if (g == 0 && on) {
+                if (lane < i) a.gram[(size_t)lane * a.ldg + i] = s_sc[lane] * w;
+                else A[(size_t)lane * lda + i] = v[1] - sfac;
+            }
         }
         __syncthreads();
         if (s_err) return;         // uniform: read after the barrier
@@ -1053,7 +1058,7 @@ __global__ void __launch_bounds__(NT) k_geqr2_resident(Geqr2ResArgs a) {
         int r = rl + warp;
         if (r0 + rl == i + 1 && rl < nr && warp == 0) { // the next top row
             const double x = fma(W[r * kQld + i], f, W[r * kQld + lane]);
-            if (lane < nb) slot_put(a.row + lane, x, tag + 1u);
+            if (lane < nb) slot_put(a.row + ((i + 1) & 1) * kQp + lane, x, tag + 1u);
             r += 4;
         }
         for (; r + 12 < nr; r += 16) {
@@ -1108,24 +1113,24 @@ cudaError_t launch_labrd_panel(int m, int n, int nb, double *A, int lda, double 
     return cudaLaunchCooperativeKernel((const void *)k_labrd_panel, dim3(G), dim3(kLT), params, 0, st);
 }
 
-// rows of a QR panel's CTA: about 64, at least 8 CTAs (the owners of 31
-// columns are a warp each), as many as there are SMs
+// rows of a QR panel's CTA: about 64, at least 11 CTAs (the owners of 31
+// columns are a warp each, three a CTA), as many as there are SMs
 static int qr_grid(int m) {
     const DevInfo d = dev_info();
-    return std::max(8, std::min({(m + 63) / 64, d.sms, kResGrid}));
+    return std::max(11, std::min({(m + 63) / 64, d.sms, kResGrid}));
 }
 static size_t qr_smem(int m, int G) { return sizeof(double) * (size_t)((m + G - 1) / G) * kQld + 64; }
 
 bool geqr2_resident_fits(int m, int nb) {
     const DevInfo d = dev_info();
-    return d.sms >= 8 && nb >= 1 && nb <= kQp && m >= nb && qr_smem(m, qr_grid(m)) <= (size_t)d.smem - 4096;
+    return d.sms >= 11 && nb >= 1 && nb <= kQp && m >= nb && qr_smem(m, qr_grid(m)) <= (size_t)d.smem - 4096;
 }
 
 cudaError_t launch_geqr2_resident(int m, int nb, double *A, int lda, double *tau, double *gram, int ldg,
                                   double *scratch, GridBar *bar, unsigned *bars, cudaStream_t st) {
     const int G = qr_grid(m);
-    Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * kQp, *sv = row + kQp, *scal = sv + kQp;
-    Geqr2ResArgs a{A, lda, m, nb, tau, gram, ldg, gp, row, sv, scal, bar, *bars};
+    Slot *gp = (Slot *)scratch, *row = gp + (size_t)kResGrid * kQp, *sv = row + 2 * kQp;
+    Geqr2ResArgs a{A, lda, m, nb, tau, gram, ldg, gp, row, sv, bar, *bars};
     *bars += (unsigned)G * (1u + 2u * (unsigned)nb);
     cudaError_t err =
         cudaFuncSetAttribute(k_geqr2_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, dev_info().smem - 4096);

@@ -25,3 +25,20 @@ def test_resident_reduction(m, n):
     bdc.ormbr(1, Ar, taup, C)
     assert float((C - A).norm()) <= 1e-15 * n * n ** 0.5 * float(A.norm())
     assert float(taup[-1]) == 0.0
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (32, 32), (33, 31), (64, 1), (352, 32), (705, 33), (9729, 32)])
+def test_resident_qr_panel(m, n):
+    """Panels held on chip: fewer rows than CTAs have, a column alone, the
+    smallest grid, one more row than a full share, the next panel's first
+    column.  Bound: n reflectors of a few ulp each, as above."""
+    from paper_2508_11467_gb300 import bdc
+    g = torch.Generator("cuda").manual_seed(m + 3 * n)
+    A = torch.randn(n, m, dtype=torch.float64, device="cuda", generator=g).t()
+    Ar, tau, info = bdc.geqrf(A.clone())   # (factors a column-major matrix of one column in place)
+    assert info == 0
+    R = torch.triu(Ar[:n])
+    Q = bdc.orgqr(Ar.clone().t().contiguous().t(), tau)
+    eye = torch.eye(n, dtype=torch.float64, device="cuda")
+    assert float((Q @ R - A).norm()) <= 1e-15 * (n + 1) * (n + 1) ** 0.5 * float(A.norm())
+    assert float((Q.t() @ Q - eye).norm()) <= 1e-15 * (n + 1) * (n + 1) ** 0.5 * n ** 0.5
