@@ -41,9 +41,11 @@ METRIC = "n=16384 bidiagonal SVD (σ+U,V) time, mixed vs FP64 at ≤1e-12 residu
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0, "sm_max_mhz": 2070.0}
 # FP64 rates of this part measured by throughput probes (per SM per clock):
-# mma.sync.m8n8k4.f64 6.66 MAC; DFMA 1.99 lane operations (independent chains
+# mma.sync.m8n8k4.f64 1.67 MAC (a warp instruction holds its sub-partition for
+# 615 cycles: the FP64 pipe's own rate); DFMA 1.99 lane operations (independent chains
 # on every SM: 626.7 G DFMA/s = 1.253 TFLOP/s at 2070 MHz; bench_fp64_peak.cu)
-FP64_DMMA_MAC_PER_CLK_SM = 6.66
+FP64_DMMA_MAC_PER_CLK_SM = 1.67
+SPLIT_PAIRS_DENSE = 34     # BF16 slice products per FP64 product of a block reflector
 FP64_ALU_OPS_PER_CLK_SM = 1.99
 SMS = 152
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_bdc_exact_uniform_n16384.md")
@@ -403,7 +405,8 @@ def dense_run(steps, warmup):
     timed with CUDA events over `steps` calls after `warmup`.  Roofline of the
     reduction: (8/3) n^3 flops, half in products with the trailing matrix
     (the BLAS2 part, FP64 ALU-bound on this part) and half in the merged
-    rank-(2b) updates (FP64 tensor cores)."""
+    rank-(2b) updates (split-BF16 products, SPLIT_PAIRS_DENSE slice pairs at
+    the measured BF16 burst rate)."""
     import torch
 
     from paper_2508_11467_gb300 import bdc, inputs
@@ -411,7 +414,7 @@ def dense_run(steps, warmup):
     out = {}
     clk = 2070e6
     alu = FP64_ALU_OPS_PER_CLK_SM * SMS * clk * 2 / 1e12          # TFLOP/s (FMA = 2)
-    dmma = 2 * FP64_DMMA_MAC_PER_CLK_SM * SMS * clk / 1e12
+    split = float(load_peaks()[0].get("bf16_tflops", FALLBACK["bf16_tflops"])) / SPLIT_PAIRS_DENSE
     for name, (m, n, kind) in {"square_n4096": (4096, 4096, "gauss"), "ts_m20000_n1000": (20000, 1000, "geo")}.items():
         if kind == "gauss":
             A0 = torch.randn(m, n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(7))
@@ -454,7 +457,7 @@ def dense_run(steps, warmup):
         ms_copy = timeit(lambda: A.copy_(A0))
         ms_brd = timeit(gebrd) - ms_copy
         flops = 4.0 * m * n * n - 4.0 * n ** 3 / 3.0
-        t_min = (flops / 2) / (alu * 1e12) + (flops / 2) / (dmma * 1e12)
+        t_min = (flops / 2) / (alu * 1e12) + (flops / 2) / (split * 1e12)
         res["gebrd_ms"] = ms_brd
         res["gebrd_gflops"] = flops / (ms_brd * 1e-3) / 1e9
         res["gebrd_roofline_frac"] = t_min / (ms_brd * 1e-3)
@@ -494,7 +497,7 @@ def dense_run(steps, warmup):
         del A, A0, U, VT, wk2
         torch.cuda.empty_cache()
     out["roofline_note"] = (f"bidiagonalization lower bound: half its (4 m n^2 - 4 n^3 / 3) flops at the FP64 ALU "
-                            f"peak {alu:.3f} TFLOP/s, half at the FP64 mma.sync peak {dmma:.2f} TFLOP/s")
+                            f"peak {alu:.3f} TFLOP/s, half as split-BF16 products at {split:.1f} TFLOP/s")
     return out
 
 
