@@ -458,6 +458,7 @@ __global__ void __launch_bounds__(256) k_final(const MatDesc *__restrict__ mats,
 // blocks that live as long as that graph (the graph replays those copies),
 // instead of the shared cache and ring of one-shot calls.
 thread_local std::vector<void *> *g_arena = nullptr;
+thread_local bool g_plan_capture = false;          // recording a plan's own graph (not a caller's)
 
 // Blocks of caller-captured graphs that have been destroyed: a CUDA user
 // object attached to the graph hands them over when its last reference goes
@@ -727,7 +728,7 @@ int run_plan(const Plan &p, const bdc_opts &o, char *work, std::vector<MatDesc> 
     }
     cudaError_t e = upload(p, work, mats, st);
     if (e != cudaSuccess) return note(e);
-    const OverlapScope overlapped(st, !g_prof.on);
+    const OverlapScope overlapped(st, !g_prof.on, g_plan_capture);
     SideStream *side = nullptr;
     if (!p.vals && !p.heights.empty() && (e = side_stream(side)) != cudaSuccess) return note(e);
     int *derr = (int *)(work + p.off_err);
@@ -1225,7 +1226,13 @@ int plan_capture(bdc_plan_s *pl, const Plan &p, const bdc_opts &r, char *w, std:
     g_arena = &pl->pinned;
     int rc = note(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
     if (rc == 0) {
-        rc = run_plan(p, r, w, mats, d_info, cs);
+        {
+            struct Flag {
+                Flag() { g_plan_capture = true; }
+                ~Flag() { g_plan_capture = false; }
+            } flag;
+            rc = run_plan(p, r, w, mats, d_info, cs);
+        }
         cudaGraph_t g = nullptr;
         const int rc2 = note(cudaStreamEndCapture(cs, &g));
         if (rc == 0) rc = rc2;

@@ -258,16 +258,20 @@ __device__ __forceinline__ void set_error(int *info, int code) {
 // (n = 16384: 6.99 ms with plain launches, 6.82 ms so, 7.35 ms with the early
 // trigger; n = 1001 1291, 1192, 1315 us; n = 100 585, 534, 541 us; values of
 // n = 10007 2.53, 2.34, 2.71 ms).  launch_pdl falls back to plain launches
-// where overlap() is off (graph capture, stage profiling).  A launch after an
+// where overlap() is off (a caller's graph capture, stage profiling).  A launch after an
 // event wait, a copy or a memset is a plain one.
 __device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 bool &overlap();   // of the calling thread (bdc_driver.cu)
-// overlap() on for a scope unless `st` is being captured
+// overlap() on for a scope unless `st` is being captured by the caller (whose
+// graph keeps plain edges); a plan's own graph (own_capture) takes them:
+// 512 matrices of order 32..1024, FP32, 3266 us with plain edges, 3191 us so;
+// 200 of order 40..300 581 and 522 us; FP64 20482 and 20349 us
 struct OverlapScope {
     bool was;
-    explicit OverlapScope(cudaStream_t st, bool allowed = true) : was(overlap()) {
+    explicit OverlapScope(cudaStream_t st, bool allowed = true, bool own_capture = false) : was(overlap()) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        overlap() = allowed && cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+        overlap() = allowed && (own_capture || (cudaStreamIsCapturing(st, &cs) == cudaSuccess &&
+                                                cs == cudaStreamCaptureStatusNone));
     }
     ~OverlapScope() { overlap() = was; }
 };
