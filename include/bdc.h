@@ -415,8 +415,9 @@ int bdc_mlp_train(const bdc_opts *o, const bdc_mlp_train_opts *t, float *params,
 /* Bidiagonalization A = Q1 B P1^T (Sec. 4.1, Algorithm 1), m >= n: per
  * panel the b column and row reflectors (H_i, G_i, Eq. gebrd-house) with the
  * vectors y_i, x_i of Eqs. (bidiag-y-k3, bidiag-x-k3), then the merged
- * rank-(2b) update A -= P Q^T of Eq. (bidiag-A-trail3) as one
- * tensor-core product.  On exit d[n] / e[n-1] hold B's diagonal and
+ * rank-(2b) update A -= P Q^T of Eq. (bidiag-A-trail3) on the
+ * tensor cores, by error-free BF16 slices that keep 56 bits below the
+ * maximum of each row of V, X, Y and U.  On exit d[n] / e[n-1] hold B's diagonal and
  * superdiagonal, A holds y_i below the diagonal of column i and u_i right of
  * the superdiagonal of row i (u_i[i+1] = 1 implicit), tauq[n], taup[n] the
  * scalars (taup[n-1] = 0).  *d_info (device): 0 or BDC_ERR_TIMEOUT. */

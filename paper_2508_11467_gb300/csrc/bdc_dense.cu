@@ -7,7 +7,8 @@
 //             corrections of the not yet updated trailing matrix merged into
 //             one pair of matrices P = [V X], Q = [Y U]; the trailing matrix
 //             then takes the merged rank-(2b) update A -= P Q^T of Eq.
-//             (bidiag-A-trail3) as ONE product.
+//             (bidiag-A-trail3): ONE product in FP64, the halves V Y^T and
+//             X U^T at a scale of their own when sliced.
 //   Sec. 4.3  QR of a tall-and-skinny A (cooperative panel k_geqr2 plus a
 //             block-reflector update of the trailing columns), the explicit Q
 //             (Eq. orgqr-q), and the back-transformations U = Q1 U2 and
@@ -24,7 +25,7 @@
 // any shape and occupancy; the plain FMA 1.9), so the FP64 products were
 // most of a large SVD: back-transformation of 4096 x 4096, one side, 181 ms
 // (165 ms without the triangular solves) -> 10.5 ms; trailing updates of its
-// reduction about 85 -> 8 ms; 333 x 333, one side, 2.4 -> 0.64 ms.  Error:
+// reduction about 85 -> 20 ms; 333 x 333, one side, 2.4 -> 0.64 ms.  Error:
 // U^T U - I and the residual of gesvd as with FP64 products (333 to 2048:
 // 5.5e-14 to 4.2e-13 and 2.8e-15 to 7.6e-15 either way).
 //
@@ -925,9 +926,9 @@ struct WideStep {
         p.sub = 1;
         if (left) {            // C -= V Z
             p.a = SplitSide{V, 0, ldv, 1, rows, 1, 0, 0, 0};
-            p.b = SplitSide{Z, zs, nb, 0, ns, np, 0, 0, 0, nullptr, 0, 0, c, ldc, 1};   // + C's first nb rows
+            p.b = SplitSide{Z, zs, nb, 0, ns, np, 0, 0, 0, c, ldc, 1};   // + C's first nb rows
         } else {               // C -= Z V^T
-            p.a = SplitSide{Z, zs, ns, 1, ns, np, 0, 0, 0, nullptr, 0, 0, c, 1, ldc};   // + C's first nb columns
+            p.a = SplitSide{Z, zs, ns, 1, ns, np, 0, 0, 0, c, 1, ldc};   // + C's first nb columns
             p.b = SplitSide{V, 0, ldv, 1, rows, 1, 0, 0, 0};
         }
         return set.add(p);
@@ -1216,7 +1217,7 @@ bool panel_split(int rows, int cols, const SplitWs &w) {
 }
 
 // Bidiagonalization, Algorithm 1 (m >= n): on chip once it fits; before that,
-// per panel of b, k_labrd_panel, then the merged rank-(2b) update of the trailing matrix (one product).
+// per panel of b, k_labrd_panel, then the merged rank-(2b) update of the trailing matrix.
 cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup, int b,
                         char *ws, cudaStream_t st) {
     const DenseWs w = dense_ws(m, n, b, n);
@@ -1237,22 +1238,27 @@ cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, 
         if (nb < nl) {
             // the merged rank-(2b) update A[nb:, nb:] -= P Q^T (Eq. bidiag-A-trail3):
             // P = [V X] (ml x 2b) and Q = [Y U] (nl x 2b) are contiguous column
-            // blocks, zero in the columns a short last panel does not use, so
-            // the whole update is ONE product with K = 2b
+            // blocks.  Sliced, it is two products of K = b, A -= V Y^T and A -= X U^T:
+            // V and U are of order one, X and Y of the trailing matrix's, and
+            // the slices keep 56 bits below a vector's maximum, which must not
+            // be the other half's: one product of K = 2b under any common
+            // scale loses V Y^T where the two differ (1900 x 1900 Gaussian,
+            // first column times 1e-8: 1.2e-9 of ||A||; so 1e-15).  Two halves
+            // cost 182 ms for 4096 x 4096, one would take 174
             const double *P = (const double *)(ws + w.PW), *Q = (const double *)(ws + w.QW);
             const SplitWs sw = split_ws(ws, w);
             const long long tr = ml - nb, tc = nl - nb;
-            if (split_scratch(tr, tc, 2 * b, ((tr + 127) / 128) * ((tc + 127) / 128)) <= sw.slice_bytes) {
-                // V and Y are brought to X's and U's scale by the exponent of
-                // the panel's first diagonal entry (a column norm)
-                SplitProd p{};
-                p.a = SplitSide{P + nb, 0, ml, 1, (int)tr, 1, 0, 0, 0, d + i0, b, 1};
-                p.b = SplitSide{Q + nb, 0, nl, 1, (int)tc, 1, 0, 0, 0, d + i0, b, -1};
-                p.C = A + i0 + nb + (size_t)(i0 + nb) * lda;
-                p.ldc = lda;
-                p.K = 2 * b;
-                p.sub = 1;
-                if ((err = split_products(&p, 1, sw.slices, sw.slice_bytes, sw.err, st)) != cudaSuccess) return err;
+            if (split_scratch(2 * tr, 2 * tc, b, ((tr + 127) / 128) * ((tc + 127) / 128)) <= sw.slice_bytes) {
+                SplitProd p[2]{};
+                for (int h = 0; h < 2; ++h) {
+                    p[h].a = SplitSide{P + (size_t)h * b * ml + nb, 0, ml, 1, (int)tr, 1, 0, 0, 0};
+                    p[h].b = SplitSide{Q + (size_t)h * b * nl + nb, 0, nl, 1, (int)tc, 1, 0, 0, 0};
+                    p[h].C = A + i0 + nb + (size_t)(i0 + nb) * lda;
+                    p[h].ldc = lda;
+                    p[h].K = b;
+                    p[h].sub = 1;
+                }
+                if ((err = split_products(p, 2, sw.slices, sw.slice_bytes, sw.err, st, 1)) != cudaSuccess) return err;
                 continue;
             }
             if ((err = dgemm(0, 1, ml - nb, nl - nb, 2 * b, -1.0, P + nb, ml, Q + nb, nl, 1.0,

@@ -53,16 +53,11 @@ cudaError_t launch_geqr2_resident(int m, int nb, double *A, int lda, double *tau
 // where row > reflector, 0 above: row moff + k of reflector v, the unit entry
 // left out (mask = 1), or row moff + v of reflector k, with it (mask = 2).
 // add: add[v add_v + k add_k] is added to entry k of vector v.
-// ref: entries k < kref are multiplied by 2^(rsign e) with e the exponent of
-// *ref (a device value): the two halves of a concatenated operand brought to
-// one scale, the other operand taking the inverse.
 struct SplitSide {
     const double *p;
     long long pstride;
     int ld, tr, n, parts, mask, moff;
     int row0;   // set by split_products
-    const double *ref;
-    int kref, rsign;
     const double *add;
     long long add_v, add_k;
 };
@@ -75,8 +70,11 @@ constexpr int kSplitMax = 32, kSplitMostK = 16384;
 // products on the tensor cores by error-free BF16 slices (bdc_gemm_mixed.cu),
 // at most kSplitMax in one launch set; scratch of split_scratch(sum of a.n,
 // sum of b.n, largest K, sum of ceil(a.n/128) ceil(b.n/128)) bytes; *err
-// (device) is set when a bounded wait gave up
+// (device) is set when a bounded wait gave up.  The products of a launch set
+// have results of their own; chained = 1: two products of one shape
+// subtracted from one C, each at a scale of its own.
 size_t split_scratch(long long rowsA, long long colsB, int K, long long tiles);
-cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t bytes, int *err, cudaStream_t st);
+cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t bytes, int *err, cudaStream_t st,
+                           int chained = 0);
 
 }  // namespace bdc

@@ -482,8 +482,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                                                      const int *__restrict__ Ea, const int *__restrict__ Fb,
                                                      int *__restrict__ err, const int2 *__restrict__ tiles,
                                                      const int *__restrict__ ntiles, unsigned long long wait_ns,
-                                                     int stall) {
+                                                     int stall, int chained) {
     pdl_begin();
+    // chained: every tile of the list is that of two products, p and p + 1, of
+    // one C, which this CTA's threads update one after the other
+    const int two = (MODE == MODE_EW || MODE == MODE_LW) ? chained : 0;
     constexpr int TILE = TM * TK * 2;                 // one 128 x 32 BF16 slice tile (A or B)
     constexpr int SL = stage_slices<S, MODE>();       // slices per operand in a stage
     constexpr int STAGE_BYTES = stage_bytes<S, MODE>();
@@ -511,6 +514,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
     // epilogue still converts and stores the current one.
     const int count = *ntiles;
     if ((int)blockIdx.x >= count) return;
+    const int mine = ((count - 1 - (int)blockIdx.x) / (int)gridDim.x + 1) << two;   // this CTA's tiles
+    auto tile_at = [&](int j) {
+        int2 tc = tiles[blockIdx.x + (j >> two) * gridDim.x];
+        tc.x += j & two;
+        return tc;
+    };
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         for (int i = 0; i < NSTAGE; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -533,16 +542,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
             int G = 0;                                  // stages loaded so far (all tiles)
             bool ok = true;
             // the next tile's coordinates are loaded while this one streams
-            int2 tcn = tiles[blockIdx.x];
+            int2 tcn = tile_at(0);
             MixProb mxn = mix[tcn.x];
             int Kn = probs[tcn.x].K;
-            for (int ti = blockIdx.x; ti < count && ok; ti += gridDim.x) {
+            for (int ti = 0; ti < mine && ok; ++ti) {
                 const int2 tc = tcn;
                 const MixProb mx = mxn;
                 const int m0 = (tc.y >> 16) * TM, n0 = (tc.y & 0xffff) * TNX;
                 const int nk = (Kn + TK - 1) / TK;
-                if (ti + (int)gridDim.x < count) {
-                    tcn = tiles[ti + gridDim.x];
+                if (ti + 1 < mine) {
+                    tcn = tile_at(ti + 1);
                     mxn = mix[tcn.x];
                     Kn = probs[tcn.x].K;
                 }
@@ -584,10 +593,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                 if (done > 0 && !mbar_wait(&accempty[set], (done - 1) & 1, err, abort_flag, wait_ns)) ok = false;
                 fence_after();
             };
-            int Kn = probs[tiles[blockIdx.x].x].K;     // the next tile's K, loaded ahead
-            for (int ti = blockIdx.x; ti < count && ok; ti += gridDim.x) {
+            int Kn = probs[tile_at(0).x].K;            // the next tile's K, loaded ahead
+            for (int ti = 0; ti < mine && ok; ++ti) {
                 const int nk = (Kn + TK - 1) / TK;
-                if (ti + (int)gridDim.x < count) Kn = probs[tiles[ti + gridDim.x].x].K;
+                if (ti + 1 < mine) Kn = probs[tile_at(ti + 1).x].K;
                 for (int s = 0; s < nk && ok; ++s, ++G) {
                     const int buf = G % NSTAGE;
                     if (!mbar_wait(&full[buf], (G / NSTAGE) & 1, err, abort_flag, wait_ns)) { ok = false; break; }
@@ -694,8 +703,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
         bool ok = true;
         int cA = 0, cB = 0;                        // drains done: set A / set B (MODE_E), tiles (MODE_X3)
         int GL = 0;                                // stages drained (MODE_L)
-        for (int ti = blockIdx.x; ti < count && ok; ti += gridDim.x) {
-            const int2 tc = tiles[ti];
+        for (int ti = 0; ti < mine && ok; ++ti) {
+            const int2 tc = tile_at(ti);
             const GemmProb pr = probs[tc.x];
             const MixProb mx = mix[tc.x];
             const int m0 = (tc.y >> 16) * TM, n0 = (tc.y & 0xffff) * TNX;
@@ -717,7 +726,28 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                     cml[h2] = cok ? (pr.cmap ? pr.cmap[col] : col) : 0;
                 }
             };
+            // the final read-modify-write of C waits on its loads while the
+            // next tile's stages wait on this warp: pull this warp's 32 rows of
+            // its CPT columns into L2 early (lane = column, 256 B each), while
+            // the stages accumulate (4096 x 4096 reduction: 184 -> 182 ms with it in
+            // MODE_EW as well)
+            auto prefetch_c = [&]() {
+                const int rw0 = m0 + 32 * q;
+#pragma unroll
+                for (int h2 = 0; h2 < CPT / 32; ++h2) {
+                    const int col = c0 + 32 * h2 + lane;
+                    if (col < pr.N && rw0 < pr.M) {
+                        const double *pc = pr.C + (long long)cml[h2] * ldc + rw0;
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(pc));
+                        if (rw0 + 16 < pr.M) asm volatile("prefetch.global.L2 [%0];" ::"l"(pc + 16));
+                    }
+                }
+            };
             if constexpr (MODE == MODE_E || MODE == MODE_EW) {
+                if constexpr (MODE == MODE_EW) {
+                    column_tables();
+                    if (mx.sub) prefetch_c();
+                }
                 // unsigned: the magic offsets wrap modulo 2^64 and cancel exactly at the end
                 unsigned long long L[CPT];
 #pragma unroll
@@ -774,7 +804,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                     const unsigned long long corr = (unsigned long long)tA * M * ((1ull << 24) + 1) +
                                                     (unsigned long long)tB * M * ((1ull << 16) + (1ull << 8));
                     const int Er = rowok ? Ea[mx.a_row0 + row] : 0;
-                    column_tables();
+                    if constexpr (MODE == MODE_E) column_tables();
 #pragma unroll
                     for (int cb = 0; cb < CPT / 8; ++cb) {
                         int F[8], cj[8];
@@ -812,24 +842,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
 #pragma unroll
                     for (int i = 0; i < CPT; ++i) I4[i] = 0;
                 }
-                // the final read-modify-write of C waits on its loads while the
-                // next tile's stages wait on this warp: pull this warp's 32 rows of
-                // its CPT columns into L2 now (lane = column, 256 B each), while
-                // the stages below accumulate
                 const int Er = rowok ? Ea[mx.a_row0 + row] : 0;
                 column_tables();
-                {
-                    const int rw0 = m0 + 32 * q;
-#pragma unroll
-                    for (int h2 = 0; h2 < CPT / 32; ++h2) {
-                        const int col = c0 + 32 * h2 + lane;
-                        if (col < pr.N && rw0 < pr.M) {
-                            const double *pc = pr.C + (long long)cml[h2] * ldc + rw0;
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(pc));
-                            if (rw0 + 16 < pr.M) asm volatile("prefetch.global.L2 [%0];" ::"l"(pc + 16));
-                        }
-                    }
-                }
+                prefetch_c();
                 for (int s = 0; s < nk; ++s, ++GL) {
                     const int b = GL & 1;
                     if (!mbar_wait(&accfull[b], (GL >> 1) & 1, err, abort_flag, wait_ns)) { ok = false; break; }
@@ -1125,12 +1140,12 @@ cudaError_t run_mixed(const GemmProb *probs, int nprobs, const std::vector<MixPr
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int grid = tiles < sm_count() ? tiles : sm_count();   // persistent: one CTA per SM
     if constexpr (EXACT) {
-        launch_pdl(k_mma<S, MODE_E>, grid, THREADS, smemE, st, mae, mbe, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, stall);
+        launch_pdl(k_mma<S, MODE_E>, grid, THREADS, smemE, st, mae, mbe, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, stall, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if constexpr (S > 4)
-            launch_pdl(k_mma<S, MODE_L>, grid, THREADS, smemL, st, ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, 0);
+            launch_pdl(k_mma<S, MODE_L>, grid, THREADS, smemL, st, ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, 0, 0);
     } else {
-        launch_pdl(k_mma<S, MODE_X3>, grid, THREADS, smemX, st, ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, stall);
+        launch_pdl(k_mma<S, MODE_X3>, grid, THREADS, smemX, st, ma, mb, probs, dmix, nprobs, E, F, err, tlist, ntiles, wait_ns, stall, 0);
     }
     return cudaGetLastError();
 }
@@ -1203,7 +1218,7 @@ constexpr int DS = 7;                      // slices: 56 bits below the row's ma
 
 struct SplitTab {
     SplitProd p[kSplitMax];
-    int count;
+    int count, chained;
 };
 
 // tables of the launch: products, exponent maxima cleared, tile list; grid
@@ -1215,7 +1230,8 @@ __global__ void __launch_bounds__(256) k_split_tab(const __grid_constant__ Split
     pdl_begin();
     const int q = blockIdx.y;
     const SplitProd &p = t.p[q];
-    const int tm = (p.a.n + TM - 1) / TM, tn = (p.b.n + TNX - 1) / TNX, cnt = tm * tn;
+    const int tm = (p.a.n + TM - 1) / TM, tn = (p.b.n + TNX - 1) / TNX;
+    const int cnt = (t.chained && q > 0) ? 0 : tm * tn;   // (chained: the first product's tiles serve both)
     int base = 0;
     for (int j = 0; j < q; ++j) base += ((t.p[j].a.n + TM - 1) / TM) * ((t.p[j].b.n + TNX - 1) / TNX);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1224,7 +1240,7 @@ __global__ void __launch_bounds__(256) k_split_tab(const __grid_constant__ Split
         m.a_row0 = p.a.row0; m.b_col0 = p.b.row0; m.tile0 = base; m.tilesN = tn;
         m.Mmax = p.a.n; m.Nmax = p.b.n; m.sub = p.sub;
         mix[q] = m;
-        if (q + 1 == t.count) *ntiles = base + cnt;
+        if (t.chained ? q == 0 : q + 1 == t.count) *ntiles = base + cnt;
     }
     constexpr int G = 8;                   // bands of 8 row blocks, as in k_tile_list
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
@@ -1252,10 +1268,6 @@ __device__ __forceinline__ double split_at(const SplitSide &s, int v, int k) {
     double x = *p;
     for (int q = 1; q < s.parts; ++q) x += p[(size_t)q * s.pstride];
     if (s.add) x += s.add[v * s.add_v + k * s.add_k];
-    if (s.ref && k < s.kref) {             // times 2^(+-e), 2^e <= |*ref| < 2^(e+1)
-        const int e = (int)((mag_bits(*s.ref) >> 52)) - 1023;
-        if (e > -1023 && e < 1024) x = ldexp_safe(x, s.rsign * e);
-    }
     return x;
 }
 constexpr int kAlongRegs = 6;              // entry pairs a lane keeps in registers: K <= 384
@@ -1290,7 +1302,7 @@ __global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ Spl
     };
     // a plain matrix of short vectors: every load issued at once, kept for
     // the digits (31 products of 480 columns x 323: 49 -> 27 us)
-    if (!s.mask && s.parts <= 1 && !s.add && !s.ref && K <= 64 * kAlongRegs) {
+    if (!s.mask && s.parts <= 1 && !s.add && K <= 64 * kAlongRegs) {
         const double *x = s.p + (size_t)v * s.ld;
         double xv[kAlongRegs][2];
 #pragma unroll
@@ -1412,10 +1424,15 @@ size_t split_scratch(long long rowsA, long long colsB, int K, long long tiles) {
     return split_layout(rowsA + TM, colsB + TNX, (K + TK - 1) / TK * TK, tiles).total + 256;
 }
 
-cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t bytes, int *err, cudaStream_t st) {
+cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t bytes, int *err, cudaStream_t st,
+                           int chained) {
     if (count <= 0) return cudaSuccess;
     if (count > kSplitMax) return cudaErrorInvalidValue;
+    if (chained && (count != 2 || prods[0].C != prods[1].C || prods[0].ldc != prods[1].ldc || !prods[0].sub ||
+                    !prods[1].sub || prods[0].a.n != prods[1].a.n || prods[0].b.n != prods[1].b.n))
+        return cudaErrorInvalidValue;
     SplitTab t{};
+    t.chained = chained;
     long long rows = 0, cols = 0, tiles = 0;
     int kmax = 1, mv = 0, mt = 0, kt = 0;
     for (int q = 0; q < count; ++q) {
@@ -1426,7 +1443,7 @@ cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t by
         rows += p.a.n;
         cols += p.b.n;
         kmax = std::max(kmax, p.K);
-        tiles += (long long)((p.a.n + TM - 1) / TM) * ((p.b.n + TNX - 1) / TNX);
+        if (!chained || q == 0) tiles += (long long)((p.a.n + TM - 1) / TM) * ((p.b.n + TNX - 1) / TNX);
         for (const SplitSide *s : {&p.a, &p.b}) {
             if (s->tr) { mt = std::max(mt, s->n); kt = std::max(kt, p.K); }
             else mv = std::max(mv, s->n);
@@ -1467,9 +1484,9 @@ cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t by
     }
     const int grid = (int)std::min<long long>(tiles, sm_count());
     const unsigned long long wait_ns = test_wait_ns();
-    launch_pdl(k_mma<DS, MODE_EW>, grid, THREADS, mma_smem<DS, MODE_EW>(), st, mae, mbe, probs, mix, count, E, F, err, tl, nt, wait_ns, 0);
+    launch_pdl(k_mma<DS, MODE_EW>, grid, THREADS, mma_smem<DS, MODE_EW>(), st, mae, mbe, probs, mix, count, E, F, err, tl, nt, wait_ns, 0, chained);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    launch_pdl(k_mma<DS, MODE_LW>, grid, THREADS, mma_smem<DS, MODE_LW>(), st, ma, mb, probs, mix, count, E, F, err, tl, nt, wait_ns, 0);
+    launch_pdl(k_mma<DS, MODE_LW>, grid, THREADS, mma_smem<DS, MODE_LW>(), st, ma, mb, probs, mix, count, E, F, err, tl, nt, wait_ns, 0, chained);
     return cudaGetLastError();
 }
 
