@@ -946,7 +946,7 @@ template <typename YK>
 cudaError_t apply_wide(int left, int rows, int other, YK yk, int nb, const double *V, int ldv, double *C, int ldc,
                        const SplitWs &w, cudaStream_t st) {
     cudaError_t e;
-    int slab = (other + 127) / 128 * 128;
+    int slab = other < kSplitMostRows ? (other + 127) / 128 * 128 : kSplitMostRows;
     auto step_of = [&](int s) {
         WideStep x = wide_step(left, rows, s, nb, V, ldv, C, ldc, w);
         x.cut(std::min(kSplitMax, 152 / std::max(x.tiles(), 1)));
@@ -1209,7 +1209,7 @@ bool use_wide(int refl, int rows, int other) {
 }
 // a QR panel's trailing update on the split products: from about 300 x 300
 bool panel_split(int rows, int cols, const SplitWs &w) {
-    return (long long)rows * cols >= 100 * 1000 && rows <= kSplitMax * (kSplitMostK - 64) &&
+    return (long long)rows * cols >= 100 * 1000 && cols <= kSplitMostRows && rows <= kSplitMax * (kSplitMostK - 64) &&
            (size_t)cols * 32 * kSplitMax <= w.zcap &&
            split_scratch((long long)kSplitMax * 32, (long long)kSplitMax * cols, (rows + kSplitMax - 1) / kSplitMax + 64,
                          (long long)kSplitMax * ((cols + 127) / 128)) <= w.slice_bytes &&
@@ -1243,12 +1243,13 @@ cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, 
             // the slices keep 56 bits below a vector's maximum, which must not
             // be the other half's: one product of K = 2b under any common
             // scale loses V Y^T where the two differ (1900 x 1900 Gaussian,
-            // first column times 1e-8: 1.2e-9 of ||A||; so 1e-15).  Two halves
+            // first column times 1e-8: 1.8e-9 of ||A||; so 1e-15).  Two halves
             // cost 182 ms for 4096 x 4096, one would take 174
             const double *P = (const double *)(ws + w.PW), *Q = (const double *)(ws + w.QW);
             const SplitWs sw = split_ws(ws, w);
             const long long tr = ml - nb, tc = nl - nb;
-            if (split_scratch(2 * tr, 2 * tc, b, ((tr + 127) / 128) * ((tc + 127) / 128)) <= sw.slice_bytes) {
+            if (tr <= kSplitMostRows &&
+                split_scratch(2 * tr, 2 * tc, b, ((tr + 127) / 128) * ((tc + 127) / 128)) <= sw.slice_bytes) {
                 SplitProd p[2]{};
                 for (int h = 0; h < 2; ++h) {
                     p[h].a = SplitSide{P + (size_t)h * b * ml + nb, 0, ml, 1, (int)tr, 1, 0, 0, 0};
@@ -1465,7 +1466,7 @@ cudaError_t dense_product(int m, int n, const double *A, int lda, const double *
     auto fits = [&](int r) {
         return split_scratch(r, n, n, (long long)((r + 127) / 128) * ((n + 127) / 128)) <= sw.slice_bytes;
     };
-    int slab = m;
+    int slab = std::min(m, kSplitMostRows);
     while (slab > 128 && !fits(slab)) slab = (slab / 2 + 127) / 128 * 128;
     if (n < 64 || n > kSplitMostK || !fits(slab))
         return dgemm(0, 0, m, n, n, 1.0, A, lda, B, n, 0.0, C, ldc, st);

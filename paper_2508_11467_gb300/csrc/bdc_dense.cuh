@@ -67,8 +67,12 @@ struct SplitProd {
     int ldc, K, sub;   // sub: C -= A B
 };
 constexpr int kSplitMax = 32, kSplitMostK = 16384;
+// rows of A and columns of B at most: a tile list entry holds the row block
+// (of 128) in 15 bits, the column block in 16
+constexpr int kSplitMostRows = 32767 * 128;
 // products on the tensor cores by error-free BF16 slices (bdc_gemm_mixed.cu),
-// at most kSplitMax in one launch set; scratch of split_scratch(sum of a.n,
+// at most kSplitMax in one launch set, K up to kSplitMostK and a.n, b.n up to
+// kSplitMostRows (cudaErrorInvalidValue beyond); scratch of split_scratch(sum of a.n,
 // sum of b.n, largest K, sum of ceil(a.n/128) ceil(b.n/128)) bytes; *err
 // (device) is set when a bounded wait gave up.  The products of a launch set
 // have results of their own; chained = 1: two products of one shape

@@ -1437,7 +1437,9 @@ cudaError_t split_products(SplitProd *prods, int count, void *scratch, size_t by
     int kmax = 1, mv = 0, mt = 0, kt = 0;
     for (int q = 0; q < count; ++q) {
         SplitProd &p = prods[q];
-        if (p.a.n <= 0 || p.b.n <= 0 || p.K <= 0 || p.K > kSplitMostK) return cudaErrorInvalidValue;
+        if (p.a.n <= 0 || p.b.n <= 0 || p.K <= 0 || p.K > kSplitMostK || p.a.n > kSplitMostRows ||
+            p.b.n > kSplitMostRows)
+            return cudaErrorInvalidValue;
         p.a.row0 = (int)rows;
         p.b.row0 = (int)cols;
         rows += p.a.n;
