@@ -1023,14 +1023,25 @@ cudaError_t apply_pair(const WideJob (&j)[kPair], cudaStream_t st) {
     return cudaSuccess;
 }
 
+// How Z = Y^T C of a QR panel is cut along K = rows: np products of kc rows,
+// a wave of tiles or so, no product longer than kSplitMostK.  (rows up to
+// kSplitMax (kSplitMostK - 64) give np <= kSplitMax and kc <= kSplitMostK.)
+struct PanelCut {
+    int np, kc;
+};
+PanelCut panel_cut(int rows, int cols) {
+    const int tiles = (cols + 127) / 128, least = (rows + kSplitMostK - 33) / (kSplitMostK - 32);
+    const int np = std::max({1, least, std::min({kSplitMax, 152 / std::max(tiles, 1), rows / 256})});
+    const int kc = ((rows + np - 1) / np + 31) / 32 * 32;
+    return PanelCut{(rows + kc - 1) / kc, kc};
+}
+
 // H^T C for one panel of at most kTB reflectors with its T (row-major, ld
 // kTB): Z = Y^T C in split-K parts, W = T^T Z in FP64 (small), C -= Y W
 cudaError_t apply_panel(const Reflectors &f, const double *T, int rows, int cols, double *C, int ldc, double *W,
                         const SplitWs &w, cudaStream_t st) {
-    const int nb = f.count, tiles = (cols + 127) / 128;
-    int np = std::max(1, std::min({kSplitMax, 152 / tiles, rows / 256}));
-    const int kc = std::max((rows + np - 1) / np + 31, 32) / 32 * 32;
-    np = (rows + kc - 1) / kc;
+    const int nb = f.count;
+    const auto [np, kc] = panel_cut(rows, cols);
     const long long zs = (long long)nb * cols;
     cudaError_t e;
     SplitSet set{w, st};
@@ -1209,7 +1220,9 @@ bool use_wide(int refl, int rows, int other) {
 }
 // a QR panel's trailing update on the split products: from about 300 x 300
 bool panel_split(int rows, int cols, const SplitWs &w) {
-    return (long long)rows * cols >= 100 * 1000 && cols <= kSplitMostRows && rows <= kSplitMax * (kSplitMostK - 64) &&
+    if ((long long)rows * cols < 100 * 1000 || cols > kSplitMostRows || rows > kSplitMax * (kSplitMostK - 64)) return false;
+    const auto [np, kc] = panel_cut(rows, cols);
+    return np <= kSplitMax && kc <= kSplitMostK && split_scratch(32, cols, kc, (cols + 127) / 128) <= w.slice_bytes &&
            (size_t)cols * 32 * kSplitMax <= w.zcap &&
            split_scratch((long long)kSplitMax * 32, (long long)kSplitMax * cols, (rows + kSplitMax - 1) / kSplitMax + 64,
                          (long long)kSplitMax * ((cols + 127) / 128)) <= w.slice_bytes &&
