@@ -211,6 +211,9 @@ __device__ __forceinline__ int scale_exp(unsigned long long maxbits) {
     return ef - 1023 + 2;
 }
 
+// above every exponent of a finite product, twice over and with room in an int
+constexpr int kNotFinite = 1 << 20;
+
 // balanced base-256 digits of round(x 2^(8S - E)): slices n_1..n_S, |n_s| <= 128
 template <int S>
 __device__ __forceinline__ void digits(double x, int E, int (&n)[S]) {
@@ -824,7 +827,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                         for (int i = 0; i < 8; ++i) {
                             const int k = 8 * cb + i;
                             if (rowok && c0 + k < pr.N) {
-                                const double v = i64_ldexp((long long)(L[k] - corr), Er + F[i] - 40);
+                                double v = i64_ldexp((long long)(L[k] - corr), Er + F[i] - 40);
+                                if (MODE == MODE_EW && Er + F[i] > kNotFinite / 2) v = __longlong_as_double(0x7ff8000000000000ll);
                                 if constexpr (MODE == MODE_EW) pr.C[cj[i] * ldc + row] = mx.sub ? cold[i] - v : v;
                                 else pr.C[cj[i] * ldc + row] = v;
                             }
@@ -1270,6 +1274,12 @@ __device__ __forceinline__ double split_at(const SplitSide &s, int v, int k) {
     if (s.add) x += s.add[v * s.add_v + k * s.add_k];
     return x;
 }
+// exponent of a vector of a dense product: a vector that holds a NaN or an
+// infinity takes kNotFinite, which leaves it no digits and makes every result
+// that it enters NaN (MODE_EW)
+__device__ __forceinline__ int split_exp(unsigned long long maxbits) {
+    return maxbits >= 0x7FF0000000000000ull ? kNotFinite : scale_exp(maxbits);
+}
 constexpr int kAlongRegs = 6;              // entry pairs a lane keeps in registers: K <= 384
 
 // vectors stored along K: a warp each, two neighbouring entries per lane (the
@@ -1288,7 +1298,7 @@ __global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ Spl
     unsigned long long m = 0;
     auto max_exp = [&] {
         for (int o = 16; o > 0; o >>= 1) m = max(m, (unsigned long long)__shfl_xor_sync(0xffffffffu, m, o));
-        const int E = scale_exp(m);
+        const int E = split_exp(m);
         if (lane == 0) (blockIdx.z ? Fb : Ea)[s.row0 + v] = E;
         return E;
     };
@@ -1373,7 +1383,7 @@ __global__ void __launch_bounds__(256) k_split_across(const __grid_constant__ Sp
     const int tr = threadIdx.x & 31, tc = threadIdx.x >> 5, v = blockIdx.x * 32 + tr;
     const int K = p.K, Kend = (K + TK - 1) / TK * TK, k0 = blockIdx.y * 64;
     if (!s.tr || blockIdx.x * 32 >= s.n || k0 >= Kend) return;
-    const int E = v < s.n ? scale_exp((side ? maxB : maxA)[s.row0 + v]) : 0;
+    const int E = v < s.n ? split_exp((side ? maxB : maxA)[s.row0 + v]) : 0;
     if (blockIdx.y == 0 && tc == 0 && v < s.n) (side ? Fb : Ea)[s.row0 + v] = E;
     double x[8];
 #pragma unroll
