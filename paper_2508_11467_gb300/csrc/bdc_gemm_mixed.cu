@@ -215,14 +215,16 @@ __device__ __forceinline__ int scale_exp(unsigned long long maxbits) {
 constexpr int kNotFinite = 1 << 20;
 
 // balanced base-256 digits of round(x 2^(8S - E)): slices n_1..n_S, |n_s| <= 128
-template <int S>
+// (SUB: subnormal x too; the merges' operands are unit vectors, whose
+// subnormal entries lie far below the digits)
+template <int S, bool SUB = false>
 __device__ __forceinline__ void digits(double x, int E, int (&n)[S]) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int ef = (int)((b >> 52) & 0x7FF);
     long long X = 0;
-    if (ef != 0) {
-        const long long mant = (long long)((b & 0xFFFFFFFFFFFFFull) | (1ull << 52));
-        const int shift = ef - 1075 - E + 8 * S;   // X = mant * 2^shift
+    if (SUB || ef != 0) {
+        const long long mant = (long long)((b & 0xFFFFFFFFFFFFFull) | ((!SUB || ef != 0) ? 1ull << 52 : 0ull));
+        const int shift = (SUB ? max(ef, 1) : ef) - 1075 - E + 8 * S;   // X = mant * 2^shift
         if (shift >= 0) X = mant << shift;
         else if (shift > -63) X = (mant + (1ll << (-shift - 1))) >> (-shift);
         if (b >> 63) X = -X;
@@ -258,11 +260,11 @@ __device__ __forceinline__ __nv_bfloat16 slice_bf16(int n, int s) {
 
 // the slices of x as BF16 patterns in the upper halves of w: the S digits at
 // scale 2^E, or (!EXACT) x rounded to BF16 and what is left of it in FP32
-template <int S, bool EXACT>
+template <int S, bool EXACT, bool SUB = false>
 __device__ __forceinline__ void slices(double x, int E, uint32_t (&w)[S]) {
     if (EXACT) {
         int n[S];
-        digits<S>(x, E, n);
+        digits<S, SUB>(x, E, n);
 #pragma unroll
         for (int s = 0; s < S; ++s) w[s] = slice_word(n[s], s);
     } else {
@@ -1304,8 +1306,8 @@ __global__ void __launch_bounds__(256) k_split_along(const __grid_constant__ Spl
     };
     auto put = [&](int k, int E, double x0, double x1) {
         uint32_t lo[DS], hi[DS];
-        slices<DS, true>(x0, E, lo);
-        slices<DS, true>(x1, E, hi);
+        slices<DS, true, true>(x0, E, lo);
+        slices<DS, true, true>(x1, E, hi);
 #pragma unroll
         for (int q = 0; q < DS; ++q)
             *reinterpret_cast<uint32_t *>(dst + (size_t)q * rows * Kld + k) = __byte_perm(lo[q], hi[q], 0x7632);
@@ -1394,7 +1396,7 @@ __global__ void __launch_bounds__(256) k_split_across(const __grid_constant__ Sp
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         int n[DS];
-        digits<DS>(x[q], E, n);
+        digits<DS, true>(x[q], E, n);
 #pragma unroll
         for (int z = 0; z < DS; ++z) tile[z][tr][tc + 8 * q] = slice_bf16(n[z], z);
     }
