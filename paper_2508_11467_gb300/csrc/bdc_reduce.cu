@@ -74,9 +74,10 @@ __device__ __forceinline__ bool grid_wait(GridBar *gb, unsigned target) {
 // takes 64 cycles here: 17 of them instead of the about 40 of a library
 // square root and two divisions (a step at n = 64: 2 x 2300 -> 2 x 1450 cycles
 // in this part).  With y the hardware estimate of 1 / sqrt(s) and r = 1 - s
-// y^2 (at most 2^-19.0 measured over [1, 4)), the series sqrt(s) = s y (1 -
-// r)^(-1/2) = s y (1 + r/2 + 3 r^2/8 + 5 r^3/16 ...) leaves 2^-58 and a residual
-// step the rounding of the last bit; the quotients are quot()'s.  Outside 2^-900..2^900 the library calls.
+// y^2 (at most 2^-19.0 measured over [1, 4)), the binomial series sqrt(s) = s y
+// (1 - r)^(-1/2) = s y (1 + r/2 + 3 r^2/8 + 5 r^3/16 ...) leaves 2^-58 and a
+// Newton step on nrm^2 = s the rounding of the last bit; the quotients are
+// quot()'s (geometric series).  Outside 2^-900..2^900 the library calls.
 __device__ __forceinline__ double reflector_fast(double alpha, double sig2, double &tau, double &beta) {
     if (__double_as_longlong(sig2) == 0) {
         tau = 0.0;
@@ -85,7 +86,8 @@ __device__ __forceinline__ double reflector_fast(double alpha, double sig2, doub
     }
     const double s = fma(alpha, alpha, sig2);
     const long long sb = __double_as_longlong(s);
-    const bool neg = __double_as_longlong(alpha) < 0;      // (alpha = -0 reflects to +||x||)
+    const bool neg = __double_as_longlong(alpha) > (long long)0x8000000000000000ull &&
+                     __double_as_longlong(alpha) < 0;       // (alpha = -0 counts as positive, as in k_geqr2)
     if (sb < (123ll << 52) || sb > (1923ll << 52)) {       // also NaN, infinity
         const double nrm = sqrt(s);
         beta = neg ? nrm : -nrm;
