@@ -1378,7 +1378,7 @@ __global__ void __launch_bounds__(256) k_split_across(const __grid_constant__ Sp
                                                       const unsigned long long *maxB, int *Ea, int *Fb, int rowsA,
                                                       int colsB, int Kld) {
     pdl_begin();
-    __shared__ __nv_bfloat16 tile[DS][32][72];
+    __shared__ __align__(16) __nv_bfloat16 tile[DS][32][72];   // read in 16-byte words
     const SplitProd &p = t.p[blockIdx.z >> 1];
     const int side = blockIdx.z & 1;
     const SplitSide s = side ? p.b : p.a;
