@@ -405,9 +405,14 @@ int bdc_mlp_train(const bdc_opts *o, const bdc_mlp_train_opts *t, float *params,
  * All matrices column-major FP64 device arrays owned by the caller; every
  * call is asynchronous on `stream` unless stated; workspaces are device
  * memory of the size the matching *_workspace function returns (any
- * alignment).  Reflectors use LAPACK's sign convention and storage: a
- * reflector I - tau y y^T maps x to beta e_1 with beta = -sign(x_1) ||x||,
- * y_1 = 1 implicit.  Panels are b = 32 columns (rows) wide.  The panel
+ * alignment): 2 KB a row and column for a reduction; for block reflectors
+ * (ormbr, geqrf / orgqr, gesvd) 10 KB a row and vector where they run in FP64
+ * (fewer than 64 reflectors or vectors, more than 131072 rows), else the
+ * reflectors once more and the slices of one product (14 bytes an entry of
+ * its operands; 14 bytes an entry of the trailing matrix for geqrf).
+ * Reflectors use LAPACK's sign convention and storage: a reflector I - tau y
+ * y^T maps x to beta e_1 with beta = -sign(x_1) ||x|| (a zero x_1 counts as
+ * positive), y_1 = 1 implicit.  Panels are b = 32 columns (rows) wide.  The panel
  * kernels are cooperative launches whose grid barriers wait at most 2 s; a
  * wait that gives up makes the call report BDC_ERR_TIMEOUT in *d_info.
  * Returns: 0, -i for an illegal argument i, BDC_ERR_CUDA. */

@@ -691,7 +691,9 @@ cudaError_t apply_block(int left, int trans, int rows, int cols, const double *Y
 // the panel through the slicing's mask), then per block Z = Y^T C (partial
 // products over K) and C -= V Z.
 constexpr int kWide = 256;
-constexpr int kGramMost = 9;     // partial products of one block's Y^T Y at most
+// partial products of a block's Y^T Y: rows of each, and how many (eight at most)
+int gram_chunk(int rows) { return std::max(512, ((rows + 7) / 8 + 31) / 32 * 32); }
+int gram_chunks(int rows) { return (rows + gram_chunk(rows) - 1) / gram_chunk(rows); }
 
 // G = Y^T Y above the diagonal from the partial products of Y without its unit
 // entries (symmetric): entry (r, c), r < c, adds reflector r's row c times
@@ -838,8 +840,7 @@ cudaError_t form_v(const WideJob *jobs, int njobs, cudaStream_t st) {
         const SplitWs &w = jobs[q].w;
         const int blocks = jobs[q].blocks();
         // (a block below the first has as many chunks or fewer)
-        const int chunk = std::max(512, ((f.rows + 7) / 8 + 31) / 32 * 32);
-        const int chunks = (f.rows + chunk - 1) / chunk;
+        const int chunk = gram_chunk(f.rows), chunks = gram_chunks(f.rows);
         for (int j = 0; j < blocks; ++j) {
             const int i0 = j * kWide, nb = std::min(kWide, f.count - i0), rows = f.rows - i0;
             for (int y = 0, k0 = 0; k0 < rows; ++y, k0 += chunk) {
@@ -941,6 +942,15 @@ WideStep wide_step(int left, int rows, int other, int nb, const double *V, int l
     return WideStep{left, rows, nb, 1, 0, other, c, ldc, V, ldv, w.Z};
 }
 
+// products along K of a block applied alone: a wave of tiles or so
+void cut_alone(WideStep &x) { x.cut(std::min(kSplitMax, 152 / std::max(x.tiles(), 1))); }
+// slice scratch of the step's products and of its update
+size_t step_slices(const WideStep &x) {
+    const long long nt = (x.ns + 127) / 128, t = nt * ((x.rows + 127) / 128);
+    return std::max({split_scratch((long long)x.np * x.nb, (long long)x.np * x.ns, x.kc, (long long)x.np * x.tiles()),
+                     split_scratch(x.ns, x.rows, x.nb, t), split_scratch(x.rows, x.ns, x.nb, t)});
+}
+
 // one block, in slabs of the untouched dimension that fit the slice scratch and the Z parts
 template <typename YK>
 cudaError_t apply_wide(int left, int rows, int other, YK yk, int nb, const double *V, int ldv, double *C, int ldc,
@@ -949,16 +959,12 @@ cudaError_t apply_wide(int left, int rows, int other, YK yk, int nb, const doubl
     int slab = other < kSplitMostRows ? (other + 127) / 128 * 128 : kSplitMostRows;
     auto step_of = [&](int s) {
         WideStep x = wide_step(left, rows, s, nb, V, ldv, C, ldc, w);
-        x.cut(std::min(kSplitMax, 152 / std::max(x.tiles(), 1)));
+        cut_alone(x);
         return x;
     };
     for (; slab > 128; slab = (slab / 2 + 127) / 128 * 128) {
         const WideStep x = step_of(slab);
-        const long long t = x.tiles();
-        if ((size_t)x.np * nb * slab <= w.zcap &&
-            split_scratch((long long)x.np * nb, (long long)x.np * slab, x.kc, x.np * t) <= w.slice_bytes &&
-            split_scratch(slab, rows, nb, (long long)(slab / 128) * ((rows + 127) / 128)) <= w.slice_bytes &&
-            split_scratch(rows, slab, nb, (long long)(slab / 128) * ((rows + 127) / 128)) <= w.slice_bytes)
+        if ((size_t)x.np * nb * slab <= w.zcap && step_slices(x) <= w.slice_bytes)
             break;
     }
     SplitSet set{w, st};
@@ -1126,69 +1132,209 @@ constexpr int kDenseBlock = 32;   // b: columns / rows per panel (reflectors per
 // Q) in FP64: wider blocks pass over C fewer times (Z = Y^T C and C -= Y W
 // with K = kApplyBlock)
 constexpr int kApplyBlock = kTB;
-constexpr int kWsBlock = kApplyBlock > kDenseBlock ? kApplyBlock : kDenseBlock;   // workspace sizing
+static_assert(kDenseBlock <= 32 && kDenseBlock <= kTB, "k_geqr2: a lane per later panel column; T of a panel");
 
-constexpr size_t kPairMost = 2048;   // largest dimension of back-transformations done side by side
+constexpr int kPairMost = 2048;   // largest dimension of back-transformations done side by side
 
-// workspace layout of the dense routines (bytes from an aligned base)
+// Blocks of kWide reflectors on the split products, or of kTB in FP64: the
+// split path's fixed cost (about 50 launches) is below one FP64 block's three
+// products from 64 reflectors on (100 x 100: 0.4 ms either way; 333 x 333:
+// 0.64 against 1.39 ms; 600 x 600: 0.88 against 2.3 ms)
+bool use_wide(int refl, int rows, int other) {
+    return refl >= 64 && other >= 64 && rows <= 8 * kSplitMostK;   // (gram_chunk)
+}
+// ---- workspaces: every routine lays out what it can reach at its shape
+// (bytes from an aligned base; the barrier and error word come first in all)
 struct DenseWs {
-    size_t bar, PW, QW, part, Y, Ti, Z, split, split_doubles, res, lab, total;
-    size_t wG, wT, wX, wV, wZ, wZcap, wS, wSbytes;   // split path
-    size_t pG, pT, pX, pV, pZ;                       // ... of a second job (order up to kPairMost)
+    size_t bar = 0, total = 256;
+    size_t PW = 0, QW = 0, lab = 0, res = 0;                             // reduction
+    size_t part = 0, Y = 0, Ti = 0, Z = 0, split = 0, split_doubles = 0; // QR panels, block reflectors in FP64
+    size_t wG[kPair] = {}, wT[kPair] = {}, wX[kPair] = {}, wV[kPair] = {}, wZ[kPair] = {}, wZcap = 0;   // per job
+    size_t wS = 0, wSbytes = 0;                                          // slices
+    size_t add(size_t bytes) {
+        const size_t at = total;
+        total += al256(bytes);
+        return at;
+    }
+    size_t doubles(size_t n) { return add(sizeof(double) * n); }
+    // partial products and sums of the FP64 block reflectors: 16 parts of kTB
+    // vectors of `len` (bound by the FP64 pipe: no more are of use)
+    void fp64(size_t rows, size_t refl, size_t other) {
+        const size_t len = std::max({rows, refl, other});
+        Y = doubles(rows * kTB);
+        Ti = doubles((size_t)kTB * (refl + kTB));
+        Z = doubles((size_t)kTB * other);
+        split_doubles = std::max<size_t>((size_t)16 * kTB * len, (size_t)16 * kTB * kTB);
+        split = doubles(split_doubles);
+    }
+    void slices(size_t bytes) {
+        wSbytes = std::max(wSbytes, bytes);
+        wS = add(bytes);
+    }
 };
 
-DenseWs dense_ws(int m, int n, int b, int zcols) {
-    DenseWs w{};
-    size_t o = 0;
-    const int grid = 4 * 256;   // upper bound of the cooperative grid (partial arrays)
-    w.bar = o; o += 256;
-    w.PW = o; o += al256(sizeof(double) * 2 * (size_t)b * m);
-    w.QW = o; o += al256(sizeof(double) * 2 * (size_t)b * n);
-    w.part = o; o += al256(sizeof(double) * (size_t)grid * (b + 1));
-    w.Y = o; o += al256(sizeof(double) * (size_t)std::max(m, n) * std::max(b, kWide));
-    w.Ti = o; o += al256(sizeof(double) * (size_t)kTB * (std::max(m, n) + kTB));   // T of every block
-    w.Z = o; o += al256(sizeof(double) * (size_t)b * std::max(std::max(m, n), zcols));
-    w.split_doubles = std::max<size_t>((size_t)16 * b * std::max(std::max(m, n), zcols), (size_t)16 * kTB * kTB);
-    w.split = o; o += al256(sizeof(double) * w.split_doubles);
-    w.lab = o; o += al256(sizeof(double) * labrd_scratch_doubles(m, n));
-    w.res = o; o += al256(sizeof(double) * resident_scratch_doubles(n));
-    // split path: every block's G, T, X; V and the partial Y^T Y; parts of Z; slices
-    {
-        const size_t D = std::max(std::max(m, n), zcols), blocks = (n + kWide - 1) / kWide, w2 = (size_t)kWide * kWide;
-        w.wG = o; o += al256(sizeof(double) * blocks * w2);
-        w.wT = o; o += al256(sizeof(double) * blocks * w2);
-        w.wX = o; o += al256(sizeof(double) * blocks * w2);
-        w.wV = o; o += al256(sizeof(double) * std::max(D * n, blocks * kGramMost * w2));
-        w.wZcap = std::max<size_t>((size_t)kWide * 2 * (D + 256), (size_t)kWide * 4096);
-        w.wZ = o; o += al256(sizeof(double) * w.wZcap);
-        if (D <= kPairMost) {
-            w.pG = o; o += al256(sizeof(double) * blocks * w2);
-            w.pT = o; o += al256(sizeof(double) * blocks * w2);
-            w.pX = o; o += al256(sizeof(double) * blocks * w2);
-            w.pV = o; o += al256(sizeof(double) * std::max(D * n, blocks * kGramMost * w2));
-            w.pZ = o; o += al256(sizeof(double) * w.wZcap);
-        }
-        // enough for whole products up to about 340 MB, then slabs of 128
-        const size_t Dp = (D + 31) / 32 * 32 + 32;
-        const size_t all = 2 * (D + 2 * kWide + 256) * std::max<size_t>(Dp, 544);
-        const size_t most = std::max<size_t>((size_t)24 << 20, (size_t)(2 * kWide + 512) * Dp);
-        w.wSbytes = 14 * std::min(all, most) + (size_t)64 * (D + 4096) + ((size_t)1 << 20);
-        w.wS = o; o += al256(w.wSbytes);
-    }
-    w.total = o + 256;
+// Slices held at most, in bytes: whole products of up to 24 M entries (340 MB),
+// or of 1024 vectors as long as the longest (`len`); above that products go in
+// slabs or sets, or in FP64
+size_t slice_cap(size_t len) {
+    const size_t lp = (len + 31) / 32 * 32 + 32;
+    return 14 * std::max<size_t>((size_t)24 << 20, (size_t)(2 * kWide + 512) * lp) + (size_t)64 * (len + 4096) +
+           ((size_t)1 << 20);
+}
+
+DenseWs ws_gebrd(int m, int n) {
+    DenseWs w;
+    constexpr int b = kDenseBlock;
+    w.PW = w.doubles(2 * (size_t)b * m);
+    w.QW = w.doubles(2 * (size_t)b * n);
+    w.lab = w.doubles(labrd_scratch_doubles(m, n));
+    w.res = w.doubles(resident_scratch_doubles(n));
+    const long long tr = m - b, tc = n - b;
+    if (tc > 0 && tr <= kSplitMostRows) w.slices(split_scratch(2 * tr, 2 * tc, b, ((tr + 127) / 128) * ((tc + 127) / 128)));
     return w;
 }
 
-SplitWs split_ws(char *ws, const DenseWs &w) {
-    return SplitWs{(double *)(ws + w.wG), (double *)(ws + w.wT), (double *)(ws + w.wX), (double *)(ws + w.wV),
-                   (double *)(ws + w.wZ), w.wZcap, ws + w.wS, w.wSbytes, &((GridBar *)(ws + w.bar))->err};
+// a QR panel's trailing update on the split products: from about 300 x 300,
+// while its slices and Z parts stay below the caps of the m x n matrix
+size_t panel_slices(int rows, int cols, const PanelCut &c) {
+    const long long tn = (cols + 127) / 128;
+    return std::max(split_scratch((long long)c.np * 32, (long long)c.np * cols, c.kc, c.np * tn),
+                    split_scratch(rows, cols, 32, (long long)((rows + 127) / 128) * tn));
+}
+bool panel_split(int rows, int cols, size_t len) {
+    if ((long long)rows * cols < 100 * 1000 || cols > kSplitMostRows || rows > kSplitMax * (kSplitMostK - 64)) return false;
+    const PanelCut c = panel_cut(rows, cols);
+    return c.np <= kSplitMax && c.kc <= kSplitMostK &&
+           (size_t)cols * 32 * kSplitMax <= std::max<size_t>((size_t)2 * kWide * (len + 256), (size_t)kWide * 4096) &&
+           panel_slices(rows, cols, c) <= slice_cap(len);
 }
 
-SplitWs split_ws2(char *ws, const DenseWs &w) {
-    SplitWs s = split_ws(ws, w);
-    s.G = (double *)(ws + w.pG); s.T = (double *)(ws + w.pT); s.X = (double *)(ws + w.pX);
-    s.V = (double *)(ws + w.pV); s.Z = (double *)(ws + w.pZ);
-    return s;
+DenseWs ws_geqrf(int m, int n) {
+    DenseWs w;
+    constexpr int b = kDenseBlock;
+    const size_t len = std::max(m, n);
+    w.part = w.doubles((size_t)4 * 256 * (b + 1));   // k_geqr2's partial sums (its grid is at most this)
+    w.res = w.doubles(resident_scratch_doubles(kQp));
+    w.Ti = w.doubles((size_t)2 * kTB * kTB);         // T, Y^T Y of a panel
+    w.Z = w.doubles((size_t)b * n);
+    size_t y = 0, parts = 0, slices = 0;
+    for (int i0 = 0; i0 < std::min(m, n); i0 += b) {
+        const int ml = m - i0, nb = std::min(b, std::min(m, n) - i0), cols = n - i0 - nb;
+        if (cols == 0) break;
+        // Y^T Y of a panel that is too long for the chip: up to four CTAs an SM
+        parts = std::max(parts, (size_t)kTB * kTB * std::min((ml + 255) / 256, 4 * sm_count_dense()));
+        if (panel_split(ml, cols, len)) {
+            const PanelCut c = panel_cut(ml, cols);
+            slices = std::max(slices, panel_slices(ml, cols, c));
+            w.wZcap = std::max(w.wZcap, (size_t)c.np * nb * cols);
+        } else {
+            y = std::max(y, (size_t)ml * nb);
+            parts = std::max(parts, (size_t)nb * cols * std::max(1, std::min(64, ml / 64)));
+        }
+    }
+    w.Y = w.doubles(y);
+    w.split_doubles = std::max((size_t)16 * kTB * kTB, parts);
+    w.split = w.doubles(w.split_doubles);
+    w.wZ[0] = w.doubles(w.wZcap);
+    w.slices(slices);
+    return w;
+}
+
+// the split path of one job, or of two side by side
+struct WideShape {
+    int left, rows, count, other;   // reflectors of `rows` entries on `other` vectors
+    int shrinks;                    // 1: block b leaves out the first b kWide vectors
+};
+void ws_wide(DenseWs &w, const WideShape *jobs, int njobs) {
+    const size_t w2 = (size_t)kWide * kWide;
+    size_t need = 0, cap = 0, zneed = 0, zmost = 0;
+    long long gram = 0, vrows = 0, vcols = 0, vtiles = 0;
+    int chunk = 0;
+    for (int q = 0; q < njobs; ++q) {
+        const WideShape &j = jobs[q];
+        const int blocks = (j.count + kWide - 1) / kWide;
+        w.wG[q] = w.doubles(blocks * w2);
+        w.wT[q] = w.doubles(blocks * w2);
+        w.wX[q] = w.doubles(blocks * w2);
+        w.wV[q] = w.doubles(std::max((size_t)j.rows * j.count, (size_t)blocks * gram_chunks(j.rows) * w2));   // V, before it Y^T Y's parts
+        gram += (long long)blocks * gram_chunks(j.rows);
+        chunk = std::max(chunk, gram_chunk(j.rows));
+        size_t step = 0;
+        for (int b = 0; b < blocks; ++b) {
+            const int nb = std::min(kWide, j.count - b * kWide), rows = j.rows - b * kWide;
+            const int ns = j.other - (j.shrinks ? b * kWide : 0);
+            WideStep x{j.left, rows, nb, 1, 0, ns < kSplitMostRows ? (ns + 127) / 128 * 128 : kSplitMostRows, nullptr, 0, nullptr, 0, nullptr};
+            cut_alone(x);
+            zneed = std::max(zneed, (size_t)x.np * nb * x.ns);
+            for (int np = x.np; np >= 1; --np) {   // (two jobs share the SMs: fewer, longer products)
+                step = std::max(step, step_slices(x));
+                if (njobs == 1) break;
+                x.cut(np - 1);
+            }
+            vrows += rows;
+            vcols += nb;
+            vtiles += (long long)((rows + 127) / 128) * ((nb + 127) / 128);
+        }
+        need += step;
+        const size_t len = std::max(j.rows, std::min(j.other, 1 << 16));
+        cap = std::max(cap, slice_cap(len));
+        zmost = std::max<size_t>({zmost, (size_t)2 * kWide * (len + 256), (size_t)kWide * 4096});
+    }
+    gram = std::min<long long>(gram, kSplitMax);
+    need = std::max({need, split_scratch(gram * kWide, gram * kWide, chunk, gram * (kWide / 128) * (kWide / 128)),
+                     split_scratch(vrows, vcols, kWide, vtiles)});
+    w.wZcap = need <= cap && zneed <= zmost ? zneed : zmost;   // whole steps, or slabs of them
+    for (int q = 0; q < njobs; ++q) w.wZ[q] = w.doubles(w.wZcap);
+    w.slices(std::min(need, cap));
+}
+
+DenseWs ws_orgqr(int m, int n) {
+    DenseWs w;
+    if (use_wide(n, m, n)) {
+        w.Y = w.doubles((size_t)m * kWide);
+        const WideShape j{1, m, n, n, 1};
+        ws_wide(w, &j, 1);
+    } else {
+        w.fp64(m, n, n);
+    }
+    return w;
+}
+
+DenseWs ws_ormbr(int vect, int m, int n, int cdim) {
+    DenseWs w;
+    const int refl = vect == 0 ? n : n - 1, rows = vect == 0 ? m : n - 1;
+    if (use_wide(refl, rows, cdim)) {
+        const WideShape j{vect == 0, rows, refl, cdim, 0};
+        ws_wide(w, &j, 1);
+    } else {
+        w.fp64(rows, std::max(refl, 0), cdim);
+    }
+    return w;
+}
+
+// U and V^T of an m x n SVD
+bool both_at_once(int m, int n) { return std::max(m, n) <= kPairMost && use_wide(n - 1, m, n); }
+DenseWs ws_both(int m, int n) {
+    DenseWs w;
+    const WideShape j[kPair] = {{1, m, n, n, 0}, {0, n - 1, n - 1, n, 0}};
+    ws_wide(w, j, kPair);
+    return w;
+}
+
+// slices of an m x n by n x n product
+DenseWs ws_product(int m, int n) {
+    DenseWs w;
+    const int rows = std::min(m, kSplitMostRows);
+    if (n >= 64 && n <= kSplitMostK)
+        w.slices(std::min(slice_cap(std::min(m, 1 << 17)),
+                          split_scratch(rows, n, n, (long long)((rows + 127) / 128) * ((n + 127) / 128))));
+    return w;
+}
+
+SplitWs split_ws(char *ws, const DenseWs &w, int job = 0) {
+    return SplitWs{(double *)(ws + w.wG[job]), (double *)(ws + w.wT[job]), (double *)(ws + w.wX[job]),
+                   (double *)(ws + w.wV[job]), (double *)(ws + w.wZ[job]), w.wZcap, ws + w.wS, w.wSbytes,
+                   &((GridBar *)(ws + w.bar))->err};
 }
 
 // the split-K scratch of the calling thread's dense routine
@@ -1211,30 +1357,12 @@ cudaError_t launch_coop(const void *fn, int grid, void *args, cudaStream_t st) {
 }  // namespace
 
 // ---------------------------------------------------------------- drivers
-// Blocks of kWide reflectors on the split products, or of kTB in FP64: the
-// split path's fixed cost (about 50 launches) is below one FP64 block's three
-// products from 64 reflectors on (100 x 100: 0.4 ms either way; 333 x 333:
-// 0.64 against 1.39 ms; 600 x 600: 0.88 against 2.3 ms)
-bool use_wide(int refl, int rows, int other) {
-    return refl >= 64 && other >= 64 && rows <= 8 * kSplitMostK;   // Y^T Y in at most kGramMost parts
-}
-// a QR panel's trailing update on the split products: from about 300 x 300
-bool panel_split(int rows, int cols, const SplitWs &w) {
-    if ((long long)rows * cols < 100 * 1000 || cols > kSplitMostRows || rows > kSplitMax * (kSplitMostK - 64)) return false;
-    const auto [np, kc] = panel_cut(rows, cols);
-    return np <= kSplitMax && kc <= kSplitMostK && split_scratch(32, cols, kc, (cols + 127) / 128) <= w.slice_bytes &&
-           (size_t)cols * 32 * kSplitMax <= w.zcap &&
-           split_scratch((long long)kSplitMax * 32, (long long)kSplitMax * cols, (rows + kSplitMax - 1) / kSplitMax + 64,
-                         (long long)kSplitMax * ((cols + 127) / 128)) <= w.slice_bytes &&
-           split_scratch(rows, cols, 32, (long long)((rows + 127) / 128) * ((cols + 127) / 128)) <= w.slice_bytes;
-}
-
 // Bidiagonalization, Algorithm 1 (m >= n): on chip once it fits; before that,
 // per panel of b, k_labrd_panel, then the merged rank-(2b) update of the trailing matrix.
-cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup, int b,
+cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup,
                         char *ws, cudaStream_t st) {
-    const DenseWs w = dense_ws(m, n, b, n);
-    SplitScope split_scope(ws, w);
+    const DenseWs w = ws_gebrd(m, n);
+    constexpr int b = kDenseBlock;
     GridBar *bar = (GridBar *)(ws + w.bar);
     cudaError_t err = cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st);   // the counters (not the error word)
     if (err != cudaSuccess) return err;
@@ -1285,9 +1413,9 @@ cudaError_t dense_gebrd(int m, int n, double *A, int lda, double *d, double *e, 
 
 // QR (Sec. 4.3): per panel, k_geqr2 and the update of the trailing columns by
 // H^T = I - Y T^T Y^T in modified compact WY
-cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, char *ws, cudaStream_t st) {
-    if (b < 1 || b > 32) return cudaErrorInvalidValue;   // k_geqr2: a lane per later panel column
-    const DenseWs w = dense_ws(m, n, b, n);
+cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, char *ws, cudaStream_t st) {
+    const DenseWs w = ws_geqrf(m, n);
+    constexpr int b = kDenseBlock;
     SplitScope split_scope(ws, w);
     GridBar *bar = (GridBar *)(ws + w.bar);
     cudaError_t err = cudaMemsetAsync(bar, 0, 3 * sizeof(unsigned), st);   // the counters (not the error word)
@@ -1315,7 +1443,7 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
             err = resident ? launch_tform(&tf, 1, 1, st)
                            : form_t(f, tau + i0, Ti, st);
             if (err != cudaSuccess) return err;
-            if (panel_split(ml, cols, sw)) {
+            if (panel_split(ml, cols, std::max(m, n))) {
                 if ((err = apply_panel(f, Ti, ml, cols, A + i0 + (size_t)(i0 + nb) * lda, lda, Z, sw, st)) !=
                     cudaSuccess)
                     return err;
@@ -1332,23 +1460,16 @@ cudaError_t dense_geqrf(int m, int n, double *A, int lda, double *tau, int b, ch
     return cudaSuccess;
 }
 
-// the first n columns of Q = H_1 ... H_k in place of A (Eq. orgqr-q): the
+// the n columns of Q = H_1 ... H_n in place of A (Eq. orgqr-q): the
 // panels from the last to the first, each panel's reflectors copied to Y
 // before its columns are reset to the identity's
-cudaError_t dense_orgqr(int m, int n, int k, double *A, int lda, const double *tau, int b, char *ws, cudaStream_t st) {
-    const DenseWs w = dense_ws(m, n, b, n);
+cudaError_t dense_orgqr(int m, int n, double *A, int lda, const double *tau, char *ws, cudaStream_t st) {
+    const DenseWs w = ws_orgqr(m, n);
+    constexpr int b = kApplyBlock;
+    const int k = n;
     SplitScope split_scope(ws, w);
     double *Y = (double *)(ws + w.Y), *Ti = (double *)(ws + w.Ti), *Z = (double *)(ws + w.Z);
     cudaError_t err = cudaSuccess;
-    // columns k..n-1 start as identity columns
-    if (k < n) {
-        const long long cnt = (long long)m * (n - k);
-        k_fill<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(A + (size_t)k * lda, m, n - k, lda, 0.0);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        const long long c2 = (long long)(m - k) * (n - k);
-        k_fill<<<(unsigned)((c2 + 255) / 256), 256, 0, st>>>(A + k + (size_t)k * lda, m - k, n - k, lda, 1.0);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    }
     if (use_wide(k, m, n)) {
         const SplitWs sw = split_ws(ws, w);
         const Reflectors f{A, 1, lda, m, k};
@@ -1392,8 +1513,9 @@ cudaError_t dense_orgqr(int m, int n, int k, double *A, int lda, const double *t
 // column reflectors of gebrd (A m x n, tauq); vect 1: C (rows x n) := C P1^T
 // with the row reflectors (taup).  Panels from the last to the first.
 cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const double *tau, double *C, int ldc,
-                        int cdim, int b, char *ws, cudaStream_t st) {
-    const DenseWs w = dense_ws(m, n, b, std::max(cdim, n));
+                        int cdim, char *ws, cudaStream_t st) {
+    const DenseWs w = ws_ormbr(vect, m, n, cdim);
+    constexpr int b = kApplyBlock;
     SplitScope split_scope(ws, w);
     double *Y = (double *)(ws + w.Y), *Ti = (double *)(ws + w.Ti), *Z = (double *)(ws + w.Z);
     cudaError_t err = cudaSuccess;
@@ -1435,29 +1557,38 @@ cudaError_t dense_ormbr(int vect, int m, int n, const double *A, int lda, const 
 
 // U := Q1 U (m x n) and VT := VT P1^T (n x n) with the reflectors of gebrd
 cudaError_t dense_ormbr_both(int m, int n, const double *A, int lda, const double *tauq, const double *taup, double *U,
-                             int ldu, double *VT, int ldvt, int b, char *ws, cudaStream_t st) {
-    const DenseWs w = dense_ws(m, n, b, n);
-    if ((size_t)std::max(m, n) <= kPairMost && use_wide(n - 1, m, n)) {
+                             int ldu, double *VT, int ldvt, char *ws, cudaStream_t st) {
+    if (both_at_once(m, n)) {
+        const DenseWs w = ws_both(m, n);
         const WideJob j[kPair] = {{{A, 1, lda, m, n}, tauq, 1, n, U, ldu, split_ws(ws, w)},
-                                  {{A + lda, lda, 1, n - 1, n - 1}, taup, 0, n, VT + ldvt, ldvt, split_ws2(ws, w)}};
+                                  {{A + lda, lda, 1, n - 1, n - 1}, taup, 0, n, VT + ldvt, ldvt, split_ws(ws, w, 1)}};
         return apply_pair(j, st);
     }
-    if (cudaError_t e = dense_ormbr(0, m, n, A, lda, tauq, U, ldu, n, b, ws, st)) return e;
-    return dense_ormbr(1, m, n, A, lda, taup, VT, ldvt, n, b, ws, st);
+    if (cudaError_t e = dense_ormbr(0, m, n, A, lda, tauq, U, ldu, n, ws, st)) return e;
+    return dense_ormbr(1, m, n, A, lda, taup, VT, ldvt, n, ws, st);
 }
 
-size_t dense_ws_bytes(int m, int n, int b) { return dense_ws(m, n, b, std::max(m, n)).total; }
+size_t gebrd_bytes(int m, int n) { return ws_gebrd(m, n).total; }
+size_t geqrf_bytes(int m, int n) { return std::max(ws_geqrf(m, n).total, n <= m ? ws_orgqr(m, n).total : 0); }
+size_t ormbr_bytes(int m, int n, int cdim) {
+    return std::max(ws_ormbr(0, m, n, cdim).total, ws_ormbr(1, m, n, cdim).total);
+}
+size_t gesvd_bytes(int m, int n, bool qr) {
+    const int r = qr ? n : m;   // rows of the reduction
+    const size_t reduce = std::max(gebrd_bytes(r, n), both_at_once(r, n) ? ws_both(r, n).total : ormbr_bytes(r, n, n));
+    return qr ? std::max({reduce, geqrf_bytes(m, n), ws_product(m, n).total}) : reduce;
+}
 // (a kernel, not a memset: overlapped launches may follow it directly)
 cudaError_t dense_clear_err(char *ws, cudaStream_t st) {
-    k_clear_bar<<<1, 1, 0, st>>>((GridBar *)(ws + dense_ws(1, 1, 1, 1).bar));
+    k_clear_bar<<<1, 1, 0, st>>>((GridBar *)(ws + DenseWs().bar));
     return cudaGetLastError();
 }
 cudaError_t dense_read_err(char *ws, int *info, cudaStream_t st) {
-    k_read_err<<<1, 1, 0, st>>>((const GridBar *)(ws + dense_ws(1, 1, 1, 1).bar), info);
+    k_read_err<<<1, 1, 0, st>>>((const GridBar *)(ws + DenseWs().bar), info);
     return cudaGetLastError();
 }
 cudaError_t dense_poison(char *ws, double *C, int rows, int cols, int ld, cudaStream_t st) {
-    k_poison<<<1, 1024, 0, st>>>(&((const GridBar *)(ws + dense_ws(1, 1, 1, 1).bar))->err, C, rows, cols, ld);
+    k_poison<<<1, 1024, 0, st>>>(&((const GridBar *)(ws + DenseWs().bar))->err, C, rows, cols, ld);
     return cudaGetLastError();
 }
 cudaError_t dense_copy_upper(const double *A, int lda, double *R, int ldr, int n, cudaStream_t st) {
@@ -1474,7 +1605,7 @@ cudaError_t dense_zero_rows(double *X, int ld, int r0, int r1, int cols, cudaStr
 // C (m x n) = A (m x n, lda) B (n x n, ld n), in row slabs that fit the slices
 cudaError_t dense_product(int m, int n, const double *A, int lda, const double *B, double *C, int ldc, char *ws,
                           cudaStream_t st) {
-    const DenseWs w = dense_ws(m, n, kWsBlock, std::max(m, n));
+    const DenseWs w = ws_product(m, n);
     const SplitWs sw = split_ws(ws, w);
     auto fits = [&](int r) {
         return split_scratch(r, n, n, (long long)((r + 127) / 128) * ((n + 127) / 128)) <= sw.slice_bytes;
@@ -1515,7 +1646,7 @@ GesvdWs gesvd_layout(int m, int n, const bdc_opts *o) {
     GesvdWs w{};
     size_t off = 0;
     const bool qr = m >= kQrRatio * n;
-    w.dense = off; off += al256(std::max(dense_ws_bytes(m, n, kWsBlock), qr ? dense_ws_bytes(n, n, kWsBlock) : 0));
+    w.dense = off; off += al256(gesvd_bytes(m, n, qr));
     w.vecs = off; off += al256(sizeof(double) * 4 * (size_t)n + 64);
     w.R = off; off += qr ? al256(sizeof(double) * (size_t)n * n) : 0;
     w.UR = off; off += qr ? al256(sizeof(double) * (size_t)n * n) : 0;
@@ -1530,7 +1661,7 @@ extern "C" {
 
 size_t bdc_gebrd_workspace(int m, int n) {
     if (m < n || n < 0) return 0;
-    return dense_ws_bytes(m, n, kWsBlock) + 512;
+    return gebrd_bytes(m, n) + 512;
 }
 
 int bdc_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *tauq, double *taup, void *work,
@@ -1550,7 +1681,7 @@ int bdc_gebrd(int m, int n, double *A, int lda, double *d, double *e, double *ta
     char *ws = align_ws(work);
     if (int r = note_cuda(dense_clear_err(ws, st))) return r;
     if (int r = note_cuda(cudaMemsetAsync(taup, 0, sizeof(double) * n, st))) return r;
-    if (int r = note_cuda(dense_gebrd(m, n, A, lda, d, e, tauq, taup, kDenseBlock, ws, st))) return r;
+    if (int r = note_cuda(dense_gebrd(m, n, A, lda, d, e, tauq, taup, ws, st))) return r;
     return note_cuda(dense_read_err(ws, d_info, st));
 }
 
@@ -1566,24 +1697,23 @@ int bdc_ormbr(int vect, int m, int n, const double *A, int lda, const double *ta
     if (ldc < std::max(1, vect == 0 ? m : cdim)) return -8;
     if (n == 0 || cdim == 0) return 0;
     if (!work) return -10;
-    const size_t need = dense_ws_bytes(std::max(m, cdim), std::max(n, cdim), kWsBlock) + 512;
-    if (lwork < need) return -11;
+    if (lwork < bdc_ormbr_workspace(m, n, cdim)) return -11;
     cudaStream_t st = (cudaStream_t)stream;
     const OverlapScope overlapped(st);
     char *ws = align_ws(work);
     if (int r = note_cuda(dense_clear_err(ws, st))) return r;
-    if (int r = note_cuda(dense_ormbr(vect, m, n, A, lda, tau, C, ldc, cdim, kApplyBlock, ws, st))) return r;
+    if (int r = note_cuda(dense_ormbr(vect, m, n, A, lda, tau, C, ldc, cdim, ws, st))) return r;
     return note_cuda(dense_poison(ws, C, vect == 0 ? m : cdim, vect == 0 ? cdim : n, ldc, st));
 }
 
 size_t bdc_ormbr_workspace(int m, int n, int cdim) {
     if (m < n || n < 0 || cdim < 0) return 0;
-    return dense_ws_bytes(std::max(m, cdim), std::max(n, cdim), kWsBlock) + 512;
+    return ormbr_bytes(m, n, cdim) + 512;
 }
 
 size_t bdc_geqrf_workspace(int m, int n) {
     if (m < 0 || n < 0) return 0;
-    return dense_ws_bytes(std::max(m, 1), std::max(n, 1), kWsBlock) + 512;
+    return geqrf_bytes(std::max(m, 1), std::max(n, 1)) + 512;
 }
 
 int bdc_geqrf(int m, int n, double *A, int lda, double *tau, void *work, size_t lwork, int *d_info,
@@ -1602,7 +1732,7 @@ int bdc_geqrf(int m, int n, double *A, int lda, double *tau, void *work, size_t 
     if (lwork < bdc_geqrf_workspace(m, n)) return -7;
     char *ws = align_ws(work);
     if (int r = note_cuda(dense_clear_err(ws, st))) return r;
-    if (int r = note_cuda(dense_geqrf(m, n, A, lda, tau, kDenseBlock, ws, st))) return r;
+    if (int r = note_cuda(dense_geqrf(m, n, A, lda, tau, ws, st))) return r;
     return note_cuda(dense_read_err(ws, d_info, st));
 }
 
@@ -1619,7 +1749,7 @@ int bdc_orgqr(int m, int n, double *A, int lda, const double *tau, void *work, s
     const OverlapScope overlapped(st);
     char *ws = align_ws(work);
     if (int r = note_cuda(dense_clear_err(ws, st))) return r;
-    if (int r = note_cuda(dense_orgqr(m, n, n, A, lda, tau, kApplyBlock, ws, st))) return r;
+    if (int r = note_cuda(dense_orgqr(m, n, A, lda, tau, ws, st))) return r;
     return note_cuda(dense_poison(ws, A, m, n, lda, st));
 }
 
@@ -1649,7 +1779,6 @@ int bdc_gesvd(int m, int n, double *A, int lda, double *S, double *U, int ldu, d
     char *ws = align_ws(work);
     char *dws = ws + L.dense;
     double *d = (double *)(ws + L.vecs), *e = d + n, *tq = e + n, *tp = tq + n;
-    const int b = kDenseBlock;
     if (int r = note_cuda(dense_clear_err(dws, st))) return r;
     if (int r = note_cuda(cudaMemsetAsync(tp, 0, sizeof(double) * n, st))) return r;
     const size_t lwb = bdc_svd_workspace(n, o);
@@ -1657,19 +1786,19 @@ int bdc_gesvd(int m, int n, double *A, int lda, double *S, double *U, int ldu, d
     if (m >= kQrRatio * n) {
         // tall and skinny: A = Q R, the SVD of R, U = Q U_R (Sec. 4.3)
         double *R = (double *)(ws + L.R), *UR = (double *)(ws + L.UR);
-        if ((rc = note_cuda(dense_geqrf(m, n, A, lda, tq, b, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_geqrf(m, n, A, lda, tq, dws, st)))) return rc;
         if ((rc = note_cuda(dense_copy_upper(A, lda, R, n, n, st)))) return rc;
-        if ((rc = note_cuda(dense_orgqr(m, n, n, A, lda, tq, kApplyBlock, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_orgqr(m, n, A, lda, tq, dws, st)))) return rc;
         if ((rc = note_cuda(cudaMemsetAsync(tq, 0, sizeof(double) * n, st)))) return rc;
-        if ((rc = note_cuda(dense_gebrd(n, n, R, n, d, e, tq, tp, b, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_gebrd(n, n, R, n, d, e, tq, tp, dws, st)))) return rc;
         if ((rc = bdc_svd_ex(n, d, e, UR, S, VT, n, ldvt, o, ws + L.bdc, lwb, d_info, stream))) return rc;
-        if ((rc = note_cuda(dense_ormbr_both(n, n, R, n, tq, tp, UR, n, VT, ldvt, kApplyBlock, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_ormbr_both(n, n, R, n, tq, tp, UR, n, VT, ldvt, dws, st)))) return rc;
         if ((rc = note_cuda(dense_product(m, n, A, lda, UR, U, ldu, dws, st)))) return rc;
     } else {
-        if ((rc = note_cuda(dense_gebrd(m, n, A, lda, d, e, tq, tp, b, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_gebrd(m, n, A, lda, d, e, tq, tp, dws, st)))) return rc;
         if ((rc = bdc_svd_ex(n, d, e, U, S, VT, ldu, ldvt, o, ws + L.bdc, lwb, d_info, stream))) return rc;
         if ((rc = note_cuda(dense_zero_rows(U, ldu, n, m, n, st)))) return rc;
-        if ((rc = note_cuda(dense_ormbr_both(m, n, A, lda, tq, tp, U, ldu, VT, ldvt, kApplyBlock, dws, st)))) return rc;
+        if ((rc = note_cuda(dense_ormbr_both(m, n, A, lda, tq, tp, U, ldu, VT, ldvt, dws, st)))) return rc;
     }
     return note_cuda(dense_read_err(dws, d_info, st));
 }

@@ -23,6 +23,7 @@ __device__ __forceinline__ unsigned long long gtime() {
 
 // CTAs of the resident kernels at most (their exchange buffers are sized by it)
 constexpr int kResGrid = 160;
+constexpr int kQp = 32;            // columns of a QR panel at most: a lane each
 // scratch doubles of the resident reduction of an m x n matrix (any m >= n
 // that resident_fits() accepts)
 size_t resident_scratch_doubles(int n);

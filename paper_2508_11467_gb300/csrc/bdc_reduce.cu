@@ -926,7 +926,6 @@ __global__ void __launch_bounds__(kLT, 1) k_labrd_panel(Labrd2Args a) {
 }
 
 // -------------------------------------------------------------- QR panel
-constexpr int kQp = 32;            // panel columns: a lane each
 constexpr int kQld = kQp + 1;      // row stride in shared memory
 
 struct Geqr2ResArgs {

@@ -1,6 +1,6 @@
 """Dense calls with more rows than a product's tile list can index (32767 row
-blocks of 128): the trailing update of a reduction and the product Q U_R of a
-tall SVD.
+blocks of 128): the trailing update of a reduction, the rows of C in a
+back-transformation, and the product Q U_R of a tall SVD.
 
 Bounds: sqrt(2 n) 4 ulp a column as for any reduction (n <= 66), on top of the
 norms' own rounding: 1e-13."""
@@ -33,6 +33,19 @@ def test_reduction_of_more_rows_than_tiles():
     bdc.ormbr(0, Ar, tauq, C)
     PT = bdc.ormbr(1, Ar, taup, torch.eye(n, dtype=torch.float64, device="cuda").t())
     assert float((C @ PT - A).norm()) <= 1e-13 * float(A.norm())
+
+
+def test_back_transformation_of_more_rows_than_tiles():
+    from paper_2508_11467_gb300 import bdc
+    n, cdim = 66, ROWS + 300
+    Ar, _, _, _, taup, info = bdc.gebrd(_gauss(n, n, 2))
+    assert info == 0
+    eye = torch.eye(n, dtype=torch.float64, device="cuda")
+    P = bdc.ormbr(1, Ar, taup, eye.clone().t())
+    C = _gauss(cdim, n, 3)
+    X = bdc.ormbr(1, Ar, taup, C.t().clone().t())
+    assert float((X - C @ P).norm()) <= 1e-13 * float(C.norm())
+    assert float((X[ROWS:] - C[ROWS:] @ P).norm()) <= 1e-13 * float(C[ROWS:].norm())
 
 
 def test_svd_of_more_rows_than_tiles():
