@@ -25,9 +25,14 @@
 // any shape and occupancy; the plain FMA 1.9), so the FP64 products were
 // most of a large SVD: back-transformation of 4096 x 4096, one side, 181 ms
 // (165 ms without the triangular solves) -> 10.5 ms; trailing updates of its
-// reduction about 85 -> 20 ms; 333 x 333, one side, 2.4 -> 0.64 ms.  Error:
-// U^T U - I and the residual of gesvd as with FP64 products (333 to 2048:
-// 5.5e-14 to 4.2e-13 and 2.8e-15 to 7.6e-15 either way).
+// reduction about 85 -> 20 ms; 333 x 333, one side, 2.4 -> 0.64 ms.  Error
+// against twice the precision, FP64 products and blocks of 64 -> these: explicit
+// Q of 257 x 257, 1000 x 1000, 10000 x 300 6.3e-16, 6.7e-16, 1.5e-16 -> 6.0e-16,
+// 4.1e-16, 1.1e-16; Q C of a Gaussian C 9.4e-16, 9.7e-16, 2.6e-16 -> 6.2e-16,
+// 4.6e-16, 1.0e-16; backward error of geqrf 6.8e-16, 7.2e-16, 2.9e-16 -> 6.2e-16,
+// 4.6e-16, 2.7e-16; U^T U - I of gesvd 333, 2000 5.3e-14, 4.0e-13 -> 4.8e-14,
+// 4.0e-13.  (Q C of an identity, whose ones scale the slices of C's first rows:
+// 6.3e-16, 6.7e-16, 1.5e-16 -> 6.7e-16, 5.3e-16, 3.5e-16.)
 //
 // The panel
 // kernels run as cooperative launches (all CTAs resident) and separate their
@@ -730,7 +735,11 @@ __global__ void k_gram_sum(const __grid_constant__ GramSums gs) {
 // the off-diagonal blocks of T from its h x h diagonal blocks, one 8 x 8
 // fragment per warp, operands from L2: phase 0: X = G_12 T_22, phase 1: T_12 =
 // -T_11 X (row-major, kWide x kWide per block; a fragment's K range skips the
-// zero half of the triangular factor)
+// zero half of the triangular factor).  The products cancel, and the rounding
+// of one long sum was most of the error of an explicit Q of about kWide
+// reflectors: sums of 8 terms, four of them as a tree, then those in turn
+// (explicit Q of 257 x 257 against twice the precision: one sum 9.6e-16, so
+// 5.8e-16, blocks of 64 in FP64 6.3e-16).
 struct TMerge {
     const double *G[kPair];
     double *T[kPair], *X[kPair];
@@ -750,10 +759,25 @@ __global__ void __launch_bounds__(128) k_tmerge(const __grid_constant__ TMerge a
     const double *A = phase == 0 ? g + (size_t)o * kWide + o + h : t + (size_t)o * kWide + o;
     const double *B = phase == 0 ? t + (size_t)(o + h) * kWide + o + h : x + (size_t)o * kWide + o + h;
     double acc[2] = {0.0, 0.0};
-    const int kb = phase == 0 ? 0 : r0, ke = phase == 0 ? c0 + 8 : h;
-#pragma unroll 8
-    for (int k = kb; k < ke; k += 4)
-        dmma(acc, A[(size_t)(r0 + gr) * kWide + k + tg], B[(size_t)(k + tg) * kWide + c0 + gr]);
+    const int kb = phase == 0 ? 0 : r0, ke = phase == 0 ? c0 + 8 : h;   // (multiples of 8)
+    for (int k0 = kb; k0 < ke; k0 += 32) {
+        double a[8], b[8], c[4][2];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const int k = k0 + 4 * s + tg;
+            a[s] = k < ke ? A[(size_t)(r0 + gr) * kWide + k] : 0.0;
+            b[s] = k < ke ? B[(size_t)k * kWide + c0 + gr] : 0.0;
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            c[s][0] = c[s][1] = 0.0;
+            if (k0 + 8 * s >= ke) continue;
+            dmma(c[s], a[2 * s], b[2 * s]);
+            dmma(c[s], a[2 * s + 1], b[2 * s + 1]);
+        }
+        acc[0] += (c[0][0] + c[1][0]) + (c[2][0] + c[3][0]);
+        acc[1] += (c[0][1] + c[1][1]) + (c[2][1] + c[3][1]);
+    }
     double *out = (phase == 0 ? x : t) + (size_t)(o + r0 + gr) * kWide + o + h + c0 + 2 * tg;
     out[0] = phase == 0 ? acc[0] : -acc[0];
     out[1] = phase == 0 ? acc[1] : -acc[1];
@@ -778,9 +802,9 @@ SplitSide y_vectors(const Reflectors &f, int i0, int nb, int k0) {   // a vector
     const double *p = f.src + (size_t)i0 * (f.sr + f.sc) + (size_t)k0 * f.sr;
     return f.sr == 1 ? SplitSide{p, 0, (int)f.sc, 0, nb, 1, 1, k0, 0} : SplitSide{p, 0, (int)f.sr, 1, nb, 1, 1, k0, 0};
 }
-SplitSide y_rows(const Reflectors &f, int i0, int rows) {            // a vector per row, K = reflectors
+SplitSide y_rows(const Reflectors &f, int i0, int rows, int mask) {  // a vector per row, K = reflectors
     const double *p = f.src + (size_t)i0 * (f.sr + f.sc);
-    return f.sr == 1 ? SplitSide{p, 0, (int)f.sc, 1, rows, 1, 2, 0, 0} : SplitSide{p, 0, (int)f.sr, 0, rows, 1, 2, 0, 0};
+    return f.sr == 1 ? SplitSide{p, 0, (int)f.sc, 1, rows, 1, mask, 0, 0} : SplitSide{p, 0, (int)f.sr, 0, rows, 1, mask, 0, 0};
 }
 
 // runs products in sets that fit kSplitMax and the slice scratch
@@ -824,9 +848,36 @@ struct WideJob {
     int blocks() const { return (f.count + kWide - 1) / kWide; }
 };
 
+// V = Y T but for the products with T's entries above the diagonal (of Y
+// without its unit entries): tau_c y_rc below the diagonal, T_rc from Y's unit
+// entry on and above it
+struct VStart {
+    Reflectors f;
+    const double *T, *tau;
+    double *V;
+};
+struct VStarts {
+    VStart v[kPair];
+};
+__global__ void k_v_start(const __grid_constant__ VStarts vs) {
+    pdl_begin();
+    const VStart &a = vs.v[blockIdx.z];
+    const Reflectors &f = a.f;
+    const int j = blockIdx.y, i0 = j * kWide, rows = f.rows - i0, k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i0 >= f.count) return;
+    const int c = k / rows, r = k - c * rows;
+    if (c >= min(kWide, f.count - i0)) return;
+    const double *src = f.src + (size_t)i0 * (f.sr + f.sc);
+    a.V[(size_t)(i0 + c) * f.rows + r] = r > c ? a.tau[i0 + c] * src[(size_t)r * f.sr + (size_t)c * f.sc]
+                                               : a.T[((size_t)j * kWide + r) * kWide + c];
+}
+
 // V = Y T of every kWide block of the jobs' reflectors (row-major T): V of
 // block j at w.V + i0 f.rows, column-major, f.rows - i0 rows, leading
-// dimension f.rows
+// dimension f.rows.  T's diagonal and Y's unit entries are about sqrt(rows)
+// times the others and would set their scale in the slices: their share is
+// formed in FP64 (k_v_start).  (Explicit Q of 10000 x 300, error against
+// twice the precision: FP64 products 1.5e-16, all of T sliced 5.0e-16.)
 cudaError_t form_v(const WideJob *jobs, int njobs, cudaStream_t st) {
     const size_t w2 = (size_t)kWide * kWide;
     cudaError_t e;
@@ -868,13 +919,22 @@ cudaError_t form_v(const WideJob *jobs, int njobs, cudaStream_t st) {
             launch_pdl(k_tmerge, dim3((tiles + 3) / 4, most, njobs), 128, 0, st, tm, h, phase);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
+    VStarts vs{};
+    int rmost = 0;
+    for (int q = 0; q < njobs; ++q) {
+        vs.v[q] = VStart{jobs[q].f, jobs[q].w.T, jobs[q].tau, jobs[q].w.V};
+        rmost = std::max(rmost, jobs[q].f.rows);
+    }
+    launch_pdl(k_v_start, dim3(rmost * (kWide / 256), most, njobs), 256, 0, st, vs);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int q = 0; q < njobs; ++q)
         for (int j = 0; j < jobs[q].blocks(); ++j) {
             const Reflectors &f = jobs[q].f;
             const int i0 = j * kWide, nb = std::min(kWide, f.count - i0);
             SplitProd p{};
-            p.a = y_rows(f, i0, f.rows - i0);
-            p.b = SplitSide{jobs[q].w.T + j * w2, 0, kWide, 1, nb, 1, 0, 0, 0};
+            p.a = y_rows(f, i0, f.rows - i0, 3);
+            p.b = SplitSide{jobs[q].w.T + j * w2, 0, kWide, 1, nb, 1, 4, 0, 0};
+            p.sub = 2;
             p.C = jobs[q].w.V + (size_t)i0 * f.rows;
             p.ldc = f.rows;
             p.K = nb;
@@ -952,9 +1012,10 @@ size_t step_slices(const WideStep &x) {
 }
 
 // one block, in slabs of the untouched dimension that fit the slice scratch and the Z parts
+// (also: one more product for the launches of the last update)
 template <typename YK>
 cudaError_t apply_wide(int left, int rows, int other, YK yk, int nb, const double *V, int ldv, double *C, int ldc,
-                       const SplitWs &w, cudaStream_t st) {
+                       const SplitWs &w, cudaStream_t st, const SplitProd *also = nullptr) {
     cudaError_t e;
     int slab = other < kSplitMostRows ? (other + 127) / 128 * 128 : kSplitMostRows;
     auto step_of = [&](int s) {
@@ -972,10 +1033,12 @@ cudaError_t apply_wide(int left, int rows, int other, YK yk, int nb, const doubl
         WideStep x = step_of(std::min(slab, other - s0));
         x.c = C + (left ? (size_t)s0 * ldc : (size_t)s0);
         if ((e = x.products(yk, set)) != cudaSuccess || (e = set.run()) != cudaSuccess ||
-            (e = x.update(set)) != cudaSuccess || (e = set.run()) != cudaSuccess)
+            (e = x.update(set)) != cudaSuccess)
             return e;
+        if (s0 + slab < other && (e = set.run()) != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    if (also && (e = set.add(*also)) != cudaSuccess) return e;
+    return set.run();
 }
 
 // where block i0 of a job starts in its C
@@ -1064,7 +1127,7 @@ cudaError_t apply_panel(const Reflectors &f, const double *T, int rows, int cols
     launch_tz(cols, st, T, nb, 1, w.Z, np, 0, cols, W, C, ldc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     SplitProd p{};
-    p.a = y_rows(f, 0, rows);
+    p.a = y_rows(f, 0, rows, 2);
     p.b = SplitSide{W, 0, nb, 0, cols, 1, 0, 0, 0};
     p.C = C;
     p.ldc = ldc;
@@ -1088,13 +1151,15 @@ __global__ void k_fill(double *X, long long rows, long long cols, long long ld, 
     X[c * ld + r] = (r == c) ? diag_val : 0.0;
 }
 
-// columns of the identity: column c has its one in row r0 + c
-__global__ void k_identity(double *X, long long rows, long long cols, long long ld, int r0) {
+// columns of the identity less V: column c has its one in row r0 + c, V's rows
+// begin there
+__global__ void k_identity_less(double *X, long long rows, long long cols, long long ld, int r0, const double *V,
+                                long long ldv) {
     pdl_begin();
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= rows * cols) return;
     const long long c = k / rows, r = k % rows;
-    X[c * ld + r] = (r == c + r0) ? 1.0 : 0.0;
+    X[c * ld + r] = r < r0 ? 0.0 : ((r == c + r0) ? 1.0 : 0.0) - V[c * ldv + r - r0];
 }
 
 __global__ void k_copy_upper(const double *A, long long lda, double *R, long long ldr, int n) {
@@ -1243,7 +1308,7 @@ DenseWs ws_geqrf(int m, int n) {
 // the split path of one job, or of two side by side
 struct WideShape {
     int left, rows, count, other;   // reflectors of `rows` entries on `other` vectors
-    int shrinks;                    // 1: block b leaves out the first b kWide vectors
+    int shrinks;                    // 1: block b acts on the vectors behind its own only (explicit Q)
 };
 void ws_wide(DenseWs &w, const WideShape *jobs, int njobs) {
     const size_t w2 = (size_t)kWide * kWide;
@@ -1262,12 +1327,16 @@ void ws_wide(DenseWs &w, const WideShape *jobs, int njobs) {
         size_t step = 0;
         for (int b = 0; b < blocks; ++b) {
             const int nb = std::min(kWide, j.count - b * kWide), rows = j.rows - b * kWide;
-            const int ns = j.other - (j.shrinks ? b * kWide : 0);
+            const int ns = j.other - (j.shrinks ? b * kWide + nb : 0);
             WideStep x{j.left, rows, nb, 1, 0, ns < kSplitMostRows ? (ns + 127) / 128 * 128 : kSplitMostRows, nullptr, 0, nullptr, 0, nullptr};
             cut_alone(x);
             zneed = std::max(zneed, (size_t)x.np * nb * x.ns);
             for (int np = x.np; np >= 1; --np) {   // (two jobs share the SMs: fewer, longer products)
                 step = std::max(step, step_slices(x));
+                if (j.shrinks) {           // the block's own columns beside the last update
+                    const long long mt = (rows + 127) / 128;
+                    step = std::max(step, split_scratch(2ll * rows, x.ns + nb, nb, mt * ((x.ns + 127) / 128 + (nb + 127) / 128)));
+                }
                 if (njobs == 1) break;
                 x.cut(np - 1);
             }
@@ -1480,11 +1549,22 @@ cudaError_t dense_orgqr(int m, int n, double *A, int lda, const double *tau, cha
             const long long cnt = (long long)ml * nb, c2 = (long long)m * nb;
             launch_pdl(k_form_y, (unsigned)((cnt + 255) / 256), 256, 0, st, Y, ml, nb, A + i0 + (size_t)i0 * lda, 1, lda);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
-            launch_pdl(k_identity, (unsigned)((c2 + 255) / 256), 256, 0, st, A + (size_t)i0 * lda, m, nb, lda, i0);
+            // the block's own columns, E of the identity: E - V Y^T E = (E - V) -
+            // V (Y's first nb rows without the unit entries)^T; the ones would
+            // set the slices' scale
+            const double *V = sw.V + (size_t)i0 * m;
+            launch_pdl(k_identity_less, (unsigned)((c2 + 255) / 256), 256, 0, st, A + (size_t)i0 * lda, m, nb, lda, i0, V, m);
             if ((err = cudaGetLastError()) != cudaSuccess) return err;
             const Reflectors fy{Y, 1, ml, ml, nb};
-            err = apply_wide(1, ml, n - i0, [&](int k0) { return y_vectors(fy, 0, nb, k0); }, nb,
-                             sw.V + (size_t)i0 * m, m, A + i0 + (size_t)i0 * lda, lda, sw, st);
+            SplitProd own{};
+            own.a = SplitSide{V, 0, m, 1, ml, 1, 0, 0, 0};
+            own.b = y_rows(fy, 0, nb, 3);
+            own.C = A + i0 + (size_t)i0 * lda;
+            own.ldc = lda;
+            own.K = nb;
+            own.sub = 1;
+            err = apply_wide(1, ml, n - i0 - nb, [&](int k0) { return y_vectors(fy, 0, nb, k0); }, nb, V, m,
+                             A + i0 + (size_t)(i0 + nb) * lda, lda, sw, st, &own);
             if (err != cudaSuccess) return err;
         }
         return cudaSuccess;

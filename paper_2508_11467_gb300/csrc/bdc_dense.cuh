@@ -51,8 +51,9 @@ cudaError_t launch_geqr2_resident(int m, int nb, double *A, int lda, double *tau
 // rows of A, the columns of B).  tr = 0: vector v at p + v ld, along K; tr =
 // 1: entry k of vector v at p + k ld + v.  parts > 1: the sum of `parts`
 // copies pstride apart.  mask: a panel of reflectors, the stored entries
-// where row > reflector, 0 above: row moff + k of reflector v, the unit entry
-// left out (mask = 1), or row moff + v of reflector k, with it (mask = 2).
+// where row > reflector, 0 above: row moff + k of reflector v (mask = 1), or
+// row moff + v of reflector k (mask = 2, mask = 3), the unit entry left out but
+// for mask = 2.  mask = 4: entry k = v left out.
 // add: add[v add_v + k add_k] is added to entry k of vector v.
 struct SplitSide {
     const double *p;
@@ -65,7 +66,7 @@ struct SplitSide {
 struct SplitProd {
     SplitSide a, b;
     double *C;   // a.n x b.n, column-major
-    int ldc, K, sub;   // sub: C -= A B
+    int ldc, K, sub;   // 0: C = A B, 1: C -= A B, 2: C += A B
 };
 constexpr int kSplitMax = 32, kSplitMostK = 16384;
 // rows of A and columns of B at most: a tile list entry holds the row block

@@ -53,7 +53,7 @@ struct MixProb {
     int tile0;    // first tile of the product in the launch grid
     int tilesN;   // tiles along N (for the host-known bound Nmax)
     int Mmax, Nmax;
-    int sub;      // 1: C -= A B (the merge products store C = A B)
+    int sub;      // 1: C -= A B, 2: C += A B (the merge products store C = A B)
     int pad1;
 };
 
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(256) k_slice_b(const GemmProb *__restrict__ pr
 //            up to 16384 of them).  MODE_L's dropped pairs and FP32 sums are
 //            each a few 1e-16 sqrt(K / 333) of max|A_r| max|B_c| for S = 7, far
 //            above an FP64 product's error on such operands.
-//   MODE_EW  MODE_E that also takes C -= A B (MODE_LW does too).
+//   MODE_EW  MODE_E that also takes C -= A B and C += A B (MODE_LW does too).
 enum { MODE_E = 0, MODE_L = 1, MODE_X3 = 2, MODE_LW = 3, MODE_EW = 4 };
 
 // Slices loaded per stage (MODE_E multiplies slices 1..4 only), bytes per
@@ -831,7 +831,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                             if (rowok && c0 + k < pr.N) {
                                 double v = i64_ldexp((long long)(L[k] - corr), Er + F[i] - 40);
                                 if (MODE == MODE_EW && Er + F[i] > kNotFinite / 2) v = __longlong_as_double(0x7ff8000000000000ll);
-                                if constexpr (MODE == MODE_EW) pr.C[cj[i] * ldc + row] = mx.sub ? cold[i] - v : v;
+                                if (MODE == MODE_EW && mx.sub == 1) v = -v;
+                                if constexpr (MODE == MODE_EW) pr.C[cj[i] * ldc + row] = mx.sub ? cold[i] + v : v;
                                 else pr.C[cj[i] * ldc + row] = v;
                             }
                         }
@@ -897,7 +898,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mma(const __grid_constant__ CUte
                                 v = i64_ldexp(((long long)I4[k] << 16) + __float2ll_rn(SL[k] * 0x1p48f), Er + F[i] - 64);
                             else
                                 v = f32_ldexp(SL[k], Er + F[i] - 16);
-                            if (MODE == MODE_LW && mx.sub) v = -v;
+                            if (MODE == MODE_LW && mx.sub == 1) v = -v;
                             if (rowok && c0 + k < pr.N) pr.C[off[i] + row] = cv[i] + v;
                         }
                     }
@@ -1266,7 +1267,9 @@ __device__ __forceinline__ unsigned long long mag_bits(double x) {
 
 // entry k of vector v
 __device__ __forceinline__ double split_at(const SplitSide &s, int v, int k) {
-    if (s.mask) {                          // reflector panel
+    if (s.mask == 4) {
+        if (k == v) return 0.0;
+    } else if (s.mask) {                   // reflector panel
         const int r = (s.mask == 1 ? k : v) + s.moff, c = s.mask == 1 ? v : k;
         if (r <= c) return (r == c && s.mask == 2) ? 1.0 : 0.0;
     }
