@@ -406,10 +406,12 @@ int bdc_mlp_train(const bdc_opts *o, const bdc_mlp_train_opts *t, float *params,
  * call is asynchronous on `stream` unless stated; workspaces are device
  * memory of the size the matching *_workspace function returns (any
  * alignment): 2 KB a row and column for a reduction; for block reflectors
- * (ormbr, geqrf / orgqr, gesvd) 10 KB a row and vector where they run in FP64
- * (fewer than 64 reflectors or vectors, more than 131072 rows), else the
- * reflectors once more and the slices of one product (14 bytes an entry of
- * its operands; 14 bytes an entry of the trailing matrix for geqrf).
+ * (ormbr, geqrf / orgqr, gesvd) 0.5 KB a row and up to 9 KB a vector where
+ * they run in FP64 (fewer than 64 reflectors or vectors, more than 131072
+ * rows), else the reflectors once more and the slices of one product (14 bytes
+ * an entry of its operands; 14 bytes an entry of the trailing matrix for
+ * geqrf).  A workspace for some sizes serves every smaller one (gesvd: with
+ * fewer rows).
  * Reflectors use LAPACK's sign convention and storage: a reflector I - tau y
  * y^T maps x to beta e_1 with beta = -sign(x_1) ||x|| (a zero x_1 counts as
  * positive), y_1 = 1 implicit.  Panels are b = 32 columns (rows) wide.  The panel

@@ -1199,6 +1199,7 @@ constexpr int kDenseBlock = 32;   // b: columns / rows per panel (reflectors per
 constexpr int kApplyBlock = kTB;
 static_assert(kDenseBlock <= 32 && kDenseBlock <= kTB, "k_geqr2: a lane per later panel column; T of a panel");
 
+constexpr double kQrRatio = 1.6;  // m >= 1.6 n: QR first (Sec. 4.3)
 constexpr int kPairMost = 2048;   // largest dimension of back-transformations done side by side
 
 // Blocks of kWide reflectors on the split products, or of kTB in FP64: the
@@ -1209,7 +1210,10 @@ bool use_wide(int refl, int rows, int other) {
     return refl >= 64 && other >= 64 && rows <= 8 * kSplitMostK;   // (gram_chunk)
 }
 // ---- workspaces: every routine lays out what it can reach at its shape
-// (bytes from an aligned base; the barrier and error word come first in all)
+// (bytes from an aligned base; the barrier and error word come first in all).
+// A workspace asked for with some sizes serves all smaller ones: the sizes
+// here are bounds that grow with every dimension (the cuts along K do not),
+// and the *_bytes functions take in what smaller shapes run instead.
 struct DenseWs {
     size_t bar = 0, total = 256;
     size_t PW = 0, QW = 0, lab = 0, res = 0;                             // reduction
@@ -1222,14 +1226,19 @@ struct DenseWs {
         return at;
     }
     size_t doubles(size_t n) { return add(sizeof(double) * n); }
-    // partial products and sums of the FP64 block reflectors: 16 parts of kTB
-    // vectors of `len` (bound by the FP64 pipe: no more are of use)
+    // block reflectors in FP64: copied reflectors, T, sums, and the partial
+    // products that dgemm_parts may use (one per 64 of K, 64 at most; 16 of as
+    // many columns as the longest dimension; one where the tiles alone fill the
+    // chip 33 times over) or k_gram's
     void fp64(size_t rows, size_t refl, size_t other) {
+        constexpr size_t kManyTiles = 340000;
         const size_t len = std::max({rows, refl, other});
         Y = doubles(rows * kTB);
         Ti = doubles((size_t)kTB * (refl + kTB));
         Z = doubles((size_t)kTB * other);
-        split_doubles = std::max<size_t>((size_t)16 * kTB * len, (size_t)16 * kTB * kTB);
+        const size_t parts = std::max<size_t>(1, std::min<size_t>(64, rows / 64));
+        split_doubles = std::max({kTB * other, std::min(parts * kTB * std::min(other, kManyTiles), 16 * kTB * len),
+                                  (size_t)kTB * kTB * std::max<size_t>(16, std::min(len / 4 + 16, (size_t)4 * sm_count_dense()))});
         split = doubles(split_doubles);
     }
     void slices(size_t bytes) {
@@ -1247,6 +1256,21 @@ size_t slice_cap(size_t len) {
            ((size_t)1 << 20);
 }
 
+// Bounds over every cut of `rows` along K into products of nb reflectors on up
+// to ns vectors (np kc < rows + 32 np; np a wave's worth of the 152 / tiles, or
+// what the length of a product asks for): doubles of the partial results, and
+// slices of the products' operands.
+int cuts_most(int rows) { return std::max((rows + kSplitMostK - 33) / (kSplitMostK - 32), std::min(kSplitMax, std::max(1, rows / 256))); }
+size_t cut_doubles(int rows, int nb, int ns) {
+    const size_t one = (size_t)nb * ns, least = (rows + kSplitMostK - 33) / (kSplitMostK - 32);
+    return std::max(least * one, std::min(cuts_most(rows) * one, (size_t)152 * 128 * 128));
+}
+size_t cut_slices(int rows, int nb, int ns) {
+    const size_t np = cuts_most(rows), len = rows + 32 * np, v = (size_t)nb + ns;
+    return 14 * (v * len + 256 * (size_t)std::min((rows + 31) / 32 * 32 + 32, kSplitMostK)) + 24 * np * (v + 256) +
+           8 * (np * 2 * ((ns + 127) / 128 + 1) + 152) + 65536;
+}
+
 DenseWs ws_gebrd(int m, int n) {
     DenseWs w;
     constexpr int b = kDenseBlock;
@@ -1254,8 +1278,8 @@ DenseWs ws_gebrd(int m, int n) {
     w.QW = w.doubles(2 * (size_t)b * n);
     w.lab = w.doubles(labrd_scratch_doubles(m, n));
     w.res = w.doubles(resident_scratch_doubles(n));
-    const long long tr = m - b, tc = n - b;
-    if (tc > 0 && tr <= kSplitMostRows) w.slices(split_scratch(2 * tr, 2 * tc, b, ((tr + 127) / 128) * ((tc + 127) / 128)));
+    const long long tr = std::min(m - b, kSplitMostRows), tc = std::min<long long>(n - b, tr);
+    if (tc > 0) w.slices(split_scratch(2 * tr, 2 * tc, b, ((tr + 127) / 128) * ((tc + 127) / 128)));
     return w;
 }
 
@@ -1282,77 +1306,71 @@ DenseWs ws_geqrf(int m, int n) {
     w.res = w.doubles(resident_scratch_doubles(kQp));
     w.Ti = w.doubles((size_t)2 * kTB * kTB);         // T, Y^T Y of a panel
     w.Z = w.doubles((size_t)b * n);
-    size_t y = 0, parts = 0, slices = 0;
-    for (int i0 = 0; i0 < std::min(m, n); i0 += b) {
-        const int ml = m - i0, nb = std::min(b, std::min(m, n) - i0), cols = n - i0 - nb;
-        if (cols == 0) break;
-        // Y^T Y of a panel that is too long for the chip: up to four CTAs an SM
-        parts = std::max(parts, (size_t)kTB * kTB * std::min((ml + 255) / 256, 4 * sm_count_dense()));
-        if (panel_split(ml, cols, len)) {
-            const PanelCut c = panel_cut(ml, cols);
-            slices = std::max(slices, panel_slices(ml, cols, c));
-            w.wZcap = std::max(w.wZcap, (size_t)c.np * nb * cols);
-        } else {
-            y = std::max(y, (size_t)ml * nb);
-            parts = std::max(parts, (size_t)nb * cols * std::max(1, std::min(64, ml / 64)));
-        }
-    }
-    w.Y = w.doubles(y);
-    w.split_doubles = std::max((size_t)16 * kTB * kTB, parts);
+    w.Y = w.doubles((size_t)b * m);
+    // The largest update that panel_split may take (its columns: at most half
+    // the longer side and 128, or 1024; a wide matrix has no fewer than n - m
+    // left); one in FP64 is small or larger than that.
+    const int rows = std::min(m, kSplitMax * (kSplitMostK - 64));
+    const long long side = std::max<long long>(m, std::min<long long>(n, 2ll * m + 256));
+    const int cols = (int)std::min<long long>({std::max(n - 1, 0), std::max((side + 256) / 2, 1024ll), kSplitMostRows});
+    const long long tiles = (long long)((rows + 127) / 128) * ((cols + 127) / 128);
+    const size_t need = std::max(cut_slices(rows, 32, cols), split_scratch(rows, cols, 32, tiles));
+    const bool large = m > rows || n - 1 > cols || need > slice_cap(len);
+    // Y^T Y of a panel that is too long for the chip: up to four CTAs an SM
+    const size_t gram = (size_t)kTB * kTB * std::max(16, std::min((m + 255) / 256, 4 * sm_count_dense()));
+    // partial products as in DenseWs::fp64
+    const size_t parts = large ? std::max(1, std::min(64, m / 64)) : 1;
+    w.split_doubles = std::max({gram, std::min((size_t)b * n * parts, 16 * b * len), (size_t)b * n, (size_t)52000});
     w.split = w.doubles(w.split_doubles);
-    w.wZ[0] = w.doubles(w.wZcap);
-    w.slices(slices);
+    if ((long long)rows * cols >= 100 * 1000) {
+        w.wZcap = cut_doubles(rows, 32, cols);
+        w.wZ[0] = w.doubles(w.wZcap);
+        w.slices(std::min(need, slice_cap(len)));
+    }
     return w;
 }
 
 // the split path of one job, or of two side by side
 struct WideShape {
     int left, rows, count, other;   // reflectors of `rows` entries on `other` vectors
-    int shrinks;                    // 1: block b acts on the vectors behind its own only (explicit Q)
+    int own;                        // 1: with a product on a block's own columns beside each update (explicit Q)
 };
 void ws_wide(DenseWs &w, const WideShape *jobs, int njobs) {
     const size_t w2 = (size_t)kWide * kWide;
-    size_t need = 0, cap = 0, zneed = 0, zmost = 0;
+    size_t need = 0, cap = 0;
     long long gram = 0, vrows = 0, vcols = 0, vtiles = 0;
     int chunk = 0;
+    w.wZcap = 0;
     for (int q = 0; q < njobs; ++q) {
         const WideShape &j = jobs[q];
-        const int blocks = (j.count + kWide - 1) / kWide;
+        const int blocks = (j.count + kWide - 1) / kWide, nb = std::min(j.count, kWide);
+        const int ns = j.other < kSplitMostRows ? (j.other + 127) / 128 * 128 : kSplitMostRows;
+        const int parts = std::min((j.rows + 511) / 512, 8);       // gram_chunks() at most
         w.wG[q] = w.doubles(blocks * w2);
         w.wT[q] = w.doubles(blocks * w2);
         w.wX[q] = w.doubles(blocks * w2);
-        w.wV[q] = w.doubles(std::max((size_t)j.rows * j.count, (size_t)blocks * gram_chunks(j.rows) * w2));   // V, before it Y^T Y's parts
-        gram += (long long)blocks * gram_chunks(j.rows);
+        w.wV[q] = w.doubles(std::max((size_t)j.rows * j.count, (size_t)blocks * parts * w2));   // V, before it Y^T Y's parts
+        gram += (long long)blocks * parts;
         chunk = std::max(chunk, gram_chunk(j.rows));
-        size_t step = 0;
         for (int b = 0; b < blocks; ++b) {
-            const int nb = std::min(kWide, j.count - b * kWide), rows = j.rows - b * kWide;
-            const int ns = j.other - (j.shrinks ? b * kWide + nb : 0);
-            WideStep x{j.left, rows, nb, 1, 0, ns < kSplitMostRows ? (ns + 127) / 128 * 128 : kSplitMostRows, nullptr, 0, nullptr, 0, nullptr};
-            cut_alone(x);
-            zneed = std::max(zneed, (size_t)x.np * nb * x.ns);
-            for (int np = x.np; np >= 1; --np) {   // (two jobs share the SMs: fewer, longer products)
-                step = std::max(step, step_slices(x));
-                if (j.shrinks) {           // the block's own columns beside the last update
-                    const long long mt = (rows + 127) / 128;
-                    step = std::max(step, split_scratch(2ll * rows, x.ns + nb, nb, mt * ((x.ns + 127) / 128 + (nb + 127) / 128)));
-                }
-                if (njobs == 1) break;
-                x.cut(np - 1);
-            }
+            const int rows = j.rows - b * kWide, c = std::min(kWide, j.count - b * kWide);
             vrows += rows;
-            vcols += nb;
-            vtiles += (long long)((rows + 127) / 128) * ((nb + 127) / 128);
+            vcols += c;
+            vtiles += (long long)((rows + 127) / 128) * ((c + 127) / 128);
         }
-        need += step;
+        // products Y^T C and the update, whole
+        const long long mt = (j.rows + 127) / 128, nt = (ns + 127) / 128 + (j.own ? (nb + 127) / 128 : 0);
+        need += std::max({cut_slices(j.rows, nb, ns), split_scratch((j.own ? 2ll : 1ll) * j.rows, ns + (j.own ? nb : 0), nb, mt * nt),
+                          split_scratch(ns, j.rows, nb, mt * nt)});
         const size_t len = std::max(j.rows, std::min(j.other, 1 << 16));
         cap = std::max(cap, slice_cap(len));
-        zmost = std::max<size_t>({zmost, (size_t)2 * kWide * (len + 256), (size_t)kWide * 4096});
+        // (the second bound: slabs of the vectors)
+        w.wZcap = std::max(w.wZcap, std::min(cut_doubles(j.rows, nb, ns),
+                                             std::max<size_t>((size_t)2 * kWide * (len + 256), (size_t)kWide * 4096)));
     }
     gram = std::min<long long>(gram, kSplitMax);
     need = std::max({need, split_scratch(gram * kWide, gram * kWide, chunk, gram * (kWide / 128) * (kWide / 128)),
                      split_scratch(vrows, vcols, kWide, vtiles)});
-    w.wZcap = need <= cap && zneed <= zmost ? zneed : zmost;   // whole steps, or slabs of them
     for (int q = 0; q < njobs; ++q) w.wZ[q] = w.doubles(w.wZcap);
     w.slices(std::min(need, cap));
 }
@@ -1398,6 +1416,29 @@ DenseWs ws_product(int m, int n) {
         w.slices(std::min(slice_cap(std::min(m, 1 << 17)),
                           split_scratch(rows, n, n, (long long)((rows + 127) / 128) * ((n + 127) / 128))));
     return w;
+}
+
+// `refl` reflectors of `rows` entries on `other` vectors, and on fewer of each
+size_t apply_bytes(int left, int rows, int refl, int other, int own) {
+    constexpr int kLongest = 8 * kSplitMostK;
+    const bool many = refl >= 64 && other >= 64;
+    DenseWs w;
+    w.fp64(rows, std::max(refl, 0), other);
+    size_t most = w.total;
+    if (many) {
+        if (rows <= kLongest) {   // fewer than 64 of one
+            DenseWs a, b;
+            a.fp64(rows, 63, other);
+            b.fp64(rows, refl, 63);
+            most = std::max(a.total, b.total);
+        }
+        DenseWs c;
+        const WideShape j{left, std::min(rows, kLongest), std::min(refl, kLongest), other, own};
+        if (own) c.Y = c.doubles((size_t)j.rows * kWide);
+        ws_wide(c, &j, 1);
+        most = std::max(most, c.total);
+    }
+    return most;
 }
 
 SplitWs split_ws(char *ws, const DenseWs &w, int job = 0) {
@@ -1649,14 +1690,16 @@ cudaError_t dense_ormbr_both(int m, int n, const double *A, int lda, const doubl
 }
 
 size_t gebrd_bytes(int m, int n) { return ws_gebrd(m, n).total; }
-size_t geqrf_bytes(int m, int n) { return std::max(ws_geqrf(m, n).total, n <= m ? ws_orgqr(m, n).total : 0); }
+size_t geqrf_bytes(int m, int n) { return std::max(ws_geqrf(m, n).total, apply_bytes(1, m, std::min(m, n), std::min(m, n), 1)); }
 size_t ormbr_bytes(int m, int n, int cdim) {
-    return std::max(ws_ormbr(0, m, n, cdim).total, ws_ormbr(1, m, n, cdim).total);
+    return std::max(apply_bytes(1, m, n, cdim, 0), apply_bytes(0, n - 1, n - 1, cdim, 0));
 }
-size_t gesvd_bytes(int m, int n, bool qr) {
-    const int r = qr ? n : m;   // rows of the reduction
-    const size_t reduce = std::max(gebrd_bytes(r, n), both_at_once(r, n) ? ws_both(r, n).total : ormbr_bytes(r, n, n));
-    return qr ? std::max({reduce, geqrf_bytes(m, n), ws_product(m, n).total}) : reduce;
+size_t gesvd_bytes(int m, int n) {
+    size_t most = std::max(gebrd_bytes(m, n), ormbr_bytes(m, n, n));
+    const int mp = std::min(m, kPairMost), np = std::min(n, kPairMost), nq = std::min(n, (int)(m / kQrRatio));
+    if (both_at_once(mp, np)) most = std::max(most, ws_both(mp, np).total);
+    if (nq > 0) most = std::max({most, geqrf_bytes(m, nq), ws_product(m, std::min(nq, kSplitMostK)).total});
+    return most;
 }
 // (a kernel, not a memset: overlapped launches may follow it directly)
 cudaError_t dense_clear_err(char *ws, cudaStream_t st) {
@@ -1713,8 +1756,6 @@ using namespace bdc;
 
 namespace {
 
-constexpr double kQrRatio = 1.6;  // m >= 1.6 n: QR first (Sec. 4.3)
-
 char *align_ws(void *work) { return (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255); }
 
 int note_cuda(cudaError_t e) { return e == cudaSuccess ? 0 : BDC_ERR_CUDA; }
@@ -1726,7 +1767,7 @@ GesvdWs gesvd_layout(int m, int n, const bdc_opts *o) {
     GesvdWs w{};
     size_t off = 0;
     const bool qr = m >= kQrRatio * n;
-    w.dense = off; off += al256(gesvd_bytes(m, n, qr));
+    w.dense = off; off += al256(gesvd_bytes(m, n));
     w.vecs = off; off += al256(sizeof(double) * 4 * (size_t)n + 64);
     w.R = off; off += qr ? al256(sizeof(double) * (size_t)n * n) : 0;
     w.UR = off; off += qr ? al256(sizeof(double) * (size_t)n * n) : 0;
