@@ -25,7 +25,7 @@
 // any shape and occupancy; the plain FMA 1.9), so the FP64 products were
 // most of a large SVD: back-transformation of 4096 x 4096, one side, 181 ms
 // (165 ms without the triangular solves) -> 10.5 ms; trailing updates of its
-// reduction about 85 -> 20 ms; 333 x 333, one side, 2.4 -> 0.64 ms.  Error
+// reduction about 85 -> 25 ms; 333 x 333, one side, 2.4 -> 0.64 ms.  Error
 // against twice the precision, FP64 products and blocks of 64 -> these: explicit
 // Q of 257 x 257, 1000 x 1000, 10000 x 300 6.3e-16, 6.7e-16, 1.5e-16 -> 6.0e-16,
 // 4.1e-16, 1.1e-16; Q C of a Gaussian C 9.4e-16, 9.7e-16, 2.6e-16 -> 6.2e-16,
